@@ -10,6 +10,7 @@
 #include <utility>
 
 #include "pkv_common.cuh"
+#include "pkv_decode.cuh"
 #include "pkv_extras.cuh"
 #include "pkv_gather.cuh"
 #include "pkv_score_generic.cuh"
@@ -756,6 +757,76 @@ bool paged_args_ok(const int32_t* block_table, int page_size, int num_pages, con
   return reinterpret_cast<uintptr_t>(k_pool) % 16 == 0 && reinterpret_cast<uintptr_t>(v_pool) % 16 == 0;
 }
 
+// CTAs of a decode cluster: doubled while the doubled grid still finds a place on the device at once (two CTAs to an
+// SM) and every CTA keeps a step's worth of rows.
+int decode_cluster(long long units, int max_count, int sms) {
+  int cluster = 1;
+  while (cluster < kDecMaxCluster && units * cluster * 2 <= 2ll * sms && max_count >= 2 * cluster * kDecMinRows) cluster *= 2;
+  return cluster;
+}
+
+// ---------------------------------------------------------------- decode attention
+template <typename T, int D, int GT, bool PAGED>
+int launch_decode(DecodeParams& dp, int batch, int max_count, cudaStream_t st) {
+  const int sms = device_sm_count();
+  if (sms <= 0) return PKV_ERR_CUDA;
+  auto kernel = decode_attention_kernel<T, D, GT, PAGED>;
+  static bool attr_done[64] = {};                  // clusters of 16 CTAs are an opt-in of the kernel, per device
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return PKV_ERR_CUDA;
+  if (dev >= 64 || !attr_done[dev]) {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return PKV_ERR_CUDA;
+    if (dev < 64) attr_done[dev] = true;
+  }
+  dp.head_blocks = (dp.group + GT - 1) / GT;
+  const long long units = static_cast<long long>(dp.num_kv_heads) * dp.head_blocks * batch;
+  const int cluster = decode_cluster(units, max_count, sms);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(cluster * dp.num_kv_heads * dp.head_blocks, batch);
+  cfg.blockDim = dim3(kDecThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  if (cudaLaunchKernelEx(&cfg, kernel, static_cast<const DecodeParams&>(dp)) != cudaSuccess) return PKV_ERR_CUDA;
+  return check_launch();
+}
+
+template <typename T, int D, bool PAGED>
+int launch_decode_group(DecodeParams& dp, int batch, int max_count, cudaStream_t st) {
+  if (dp.group == 1) return launch_decode<T, D, 1, PAGED>(dp, batch, max_count, st);
+  if (dp.group == 2) return launch_decode<T, D, 2, PAGED>(dp, batch, max_count, st);
+  if (dp.group <= 4) return launch_decode<T, D, 4, PAGED>(dp, batch, max_count, st);
+  return launch_decode<T, D, 8, PAGED>(dp, batch, max_count, st);
+}
+
+template <bool PAGED>
+int run_decode(const pkv_config* c, DecodeParams& dp, int batch, cudaStream_t st) {
+  dp.num_kv_heads = c->num_kv_heads;
+  dp.group = c->num_q_heads / c->num_kv_heads;
+  dp.scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(c->head_dim)));
+  int max_count = 0;
+  for (int b = 0; b < batch; ++b) max_count = std::max(max_count, dp.seq.count[b]);
+  const bool wide = c->head_dim == 128;
+  switch (c->dtype) {
+    case PKV_DTYPE_FP32:
+      return wide ? launch_decode_group<float, 128, PAGED>(dp, batch, max_count, st)
+                  : launch_decode_group<float, 64, PAGED>(dp, batch, max_count, st);
+    case PKV_DTYPE_FP16:
+      return wide ? launch_decode_group<__half, 128, PAGED>(dp, batch, max_count, st)
+                  : launch_decode_group<__half, 64, PAGED>(dp, batch, max_count, st);
+    default:
+      return wide ? launch_decode_group<__nv_bfloat16, 128, PAGED>(dp, batch, max_count, st)
+                  : launch_decode_group<__nv_bfloat16, 64, PAGED>(dp, batch, max_count, st);
+  }
+}
+
 // Table of a call on one shard of each sequence: n = keys held here, prefix = those that are scored.
 int build_shard_table(const pkv_config* c, const int32_t* shard_keys, const int32_t* window_keys, int batch,
                       SeqTable* t, int* max_n) {
@@ -1090,22 +1161,7 @@ int pyramidkv_decode_attention(const pkv_config* cfg, const void* q, const void*
   dp.v_cache = v_cache;
   dp.out = out;
   dp.seq = table;
-  dp.num_kv_heads = cfg->num_kv_heads;
-  dp.group = cfg->num_q_heads / cfg->num_kv_heads;
-  dp.scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(cfg->head_dim)));
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const dim3 grid(cfg->num_q_heads, batch);
-  if (cfg->dtype == PKV_DTYPE_FP32) {
-    if (cfg->head_dim == 64) launch_pdl(decode_attention_kernel<float, 64>, grid, kDecThreads, 0, st, dp);
-    else launch_pdl(decode_attention_kernel<float, 128>, grid, kDecThreads, 0, st, dp);
-  } else if (cfg->dtype == PKV_DTYPE_FP16) {
-    if (cfg->head_dim == 64) launch_pdl(decode_attention_kernel<__half, 64>, grid, kDecThreads, 0, st, dp);
-    else launch_pdl(decode_attention_kernel<__half, 128>, grid, kDecThreads, 0, st, dp);
-  } else {
-    if (cfg->head_dim == 64) launch_pdl(decode_attention_kernel<__nv_bfloat16, 64>, grid, kDecThreads, 0, st, dp);
-    else launch_pdl(decode_attention_kernel<__nv_bfloat16, 128>, grid, kDecThreads, 0, st, dp);
-  }
-  return check_launch();
+  return run_decode<false>(cfg, dp, batch, static_cast<cudaStream_t>(stream));
 }
 
 int pyramidkv_attention_recall(const pkv_config* cfg, const float* scores, int64_t ld_scores, const int32_t* indices,
@@ -1210,23 +1266,7 @@ int pyramidkv_decode_attention_paged(const pkv_config* cfg, const void* q, const
   dp.seq = table;
   fill_page_table(cfg, table, block_table, page_size, num_pages, &dp.pt);
   dp.status = static_cast<uint32_t*>(workspace);
-  dp.num_kv_heads = cfg->num_kv_heads;
-  dp.group = cfg->num_q_heads / cfg->num_kv_heads;
-  dp.scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(cfg->head_dim)));
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const dim3 grid(cfg->num_q_heads, batch);
-  const bool wide = cfg->head_dim == 128;
-  if (cfg->dtype == PKV_DTYPE_FP32) {
-    if (wide) launch_pdl(decode_attention_kernel<float, 128, true>, grid, kDecThreads, 0, st, dp);
-    else launch_pdl(decode_attention_kernel<float, 64, true>, grid, kDecThreads, 0, st, dp);
-  } else if (cfg->dtype == PKV_DTYPE_FP16) {
-    if (wide) launch_pdl(decode_attention_kernel<__half, 128, true>, grid, kDecThreads, 0, st, dp);
-    else launch_pdl(decode_attention_kernel<__half, 64, true>, grid, kDecThreads, 0, st, dp);
-  } else {
-    if (wide) launch_pdl(decode_attention_kernel<__nv_bfloat16, 128, true>, grid, kDecThreads, 0, st, dp);
-    else launch_pdl(decode_attention_kernel<__nv_bfloat16, 64, true>, grid, kDecThreads, 0, st, dp);
-  }
-  return check_launch();
+  return run_decode<true>(cfg, dp, batch, static_cast<cudaStream_t>(stream));
 }
 
 int pyramidkv_shard_window_lse(const pkv_config* cfg, pkv_tensor q_win, pkv_tensor k_shard,
