@@ -1,4 +1,8 @@
-"""ctypes binding of libpyramidkv.so: same names as the C boundary, argument marshalling only.
+"""Binding of libpyramidkv.so: same names as the C boundary, argument marshalling only.
+
+The calls that a prefill or a decode step makes once per layer go through the native
+module (native/pkv_bind.cpp), which checks and marshals in about a microsecond; what it
+does not take (and all other calls) goes through the checks below and ctypes.
 
 Every step of the path runs in the library's CUDA kernels.  torch supplies device
 memory and the stream, nothing else.  There is no CPU fallback: the library is
@@ -11,7 +15,8 @@ configuration and the sequence lengths say, of the configured type, and on a dev
 from __future__ import annotations
 
 import ctypes
-import os
+import importlib.machinery
+import importlib.util
 from typing import List, Optional, Sequence
 
 import torch
@@ -128,6 +133,28 @@ class _LazyLibrary:
 
 
 _lib = _LazyLibrary()
+
+
+class _LazyNative:
+    """The functions of _pkv_native.so, loaded on first use (after libpyramidkv.so, which it is linked against) and
+    kept as attributes."""
+
+    def __getattr__(self, name):
+        if name.startswith("__"):
+            raise AttributeError(name)
+        _lib.pyramidkv_strerror                     # loads libpyramidkv.so
+        path = _build.build_binding()
+        spec = importlib.util.spec_from_loader("_pkv_native", importlib.machinery.ExtensionFileLoader("_pkv_native", path))
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        for f in dir(module):
+            if not f.startswith("__"):
+                setattr(self, f, getattr(module, f))
+        return self.__dict__[name]
+
+
+_native = _LazyNative()
+_NOT_TAKEN = -1        # the native call left the arguments to the checks here; nothing was enqueued
 
 
 def library_path() -> str:
@@ -328,6 +355,10 @@ def score_window(cfg: PkvConfig, q_win: torch.Tensor, k: torch.Tensor, seq_lens:
                  scores: torch.Tensor, workspace: torch.Tensor, stream=None,
                  window_lse: Optional[torch.Tensor] = None) -> None:
     """window_lse given: the prefill's natural-log row normalisers are used and one K sweep is skipped."""
+    st = _native.score_window(cfg, q_win, k, seq_lens, scores, workspace, stream, window_lse)
+    if st != _NOT_TAKEN:
+        _check(st, "pyramidkv_score_window" + ("" if window_lse is None else "_lse"))
+        return
     lens, batch = _lens(seq_lens)
     _check_q(cfg, q_win, batch)
     _check_kv(cfg, k, "k", batch, max(seq_lens))
@@ -393,6 +424,10 @@ def check_status_static(stream=None) -> int:
 
 def select_topk(cfg: PkvConfig, scores: torch.Tensor, seq_lens: Sequence[int], k_layer: int,
                 indices: torch.Tensor, workspace: torch.Tensor, stream=None) -> None:
+    st = _native.select_topk(cfg, scores, seq_lens, k_layer, indices, workspace, stream)
+    if st != _NOT_TAKEN:
+        _check(st, "pyramidkv_select_topk")
+        return
     lens, batch = _lens(seq_lens)
     _check_scores(cfg, scores, batch, max(seq_lens) - cfg.window)
     _check_rows(cfg, total_rows(cfg, k_layer, seq_lens), None, None, indices)
@@ -405,6 +440,10 @@ def select_topk(cfg: PkvConfig, scores: torch.Tensor, seq_lens: Sequence[int], k
 def gather_compact(cfg: PkvConfig, k: torch.Tensor, v: Optional[torch.Tensor], indices: torch.Tensor,
                    seq_lens: Sequence[int], k_layer: int, k_out: torch.Tensor, v_out: Optional[torch.Tensor],
                    stream=None) -> None:
+    st = _native.gather_compact(cfg, k, v, indices, seq_lens, k_layer, k_out, v_out, stream)
+    if st != _NOT_TAKEN:
+        _check(st, "pyramidkv_gather_compact")
+        return
     lens, batch = _lens(seq_lens)
     _check_kv(cfg, k, "k", batch, max(seq_lens))
     if v is not None:
@@ -420,6 +459,10 @@ def compress_layer(cfg: PkvConfig, layer: int, q_win: torch.Tensor, k: torch.Ten
                    seq_lens: Sequence[int], k_out: torch.Tensor, v_out: torch.Tensor, indices: torch.Tensor,
                    workspace: torch.Tensor, scores: Optional[torch.Tensor] = None, stream=None,
                    window_lse: Optional[torch.Tensor] = None) -> None:
+    st = _native.compress_layer(cfg, layer, q_win, k, v, seq_lens, k_out, v_out, indices, workspace, scores, stream, window_lse)
+    if st != _NOT_TAKEN:
+        _check(st, "pyramidkv_compress_layer" + ("" if window_lse is None else "_lse"))
+        return
     lens, batch = _lens(seq_lens)
     _check_layer_call(cfg, layer, q_win, k, v, seq_lens, k_out, v_out, indices, workspace, scores)
     if window_lse is not None:
@@ -464,6 +507,10 @@ def attend_compress_layer(cfg: PkvConfig, layer: int, q_win: torch.Tensor, k: to
                           indices: torch.Tensor, workspace: torch.Tensor, scores: Optional[torch.Tensor] = None,
                           stream=None) -> None:
     """compress_layer that also returns the window rows' attention output."""
+    st = _native.attend_compress_layer(cfg, layer, q_win, k, v, seq_lens, attn_out, k_out, v_out, indices, workspace, scores, stream)
+    if st != _NOT_TAKEN:
+        _check(st, "pyramidkv_attend_compress_layer")
+        return
     lens, batch = _lens(seq_lens)
     _check_layer_call(cfg, layer, q_win, k, v, seq_lens, k_out, v_out, indices, workspace, scores)
     _check_attn_out(cfg, attn_out, batch)
@@ -508,6 +555,10 @@ def profile_layer(cfg: PkvConfig, layer: int, q_win: torch.Tensor, k: torch.Tens
 def decode_attention(cfg: PkvConfig, q: torch.Tensor, k_cache: torch.Tensor, v_cache: torch.Tensor,
                      seq_lens: Sequence[int], k_layer: int, out: torch.Tensor, stream=None) -> None:
     """One new token per sequence attends to the compact cache of a layer: q [batch][H_q][d] -> out fp32."""
+    st = _native.decode_attention(cfg, q, k_cache, v_cache, seq_lens, k_layer, out, stream)
+    if st != _NOT_TAKEN:
+        _check(st, "pyramidkv_decode_attention")
+        return
     lens, batch = _lens(seq_lens)
     if not (q.is_contiguous() and k_cache.is_contiguous() and v_cache.is_contiguous() and out.is_contiguous()):
         raise ValueError("decode_attention takes contiguous tensors")
@@ -558,6 +609,11 @@ def compress_layer_paged(cfg: PkvConfig, layer: int, q_win: torch.Tensor, k: tor
                          v_pool: torch.Tensor, indices: torch.Tensor, workspace: torch.Tensor,
                          scores: Optional[torch.Tensor] = None, stream=None,
                          window_lse: Optional[torch.Tensor] = None) -> None:
+    st = _native.compress_layer_paged(cfg, layer, q_win, k, v, seq_lens, block_table, k_pool, v_pool, indices, workspace, scores, stream,
+                                     window_lse)
+    if st != _NOT_TAKEN:
+        _check(st, "pyramidkv_compress_layer_paged")
+        return
     lens, batch = _lens(seq_lens)
     tab, page_size, num_pages, kp, vp = _paged(block_table, k_pool, v_pool)
     _check(_lib.pyramidkv_compress_layer_paged(
@@ -571,6 +627,10 @@ def compress_layer_paged(cfg: PkvConfig, layer: int, q_win: torch.Tensor, k: tor
 def decode_attention_paged(cfg: PkvConfig, q: torch.Tensor, block_table: torch.Tensor, k_pool: torch.Tensor,
                            v_pool: torch.Tensor, seq_lens: Sequence[int], k_layer: int, out: torch.Tensor,
                            workspace: torch.Tensor, stream=None) -> None:
+    st = _native.decode_attention_paged(cfg, q, block_table, k_pool, v_pool, seq_lens, k_layer, out, workspace, stream)
+    if st != _NOT_TAKEN:
+        _check(st, "pyramidkv_decode_attention_paged")
+        return
     lens, batch = _lens(seq_lens)
     if not (q.is_contiguous() and out.is_contiguous()):
         raise ValueError("decode_attention_paged takes contiguous q and out")

@@ -8,6 +8,7 @@
 #include <atomic>
 #include <mutex>
 #include <utility>
+#include <vector>
 
 #include "pkv_common.cuh"
 #include "pkv_decode.cuh"
@@ -971,14 +972,21 @@ int pyramidkv_gather_compact(const pkv_config* cfg, pkv_tensor k, pkv_tensor v, 
   return run_gather(cfg, k, v, indices, table, rows, k_out, v_out, static_cast<cudaStream_t>(stream));
 }
 
-// Budget of one layer: the schedule is O(m) integer work, small enough to redo per call.
+// Budget of one layer.  The schedule of a model is worked out once and remembered per thread (the last one asked for:
+// the layers of a model come one after another): 1 us per call for Eq. 1 over 32 layers, some 30 us for the geometric
+// schedule's bisection over 80.
 static int32_t layer_budget(const pkv_config* cfg, int32_t layer) {
-  int32_t stack_buf[512];
-  int32_t* all = cfg->num_layers <= 512 ? stack_buf : new int32_t[cfg->num_layers];
-  budgets(cfg, all);
-  const int32_t k_layer = all[layer];
-  if (all != stack_buf) delete[] all;
-  return k_layer;
+  struct Key { int32_t num_layers, window, avg_budget, schedule; double beta; };
+  thread_local Key last{};
+  thread_local std::vector<int32_t> all;
+  const Key key{cfg->num_layers, cfg->window, cfg->avg_budget, cfg->schedule, cfg->beta};
+  if (all.empty() || last.num_layers != key.num_layers || last.window != key.window || last.avg_budget != key.avg_budget ||
+      last.schedule != key.schedule || last.beta != key.beta) {
+    all.resize(static_cast<size_t>(cfg->num_layers));
+    budgets(cfg, all.data());
+    last = key;
+  }
+  return all[static_cast<size_t>(layer)];
 }
 
 static int compress_layer_impl(const pkv_config* cfg, int32_t layer, pkv_tensor q_win, pkv_tensor k, pkv_tensor v,
