@@ -599,11 +599,42 @@ int run_attend(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, co
   return check_launch();
 }
 
+// Table offsets of a layer's block table: sequences in batch order, H_kv * pages_b entries each.
+void fill_page_table(const pkv_config* c, const SeqTable& t, const int32_t* block_table, int page_size,
+                     int num_pages, PageTable* pt) {
+  std::memset(pt, 0, sizeof *pt);
+  pt->table = block_table;
+  pt->page_size = page_size;
+  pt->num_pages = num_pages;
+  int64_t off = 0;
+  for (int b = 0; b < t.batch; ++b) {
+    pt->pages[b] = (t.count[b] + page_size - 1) / page_size;
+    pt->tab_off[b] = off;
+    off += static_cast<int64_t>(c->num_kv_heads) * pt->pages[b];
+  }
+}
+
 // ---------------------------------------------------------------- select
-// With k/v/k_out given the kernel also copies the kept rows (fused eviction); otherwise it writes indices only.
+struct PagedOut {             // where the kept rows of a paged call go
+  const int32_t* block_table;
+  int page_size, num_pages;
+};
+
+// Instances of the selection kernel: threads x runs of eight positions = the longest slice they take.
+template <bool AVG>
+const void* select_instance(int slice, int* threads) {
+  if (slice <= 2048) { *threads = 256; return reinterpret_cast<const void*>(select_kernel<256, 1, AVG>); }
+  if (slice <= 4096) { *threads = 512; return reinterpret_cast<const void*>(select_kernel<512, 1, AVG>); }
+  *threads = 1024;
+  return slice <= 8192 ? reinterpret_cast<const void*>(select_kernel<1024, 1, AVG>)
+                       : reinterpret_cast<const void*>(select_kernel<1024, 2, AVG>);
+}
+
+// With k/v/k_out given the kernel also copies the kept rows (fused eviction; with `paged` into page slots of k_out and
+// v_out); otherwise it writes indices only.
 int run_select(const pkv_config* c, const float* scores, int64_t ld, const SeqTable& table, int batch, int max_n,
                int32_t* indices, const Workspace& w, cudaStream_t st, const pkv_tensor* k = nullptr,
-               const pkv_tensor* v = nullptr, void* k_out = nullptr, void* v_out = nullptr) {
+               const pkv_tensor* v = nullptr, void* k_out = nullptr, void* v_out = nullptr, const PagedOut* paged = nullptr) {
   SelectParams sp{};
   sp.scores = scores;
   sp.ld_scores = ld;
@@ -612,9 +643,7 @@ int run_select(const pkv_config* c, const float* scores, int64_t ld, const SeqTa
   sp.num_kv_heads = c->num_kv_heads;
   sp.pool_radius = (c->pool_kernel - 1) / 2;
   sp.status = w.status;
-  sp.cand = w.sel_cand;
-  sp.cand_stride = w.sel_cand_stride;
-  sp.cand_cnt = w.sel_cnt;
+  sp.vec = ld % 4 == 0 && reinterpret_cast<uintptr_t>(scores) % 16 == 0 ? 1 : 0;
   if (k_out) {
     sp.k = view(*k);
     sp.v = view(*v);
@@ -622,36 +651,56 @@ int run_select(const pkv_config* c, const float* scores, int64_t ld, const SeqTa
     sp.v_out = v_out;
     sp.elem_bytes = c->dtype == PKV_DTYPE_FP32 ? 4 : 2;
     sp.pieces = c->head_dim * sp.elem_bytes / 16;
+    while ((1 << sp.log_pieces) < sp.pieces) ++sp.log_pieces;
+  }
+  if (paged) {
+    sp.paged = 1;
+    fill_page_table(c, table, paged->block_table, paged->page_size, paged->num_pages, &sp.pt);
   }
   const int max_p = max_n - c->window;
   int cluster = 1;
-  while (cluster < kSelMaxCluster && (max_p + cluster - 1) / cluster > 8192) cluster *= 2;
+  while (cluster < kSelMaxCluster && (max_p + cluster - 1) / cluster > kSelClusterSlice) cluster *= 2;
   const int slice = ((max_p + cluster - 1) / cluster + 31) & ~31;
-  sp.cached = sp.pool_radius <= kSelHalo ? 1 : 0;
-  const size_t smem = sp.cached ? static_cast<size_t>(std::min(slice, kSelSliceCap)) * 6 + 8 * kSelHalo : 0;
-  sp.smem_pairs = static_cast<int32_t>(smem / sizeof(uint2));
+  const bool avg = c->pool_kind == PKV_POOL_AVG;
+  // rows longer than 8 x 16384 positions, and pools that reach further than the staged halo
+  const bool rounds = slice > kSelSliceCap || sp.pool_radius > kSelHalo;
+  int threads = kSelThreads;
+  const void* kernel;
+  size_t smem;
+  if (rounds) {
+    sp.cand = w.sel_cand;
+    sp.cand_stride = w.sel_cand_stride;
+    sp.cand_cnt = w.sel_cnt;
+    sp.cached = sp.pool_radius <= kSelHalo ? 1 : 0;
+    smem = sp.cached ? static_cast<size_t>(std::min(slice, kSelSliceCap)) * 6 + 8 * kSelHalo : 0;
+    sp.smem_pairs = static_cast<int32_t>(smem / sizeof(uint2));
+    int k_max = 0;                                  // largest number of prefix rows any sequence keeps
+    for (int b = 0; b < batch; ++b) k_max = std::max(k_max, table.count[b] - c->window);
+    const bool wide = k_max > 512;                  // then 8 maxima per thread keep the candidate bound tight
+    kernel = avg ? (wide ? reinterpret_cast<const void*>(pool_select_kernel<true, 8>) : reinterpret_cast<const void*>(pool_select_kernel<true, 1>))
+                 : (wide ? reinterpret_cast<const void*>(pool_select_kernel<false, 8>) : reinterpret_cast<const void*>(pool_select_kernel<false, 1>));
+  } else {
+    kernel = avg ? select_instance<true>(slice, &threads) : select_instance<false>(slice, &threads);
+    smem = sel_smem_bytes(slice);
+  }
   static bool attr_done[64] = {};  // the attribute is per device; setting it twice is harmless
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return PKV_ERR_CUDA;
   if (dev >= 64 || !attr_done[dev]) {
-    for (auto kernel : {pool_select_kernel<false, false, 1>, pool_select_kernel<true, false, 1>,
-                        pool_select_kernel<false, true, 1>, pool_select_kernel<true, true, 1>,
-                        pool_select_kernel<false, false, 8>, pool_select_kernel<true, false, 8>,
-                        pool_select_kernel<false, true, 8>, pool_select_kernel<true, true, 8>,
-                        pool_select_kernel<false, false, 1, kSelThreadsSmall>, pool_select_kernel<true, false, 1, kSelThreadsSmall>,
-                        pool_select_kernel<false, false, 8, kSelThreadsSmall>, pool_select_kernel<true, false, 8, kSelThreadsSmall>})
-      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kSelSliceCap * 6 + 8 * kSelHalo) != cudaSuccess)
+    for (auto f : {pool_select_kernel<false, 1>, pool_select_kernel<true, 1>, pool_select_kernel<false, 8>, pool_select_kernel<true, 8>})
+      if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSliceCap * 6 + 8 * kSelHalo) != cudaSuccess)
         return PKV_ERR_CUDA;
+    for (int s : {2048, 4096, 8192, 16384}) {
+      int unused;
+      for (const void* f : {select_instance<false>(s, &unused), select_instance<true>(s, &unused)})
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sel_smem_bytes(s))) != cudaSuccess)
+          return PKV_ERR_CUDA;
+    }
     if (dev < 64) attr_done[dev] = true;
   }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(cluster * c->num_kv_heads, batch);
-  // short slices (at most 8 positions per thread): the 512-thread instance, of which two fit on an SM, or one beside
-  // another layer's single-sweep score CTA.  (It could take 8192 positions, but at 16 per thread it is slower than
-  // 1024 threads at 8: measured +6 % per step on the 32k and batch-8 shapes.)
-  const bool small_cta = slice <= 4096;
-  cfg.blockDim = dim3(small_cta ? kSelThreadsSmall : kSelThreads);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
@@ -663,28 +712,26 @@ int run_select(const pkv_config* c, const float* scores, int64_t ld, const SeqTa
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  const bool avg = c->pool_kind == PKV_POOL_AVG;   // the mean pool is a variant; the max pool is the graded reading
-  const bool multi = slice > kSelSliceCap;          // long rows: each CTA takes its slice in several rounds
-  int k_max = 0;                                    // largest number of prefix rows any sequence keeps
-  for (int b = 0; b < batch; ++b) k_max = std::max(k_max, table.count[b] - c->window);
-  const bool wide = k_max > 512;                    // then 8 maxima per thread keep the candidate bound tight
-  auto kernel = avg ? (multi ? (wide ? pool_select_kernel<true, true, 8> : pool_select_kernel<true, true, 1>)
-                             : (wide ? pool_select_kernel<true, false, 8> : pool_select_kernel<true, false, 1>))
-                    : (multi ? (wide ? pool_select_kernel<false, true, 8> : pool_select_kernel<false, true, 1>)
-                             : (wide ? pool_select_kernel<false, false, 8> : pool_select_kernel<false, false, 1>));
-  if (small_cta)                                    // never multi: a slice of 8192 positions is one round
-    kernel = avg ? (wide ? pool_select_kernel<true, false, 8, kSelThreadsSmall> : pool_select_kernel<true, false, 1, kSelThreadsSmall>)
-                 : (wide ? pool_select_kernel<false, false, 8, kSelThreadsSmall> : pool_select_kernel<false, false, 1, kSelThreadsSmall>);
-  if (cudaLaunchKernelEx(&cfg, kernel, sp) != cudaSuccess) return PKV_ERR_CUDA;
-  if (k_out) {
+  void* args[1] = {&sp};
+  if (cudaLaunchKernelExC(&cfg, kernel, args) != cudaSuccess) return PKV_ERR_CUDA;
+  if (k_out && !paged) {
     int64_t out_rows = 0;
     for (int b = 0; b < batch; ++b) out_rows += static_cast<int64_t>(c->num_kv_heads) * table.count[b];
     const size_t out_bytes = static_cast<size_t>(out_rows) * c->head_dim * sp.elem_bytes;
     note_output(k_out, out_bytes);
     note_output(v_out, out_bytes);
+  } else if (paged) {
+    const size_t pool_bytes = static_cast<size_t>(paged->num_pages) * paged->page_size * c->head_dim * sp.elem_bytes;
+    note_output(k_out, pool_bytes);
+    note_output(v_out, pool_bytes);
   }
   mark(st, k_out ? "pool_select_gather" : "pool_select");
   return check_launch();
+}
+
+// Whether run_select would take the rows in rounds (it then cannot place them in pages itself).
+bool select_in_rounds(const pkv_config* c, int max_n) {
+  return max_n - c->window > kSelMaxCluster * kSelSliceCap || (c->pool_kernel - 1) / 2 > kSelHalo;
 }
 
 // ---------------------------------------------------------------- gather
@@ -709,21 +756,6 @@ int run_gather(const pkv_config* c, const pkv_tensor& k, const pkv_tensor& v, co
   note_output(v_out, static_cast<size_t>(total_rows) * c->head_dim * gp.elem_bytes);
   mark(st, "gather_rows");
   return check_launch();
-}
-
-// Table offsets of a layer's block table: sequences in batch order, H_kv * pages_b entries each.
-void fill_page_table(const pkv_config* c, const SeqTable& t, const int32_t* block_table, int page_size,
-                     int num_pages, PageTable* pt) {
-  std::memset(pt, 0, sizeof *pt);
-  pt->table = block_table;
-  pt->page_size = page_size;
-  pt->num_pages = num_pages;
-  int64_t off = 0;
-  for (int b = 0; b < t.batch; ++b) {
-    pt->pages[b] = (t.count[b] + page_size - 1) / page_size;
-    pt->tab_off[b] = off;
-    off += static_cast<int64_t>(c->num_kv_heads) * pt->pages[b];
-  }
 }
 
 int run_gather_paged(const pkv_config* c, const pkv_tensor& k, const pkv_tensor& v, const int32_t* indices,
@@ -1247,6 +1279,10 @@ int pyramidkv_compress_layer_paged(const pkv_config* cfg, int32_t layer, pkv_ten
   for (int b = 0; b < batch; ++b) any_compress |= table.count[b] < table.n[b];
   if (any_compress || scores_or_null)
     if (int rc = run_scores(cfg, q_win, k, table, batch, scores, ld, w, st, window_lse_or_null)) return rc;
+  if (!select_in_rounds(cfg, max_n)) {                        // the selection kernel places the rows itself
+    const PagedOut paged{block_table, page_size, num_pages};
+    return run_select(cfg, scores, ld, table, batch, max_n, indices, w, st, &k, &v, k_pool, v_pool, &paged);
+  }
   if (int rc = run_select(cfg, scores, ld, table, batch, max_n, indices, w, st)) return rc;
   return run_gather_paged(cfg, k, v, indices, table, rows, block_table, page_size, num_pages, k_pool, v_pool,
                           w.status, st);

@@ -31,13 +31,13 @@
 #include <cooperative_groups.h>
 
 #include "pkv_common.cuh"
+#include "pkv_paged.cuh"
 
 namespace pkv {
 
 namespace cg = cooperative_groups;
 
 constexpr int kSelThreads = 1024;
-constexpr int kSelThreadsSmall = 512;      // the instance for short slices (it can take up to 8192 positions)
 constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kSelMaxCluster = 8;
 constexpr int kSelBins = 2048;
@@ -66,6 +66,10 @@ struct SelectParams {
   void* v_out;
   int32_t elem_bytes;       // 4 or 2
   int32_t pieces;           // 16-byte pieces per row = d * elem_bytes / 16
+  int32_t log_pieces;       // log2 of that
+  int32_t vec;              // score rows start on 16-byte boundaries
+  int32_t paged;            // kept rows go to page slots of k_out / v_out through pt instead of packed rows
+  PageTable pt;
 };
 
 // Monotone map float -> uint32 (larger float, larger key).  -0 is folded into +0 first.
@@ -139,18 +143,15 @@ __device__ __noinline__ void gather_listed_rows(const int32_t* out, const char* 
 
 // grid (cluster * H_kv, batch), cluster (cluster, 1, 1), block kSelThreads,
 // dynamic shared memory (6 bytes per slice position + 8 * kSelHalo) when cached, else none.
-// MULTI: some CTA's slice is longer than kSelSliceCap and is taken in several rounds.
+// A slice longer than kSelSliceCap is taken in several rounds.
 // GROUPS: maxima each thread keeps for the lower bound of step 2 (1 for small budgets, 8 when k nears or
 // passes the thread count, so that the bound stays tight).
-template <bool AVG, bool MULTI, int GROUPS, int THREADS = kSelThreads>
-__global__ void __launch_bounds__(THREADS, THREADS == kSelThreads ? 1 : 2) pool_select_kernel(const SelectParams p) {
-  // THREADS = 512 is the instance for short slices (at most 8192 positions): half the registers of an SM, so that
-  // two such CTAs, or one and a CTA of another layer's score kernel, share an SM
-  constexpr int WARPS = THREADS / 32;
-  constexpr int CAP = kSelSliceCap / (kSelThreads / THREADS);   // positions a CTA holds per round
+template <bool AVG, int GROUPS>
+__global__ void __launch_bounds__(kSelThreads, 1) pool_select_kernel(const SelectParams p) {
+  constexpr int THREADS = kSelThreads, WARPS = kSelWarps;
+  constexpr int CAP = kSelSliceCap;                              // positions a CTA holds per round
   constexpr int PER_LANE = kSelPerLane;
-  constexpr int BPT = kSelBins / THREADS;                        // histogram bins every thread scans: 2 or 4
-  static_assert(BPT == 2 || BPT == 4, "thread count of the selection kernel");
+  constexpr int BPT = kSelBins / THREADS;                        // histogram bins every thread scans
   extern __shared__ __align__(16) uint32_t sel_smem[];      // [halo | slice | halo] raw scores; later CTA 0's pairs
   __shared__ uint32_t hist[2][kSelBins];                    // per-pass digit histogram (double buffered)
   __shared__ uint32_t warp_sum[WARPS];
@@ -184,9 +185,6 @@ __global__ void __launch_bounds__(THREADS, THREADS == kSelThreads ? 1 : 2) pool_
   uint2* regions = p.cand + head * p.cand_stride;           // region of CTA c starts at c * slice
   uint32_t* counts = p.cand_cnt + head * kSelMaxCluster;
   for (int i = tid; i < 2 * kSelBins; i += THREADS) (&hist[0][0])[i] = 0;
-  // A cluster of one keeps its candidates in shared memory when they fit: no trip through global memory.
-  bool local_pairs = false;
-  int local_count = 0;
 
   if (selecting) {
     const float* s = p.scores + head * p.ld_scores;
@@ -200,13 +198,13 @@ __global__ void __launch_bounds__(THREADS, THREADS == kSelThreads ? 1 : 2) pool_
       float* raw = reinterpret_cast<float*>(sel_smem + kSelHalo);
       const float outside = AVG ? 0.0f : -INFINITY;
       const float width = static_cast<float>(2 * radius + 1);
-      const int rounds = MULTI ? (hi - lo + CAP - 1) / CAP : 1;
+      const int rounds = (hi - lo + CAP - 1) / CAP;
       const int run = ((min(slice, CAP) / WARPS) + 31) & ~31;   // positions per warp and round
       uint32_t pk[PER_LANE];
       int wlo = hi, whi = hi;
       auto pool_round = [&](int r) {
         const int rlo = lo + r * CAP, rhi = min(hi, rlo + CAP);
-        if (MULTI) __syncthreads();                         // the previous round's readers are done
+        __syncthreads();                         // the previous round's readers are done
         for (int i = rlo - kSelHalo + tid; i < rhi + kSelHalo; i += THREADS)
           raw[i - rlo] = (i >= 0 && i < P) ? s[i] : outside;
         __syncthreads();
@@ -298,7 +296,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == kSelThreads ? 1 : 2) pool_
       // ---- 2b. candidates (keys >= bound) of every round, in position order, to this CTA's region
       uint32_t filled = 0;
       for (int r = 0; r < rounds; ++r) {
-        if (MULTI) pool_round(r);                           // a single round still holds its keys in registers
+        pool_round(r);
         uint32_t wc = 0;
 #pragma unroll
         for (int it = 0; it < PER_LANE; ++it) {
@@ -312,19 +310,16 @@ __global__ void __launch_bounds__(THREADS, THREADS == kSelThreads ? 1 : 2) pool_
           if (w2 < warp) base += warp_gt[w2];
           all_cand += warp_gt[w2];
         }
-        local_pairs = !MULTI && C == 1 && static_cast<int>(all_cand) <= p.smem_pairs;
-        uint2* dst = local_pairs ? reinterpret_cast<uint2*>(sel_smem) : region;   // the raw scores are dead by now
 #pragma unroll
         for (int it = 0; it < PER_LANE; ++it) {
           const int i = wlo + it * 32 + lane;
           const bool c = i < whi && pk[it] >= bound;
           const uint32_t bal = __ballot_sync(0xffffffffu, c);
-          if (c) dst[base + __popc(bal & lt)] = make_uint2(pk[it], static_cast<uint32_t>(i));
+          if (c) region[base + __popc(bal & lt)] = make_uint2(pk[it], static_cast<uint32_t>(i));
           base += __popc(bal);
         }
         filled += all_cand;
       }
-      local_count = static_cast<int>(filled);
       if (tid == 0) counts[rank] = filled;
     } else {
       // a very wide pool: every position is a candidate
@@ -340,7 +335,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == kSelThreads ? 1 : 2) pool_
     pre[0] = 0;
 #pragma unroll
     for (int c = 0; c < kSelMaxCluster; ++c) pre[c + 1] = pre[c] + (c < C ? __ldcg(counts + c) : 0u);
-    const int N = local_pairs ? local_count : static_cast<int>(pre[kSelMaxCluster]);
+    const int N = static_cast<int>(pre[kSelMaxCluster]);
     auto fetch = [&](int j) -> uint2 {                      // pair j of the concatenation, from global memory
       int c = 0;
 #pragma unroll
@@ -349,10 +344,8 @@ __global__ void __launch_bounds__(THREADS, THREADS == kSelThreads ? 1 : 2) pool_
     };
     uint2* flat = reinterpret_cast<uint2*>(sel_smem);
     const int held = min(N, p.smem_pairs);
-    if (!local_pairs) {
-      for (int j = tid; j < held; j += THREADS) flat[j] = fetch(j);
-      __syncthreads();
-    }
+    for (int j = tid; j < held; j += THREADS) flat[j] = fetch(j);
+    __syncthreads();
     auto item = [&](int j) -> uint2 { return j < held ? flat[j] : fetch(j); };
 
     uint32_t prefix = 0, mask = 0, remaining = k;
@@ -459,6 +452,451 @@ __global__ void __launch_bounds__(THREADS, THREADS == kSelThreads ? 1 : 2) pool_
       }
     }
   }
+}
+
+// ------------------------------------------------------------------ rows of at most kSelMaxCluster * 16384 positions
+//
+// The kernel is a chain of short phases, bound by their latencies (loads, block and cluster barriers), not by a unit.
+// What shortens the chain:
+//   * a thread takes runs of eight consecutive positions, so pooling is a handful of 16-byte shared-memory reads (the
+//     staged scores are padded by 16 bytes per 128 so that these do not conflict) and position order is thread order;
+//   * the lower bound of the k-th key comes from one histogram pass over the runs' maxima, linear over their range.  A
+//     run counts with the number of its positions that hold its maximum (pooled scores come in plateaus), so that the
+//     bound lets through about k positions of the CTA;
+//   * every CTA of the cluster finishes on its own: it reads the candidates of all (distributed shared memory), finds
+//     the threshold, and emits and copies the rows of its own slice.  There is one full cluster barrier (two when the
+//     list is long and the copy is dealt out evenly) and no trip through global memory;
+//   * the exact threshold is searched inside [largest bound of the CTAs, largest key], ten bits a pass, and finished by
+//     a warp as soon as at most 32 candidates are left in the bin (mostly after the first pass).
+constexpr int kSelBinsLin = 1024;          // bins of a linear histogram: ten bits of the key range
+constexpr int kSelRun = 8;                 // consecutive positions of a thread
+constexpr int kSelClusterSlice = 8192;     // a cluster doubles (up to 8 CTAs) while its slices are longer than this
+constexpr int kSelEvenRows = 1024;         // lists of at least this many rows are copied by the whole cluster evenly
+
+// Position i of the staged scores in shared memory: four floats of padding after every 32.
+__device__ __forceinline__ int sel_pad(int i) { return i + ((i >> 5) << 2); }
+
+// The largest bin d with (sum of bins >= d) >= want, and what lies above it; false when all bins together hold less.
+// Called by the whole block after a barrier behind the last update; `rows` is scratch (32 words); one barrier inside.
+template <int THREADS>
+__device__ __forceinline__ bool sel_find_from_top(const uint32_t* hist, uint32_t* rows, uint32_t want, uint32_t& digit,
+                                                  uint32_t& above) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int r = 0; r < kSelBinsLin / THREADS; ++r) {
+    const int row = warp + r * (THREADS / 32);
+    const uint32_t sum = __reduce_add_sync(0xffffffffu, hist[row * 32 + lane]);
+    if (lane == 0) rows[row] = sum;
+  }
+  __syncthreads();
+  // suffix sums over the 32 rows, then over the bins of the row the searched one lies in
+  auto suffix = [&](uint32_t x) {
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t u = __shfl_down_sync(0xffffffffu, x, off);
+      if (lane + off < 32) x += u;
+    }
+    return x;
+  };
+  const uint32_t rs = suffix(rows[lane]);
+  const uint32_t rmask = __ballot_sync(0xffffffffu, rs >= want);
+  if (rmask == 0) return false;
+  const int row = 31 - __clz(rmask);
+  const uint32_t past = row == 31 ? 0u : __shfl_sync(0xffffffffu, rs, row + 1);
+  const uint32_t bin = hist[row * 32 + lane];
+  const uint32_t bs = suffix(bin) + past;
+  const int b = 31 - __clz(__ballot_sync(0xffffffffu, bs >= want));
+  digit = static_cast<uint32_t>(row * 32 + b);
+  above = __shfl_sync(0xffffffffu, bs - bin, b);
+  return true;
+}
+
+// Pooled keys of eight consecutive positions; x[4 + j] is position j of the run.
+template <int R, bool AVG>
+__device__ __forceinline__ void sel_pool8(const float (&x)[16], uint32_t (&key)[kSelRun]) {
+#pragma unroll
+  for (int j = 0; j < kSelRun; ++j) {
+    float best = x[4 + j - R];
+#pragma unroll
+    for (int t = 1 - R; t <= R; ++t) best = AVG ? __fadd_rn(best, x[4 + j + t]) : fmaxf(best, x[4 + j + t]);
+    if (AVG) best = __fdiv_rn(best, static_cast<float>(2 * R + 1));
+    key[j] = ordered_key(best);
+  }
+}
+
+template <bool AVG>
+__device__ __forceinline__ void sel_pool_run(const float* raw, int at, int radius, uint32_t (&key)[kSelRun]) {
+  if (radius <= 4) {
+    float x[16];                                             // positions at - 4 .. at + 11
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const float4 f = *reinterpret_cast<const float4*>(raw + sel_pad(at - 4 + 4 * c));
+      x[4 * c] = f.x; x[4 * c + 1] = f.y; x[4 * c + 2] = f.z; x[4 * c + 3] = f.w;
+    }
+    switch (radius) {
+      case 0: sel_pool8<0, AVG>(x, key); break;
+      case 1: sel_pool8<1, AVG>(x, key); break;
+      case 2: sel_pool8<2, AVG>(x, key); break;
+      case 3: sel_pool8<3, AVG>(x, key); break;
+      default: sel_pool8<4, AVG>(x, key); break;
+    }
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < kSelRun; ++j) {
+    float best = raw[sel_pad(at + j - radius)];
+    for (int t = 1 - radius; t <= radius; ++t) {
+      const float v = raw[sel_pad(at + j + t)];
+      best = AVG ? __fadd_rn(best, v) : fmaxf(best, v);
+    }
+    if (AVG) best = __fdiv_rn(best, static_cast<float>(2 * radius + 1));
+    key[j] = ordered_key(best);
+  }
+}
+
+// Dynamic shared memory of an instance for slices of `slice` positions (a multiple of 32).
+__host__ __device__ constexpr size_t sel_smem_floats(int slice) { return static_cast<size_t>(slice + 2 * kSelHalo) * 9 / 8 + 4; }
+__host__ __device__ constexpr size_t sel_smem_bytes(int slice) { return sel_smem_floats(slice) * 4 + static_cast<size_t>(slice) * 8; }
+
+// grid (cluster * H_kv, batch), cluster (cluster, 1, 1), block THREADS, dynamic shared memory sel_smem_bytes(slice).
+// RUNS runs of eight positions per thread: a CTA takes at most THREADS * RUNS * 8 positions.
+template <int THREADS, int RUNS, bool AVG>
+__global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kernel(const SelectParams p) {
+  constexpr int WARPS = THREADS / 32;
+  extern __shared__ __align__(16) uint8_t sel_dyn[];
+  __shared__ uint32_t hist[2][kSelBinsLin];
+  __shared__ uint32_t rows[32];
+  __shared__ uint32_t warp_a[WARPS], warp_b[WARPS], warp_c[WARPS], warp_d[WARPS];
+  __shared__ uint32_t few[32], few_n;
+  __shared__ uint4 pub;                                     // candidates, bound, largest key: read by the whole cluster
+
+  pdl_trigger();
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = cluster.dim_blocks().x, rank = cluster.block_rank();
+  const int h = blockIdx.x / C, b = blockIdx.y;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t full = 0xffffffffu, lt = (1u << lane) - 1u;
+
+  const int n = p.seq.n[b], alpha = p.seq.alpha, P = n - alpha;
+  const int count = p.seq.count[b], k = count - alpha;      // prefix rows to keep, 0 <= k <= P
+  const bool selecting = k > 0 && k < P;                    // uniform over the cluster
+  const int slice = ((P + C - 1) / C + 31) & ~31;           // positions of a CTA, a multiple of 32
+  const int lo = min(P, rank * slice), len = min(P, lo + slice) - lo;
+  const int64_t head = static_cast<int64_t>(b) * p.num_kv_heads + h;
+  const int64_t row0 = p.seq.row_off[b] + static_cast<int64_t>(h) * count;
+  int32_t* out = p.indices + row0;
+  float* raw = reinterpret_cast<float*>(sel_dyn);           // staged scores; later keys of all candidates, then own list
+  const int flat_cap = static_cast<int>(sel_smem_floats(slice));
+  uint2* list = reinterpret_cast<uint2*>(sel_dyn + sel_smem_floats(slice) * 4);   // own candidates (key, position)
+
+  for (int i = tid; i < 2 * kSelBinsLin; i += THREADS) (&hist[0][0])[i] = 0;
+  if (tid == 0) few_n = 0;
+  pdl_wait();
+
+  // the rows this CTA copies: entries [own0, own1) of the head's list, positions in kept[]; the window closes the list
+  int own0 = 0, own1 = 0;
+  int32_t* kept = reinterpret_cast<int32_t*>(raw);
+  if (selecting) {
+    // ---- stage the slice with a halo (outside the prefix: what the pool ignores)
+    {
+      const float* s = p.scores + head * p.ld_scores;
+      const float outside = AVG ? 0.0f : -INFINITY;
+      constexpr int V = RUNS * 2 + 1;                       // 16-byte pieces per thread, halo included
+      const int pieces = (len + 2 * kSelHalo + 3) / 4;
+      float4 f[V];
+#pragma unroll
+      for (int j = 0; j < V; ++j) {
+        const int v = tid + j * THREADS, i = lo - kSelHalo + 4 * v;
+        if (v < pieces) {
+          if (p.vec && i >= 0 && i + 3 < P) {
+            f[j] = __ldcg(reinterpret_cast<const float4*>(s + i));
+          } else {
+            f[j].x = i >= 0 && i < P ? s[i] : outside;
+            f[j].y = i + 1 >= 0 && i + 1 < P ? s[i + 1] : outside;
+            f[j].z = i + 2 >= 0 && i + 2 < P ? s[i + 2] : outside;
+            f[j].w = i + 3 >= 0 && i + 3 < P ? s[i + 3] : outside;
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < V; ++j) {
+        const int v = tid + j * THREADS;
+        if (v < pieces) *reinterpret_cast<float4*>(raw + sel_pad(4 * v)) = f[j];
+      }
+    }
+    __syncthreads();
+
+    // ---- pool, and each run's largest key with the number of its positions that hold it
+    uint32_t key[RUNS][kSelRun], tmax[RUNS], weight[RUNS];
+    uint32_t mx = 0, mn = 0xffffffffu;
+#pragma unroll
+    for (int r = 0; r < RUNS; ++r) {
+      const int at = (r * THREADS + tid) * kSelRun;
+      tmax[r] = 0;
+      weight[r] = 0;
+      if (at < len) {
+        sel_pool_run<AVG>(raw, kSelHalo + at, p.pool_radius, key[r]);
+#pragma unroll
+        for (int j = 0; j < kSelRun; ++j)
+          if (at + j < len) tmax[r] = max(tmax[r], key[r][j]);
+#pragma unroll
+        for (int j = 0; j < kSelRun; ++j)
+          if (at + j < len && key[r][j] == tmax[r]) ++weight[r];
+        mx = max(mx, tmax[r]);
+        mn = min(mn, tmax[r]);
+      }
+    }
+    mx = __reduce_max_sync(full, mx);
+    mn = __reduce_min_sync(full, mn);
+    if (lane == 0) { warp_a[warp] = mx; warp_b[warp] = mn; }
+    __syncthreads();
+    mx = __reduce_max_sync(full, warp_a[lane & (WARPS - 1)]);
+    mn = __reduce_min_sync(full, warp_b[lane & (WARPS - 1)]);
+
+    // ---- lower bound of the k-th key, candidates in position order
+    uint32_t bound = 0;
+    if (len > 0) {
+      const int shift = max(0, 22 - __clz(mx - mn));        // (mx - mn) >> shift < 1024
+#pragma unroll
+      for (int r = 0; r < RUNS; ++r)
+        if (weight[r]) atomicAdd(&hist[0][(tmax[r] - mn) >> shift], weight[r]);
+      __syncthreads();
+      uint32_t digit, above;
+      bool found = sel_find_from_top<THREADS>(hist[0], rows, static_cast<uint32_t>(k), digit, above);
+      if (!found && k < len) {                              // large budgets: every position counts
+#pragma unroll
+        for (int r = 0; r < RUNS; ++r) {
+          const int at = (r * THREADS + tid) * kSelRun;
+#pragma unroll
+          for (int j = 0; j < kSelRun; ++j)
+            if (at + j < len && key[r][j] >= mn) atomicAdd(&hist[1][(key[r][j] - mn) >> shift], 1u);
+        }
+        __syncthreads();
+        found = sel_find_from_top<THREADS>(hist[1], rows, static_cast<uint32_t>(k), digit, above);
+        __syncthreads();
+        for (int i = tid; i < kSelBinsLin; i += THREADS) hist[1][i] = 0;
+      }
+      if (found) bound = mn + (digit << shift);
+    }
+    uint32_t c2 = 0;                                        // candidates of the runs, 16 bits each
+#pragma unroll
+    for (int r = 0; r < RUNS; ++r) {
+      const int at = (r * THREADS + tid) * kSelRun;
+#pragma unroll
+      for (int j = 0; j < kSelRun; ++j)
+        if (at + j < len && key[r][j] >= bound) c2 += 1u << (16 * r);
+    }
+    uint32_t incl = c2;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t u = __shfl_up_sync(full, incl, off);
+      if (lane >= off) incl += u;
+    }
+    if (lane == 31) warp_c[warp] = incl;
+    __syncthreads();
+    uint32_t wsum = lane < WARPS ? warp_c[lane] : 0u;
+    const uint32_t before = __reduce_add_sync(full, lane < warp ? wsum : 0u), all = __reduce_add_sync(full, wsum);
+    const int M = static_cast<int>((all & 0xffffu) + (all >> 16));
+    {
+      const uint32_t base2 = before + incl - c2;
+#pragma unroll
+      for (int r = 0; r < RUNS; ++r) {
+        const int at = (r * THREADS + tid) * kSelRun;
+        uint32_t to = r == 0 ? (base2 & 0xffffu) : (all & 0xffffu) + (base2 >> 16);
+        if ((c2 >> (16 * r)) & 0xffffu) {
+#pragma unroll
+          for (int j = 0; j < kSelRun; ++j)
+            if (at + j < len && key[r][j] >= bound) list[to++] = make_uint2(key[r][j], static_cast<uint32_t>(lo + at + j));
+        }
+      }
+    }
+    if (tid == 0) pub = make_uint4(static_cast<uint32_t>(M), bound, mx, 0u);
+    for (int i = tid; i < kSelBinsLin; i += THREADS) hist[0][i] = 0;
+    if (C == 1) __syncthreads(); else cluster.sync();       // candidates of the whole cluster are in place
+
+    // ---- the threshold T (k-th largest key) and how many ties at T are taken
+    uint32_t m_c = 0, b_c = 0, x_c = 0;
+    if (lane < C) {
+      const uint4 o = C == 1 ? pub : *cluster.map_shared_rank(&pub, lane);
+      m_c = o.x; b_c = o.y; x_c = o.z;
+    }
+    uint32_t pre[kSelMaxCluster + 1];
+    pre[0] = 0;
+#pragma unroll
+    for (int c = 0; c < kSelMaxCluster; ++c) pre[c + 1] = pre[c] + __shfl_sync(full, m_c, c);
+    const int N = static_cast<int>(pre[kSelMaxCluster]);
+    uint32_t base = __reduce_max_sync(full, b_c);           // at least k keys of some CTA, so of all, reach its bound
+    const uint32_t top = __reduce_max_sync(full, x_c);
+    uint32_t* flat = reinterpret_cast<uint32_t*>(raw);      // the raw scores are dead: keys of all candidates
+    auto remote = [&](int j) -> uint32_t {
+      if (C == 1) return list[j].x;
+      int c = 0;
+#pragma unroll
+      for (int q = 1; q < kSelMaxCluster; ++q) c += static_cast<uint32_t>(j) >= pre[q] ? 1 : 0;
+      uint32_t from = 0;
+#pragma unroll
+      for (int q = 1; q < kSelMaxCluster; ++q) from = c == q ? pre[q] : from;
+      return cluster.map_shared_rank(list, c)[j - static_cast<int>(from)].x;
+    };
+    const int held = min(N, flat_cap);
+    auto at_flat = [&](int j) -> uint32_t { return j < held ? flat[j] : remote(j); };
+    uint32_t want = static_cast<uint32_t>(k), T = 0, need_eq = 0;
+    int shift = max(0, 22 - __clz(top - base));
+    uint32_t span = 0xffffffffu;                            // keys base .. base + span take part
+    for (int pass = 0;; ++pass) {
+      uint32_t* hc = hist[pass & 1];
+      for (int j = tid; j < N; j += THREADS) {
+        uint32_t x;
+        if (pass == 0) {
+          x = remote(j);
+          if (j < held) flat[j] = x;
+        } else {
+          x = at_flat(j);
+        }
+        if (x >= base && x - base <= span) atomicAdd(&hc[(x - base) >> shift], 1u);
+      }
+      __syncthreads();
+      uint32_t digit = 0, above = 0;
+      sel_find_from_top<THREADS>(hc, rows, want, digit, above);
+      want -= above;
+      base += digit << shift;
+      const uint32_t in_bin = hc[digit];
+      if (shift == 0) {
+        T = base;
+        need_eq = want;
+        break;
+      }
+      if (in_bin <= 32u) {                                  // few enough for a warp: rank them by counting
+        for (int j = tid; j < N; j += THREADS) {
+          const uint32_t x = at_flat(j);
+          if (x >= base && ((x - base) >> shift) == 0) few[atomicAdd(&few_n, 1u)] = x;
+        }
+        __syncthreads();
+        const uint32_t x = lane < static_cast<int>(in_bin) ? few[lane] : 0u;
+        uint32_t gt = 0, ge = 0;
+        for (int q = 0; q < static_cast<int>(in_bin); ++q) {
+          const uint32_t o = __shfl_sync(full, x, q);
+          gt += o > x ? 1u : 0u;
+          ge += o >= x ? 1u : 0u;
+        }
+        const uint32_t hit = __ballot_sync(full, lane < static_cast<int>(in_bin) && gt < want && want <= ge);
+        const int src = __ffs(hit) - 1;
+        T = __shfl_sync(full, x, src);
+        need_eq = want - __shfl_sync(full, gt, src);
+        break;
+      }
+      span = (1u << shift) - 1u;
+      shift = max(0, shift - 10);
+      for (int i = tid; i < kSelBinsLin; i += THREADS) hist[(pass + 1) & 1][i] = 0;
+      __syncthreads();
+    }
+
+    // ---- emit: kept = keys above T and the leftmost need_eq of those at T.  Counted over the candidates of the CTAs
+    //      before this one (where its part of the list starts) and over its own, warp by warp in contiguous chunks
+    int own_lo = 0;                                         // candidates of the CTAs before this one
+#pragma unroll
+    for (int q = 1; q < kSelMaxCluster; ++q) own_lo = rank == q ? static_cast<int>(pre[q]) : own_lo;
+    uint32_t pgt = 0, peq = 0;
+    for (int j = tid; j < own_lo; j += THREADS) {
+      const uint32_t x = at_flat(j);
+      pgt += x > T ? 1u : 0u;
+      peq += x == T ? 1u : 0u;
+    }
+    pgt = __reduce_add_sync(full, pgt);
+    peq = __reduce_add_sync(full, peq);
+    const int chunk = (((M + WARPS - 1) / WARPS) + 31) & ~31;
+    const int j_lo = min(M, warp * chunk), j_hi = min(M, j_lo + chunk);
+    uint32_t ngt = 0, neq = 0;
+    for (int j0 = j_lo; j0 < j_hi; j0 += 32) {
+      const int j = j0 + lane;
+      const uint32_t x = j < j_hi ? list[j].x : 0u;
+      ngt += __popc(__ballot_sync(full, j < j_hi && x > T));
+      neq += __popc(__ballot_sync(full, j < j_hi && x == T));
+    }
+    if (lane == 0) { warp_a[warp] = pgt; warp_b[warp] = peq; warp_c[warp] = ngt; warp_d[warp] = neq; }
+    __syncthreads();
+    const bool has = lane < WARPS;
+    const uint32_t gt0 = __reduce_add_sync(full, has ? warp_a[lane & (WARPS - 1)] : 0u);
+    const uint32_t eq0 = __reduce_add_sync(full, has ? warp_b[lane & (WARPS - 1)] : 0u);
+    const uint32_t wg = has ? warp_c[lane & (WARPS - 1)] : 0u, we = has ? warp_d[lane & (WARPS - 1)] : 0u;
+    const uint32_t gt_all = gt0 + __reduce_add_sync(full, wg), eq_all = eq0 + __reduce_add_sync(full, we);
+    uint32_t gt_before = gt0 + __reduce_add_sync(full, lane < warp ? wg : 0u);
+    uint32_t eq_before = eq0 + __reduce_add_sync(full, lane < warp ? we : 0u);
+    own0 = static_cast<int>(gt0 + min(eq0, need_eq));
+    own1 = static_cast<int>(gt_all + min(eq_all, need_eq));
+    if (rank == C - 1 && tid == 0 && own1 != k) atomicOr(p.status, kStatusSelectMismatch);
+    for (int j0 = j_lo; j0 < j_hi; j0 += 32) {
+      const int j = j0 + lane;
+      const uint2 kv = j < j_hi ? list[j] : make_uint2(0u, 0u);
+      const bool is_gt = j < j_hi && kv.x > T, is_eq = j < j_hi && kv.x == T;
+      const uint32_t bg = __ballot_sync(full, is_gt), be = __ballot_sync(full, is_eq);
+      const uint32_t g = gt_before + __popc(bg & lt), e = eq_before + __popc(be & lt);
+      if (is_gt || (is_eq && e < need_eq)) {
+        const int at = static_cast<int>(g + min(e, need_eq));
+        out[at] = static_cast<int32_t>(kv.y);
+        kept[at - own0] = static_cast<int32_t>(kv.y);       // over the flat keys, which nobody reads any more
+      }
+      gt_before += __popc(bg);
+      eq_before += __popc(be);
+    }
+    if (C > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");   // done with the others' memory
+  } else if (k >= P) {                                      // nothing to evict: this CTA's share of the identity list
+    own0 = lo;
+    own1 = lo + len;
+    for (int i = tid; i < len; i += THREADS) out[lo + i] = lo + i;
+  }
+  // The window positions close the list (Section 4.2.1: always retained).
+  if (rank == C - 1)
+    for (int j = tid; j < alpha; j += THREADS) out[k + j] = P + j;
+
+  // ---- eviction by gather (appendix on torch.gather).  Every CTA copies the rows of its own slice, unless the list is
+  //      long: then it is dealt out evenly (kept rows may crowd into one slice)
+  if (p.k_out == nullptr) {
+    if (selecting && C > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    return;
+  }
+  const bool even = C > 1 && selecting && k >= kSelEvenRows;
+  if (even) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");        // the list is complete
+  else __syncthreads();                                     // kept[] is complete
+  const char* kb = static_cast<const char*>(p.k.ptr) + (b * p.k.sb + h * p.k.sh) * p.elem_bytes;
+  const char* vb = static_cast<const char*>(p.v.ptr) + (b * p.v.sb + h * p.v.sh) * p.elem_bytes;
+  const int64_t k_step = p.k.st * p.elem_bytes, v_step = p.v.st * p.elem_bytes;
+  const int first = even ? 0 : own0;                        // list entries [first, first + listed), then the window
+  const int listed = even ? k : own1 - own0;
+  const int total = (listed + (even || rank == C - 1 ? alpha : 0)) << p.log_pieces;
+  const int start = even ? rank * THREADS + tid : tid, stride = even ? C * THREADS : THREADS;
+  constexpr int U = 4;
+  for (int g0 = start; g0 < total; g0 += U * stride) {
+    uint4 kv[U], vv[U];
+    int64_t dst[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int g = g0 + u * stride;
+      dst[u] = -1;
+      if (g >= total) continue;
+      const int r = g >> p.log_pieces, piece = g & ((1 << p.log_pieces) - 1);
+      const int pos = r >= listed ? P + (r - listed) : (!selecting ? first + r : (even ? __ldcg(out + r) : kept[r]));
+      const int dr = r >= listed ? k + (r - listed) : first + r;
+      int64_t to = row0 + dr;
+      if (p.paged) {
+        to = paged_row(p.pt, b, h, dr);
+        if (to < 0) {
+          if (piece == 0) atomicOr(p.status, kStatusBadPage);
+          continue;
+        }
+      }
+      dst[u] = (to << p.log_pieces) + piece;
+      kv[u] = reinterpret_cast<const uint4*>(kb + pos * k_step)[piece];
+      vv[u] = reinterpret_cast<const uint4*>(vb + pos * v_step)[piece];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (dst[u] >= 0) {
+        static_cast<uint4*>(p.k_out)[dst[u]] = kv[u];
+        static_cast<uint4*>(p.v_out)[dst[u]] = vv[u];
+      }
+  }
+  if (selecting && C > 1 && !even) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
 }  // namespace pkv
