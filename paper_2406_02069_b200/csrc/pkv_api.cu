@@ -31,7 +31,8 @@ std::atomic<int> g_test_withhold_attend{0};  // 1: the withheld K tile, in the w
 std::atomic<int> g_test_two_sweeps{0};     // 1: never take the single-sweep kernel for short contexts
 
 constexpr size_t kAlign = 256;
-constexpr int kPartialChunk = 128;   // smallest key chunk any row-statistics kernel uses (sizes the workspace)
+constexpr int kPartialChunk = 128;   // keys per two partial slots at least (sizes the workspace): chunks of 64 keys or more
+constexpr size_t kMaxLogitBytes = size_t{256} << 20;   // fp32-pipe path: logits are kept between its passes up to this size
 
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
@@ -134,6 +135,8 @@ struct Workspace {
   uint2* sel_cand;           // selection: candidate (key, position) pairs, [heads][sel_cand_stride]
   int64_t sel_cand_stride;
   uint32_t* sel_cnt;         // selection: pairs per cluster rank, [heads][kSelMaxCluster]
+  float* logits;             // fp32-pipe path: [heads][rows][ld_logits] logits between its two passes, or null
+  int64_t ld_logits;
   float* o_partial;          // window attention: per-segment accumulators [kAtMaxGrid + heads][R][d], or null
   size_t score_scratch_bytes;   // bytes of the leading regions that the score kernels alone need
   size_t bytes;
@@ -172,6 +175,11 @@ Workspace carve(const pkv_config* c, int batch, int max_n, void* base) {
   w.sel_cand_stride = static_cast<int64_t>(max_n) + 32 * kSelMaxCluster;   // cluster * slice never exceeds this
   w.sel_cand = reinterpret_cast<uint2*>(take(heads * w.sel_cand_stride * sizeof(uint2)));
   w.sel_cnt = reinterpret_cast<uint32_t*>(take(heads * kSelMaxCluster * sizeof(uint32_t)));
+  if (!tc_eligible(c)) {
+    w.ld_logits = static_cast<int64_t>((static_cast<size_t>(max_n) + 127) / 128 * 128);
+    const size_t bytes = heads * rows * static_cast<size_t>(w.ld_logits) * sizeof(float);
+    if (bytes <= kMaxLogitBytes) w.logits = reinterpret_cast<float*>(take(bytes));
+  }
   if (attend_eligible(c))
     w.o_partial = reinterpret_cast<float*>(take((static_cast<size_t>(kAtMaxGrid) + heads) * rows * kAtD * sizeof(float)));
   w.bytes = off;
@@ -275,30 +283,94 @@ bool overlaps_recent_output(const pkv_tensor& t, int batch, int heads, int token
   return false;
 }
 
-// ---------------------------------------------------------------- scores
-template <typename T, int D>
-int launch_scores_generic(ScoreParams& sp, int batch, cudaStream_t st) {
-  int stat_tiles = 0, score_tiles = 0;
-  for (int b = 0; b < batch; ++b) {
-    sp.seq.stat_off[b] = stat_tiles;
-    sp.seq.score_off[b] = score_tiles;
-    stat_tiles += (sp.seq.n[b] + kGenChunk - 1) / kGenChunk;
-    score_tiles += (sp.seq.prefix[b] + kGenScoreKeys - 1) / kGenScoreKeys;
+// SMs the persistent score kernels may count on: the device's, or fewer while a call runs them on a lane that
+// owns only a group of the SMs (pyramidkv_compress_model_lanes sets the limit for its own thread).
+thread_local int tl_sm_limit = 0;
+
+int device_sm_count() {
+  static int sms[64] = {};
+  if (tl_sm_limit > 0) return tl_sm_limit;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (!sms[dev]) {
+    int n = 0;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    sms[dev] = n;
   }
-  sp.seq.stat_off[batch] = stat_tiles;
-  sp.seq.score_off[batch] = score_tiles;
+  return sms[dev];
+}
+
+// ---------------------------------------------------------------- scores
+template <typename T, int D, int ROWS, int KEYS>
+int launch_logit_tiles(ScoreParams& sp, int batch, cudaStream_t st) {
+  constexpr int kSmem = gen_smem_bytes<D, ROWS, KEYS>();
+  const int sms = device_sm_count();
+  if (sms <= 0) return PKV_ERR_CUDA;
+  static bool attr_done[64] = {};  // the attribute is per device; setting it twice is harmless
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return PKV_ERR_CUDA;
+  if (dev >= 64 || !attr_done[dev]) {
+    if (cudaFuncSetAttribute(logit_tiles_kernel<T, D, ROWS, KEYS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess ||
+        cudaFuncSetAttribute(logit_tiles_kernel<T, D, ROWS, KEYS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
+      return PKV_ERR_CUDA;
+    if (dev < 64) attr_done[dev] = true;
+  }
+  const bool given = sp.lse_in != sp.lse2;           // normalisers supplied by the caller: no statistics
+  // Tiles per chunk: as many as keep the busiest of the CTA slots (two to an SM) as short as possible; a chunk loads
+  // the window queries once and writes one partial per row.  With several row blocks a chunk is one tile.
+  auto tiles_of = [&](int b, bool prefix) { return ((prefix ? sp.seq.prefix[b] : sp.seq.n[b]) + KEYS - 1) / KEYS; };
+  sp.chunk_tiles = 1;
+  if (sp.rows <= ROWS) {
+    long long best = 0;
+    for (int ct = 1; ct <= 16; ++ct) {
+      long long items = 0;
+      for (int b = 0; b < batch; ++b) items += (tiles_of(b, false) + ct - 1) / ct;
+      const long long cost = (items * sp.num_kv_heads + 2 * sms - 1) / (2 * sms) * ct;
+      if (ct == 1 || cost <= best) { best = cost; sp.chunk_tiles = ct; }
+    }
+  }
+  int stat_chunks = 0, score_chunks = 0;
+  for (int b = 0; b < batch; ++b) {
+    sp.seq.stat_off[b] = stat_chunks;
+    sp.seq.score_off[b] = score_chunks;
+    stat_chunks += (tiles_of(b, false) + sp.chunk_tiles - 1) / sp.chunk_tiles;
+    score_chunks += (tiles_of(b, true) + sp.chunk_tiles - 1) / sp.chunk_tiles;
+  }
+  sp.seq.stat_off[batch] = stat_chunks;
+  sp.seq.score_off[batch] = score_chunks;
   sp.slots_per_chunk = 1;
-  if (sp.lse_in == sp.lse2) {                    // normalisers not supplied: sweep A and its merge
-    launch_pdl(rowstats_generic_kernel<T, D>, dim3(stat_tiles, sp.num_kv_heads), kGenRowBlock, 0, st, sp);
+  sp.log2_group = std::log2(static_cast<float>(sp.group));
+  if (sp.stats_only || given || sp.rows > 8192) sp.logits = nullptr;   // (scores_of_logits keeps the normalisers in shared memory)
+  if (!given) {
+    launch_pdl(logit_tiles_kernel<T, D, ROWS, KEYS, false>, dim3(stat_chunks, sp.num_kv_heads), kGenThreads, kSmem, st, sp);
     mark(st, "rowstats_generic");
-    launch_pdl(combine_stats_kernel, dim3((sp.rows + 31) / 32, sp.num_kv_heads, batch), kCombineThreads, 0, st, sp,
-               std::log2(static_cast<float>(sp.group)));
-    mark(st, "combine_stats");
+    if (!sp.logits) {
+      launch_pdl(combine_stats_kernel, dim3((sp.rows + 31) / 32, sp.num_kv_heads, batch), kCombineThreads, 0, st, sp, sp.log2_group);
+      mark(st, "combine_stats");
+    }
   }
   if (sp.stats_only) return check_launch();
-  launch_pdl(scores_generic_kernel<T, D>, dim3(score_tiles, sp.num_kv_heads), kGenScoreKeys, 0, st, sp);
+  if (sp.logits) {
+    int max_p = 0;
+    for (int b = 0; b < batch; ++b) max_p = std::max(max_p, sp.seq.prefix[b]);
+    constexpr int kKeys = 4 * kGenSumThreads;
+    launch_pdl(scores_of_logits_kernel, dim3((max_p + kKeys - 1) / kKeys, sp.num_kv_heads, batch), kGenSumThreads,
+               static_cast<size_t>(sp.rows) * sizeof(float), st, sp);
+  } else {
+    launch_pdl(logit_tiles_kernel<T, D, ROWS, KEYS, true>, dim3(score_chunks, sp.num_kv_heads), kGenThreads, kSmem, st, sp);
+  }
   mark(st, "scores_generic");
   return check_launch();
+}
+
+// Row blocks as large as the window rows need (16-bit inputs only come here with more than 256 rows).
+template <typename T, int D>
+int launch_scores_generic(ScoreParams& sp, int batch, cudaStream_t st) {
+  if constexpr (sizeof(T) == 4) {
+    if (sp.rows <= 32) return launch_logit_tiles<T, D, 32, 128>(sp, batch, st);
+    if (sp.rows <= 64) return launch_logit_tiles<T, D, 64, 64>(sp, batch, st);
+  }
+  return launch_logit_tiles<T, D, 128, 64>(sp, batch, st);
 }
 
 // ---------------------------------------------------------------- tensor-core scores
@@ -337,23 +409,6 @@ bool make_map(CUtensorMap* map, const pkv_tensor& t, bool fp16, int d, uint64_t 
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-
-// SMs the persistent score kernels may count on: the device's, or fewer while a call runs them on a lane that
-// owns only a group of the SMs (pyramidkv_compress_model_lanes sets the limit for its own thread).
-thread_local int tl_sm_limit = 0;
-
-int device_sm_count() {
-  static int sms[64] = {};
-  if (tl_sm_limit > 0) return tl_sm_limit;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (!sms[dev]) {
-    int n = 0;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    sms[dev] = n;
-  }
-  return sms[dev];
-}
 
 template <int D>
 int launch_scores_tc(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, ScoreParams& sp, int batch,
@@ -516,6 +571,8 @@ int run_scores(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, co
   sp.lse_add = window_lse ? std::log2(static_cast<float>(sp.group)) : 0.0f;
   sp.scores = scores;
   sp.ld_scores = ld;
+  sp.logits = w.logits;
+  sp.ld_logits = w.ld_logits;
   if (tc_eligible(c)) {
     int max_n = 0;
     for (int b = 0; b < batch; ++b) max_n = std::max(max_n, table.n[b]);
@@ -1665,7 +1722,8 @@ extern "C" int pyramidkv_score_window_static(const pkv_config* cfg, pkv_tensor q
   if (need > PKV_STATIC_SCRATCH_BYTES) return PKV_ERR_STATIC_SCRATCH;
   void* base = static_scratch_address();
   if (!base) return PKV_ERR_CUDA;
-  const Workspace w = carve(cfg, batch, max_n, base);
+  Workspace w = carve(cfg, batch, max_n, base);
+  w.logits = nullptr;                              // no room for logits here: they are formed again instead
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // The array keeps whatever the previous call left.  Only the status word has to start from zero;
   // statistics and normalisers are fully rewritten before they are read.

@@ -42,25 +42,6 @@ struct DecodeParams {
   float scale_log2;         // log2(e) / sqrt(d)
 };
 
-__device__ __forceinline__ unsigned long long dec_pack(float lo, float hi) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void dec_unpack(unsigned long long r, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(r));
-}
-__device__ __forceinline__ unsigned long long dec_fma(unsigned long long a, unsigned long long b, unsigned long long c) {
-  unsigned long long d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ unsigned long long dec_mul(unsigned long long a, unsigned long long b) {
-  unsigned long long d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
 // Eight consecutive elements of a row, as loaded and as four packed pairs of floats.
 template <typename T>
 struct Dec8 {
@@ -71,9 +52,9 @@ struct Dec8 {
     const uint32_t w = i == 0 ? u.x : (i == 1 ? u.y : (i == 2 ? u.z : u.w));
     if (sizeof(T) == 2 && __is_same(T, __half)) {
       const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w));
-      return dec_pack(f.x, f.y);
+      return pack2(f.x, f.y);
     }
-    return dec_pack(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));      // bfloat16: the upper half of a float
+    return pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));      // bfloat16: the upper half of a float
   }
 };
 template <>
@@ -85,7 +66,7 @@ struct Dec8<float> {
   }
   __device__ __forceinline__ void zero() { a = b = make_float4(0.f, 0.f, 0.f, 0.f); }
   __device__ __forceinline__ unsigned long long pair(int i) const {
-    return i == 0 ? dec_pack(a.x, a.y) : (i == 1 ? dec_pack(a.z, a.w) : (i == 2 ? dec_pack(b.x, b.y) : dec_pack(b.z, b.w)));
+    return i == 0 ? pack2(a.x, a.y) : (i == 1 ? pack2(a.z, a.w) : (i == 2 ? pack2(b.x, b.y) : pack2(b.z, b.w)));
   }
 };
 
@@ -160,11 +141,11 @@ __global__ void __launch_bounds__(kDecThreads) decode_attention_kernel(const Dec
       for (int c = 0; c < 4; ++c) k2[c] = kr[u].pair(c);
 #pragma unroll
       for (int g = 0; g < GT; ++g) {
-        unsigned long long d = dec_mul(q2[g][0], k2[0]);
+        unsigned long long d = mul2(q2[g][0], k2[0]);
 #pragma unroll
-        for (int c = 1; c < 4; ++c) d = dec_fma(q2[g][c], k2[c], d);
+        for (int c = 1; c < 4; ++c) d = fma2(q2[g][c], k2[c], d);
         float x, y;
-        dec_unpack(d, x, y);
+        unpack2(d, x, y);
         val[g * U + u] = x + y;
       }
     }
@@ -213,9 +194,9 @@ __global__ void __launch_bounds__(kDecThreads) decode_attention_kernel(const Dec
 #pragma unroll
       for (int g = 0; g < GT; ++g) {
         const float f = __shfl_sync(0xffffffffu, corr, g * U / PER * SHARE, L);
-        const unsigned long long f2 = dec_pack(f, f);
+        const unsigned long long f2 = pack2(f, f);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[g][c] = dec_mul(acc[g][c], f2);
+        for (int c = 0; c < 4; ++c) acc[g][c] = mul2(acc[g][c], f2);
       }
     }
 #pragma unroll
@@ -227,9 +208,9 @@ __global__ void __launch_bounds__(kDecThreads) decode_attention_kernel(const Dec
       for (int g = 0; g < GT; ++g) {
         const int i = g * U + u;
         const float w = __shfl_sync(0xffffffffu, val[i % PER], i / PER * SHARE, L);
-        const unsigned long long w2 = dec_pack(w, w);
+        const unsigned long long w2 = pack2(w, w);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[g][c] = dec_fma(w2, v2[c], acc[g][c]);
+        for (int c = 0; c < 4; ++c) acc[g][c] = fma2(w2, v2[c], acc[g][c]);
       }
     }
   }
@@ -250,7 +231,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_attention_kernel(const Dec
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       float x, y;
-      dec_unpack(acc[g][c], x, y);
+      unpack2(acc[g][c], x, y);
       x *= f;
       y *= f;
 #pragma unroll

@@ -1,32 +1,36 @@
 // Window-score kernels on the plain fp32 pipes (Section 4.2.2, Eq. 2 and Eq. 3).
 //
-// These cover every dtype / shape the boundary admits (fp32 inputs, any window,
-// any group size) and are the path of small fp32 problems.  The tensor-core
-// kernels in pkv_score_tc.cuh take over for bf16 inputs when their shape rules hold.
+// These cover every dtype / shape the boundary admits (fp32 inputs, any window, any group size) and are the path of
+// small fp32 problems.  The tensor-core kernels in pkv_score_tc.cuh take over for 16-bit inputs when their shape rules
+// hold.
 //
-// The score of a key mixes softmax rows that each have their own normaliser, so
-// the normalisers must be known before any score can be formed.  Three launches:
-//   rowstats    one thread per window row r = (query head g, window row j): running
-//               max and sum of exp over one chunk of keys     -> partial (max, sum)
-//   combine     merges the chunks of a (sequence, KV head)     -> lse2[r] = log2 sum_i 2^(x_ri)
-//   scores      one thread per key: s_i = sum_r 2^(x_ri - lse2[r] - log2 G)
-// with x_ri = q_r . k_i * log2(e) / sqrt(d); both sweeps form x with the same
-// sequence of operations, so the two agree bit for bit.
+// The score of a key mixes softmax rows that each have their own normaliser, so the normalisers must be known before
+// any score can be formed:
+//   logit_tiles<STATS>   x_ri = q_r . k_i * log2(e) / sqrt(d) of a block of window rows and a chunk of keys, tile by tile;
+//                        per row the maximum and the sum of 2^(x - max) -> partial (max, sum), and x itself to the
+//                        workspace when that has room for it (w.logits)
+//   scores_of_logits     s_i = sum_r 2^(x_ri - lse2[r] - log2 G) from the stored x; merges a head's partials first
+//   logit_tiles<SCORES>  the same sum straight from the tiles, with the normalisers known (the caller's, or those of
+//                        combine_stats): when x was not stored
+// Both ways form x with the same sequence of operations (one multiply-add chain over the channels per logit).
+//
+// What bounds it: 2 R n d flops per KV head on the fp32 pipe (128 multiply-adds per clock and SM).  Storing x (4 R n
+// bytes, mostly in the L2) costs a quarter of forming it again.  A tile is a register-blocked product: 256 threads with
+// 8 x 4 (4 x 4) logits each, fed by 16-byte shared-memory reads of channel-major Q and K, two logits per packed
+// multiply-add, so that the pipe and not the reads are the limit.
 #pragma once
 
 #include "pkv_common.cuh"
 
 namespace pkv {
 
-constexpr int kGenChunk = 128;       // keys per rowstats CTA (= the chunk the workspace is sized for)
-constexpr int kGenKeyTile = 16;      // keys staged in shared memory at a time
-constexpr int kGenRowBlock = 256;    // window rows per rowstats CTA pass (= its thread count)
-constexpr int kGenScoreKeys = 128;   // keys (= threads) per scores CTA
-constexpr int kGenQRows = 32;        // window rows staged per pass in the scores kernel
+constexpr int kGenThreads = 256;
+constexpr int kGenMinTile = 64;      // fewest keys per tile (a chunk of partial statistics is at least one tile)
+constexpr int kGenSumThreads = 128;  // scores_of_logits: threads per CTA, four keys each
 
 struct ScoreParams {
   TensorView q, k;
-  SeqTable seq;
+  SeqTable seq;                          // stat_off / score_off count chunks of chunk_tiles tiles
   int32_t num_kv_heads, group, rows;     // rows = group * alpha
   float scale_log2;                      // log2(e) / sqrt(d)
   float2* partial;                       // [sum_b chunks_b][slots_per_chunk][H_kv][rows] (max, sum)
@@ -40,70 +44,245 @@ struct ScoreParams {
   int32_t stat_grid;                     // 0: partial is [chunk][slot][H_kv][rows] (fp32-pipe sweep).  > 0: CTAs of
                                          // the tensor-core sweep, which writes [segment][slot][rows] with segment =
                                          // CTA + head for every run of a CTA over one head's chunks
+  float* logits;                         // fp32-pipe path: [batch][H_kv][rows][ld_logits] x values, or null
+  int64_t ld_logits;
+  int32_t chunk_tiles;                   // tiles per chunk (1 when there are several row blocks)
+  float log2_group;
 };
 
-// grid (total chunks, H_kv), block kGenRowBlock.
-template <typename T, int D>
-__global__ void __launch_bounds__(kGenRowBlock) rowstats_generic_kernel(const ScoreParams p) {
-  __shared__ __align__(16) float ktile[kGenKeyTile][D];
-  pdl_trigger();
-  pdl_wait();
-  const int tile = blockIdx.x, h = blockIdx.y;
-  const int b = find_sequence(p.seq.stat_off, p.seq.batch, tile);
-  const int n = p.seq.n[b], alpha = p.seq.alpha, P = p.seq.prefix[b];
-  const int key0 = (tile - p.seq.stat_off[b]) * kGenChunk;
-  const int key1 = min(n, key0 + kGenChunk);
-  const T* kbase = static_cast<const T*>(p.k.ptr) + b * p.k.sb + h * p.k.sh;
+// Four consecutive channels of a row as floats.
+__device__ __forceinline__ float4 gen_load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 gen_load4(const __nv_bfloat16* p) {
+  const uint2 u = *reinterpret_cast<const uint2*>(p);
+  return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
+                     __uint_as_float(u.y & 0xffff0000u));
+}
+__device__ __forceinline__ float4 gen_load4(const __half* p) {
+  const uint2 u = *reinterpret_cast<const uint2*>(p);
+  const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u.x)), b = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
+  return make_float4(a.x, a.y, b.x, b.y);
+}
 
-  for (int r0 = 0; r0 < p.rows; r0 += kGenRowBlock) {
-    const int r = r0 + threadIdx.x;
-    const bool live = r < p.rows;
-    const int g = live ? r / alpha : 0, j = live ? r % alpha : 0;
-    const int last_visible = P + j;                  // row j sees keys 0 .. P + j
-    float qreg[D];
-    {
-      const T* qrow = static_cast<const T*>(p.q.ptr) + b * p.q.sb +
-                      static_cast<int64_t>(h * p.group + g) * p.q.sh + j * p.q.st;
+// Channel-major tile in shared memory: element (channel c, column x) of a tile of W columns.  Columns are exchanged in
+// groups of four by a function of the channel, so that both the transposing stores (eight lanes along the channels,
+// four along the columns) and the 16-byte reads along the columns touch every bank once.
+template <int W>
+__device__ __forceinline__ int gen_at(int c, int x) { return c * W + (x ^ (((c >> 2) & 7) << 2)); }
+
+// Fills a channel-major tile from `count` rows (row(x) = address of row x; the columns from `count` to W become zero).
+template <int W, int D, typename F>
+__device__ __forceinline__ void gen_fill(float* tile, int count, F&& row) {
+  constexpr int kSteps = W * D / 4 / kGenThreads, kBatch = kSteps < 4 ? kSteps : 4;
+  static_assert(W * D / 4 % kGenThreads == 0, "tile of whole steps");
+  const int dq = threadIdx.x & 7;                            // 32 channels = 8 lanes of 4
 #pragma unroll
-      for (int c = 0; c < D; ++c) qreg[c] = live ? to_float(qrow[c]) : 0.f;
+  for (int s0 = 0; s0 < kSteps; s0 += kBatch) {
+    float4 f[kBatch];
+#pragma unroll
+    for (int s = 0; s < kBatch; ++s) {
+      const int e = (s0 + s) * (kGenThreads / 8) + threadIdx.x / 8;        // (channel block of 32, column), column fastest
+      const int x = e % W, cb = e / W;
+      f[s] = x < count ? gen_load4(row(x) + cb * 32 + dq * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    float m = -INFINITY, z = 0.f;
-    for (int t0 = key0; t0 < key1; t0 += kGenKeyTile) {
-      __syncthreads();
-      for (int e = threadIdx.x; e < kGenKeyTile * D; e += blockDim.x) {
-        const int kk = e / D, c = e % D;
-        const int i = t0 + kk;
-        ktile[kk][c] = i < key1 ? to_float(kbase[static_cast<int64_t>(i) * p.k.st + c]) : 0.f;
+#pragma unroll
+    for (int s = 0; s < kBatch; ++s) {
+      const int e = (s0 + s) * (kGenThreads / 8) + threadIdx.x / 8;
+      const int x = e % W, c = (e / W) * 32 + dq * 4;
+      tile[gen_at<W>(c, x)] = f[s].x;
+      tile[gen_at<W>(c + 1, x)] = f[s].y;
+      tile[gen_at<W>(c + 2, x)] = f[s].z;
+      tile[gen_at<W>(c + 3, x)] = f[s].w;
+    }
+  }
+}
+
+// grid (chunks over all sequences, H_kv), block kGenThreads, dynamic shared memory gen_smem_bytes.
+// ROWS x KEYS: window rows and keys of a tile; TR rows x 4 keys per thread.
+template <int D, int ROWS, int KEYS>
+__host__ __device__ constexpr int gen_smem_bytes() { return (ROWS + KEYS) * D * 4; }
+
+template <typename T, int D, int ROWS, int KEYS, bool SCORES>
+__global__ void __launch_bounds__(kGenThreads, 2) logit_tiles_kernel(const ScoreParams p) {
+  constexpr int KT = KEYS / 4;                               // threads along the keys
+  constexpr int RT = kGenThreads / KT;                       // threads along the rows
+  constexpr int TR = ROWS / RT;                              // rows per thread
+  static_assert(KT <= 32 && TR % 4 == 0, "a warp holds whole rows of threads");
+  extern __shared__ __align__(16) float gen_smem[];
+  float* qs = gen_smem;                                      // channel-major [D][ROWS]
+  float* ks = gen_smem + ROWS * D;                           // channel-major [D][KEYS]
+  __shared__ float lse_s[SCORES ? ROWS : 1];
+  __shared__ __align__(16) float part[SCORES ? RT : 1][SCORES ? KEYS : 4];
+  pdl_trigger();
+  const int32_t* off = SCORES ? p.seq.score_off : p.seq.stat_off;
+  const int h = blockIdx.y, b = find_sequence(off, p.seq.batch, blockIdx.x);
+  const int n = p.seq.n[b], alpha = p.seq.alpha, P = p.seq.prefix[b];
+  const int keys = SCORES ? P : n;
+  const int tile0 = (blockIdx.x - off[b]) * p.chunk_tiles, tile1 = min(tile0 + p.chunk_tiles, (keys + KEYS - 1) / KEYS);
+  const T* kbase = static_cast<const T*>(p.k.ptr) + b * p.k.sb + h * p.k.sh;
+  const T* qbase = static_cast<const T*>(p.q.ptr) + b * p.q.sb + static_cast<int64_t>(h * p.group) * p.q.sh;
+  const int tk = threadIdx.x % KT, tr = threadIdx.x / KT;
+  const int blocks = (p.rows + ROWS - 1) / ROWS;
+  const int64_t head = static_cast<int64_t>(b) * p.num_kv_heads + h;
+  pdl_wait();
+
+  float m[TR], z[TR];                                        // STATS: per row over this thread's keys of the chunk
+#pragma unroll
+  for (int i = 0; i < TR; ++i) { m[i] = -INFINITY; z[i] = 0.f; }
+  for (int t = tile0; t < tile1; ++t) {
+    const int key0 = t * KEYS;
+    float sum[4] = {0.f, 0.f, 0.f, 0.f};                     // SCORES: of this thread's keys
+    for (int rb = 0; rb < blocks; ++rb) {
+      const int r0 = rb * ROWS;
+      __syncthreads();                                       // the tiles before have been read
+      if (blocks > 1 || t == tile0) {
+        gen_fill<ROWS, D>(qs, min(ROWS, p.rows - r0), [&](int x) {
+          const int r = r0 + x;
+          return qbase + (r / alpha) * p.q.sh + (r % alpha) * p.q.st;
+        });
+        if (SCORES)
+          for (int x = threadIdx.x; x < ROWS; x += kGenThreads)
+            lse_s[x] = r0 + x < p.rows ? fmaf(p.lse_in[head * p.rows + r0 + x], p.lse_scale, p.lse_add) : INFINITY;
       }
+      if (rb == 0) gen_fill<KEYS, D>(ks, min(KEYS, n - key0), [&](int x) { return kbase + static_cast<int64_t>(key0 + x) * p.k.st; });
       __syncthreads();
-      float x[kGenKeyTile];
-      float tmax = -INFINITY;
+      unsigned long long acc[TR][2];
 #pragma unroll
-      for (int kk = 0; kk < kGenKeyTile; ++kk) {
-        float dot = 0.f;
+      for (int i = 0; i < TR; ++i) acc[i][0] = acc[i][1] = 0ull;
+#pragma unroll 32
+      for (int c = 0; c < D; ++c) {
+        const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(ks + gen_at<KEYS>(c, tk * 4));
 #pragma unroll
-        for (int c = 0; c < D; c += 4) {
-          const float4 kv = *reinterpret_cast<const float4*>(&ktile[kk][c]);
-          dot = fmaf(qreg[c], kv.x, dot);
-          dot = fmaf(qreg[c + 1], kv.y, dot);
-          dot = fmaf(qreg[c + 2], kv.z, dot);
-          dot = fmaf(qreg[c + 3], kv.w, dot);
+        for (int i = 0; i < TR; i += 4) {
+          const float4 q = *reinterpret_cast<const float4*>(qs + gen_at<ROWS>(c, tr * TR + i));
+          const float qv[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const unsigned long long q2 = pack2(qv[j], qv[j]);
+            acc[i + j][0] = fma2(q2, kk.x, acc[i + j][0]);
+            acc[i + j][1] = fma2(q2, kk.y, acc[i + j][1]);
+          }
         }
-        const int i = t0 + kk;
-        x[kk] = (i < key1 && i <= last_visible) ? dot * p.scale_log2 : -INFINITY;
-        tmax = fmaxf(tmax, x[kk]);
       }
-      if (tmax > -INFINITY) {
-        const float mn = fmaxf(m, tmax);
-        float acc = 0.f;
+      const int i0 = key0 + tk * 4;                          // this thread's keys
 #pragma unroll
-        for (int kk = 0; kk < kGenKeyTile; ++kk) acc += exp2f(x[kk] - mn);
-        z = z * exp2f(m - mn) + acc;                 // exp2f(-inf) = 0 on the first tile
+      for (int i = 0; i < TR; ++i) {
+        const int r = r0 + tr * TR + i;
+        float x[4];
+        unpack2(acc[i][0], x[0], x[1]);
+        unpack2(acc[i][1], x[2], x[3]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x[j] *= p.scale_log2;
+        if (SCORES) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) sum[j] += exp2f(x[j] - lse_s[tr * TR + i]);
+          continue;
+        }
+        if (r >= p.rows) continue;
+        if (p.logits && i0 < P)
+          *reinterpret_cast<float4*>(p.logits + (head * p.rows + r) * p.ld_logits + i0) = make_float4(x[0], x[1], x[2], x[3]);
+        const int last = min(P + r % alpha, n - 1);          // row (g, j) sees keys 0 .. P + j that exist here
+        if (i0 + 3 > last) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) x[j] = i0 + j <= last ? x[j] : -INFINITY;
+        }
+        const float mn = fmaxf(fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3])), m[i]);
+        if (mn > -INFINITY) {
+          z[i] = z[i] * exp2f(m[i] - mn) + ((exp2f(x[0] - mn) + exp2f(x[1] - mn)) + (exp2f(x[2] - mn) + exp2f(x[3] - mn)));
+          m[i] = mn;
+        }
+      }
+      if (!SCORES && (blocks > 1 || t + 1 == tile1)) {       // the rows' statistics over the chunk: merge the threads along the keys
+#pragma unroll
+        for (int i = 0; i < TR; ++i) {
+#pragma unroll
+          for (int o = 1; o < KT; o <<= 1) {
+            const float m2 = __shfl_xor_sync(0xffffffffu, m[i], o), z2 = __shfl_xor_sync(0xffffffffu, z[i], o);
+            const float mm = fmaxf(m[i], m2);
+            if (mm > -INFINITY) z[i] = z[i] * exp2f(m[i] - mm) + z2 * exp2f(m2 - mm);
+            m[i] = mm;
+          }
+          const int r = r0 + tr * TR + i;
+          if (tk == 0 && r < p.rows)
+            p.partial[(static_cast<int64_t>(blockIdx.x) * p.num_kv_heads + h) * p.rows + r] = make_float2(m[i], z[i]);
+          m[i] = -INFINITY;
+          z[i] = 0.f;
+        }
+      }
+    }
+    if (SCORES) {                                            // the rows of a key are spread over RT threads
+      *reinterpret_cast<float4*>(&part[tr][tk * 4]) = make_float4(sum[0], sum[1], sum[2], sum[3]);
+      __syncthreads();
+      for (int x = threadIdx.x; x < KEYS; x += kGenThreads) {
+        float s = 0.f;
+#pragma unroll
+        for (int q = 0; q < RT; ++q) s += part[q][x];
+        if (key0 + x < P) p.scores[head * p.ld_scores + key0 + x] = s;
+      }
+    }
+  }
+}
+
+// grid (blocks of 4 * kGenSumThreads prefix keys of the longest sequence, H_kv, batch), block kGenSumThreads, dynamic
+// shared memory rows floats: scores from stored logits.  Four keys per thread; the row normalisers are merged from the
+// partials by every CTA for itself (a few hundred kilobytes from the L2), which saves a launch between the two.
+__global__ void __launch_bounds__(kGenSumThreads) scores_of_logits_kernel(const ScoreParams p) {
+  extern __shared__ float lse_all[];
+  pdl_trigger();
+  const int h = blockIdx.y, b = blockIdx.z, P = p.seq.prefix[b];
+  const int i0 = (blockIdx.x * kGenSumThreads + threadIdx.x) * 4;
+  pdl_wait();
+  if (blockIdx.x * kGenSumThreads * 4 >= P) return;
+  const int64_t head = static_cast<int64_t>(b) * p.num_kv_heads + h;
+  const int t0 = p.seq.stat_off[b], t1 = p.seq.stat_off[b + 1];
+  const int64_t step = static_cast<int64_t>(p.num_kv_heads) * p.rows;
+  for (int r = threadIdx.x; r < p.rows; r += kGenSumThreads) {
+    const float2* src = p.partial + static_cast<int64_t>(h) * p.rows + r;
+    float m = -INFINITY, z = 0.f;
+    for (int t = t0; t < t1; t += 8) {
+      float2 pz[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) pz[u] = t + u < t1 ? __ldcg(src + (t + u) * step) : make_float2(-INFINITY, 0.f);
+      float mn = m;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) mn = fmaxf(mn, pz[u].x);
+      if (mn > -INFINITY) {
+        z *= exp2f(m - mn);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) z += pz[u].y * exp2f(pz[u].x - mn);
         m = mn;
       }
     }
-    if (live) p.partial[(static_cast<int64_t>(tile) * p.num_kv_heads + h) * p.rows + r] = make_float2(m, z);
+    lse_all[r] = m + log2f(z) + p.log2_group;
   }
+  __syncthreads();
+  if (i0 >= P) return;
+  const float* x = p.logits + head * p.rows * p.ld_logits + i0;
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
+  int r = 0;
+  for (; r + 8 <= p.rows; r += 8) {
+    float4 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = __ldcs(reinterpret_cast<const float4*>(x + (r + u) * p.ld_logits));
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const float l = lse_all[r + u];
+      s[0] += exp2f(v[u].x - l);
+      s[1] += exp2f(v[u].y - l);
+      s[2] += exp2f(v[u].z - l);
+      s[3] += exp2f(v[u].w - l);
+    }
+  }
+  for (; r < p.rows; ++r) {
+    const float4 v = *reinterpret_cast<const float4*>(x + r * p.ld_logits);
+    const float l = lse_all[r];
+    s[0] += exp2f(v.x - l);
+    s[1] += exp2f(v.y - l);
+    s[2] += exp2f(v.z - l);
+    s[3] += exp2f(v.w - l);
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (i0 + j < P) p.scores[head * p.ld_scores + i0 + j] = s[j];
 }
 
 // grid (ceil(rows / 32), H_kv, batch), block 1024: merge the chunk partials of each window row.
@@ -166,62 +345,6 @@ __global__ void __launch_bounds__(kCombineThreads) combine_stats_kernel(const Sc
       if (sm[g][rl] > -INFINITY) zz += sz[g][rl] * exp2f(sm[g][rl] - mm);
     p.lse2[(static_cast<int64_t>(b) * p.num_kv_heads + h) * p.rows + r] = mm + log2f(zz) + extra_log2;
   }
-}
-
-// grid (total prefix tiles, H_kv), block kGenScoreKeys: one thread per prefix key.
-template <typename T, int D>
-__global__ void __launch_bounds__(kGenScoreKeys) scores_generic_kernel(const ScoreParams p) {
-  __shared__ __align__(16) float qs[kGenQRows][D];
-  __shared__ float lse_s[kGenQRows];
-  pdl_trigger();
-  pdl_wait();
-  const int tile = blockIdx.x, h = blockIdx.y;
-  const int b = find_sequence(p.seq.score_off, p.seq.batch, tile);
-  const int alpha = p.seq.alpha, P = p.seq.prefix[b];
-  const int i = (tile - p.seq.score_off[b]) * kGenScoreKeys + threadIdx.x;
-  const bool live = i < P;
-  float kreg[D];
-  {
-    const T* krow = static_cast<const T*>(p.k.ptr) + b * p.k.sb + h * p.k.sh +
-                    static_cast<int64_t>(live ? i : 0) * p.k.st;
-#pragma unroll
-    for (int c = 0; c < D; ++c) kreg[c] = to_float(krow[c]);
-  }
-  float s = 0.f;
-  for (int r0 = 0; r0 < p.rows; r0 += kGenQRows) {
-    __syncthreads();
-    for (int e = threadIdx.x; e < kGenQRows * D; e += blockDim.x) {
-      const int rr = e / D, c = e % D, r = r0 + rr;
-      float v = 0.f;
-      if (r < p.rows) {
-        const int g = r / alpha, j = r % alpha;
-        v = to_float(static_cast<const T*>(p.q.ptr)[b * p.q.sb + static_cast<int64_t>(h * p.group + g) * p.q.sh +
-                                                     j * p.q.st + c]);
-      }
-      qs[rr][c] = v;
-    }
-    if (threadIdx.x < kGenQRows) {
-      const int r = r0 + threadIdx.x;
-      lse_s[threadIdx.x] =
-          r < p.rows ? fmaf(p.lse_in[(static_cast<int64_t>(b) * p.num_kv_heads + h) * p.rows + r], p.lse_scale, p.lse_add)
-                     : INFINITY;
-    }
-    __syncthreads();
-    const int rn = min(kGenQRows, p.rows - r0);
-    for (int rr = 0; rr < rn; ++rr) {
-      float dot = 0.f;
-#pragma unroll
-      for (int c = 0; c < D; c += 4) {
-        const float4 qv = *reinterpret_cast<const float4*>(&qs[rr][c]);
-        dot = fmaf(qv.x, kreg[c], dot);
-        dot = fmaf(qv.y, kreg[c + 1], dot);
-        dot = fmaf(qv.z, kreg[c + 2], dot);
-        dot = fmaf(qv.w, kreg[c + 3], dot);
-      }
-      s += exp2f(dot * p.scale_log2 - lse_s[rr]);
-    }
-  }
-  if (live) p.scores[(static_cast<int64_t>(b) * p.num_kv_heads + h) * p.ld_scores + i] = s;
 }
 
 }  // namespace pkv
