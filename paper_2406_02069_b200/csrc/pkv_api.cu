@@ -353,8 +353,7 @@ int launch_logit_tiles(ScoreParams& sp, int batch, cudaStream_t st) {
   if (sp.logits) {
     int max_p = 0;
     for (int b = 0; b < batch; ++b) max_p = std::max(max_p, sp.seq.prefix[b]);
-    constexpr int kKeys = 4 * kGenSumThreads;
-    launch_pdl(scores_of_logits_kernel, dim3((max_p + kKeys - 1) / kKeys, sp.num_kv_heads, batch), kGenSumThreads,
+    launch_pdl(scores_of_logits_kernel, dim3((max_p + kGenSumKeys - 1) / kGenSumKeys, sp.num_kv_heads, batch), kGenSumThreads,
                static_cast<size_t>(sp.rows) * sizeof(float), st, sp);
   } else {
     launch_pdl(logit_tiles_kernel<T, D, ROWS, KEYS, true>, dim3(score_chunks, sp.num_kv_heads), kGenThreads, kSmem, st, sp);
@@ -717,6 +716,15 @@ int run_select(const pkv_config* c, const float* scores, int64_t ld, const SeqTa
   const int max_p = max_n - c->window;
   int cluster = 1;
   while (cluster < kSelMaxCluster && (max_p + cluster - 1) / cluster > kSelClusterSlice) cluster *= 2;
+  // A CTA moves some 50 GB/s of rows: more of them for heads that keep many bytes, while SMs are idle.
+  if (k_out) {
+    int most = 0;
+    for (int b = 0; b < batch; ++b) most = std::max(most, table.count[b]);
+    const int64_t bytes = static_cast<int64_t>(most) * c->head_dim * sp.elem_bytes * 2;   // K and V of a head
+    while (cluster < kSelMaxCluster && bytes / cluster > kSelCopyBytes && max_p / cluster >= 1024 &&
+           2ll * cluster * c->num_kv_heads * batch <= device_sm_count())
+      cluster *= 2;
+  }
   const int slice = ((max_p + cluster - 1) / cluster + 31) & ~31;
   const bool avg = c->pool_kind == PKV_POOL_AVG;
   // rows longer than 8 x 16384 positions, and pools that reach further than the staged halo
@@ -738,7 +746,14 @@ int run_select(const pkv_config* c, const float* scores, int64_t ld, const SeqTa
                  : (wide ? reinterpret_cast<const void*>(pool_select_kernel<false, 8>) : reinterpret_cast<const void*>(pool_select_kernel<false, 1>));
   } else {
     kernel = avg ? select_instance<true>(slice, &threads) : select_instance<false>(slice, &threads);
-    smem = sel_smem_bytes(slice);
+    // room for the staged scores, and for the keys of all candidates (about k per CTA, or about k in all)
+    int k_max = 0;
+    for (int b = 0; b < batch; ++b) k_max = std::max(k_max, table.count[b] - c->window);
+    sp.common_rows = kSelCommonCandidates / cluster;
+    const int expect = k_max > sp.common_rows ? k_max + k_max / 4 : cluster * (k_max + k_max / 4);
+    const int raw = static_cast<int>(sel_smem_floats(slice)), most = static_cast<int>((kSelSmemMax - static_cast<size_t>(slice) * 8) / 4);
+    sp.flat_cap = std::max(raw, std::min(std::min(max_p, expect) + 256, most)) & ~3;
+    smem = static_cast<size_t>(sp.flat_cap) * 4 + static_cast<size_t>(slice) * 8;
   }
   static bool attr_done[64] = {};  // the attribute is per device; setting it twice is harmless
   int dev = 0;
@@ -750,7 +765,7 @@ int run_select(const pkv_config* c, const float* scores, int64_t ld, const SeqTa
     for (int s : {2048, 4096, 8192, 16384}) {
       int unused;
       for (const void* f : {select_instance<false>(s, &unused), select_instance<true>(s, &unused)})
-        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sel_smem_bytes(s))) != cudaSuccess)
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSelSmemMax)) != cudaSuccess)
           return PKV_ERR_CUDA;
     }
     if (dev < 64) attr_done[dev] = true;

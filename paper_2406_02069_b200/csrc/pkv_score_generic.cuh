@@ -26,7 +26,9 @@ namespace pkv {
 
 constexpr int kGenThreads = 256;
 constexpr int kGenMinTile = 64;      // fewest keys per tile (a chunk of partial statistics is at least one tile)
-constexpr int kGenSumThreads = 128;  // scores_of_logits: threads per CTA, four keys each
+constexpr int kGenSumThreads = 256;  // scores_of_logits: threads per CTA,
+constexpr int kGenSumKeys = 256;     // keys per CTA (four per thread),
+constexpr int kGenSumGroups = kGenSumThreads * 4 / kGenSumKeys;   // and groups of threads that share the rows
 
 struct ScoreParams {
   TensorView q, k;
@@ -145,21 +147,22 @@ __global__ void __launch_bounds__(kGenThreads, 2) logit_tiles_kernel(const Score
       }
       if (rb == 0) gen_fill<KEYS, D>(ks, min(KEYS, n - key0), [&](int x) { return kbase + static_cast<int64_t>(key0 + x) * p.k.st; });
       __syncthreads();
-      unsigned long long acc[TR][2];
+      unsigned long long acc[TR / 2][4];                     // pairs of rows: the queries come in pairs as they are, only the
+#pragma unroll                                               // four keys have to be doubled
+      for (int i = 0; i < TR / 2; ++i)
 #pragma unroll
-      for (int i = 0; i < TR; ++i) acc[i][0] = acc[i][1] = 0ull;
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
 #pragma unroll 32
       for (int c = 0; c < D; ++c) {
-        const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(ks + gen_at<KEYS>(c, tk * 4));
+        const float4 kf = *reinterpret_cast<const float4*>(ks + gen_at<KEYS>(c, tk * 4));
+        const unsigned long long k2[4] = {pack2(kf.x, kf.x), pack2(kf.y, kf.y), pack2(kf.z, kf.z), pack2(kf.w, kf.w)};
 #pragma unroll
         for (int i = 0; i < TR; i += 4) {
-          const float4 q = *reinterpret_cast<const float4*>(qs + gen_at<ROWS>(c, tr * TR + i));
-          const float qv[4] = {q.x, q.y, q.z, q.w};
+          const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(qs + gen_at<ROWS>(c, tr * TR + i));
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const unsigned long long q2 = pack2(qv[j], qv[j]);
-            acc[i + j][0] = fma2(q2, kk.x, acc[i + j][0]);
-            acc[i + j][1] = fma2(q2, kk.y, acc[i + j][1]);
+            acc[i / 2][j] = fma2(q.x, k2[j], acc[i / 2][j]);
+            acc[i / 2 + 1][j] = fma2(q.y, k2[j], acc[i / 2 + 1][j]);
           }
         }
       }
@@ -168,10 +171,12 @@ __global__ void __launch_bounds__(kGenThreads, 2) logit_tiles_kernel(const Score
       for (int i = 0; i < TR; ++i) {
         const int r = r0 + tr * TR + i;
         float x[4];
-        unpack2(acc[i][0], x[0], x[1]);
-        unpack2(acc[i][1], x[2], x[3]);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) x[j] *= p.scale_log2;
+        for (int j = 0; j < 4; ++j) {
+          float even, odd;
+          unpack2(acc[i / 2][j], even, odd);
+          x[j] = (i & 1 ? odd : even) * p.scale_log2;
+        }
         if (SCORES) {
 #pragma unroll
           for (int j = 0; j < 4; ++j) sum[j] += exp2f(x[j] - lse_s[tr * TR + i]);
@@ -222,16 +227,20 @@ __global__ void __launch_bounds__(kGenThreads, 2) logit_tiles_kernel(const Score
   }
 }
 
-// grid (blocks of 4 * kGenSumThreads prefix keys of the longest sequence, H_kv, batch), block kGenSumThreads, dynamic
-// shared memory rows floats: scores from stored logits.  Four keys per thread; the row normalisers are merged from the
-// partials by every CTA for itself (a few hundred kilobytes from the L2), which saves a launch between the two.
+// grid (blocks of kGenSumKeys prefix keys of the longest sequence, H_kv, batch), block kGenSumThreads, dynamic shared
+// memory rows floats: scores from stored logits.  Latency is what it has to hide (a thread's loads are strided by whole
+// rows): four keys per thread, the rows dealt round to the CTA's four groups of threads in batches of eight loads, the
+// groups' sums added in a fixed order.  The row normalisers are merged from the partials by every CTA for itself (a few
+// hundred kilobytes from the L2), which saves a launch between the two.
 __global__ void __launch_bounds__(kGenSumThreads) scores_of_logits_kernel(const ScoreParams p) {
   extern __shared__ float lse_all[];
+  __shared__ float4 part[kGenSumGroups - 1][kGenSumKeys / 4];
   pdl_trigger();
   const int h = blockIdx.y, b = blockIdx.z, P = p.seq.prefix[b];
-  const int i0 = (blockIdx.x * kGenSumThreads + threadIdx.x) * 4;
+  const int kt = threadIdx.x % (kGenSumKeys / 4), grp = threadIdx.x / (kGenSumKeys / 4);
+  const int i0 = blockIdx.x * kGenSumKeys + kt * 4;
   pdl_wait();
-  if (blockIdx.x * kGenSumThreads * 4 >= P) return;
+  if (blockIdx.x * kGenSumKeys >= P) return;
   const int64_t head = static_cast<int64_t>(b) * p.num_kv_heads + h;
   const int t0 = p.seq.stat_off[b], t1 = p.seq.stat_off[b + 1];
   const int64_t step = static_cast<int64_t>(p.num_kv_heads) * p.rows;
@@ -255,30 +264,34 @@ __global__ void __launch_bounds__(kGenSumThreads) scores_of_logits_kernel(const 
     lse_all[r] = m + log2f(z) + p.log2_group;
   }
   __syncthreads();
-  if (i0 >= P) return;
-  const float* x = p.logits + head * p.rows * p.ld_logits + i0;
   float s[4] = {0.f, 0.f, 0.f, 0.f};
-  int r = 0;
-  for (; r + 8 <= p.rows; r += 8) {
-    float4 v[8];
+  if (i0 < P) {
+    const float* x = p.logits + head * p.rows * p.ld_logits + i0;
+    for (int r0 = grp; r0 < p.rows; r0 += 8 * kGenSumGroups) {
+      float4 v[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = __ldcs(reinterpret_cast<const float4*>(x + (r + u) * p.ld_logits));
+      for (int u = 0; u < 8; ++u) {
+        const int r = r0 + u * kGenSumGroups;
+        v[u] = r < p.rows ? __ldcg(reinterpret_cast<const float4*>(x + r * p.ld_logits)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const float l = lse_all[r + u];
-      s[0] += exp2f(v[u].x - l);
-      s[1] += exp2f(v[u].y - l);
-      s[2] += exp2f(v[u].z - l);
-      s[3] += exp2f(v[u].w - l);
+      for (int u = 0; u < 8; ++u) {
+        const int r = r0 + u * kGenSumGroups;
+        const float l = r < p.rows ? lse_all[r] : INFINITY;
+        s[0] += exp2f(v[u].x - l);
+        s[1] += exp2f(v[u].y - l);
+        s[2] += exp2f(v[u].z - l);
+        s[3] += exp2f(v[u].w - l);
+      }
     }
   }
-  for (; r < p.rows; ++r) {
-    const float4 v = *reinterpret_cast<const float4*>(x + r * p.ld_logits);
-    const float l = lse_all[r];
-    s[0] += exp2f(v.x - l);
-    s[1] += exp2f(v.y - l);
-    s[2] += exp2f(v.z - l);
-    s[3] += exp2f(v.w - l);
+  if (grp > 0) part[grp - 1][kt] = make_float4(s[0], s[1], s[2], s[3]);
+  __syncthreads();
+  if (grp > 0) return;
+#pragma unroll
+  for (int q = 0; q < kGenSumGroups - 1; ++q) {
+    const float4 o = part[q][kt];
+    s[0] += o.x; s[1] += o.y; s[2] += o.z; s[3] += o.w;
   }
 #pragma unroll
   for (int j = 0; j < 4; ++j)

@@ -68,6 +68,8 @@ struct SelectParams {
   int32_t pieces;           // 16-byte pieces per row = d * elem_bytes / 16
   int32_t log_pieces;       // log2 of that
   int32_t vec;              // score rows start on 16-byte boundaries
+  int32_t flat_cap;         // floats in front of a CTA's candidate list in shared memory (a multiple of 4)
+  int32_t common_rows;      // lists of more rows than this take one bound for the whole cluster
   int32_t paged;            // kept rows go to page slots of k_out / v_out through pt instead of packed rows
   PageTable pt;
 };
@@ -460,17 +462,20 @@ __global__ void __launch_bounds__(kSelThreads, 1) pool_select_kernel(const Selec
 // What shortens the chain:
 //   * a thread takes runs of eight consecutive positions, so pooling is a handful of 16-byte shared-memory reads (the
 //     staged scores are padded by 16 bytes per 128 so that these do not conflict) and position order is thread order;
-//   * the lower bound of the k-th key comes from one histogram pass over the runs' maxima, linear over their range.  A
-//     run counts with the number of its positions that hold its maximum (pooled scores come in plateaus), so that the
-//     bound lets through about k positions of the CTA;
+//   * the lower bound of the k-th key comes from one histogram pass over the runs' maxima on an absolute scale.  A run
+//     counts with the number of its positions that hold its maximum (pooled scores come in plateaus), so that the bound
+//     lets through about k positions.  Short lists take a bound per CTA (about k candidates each); for long ones the
+//     CTAs' histograms are added up first, one cluster barrier more, and about k candidates are left in all;
 //   * every CTA of the cluster finishes on its own: it reads the candidates of all (distributed shared memory), finds
-//     the threshold, and emits and copies the rows of its own slice.  There is one full cluster barrier (two when the
-//     list is long and the copy is dealt out evenly) and no trip through global memory;
+//     the threshold, and emits and copies the rows of its own slice.  There is one full cluster barrier (up to three
+//     when the list is long) and no trip through global memory;
 //   * the exact threshold is searched inside [largest bound of the CTAs, largest key], ten bits a pass, and finished by
 //     a warp as soon as at most 32 candidates are left in the bin (mostly after the first pass).
 constexpr int kSelBinsLin = 1024;          // bins of a linear histogram: ten bits of the key range
 constexpr int kSelRun = 8;                 // consecutive positions of a thread
 constexpr int kSelClusterSlice = 8192;     // a cluster doubles (up to 8 CTAs) while its slices are longer than this
+constexpr int kSelCopyBytes = 128 << 10;   // ... or while a CTA would copy more than this and SMs are idle
+constexpr int kSelCommonCandidates = 4096; // more expected candidates (k per CTA) than this: one bound for the cluster
 constexpr int kSelEvenRows = 1024;         // lists of at least this many rows are copied by the whole cluster evenly
 
 // Position i of the staged scores in shared memory: four floats of padding after every 32.
@@ -482,8 +487,9 @@ template <int THREADS>
 __device__ __forceinline__ bool sel_find_from_top(const uint32_t* hist, uint32_t* rows, uint32_t want, uint32_t& digit,
                                                   uint32_t& above) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int kRowsPerWarp = kSelBinsLin / THREADS;       // a row: 32 bins
 #pragma unroll
-  for (int r = 0; r < kSelBinsLin / THREADS; ++r) {
+  for (int r = 0; r < kRowsPerWarp; ++r) {
     const int row = warp + r * (THREADS / 32);
     const uint32_t sum = __reduce_add_sync(0xffffffffu, hist[row * 32 + lane]);
     if (lane == 0) rows[row] = sum;
@@ -510,6 +516,14 @@ __device__ __forceinline__ bool sel_find_from_top(const uint32_t* hist, uint32_t
   above = __shfl_sync(0xffffffffu, bs - bin, b);
   return true;
 }
+
+// Bin of a key for the candidate bound: an absolute scale (the same in every CTA of a cluster), 32 bins an octave over the
+// 32 octaves below 2^6 (scores lie between 0 and alpha); what lies below or above goes to the first and last bin.
+constexpr uint32_t kSelBinBase = 0x80000000u | ((127u + 6u - 32u) << 23);      // key of 2^-26
+__device__ __forceinline__ uint32_t sel_bin(uint32_t key) {
+  return key < kSelBinBase ? 0u : min((key - kSelBinBase) >> 18, static_cast<uint32_t>(kSelBinsLin - 1));
+}
+__device__ __forceinline__ uint32_t sel_bin_edge(uint32_t bin) { return bin == 0 ? 0u : kSelBinBase + (bin << 18); }
 
 // Pooled keys of eight consecutive positions; x[4 + j] is position j of the run.
 template <int R, bool AVG>
@@ -556,15 +570,17 @@ __device__ __forceinline__ void sel_pool_run(const float* raw, int at, int radiu
 
 // Dynamic shared memory of an instance for slices of `slice` positions (a multiple of 32).
 __host__ __device__ constexpr size_t sel_smem_floats(int slice) { return static_cast<size_t>(slice + 2 * kSelHalo) * 9 / 8 + 4; }
-__host__ __device__ constexpr size_t sel_smem_bytes(int slice) { return sel_smem_floats(slice) * 4 + static_cast<size_t>(slice) * 8; }
+constexpr size_t kSelSmemMax = 208 * 1024;
 
-// grid (cluster * H_kv, batch), cluster (cluster, 1, 1), block THREADS, dynamic shared memory sel_smem_bytes(slice).
+// grid (cluster * H_kv, batch), cluster (cluster, 1, 1), block THREADS, dynamic shared memory flat_cap floats and
+// eight bytes per position of a slice.
 // RUNS runs of eight positions per thread: a CTA takes at most THREADS * RUNS * 8 positions.
 template <int THREADS, int RUNS, bool AVG>
 __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kernel(const SelectParams p) {
   constexpr int WARPS = THREADS / 32;
   extern __shared__ __align__(16) uint8_t sel_dyn[];
-  __shared__ uint32_t hist[2][kSelBinsLin];
+  __shared__ uint32_t hist[2][kSelBinsLin];                 // [0]: read by the whole cluster when the bound is a common one
+  __shared__ uint32_t local[2][kSelBinsLin];                // threshold search
   __shared__ uint32_t rows[32];
   __shared__ uint32_t warp_a[WARPS], warp_b[WARPS], warp_c[WARPS], warp_d[WARPS];
   __shared__ uint32_t few[32], few_n;
@@ -586,8 +602,8 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
   const int64_t row0 = p.seq.row_off[b] + static_cast<int64_t>(h) * count;
   int32_t* out = p.indices + row0;
   float* raw = reinterpret_cast<float*>(sel_dyn);           // staged scores; later keys of all candidates, then own list
-  const int flat_cap = static_cast<int>(sel_smem_floats(slice));
-  uint2* list = reinterpret_cast<uint2*>(sel_dyn + sel_smem_floats(slice) * 4);   // own candidates (key, position)
+  const int flat_cap = p.flat_cap;
+  uint2* list = reinterpret_cast<uint2*>(sel_dyn + static_cast<size_t>(flat_cap) * 4);   // own candidates (key, position)
 
   for (int i = tid; i < 2 * kSelBinsLin; i += THREADS) (&hist[0][0])[i] = 0;
   if (tid == 0) few_n = 0;
@@ -628,7 +644,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
 
     // ---- pool, and each run's largest key with the number of its positions that hold it
     uint32_t key[RUNS][kSelRun], tmax[RUNS], weight[RUNS];
-    uint32_t mx = 0, mn = 0xffffffffu;
+    uint32_t mx = 0;
 #pragma unroll
     for (int r = 0; r < RUNS; ++r) {
       const int at = (r * THREADS + tid) * kSelRun;
@@ -643,40 +659,52 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
         for (int j = 0; j < kSelRun; ++j)
           if (at + j < len && key[r][j] == tmax[r]) ++weight[r];
         mx = max(mx, tmax[r]);
-        mn = min(mn, tmax[r]);
+        atomicAdd(&hist[0][sel_bin(tmax[r])], weight[r]);
       }
     }
     mx = __reduce_max_sync(full, mx);
-    mn = __reduce_min_sync(full, mn);
-    if (lane == 0) { warp_a[warp] = mx; warp_b[warp] = mn; }
-    __syncthreads();
-    mx = __reduce_max_sync(full, warp_a[lane & (WARPS - 1)]);
-    mn = __reduce_min_sync(full, warp_b[lane & (WARPS - 1)]);
+    if (lane == 0) warp_a[warp] = mx;
 
     // ---- lower bound of the k-th key, candidates in position order
-    uint32_t bound = 0;
-    if (len > 0) {
-      const int shift = max(0, 22 - __clz(mx - mn));        // (mx - mn) >> shift < 1024
+    const bool common = C > 1 && k > p.common_rows;         // uniform over the cluster
+    if (common) {
+      cluster.sync();
+      for (int i = tid; i < kSelBinsLin; i += THREADS) {
+        uint32_t sum = 0;
 #pragma unroll
-      for (int r = 0; r < RUNS; ++r)
-        if (weight[r]) atomicAdd(&hist[0][(tmax[r] - mn) >> shift], weight[r]);
-      __syncthreads();
+        for (int c = 0; c < kSelMaxCluster; ++c) sum += c < C ? cluster.map_shared_rank(&hist[0][0], c)[i] : 0u;
+        hist[1][i] = sum;
+      }
+    }
+    __syncthreads();
+    uint32_t bound = 0;
+    {
       uint32_t digit, above;
-      bool found = sel_find_from_top<THREADS>(hist[0], rows, static_cast<uint32_t>(k), digit, above);
-      if (!found && k < len) {                              // large budgets: every position counts
+      if (sel_find_from_top<THREADS>(hist[common ? 1 : 0], rows, static_cast<uint32_t>(k), digit, above)) {
+        bound = sel_bin_edge(digit);
+      } else if (common || k < len) {                       // the plateaus do not add up to k: count every position
+        if (common) cluster.sync(); else __syncthreads();   // everybody has read the first counts
+        for (int i = tid; i < 2 * kSelBinsLin; i += THREADS) (&hist[0][0])[i] = 0;
+        __syncthreads();
 #pragma unroll
         for (int r = 0; r < RUNS; ++r) {
           const int at = (r * THREADS + tid) * kSelRun;
 #pragma unroll
           for (int j = 0; j < kSelRun; ++j)
-            if (at + j < len && key[r][j] >= mn) atomicAdd(&hist[1][(key[r][j] - mn) >> shift], 1u);
+            if (at + j < len) atomicAdd(&hist[0][sel_bin(key[r][j])], 1u);
+        }
+        if (common) {
+          cluster.sync();
+          for (int i = tid; i < kSelBinsLin; i += THREADS) {
+            uint32_t sum = 0;
+#pragma unroll
+            for (int c = 0; c < kSelMaxCluster; ++c) sum += c < C ? cluster.map_shared_rank(&hist[0][0], c)[i] : 0u;
+            hist[1][i] = sum;
+          }
         }
         __syncthreads();
-        found = sel_find_from_top<THREADS>(hist[1], rows, static_cast<uint32_t>(k), digit, above);
-        __syncthreads();
-        for (int i = tid; i < kSelBinsLin; i += THREADS) hist[1][i] = 0;
+        if (sel_find_from_top<THREADS>(hist[common ? 1 : 0], rows, static_cast<uint32_t>(k), digit, above)) bound = sel_bin_edge(digit);
       }
-      if (found) bound = mn + (digit << shift);
     }
     uint32_t c2 = 0;                                        // candidates of the runs, 16 bits each
 #pragma unroll
@@ -710,8 +738,9 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
         }
       }
     }
+    mx = __reduce_max_sync(full, warp_a[lane & (WARPS - 1)]);
     if (tid == 0) pub = make_uint4(static_cast<uint32_t>(M), bound, mx, 0u);
-    for (int i = tid; i < kSelBinsLin; i += THREADS) hist[0][i] = 0;
+    for (int i = tid; i < 2 * kSelBinsLin; i += THREADS) (&local[0][0])[i] = 0;
     if (C == 1) __syncthreads(); else cluster.sync();       // candidates of the whole cluster are in place
 
     // ---- the threshold T (k-th largest key) and how many ties at T are taken
@@ -744,7 +773,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
     int shift = max(0, 22 - __clz(top - base));
     uint32_t span = 0xffffffffu;                            // keys base .. base + span take part
     for (int pass = 0;; ++pass) {
-      uint32_t* hc = hist[pass & 1];
+      uint32_t* hc = local[pass & 1];
       for (int j = tid; j < N; j += THREADS) {
         uint32_t x;
         if (pass == 0) {
@@ -787,7 +816,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
       }
       span = (1u << shift) - 1u;
       shift = max(0, shift - 10);
-      for (int i = tid; i < kSelBinsLin; i += THREADS) hist[(pass + 1) & 1][i] = 0;
+      for (int i = tid; i < kSelBinsLin; i += THREADS) local[(pass + 1) & 1][i] = 0;
       __syncthreads();
     }
 
