@@ -31,7 +31,8 @@ std::atomic<int> g_test_withhold_attend{0};  // 1: the withheld K tile, in the w
 std::atomic<int> g_test_two_sweeps{0};     // 1: never take the single-sweep kernel for short contexts
 
 constexpr size_t kAlign = 256;
-constexpr int kPartialChunk = 128;   // keys per two partial slots at least (sizes the workspace): chunks of 64 keys or more
+constexpr int kPartialChunk = 128;   // keys per partial slot of the fp32-pipe path (sizes the workspace)
+static_assert(kPartialChunk == kGenTile, "one partial per tile");
 constexpr size_t kMaxLogitBytes = size_t{256} << 20;   // fp32-pipe path: logits are kept between its passes up to this size
 
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
@@ -164,7 +165,7 @@ Workspace carve(const pkv_config* c, int batch, int max_n, void* base) {
   const size_t chunks = (static_cast<size_t>(max_n) + kPartialChunk - 1) / kPartialChunk;
   w.status = reinterpret_cast<uint32_t*>(take(kAlign));
   w.lse2 = reinterpret_cast<float*>(take(heads * rows * sizeof(float)));
-  // fp32-pipe sweep: 2 slots per chunk and head; tensor-core sweep: kTcStatSlots slots per segment, one segment
+  // fp32-pipe path: a slot per tile of 128 keys and head (room for two); tensor-core sweep: kTcStatSlots slots per segment, one segment
   // per run of a CTA over a head (at most CTAs + heads of them), whatever the context length
   const size_t partial_slots =
       tc_eligible(c) ? (static_cast<size_t>(kTcMaxGrid) + heads) * kTcStatSlots : heads * chunks * 2;
@@ -301,8 +302,9 @@ int device_sm_count() {
 }
 
 // ---------------------------------------------------------------- scores
-template <typename T, int D, int ROWS, int KEYS>
+template <typename T, int D, int ROWS, int TR, int TK>
 int launch_logit_tiles(ScoreParams& sp, int batch, cudaStream_t st) {
+  constexpr int KEYS = kGenTile;
   constexpr int kSmem = gen_smem_bytes<D, ROWS, KEYS>();
   const int sms = device_sm_count();
   if (sms <= 0) return PKV_ERR_CUDA;
@@ -310,14 +312,14 @@ int launch_logit_tiles(ScoreParams& sp, int batch, cudaStream_t st) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return PKV_ERR_CUDA;
   if (dev >= 64 || !attr_done[dev]) {
-    if (cudaFuncSetAttribute(logit_tiles_kernel<T, D, ROWS, KEYS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess ||
-        cudaFuncSetAttribute(logit_tiles_kernel<T, D, ROWS, KEYS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
+    if (cudaFuncSetAttribute(logit_tiles_kernel<T, D, ROWS, KEYS, TR, TK, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess ||
+        cudaFuncSetAttribute(logit_tiles_kernel<T, D, ROWS, KEYS, TR, TK, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
       return PKV_ERR_CUDA;
     if (dev < 64) attr_done[dev] = true;
   }
   const bool given = sp.lse_in != sp.lse2;           // normalisers supplied by the caller: no statistics
-  // Tiles per chunk: as many as keep the busiest of the CTA slots (two to an SM) as short as possible; a chunk loads
-  // the window queries once and writes one partial per row.  With several row blocks a chunk is one tile.
+  // Tiles per CTA: as many as keep the busiest of the CTA slots (two to an SM) as short as possible (the window queries
+  // are loaded once per CTA).  With several row blocks it is one tile.
   auto tiles_of = [&](int b, bool prefix) { return ((prefix ? sp.seq.prefix[b] : sp.seq.n[b]) + KEYS - 1) / KEYS; };
   sp.chunk_tiles = 1;
   if (sp.rows <= ROWS) {
@@ -329,20 +331,22 @@ int launch_logit_tiles(ScoreParams& sp, int batch, cudaStream_t st) {
       if (ct == 1 || cost <= best) { best = cost; sp.chunk_tiles = ct; }
     }
   }
-  int stat_chunks = 0, score_chunks = 0;
+  int stat_chunks = 0, score_chunks = 0, tiles = 0;
   for (int b = 0; b < batch; ++b) {
     sp.seq.stat_off[b] = stat_chunks;
     sp.seq.score_off[b] = score_chunks;
+    sp.seq.tile_off[b] = tiles;
+    tiles += tiles_of(b, false);
     stat_chunks += (tiles_of(b, false) + sp.chunk_tiles - 1) / sp.chunk_tiles;
     score_chunks += (tiles_of(b, true) + sp.chunk_tiles - 1) / sp.chunk_tiles;
   }
   sp.seq.stat_off[batch] = stat_chunks;
   sp.seq.score_off[batch] = score_chunks;
-  sp.slots_per_chunk = 1;
+  sp.seq.tile_off[batch] = tiles;
   sp.log2_group = std::log2(static_cast<float>(sp.group));
   if (sp.stats_only || given || sp.rows > 8192) sp.logits = nullptr;   // (scores_of_logits keeps the normalisers in shared memory)
   if (!given) {
-    launch_pdl(logit_tiles_kernel<T, D, ROWS, KEYS, false>, dim3(stat_chunks, sp.num_kv_heads), kGenThreads, kSmem, st, sp);
+    launch_pdl(logit_tiles_kernel<T, D, ROWS, KEYS, TR, TK, false>, dim3(stat_chunks, sp.num_kv_heads), kGenThreads, kSmem, st, sp);
     mark(st, "rowstats_generic");
     if (!sp.logits) {
       launch_pdl(combine_stats_kernel, dim3((sp.rows + 31) / 32, sp.num_kv_heads, batch), kCombineThreads, 0, st, sp, sp.log2_group);
@@ -356,7 +360,7 @@ int launch_logit_tiles(ScoreParams& sp, int batch, cudaStream_t st) {
     launch_pdl(scores_of_logits_kernel, dim3((max_p + kGenSumKeys - 1) / kGenSumKeys, sp.num_kv_heads, batch), kGenSumThreads,
                static_cast<size_t>(sp.rows) * sizeof(float), st, sp);
   } else {
-    launch_pdl(logit_tiles_kernel<T, D, ROWS, KEYS, true>, dim3(score_chunks, sp.num_kv_heads), kGenThreads, kSmem, st, sp);
+    launch_pdl(logit_tiles_kernel<T, D, ROWS, KEYS, TR, TK, true>, dim3(score_chunks, sp.num_kv_heads), kGenThreads, kSmem, st, sp);
   }
   mark(st, "scores_generic");
   return check_launch();
@@ -366,10 +370,10 @@ int launch_logit_tiles(ScoreParams& sp, int batch, cudaStream_t st) {
 template <typename T, int D>
 int launch_scores_generic(ScoreParams& sp, int batch, cudaStream_t st) {
   if constexpr (sizeof(T) == 4) {
-    if (sp.rows <= 32) return launch_logit_tiles<T, D, 32, 128>(sp, batch, st);
-    if (sp.rows <= 64) return launch_logit_tiles<T, D, 64, 64>(sp, batch, st);
+    if (sp.rows <= 32) return launch_logit_tiles<T, D, 32, 4, 4>(sp, batch, st);
+    if (sp.rows <= 64) return launch_logit_tiles<T, D, 64, 4, 8>(sp, batch, st);
   }
-  return launch_logit_tiles<T, D, 128, 64>(sp, batch, st);
+  return launch_logit_tiles<T, D, 128, 8, 8>(sp, batch, st);
 }
 
 // ---------------------------------------------------------------- tensor-core scores

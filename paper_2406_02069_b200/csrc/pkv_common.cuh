@@ -21,6 +21,7 @@ struct SeqTable {
   int64_t row_off[PKV_MAX_BATCH];        // first packed output row of sequence b
   int32_t stat_off[PKV_MAX_BATCH + 1];   // running sum of key chunks per sequence (row statistics sweep)
   int32_t score_off[PKV_MAX_BATCH + 1];  // running sum of prefix key tiles per sequence (score sweep)
+  int32_t tile_off[PKV_MAX_BATCH + 1];   // fp32-pipe path: running sum of key tiles per sequence (partial statistics)
 };
 
 // Strided view of a [batch][head][token][d] tensor.
@@ -48,6 +49,12 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ float to_float(float x) { return x; }
 __device__ __forceinline__ float to_float(__nv_bfloat16 x) { return __bfloat162float(x); }
 __device__ __forceinline__ float to_float(__half x) { return __half2float(x); }
+
+__device__ __forceinline__ float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 
 // Packed pairs of fp32 (one instruction for two multiply-adds, adds or multiplications): they halve the issue slots of
 // whatever the fp32 pipe is fed with.

@@ -7,17 +7,17 @@
 // The score of a key mixes softmax rows that each have their own normaliser, so the normalisers must be known before
 // any score can be formed:
 //   logit_tiles<STATS>   x_ri = q_r . k_i * log2(e) / sqrt(d) of a block of window rows and a chunk of keys, tile by tile;
-//                        per row the maximum and the sum of 2^(x - max) -> partial (max, sum), and x itself to the
-//                        workspace when that has room for it (w.logits)
+//                        per row and tile the maximum and the sum of 2^(x - max) -> partial (max, sum), and x itself to
+//                        the workspace when that has room for it (w.logits)
 //   scores_of_logits     s_i = sum_r 2^(x_ri - lse2[r] - log2 G) from the stored x; merges a head's partials first
 //   logit_tiles<SCORES>  the same sum straight from the tiles, with the normalisers known (the caller's, or those of
 //                        combine_stats): when x was not stored
-// Both ways form x with the same sequence of operations (one multiply-add chain over the channels per logit).
+// Both ways form x with the same sequence of operations.
 //
-// What bounds it: 2 R n d flops per KV head on the fp32 pipe (128 multiply-adds per clock and SM).  Storing x (4 R n
-// bytes, mostly in the L2) costs a quarter of forming it again.  A tile is a register-blocked product: 256 threads with
-// 8 x 4 (4 x 4) logits each, fed by 16-byte shared-memory reads of channel-major Q and K, two logits per packed
-// multiply-add, so that the pipe and not the reads are the limit.
+// What bounds it: 2 R n d flops per KV head on the fp32 pipe (a loop of packed multiply-adds reaches 63 TFLOP/s on this
+// device, scalar ones 50).  Storing x (4 R n bytes, mostly in the L2) costs a quarter of forming it again.  A tile is a
+// register-blocked product: 256 threads with 8 x 8 (4 x 8, 4 x 4) logits each.  At 8 x 4 the 16-byte shared-memory reads
+// (four wavefronts each) and not the multiply-adds were the limit, whichever way the operands lay.
 #pragma once
 
 #include "pkv_common.cuh"
@@ -25,7 +25,7 @@
 namespace pkv {
 
 constexpr int kGenThreads = 256;
-constexpr int kGenMinTile = 64;      // fewest keys per tile (a chunk of partial statistics is at least one tile)
+constexpr int kGenTile = 128;        // keys per tile: one (max, sum) per row and tile
 constexpr int kGenSumThreads = 256;  // scores_of_logits: threads per CTA,
 constexpr int kGenSumKeys = 256;     // keys per CTA (four per thread),
 constexpr int kGenSumGroups = kGenSumThreads * 4 / kGenSumKeys;   // and groups of threads that share the rows
@@ -36,7 +36,7 @@ struct ScoreParams {
   int32_t num_kv_heads, group, rows;     // rows = group * alpha
   float scale_log2;                      // log2(e) / sqrt(d)
   float2* partial;                       // [sum_b chunks_b][slots_per_chunk][H_kv][rows] (max, sum)
-  int32_t slots_per_chunk;               // partial slots each chunk writes (1 here, 2 for the tensor-core sweep)
+  int32_t slots_per_chunk;               // partial slots each chunk writes (tensor-core sweep)
   float* lse2;                           // [batch][H_kv][rows]
   const float* lse_in;                   // normalisers the score sweep reads: lse2, or the caller's
   float lse_scale, lse_add;              // applied on load: (1, 0), or (log2 e, log2 G) for natural-log input
@@ -48,7 +48,7 @@ struct ScoreParams {
                                          // CTA + head for every run of a CTA over one head's chunks
   float* logits;                         // fp32-pipe path: [batch][H_kv][rows][ld_logits] x values, or null
   int64_t ld_logits;
-  int32_t chunk_tiles;                   // tiles per chunk (1 when there are several row blocks)
+  int32_t chunk_tiles;                   // tiles per CTA (1 when there are several row blocks)
   float log2_group;
 };
 
@@ -71,158 +71,188 @@ __device__ __forceinline__ float4 gen_load4(const __half* p) {
 template <int W>
 __device__ __forceinline__ int gen_at(int c, int x) { return c * W + (x ^ (((c >> 2) & 7) << 2)); }
 
-// Fills a channel-major tile from `count` rows (row(x) = address of row x; the columns from `count` to W become zero).
-template <int W, int D, typename F>
-__device__ __forceinline__ void gen_fill(float* tile, int count, F&& row) {
-  constexpr int kSteps = W * D / 4 / kGenThreads, kBatch = kSteps < 4 ? kSteps : 4;
-  static_assert(W * D / 4 % kGenThreads == 0, "tile of whole steps");
-  const int dq = threadIdx.x & 7;                            // 32 channels = 8 lanes of 4
+constexpr int kGenSlice = 32;        // channels of K in shared memory at a time (two buffers)
+
+// 32 channels of W rows, global memory -> registers -> channel-major tile: eight lanes take a row's 32 channels.
+template <int W>
+struct GenSlice {
+  static constexpr int kSteps = W * kGenSlice / 4 / kGenThreads;
+  static_assert(W * kGenSlice / 4 % kGenThreads == 0, "slice of whole steps");
+  float4 f[kSteps];
+  // row(x) = address of the first of the 32 channels of row x; rows from `count` on are zero
+  template <typename F>
+  __device__ __forceinline__ void load(int count, F&& row) {
 #pragma unroll
-  for (int s0 = 0; s0 < kSteps; s0 += kBatch) {
-    float4 f[kBatch];
-#pragma unroll
-    for (int s = 0; s < kBatch; ++s) {
-      const int e = (s0 + s) * (kGenThreads / 8) + threadIdx.x / 8;        // (channel block of 32, column), column fastest
-      const int x = e % W, cb = e / W;
-      f[s] = x < count ? gen_load4(row(x) + cb * 32 + dq * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s = 0; s < kSteps; ++s) {
+      const int x = s * (kGenThreads / 8) + threadIdx.x / 8;
+      f[s] = x < count ? gen_load4(row(x) + (threadIdx.x & 7) * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
+  }
+  __device__ __forceinline__ void store(float* tile) const {       // tile: the slice's first channel
+    const int c = (threadIdx.x & 7) * 4;
 #pragma unroll
-    for (int s = 0; s < kBatch; ++s) {
-      const int e = (s0 + s) * (kGenThreads / 8) + threadIdx.x / 8;
-      const int x = e % W, c = (e / W) * 32 + dq * 4;
+    for (int s = 0; s < kSteps; ++s) {
+      const int x = s * (kGenThreads / 8) + threadIdx.x / 8;
       tile[gen_at<W>(c, x)] = f[s].x;
       tile[gen_at<W>(c + 1, x)] = f[s].y;
       tile[gen_at<W>(c + 2, x)] = f[s].z;
       tile[gen_at<W>(c + 3, x)] = f[s].w;
     }
   }
-}
+};
 
 // grid (chunks over all sequences, H_kv), block kGenThreads, dynamic shared memory gen_smem_bytes.
-// ROWS x KEYS: window rows and keys of a tile; TR rows x 4 keys per thread.
+// ROWS x KEYS: window rows and keys of a tile; TR rows x TK keys per thread, in groups of four.
 template <int D, int ROWS, int KEYS>
-__host__ __device__ constexpr int gen_smem_bytes() { return (ROWS + KEYS) * D * 4; }
+__host__ __device__ constexpr int gen_smem_bytes() { return (ROWS * D + 2 * KEYS * kGenSlice) * 4; }
 
-template <typename T, int D, int ROWS, int KEYS, bool SCORES>
+template <typename T, int D, int ROWS, int KEYS, int TR, int TK, bool SCORES>
 __global__ void __launch_bounds__(kGenThreads, 2) logit_tiles_kernel(const ScoreParams p) {
-  constexpr int KT = KEYS / 4;                               // threads along the keys
+  constexpr int KT = KEYS / TK;                              // threads along the keys
   constexpr int RT = kGenThreads / KT;                       // threads along the rows
-  constexpr int TR = ROWS / RT;                              // rows per thread
-  static_assert(KT <= 32 && TR % 4 == 0, "a warp holds whole rows of threads");
+  constexpr int SLICES = D / kGenSlice;
+  static_assert(KT <= 32 && RT * TR == ROWS && TR % 4 == 0 && TK % 4 == 0, "whole rows of threads in a warp");
   extern __shared__ __align__(16) float gen_smem[];
   float* qs = gen_smem;                                      // channel-major [D][ROWS]
-  float* ks = gen_smem + ROWS * D;                           // channel-major [D][KEYS]
+  float* ks = gen_smem + ROWS * D;                           // channel-major [2][kGenSlice][KEYS]
   __shared__ float lse_s[SCORES ? ROWS : 1];
-  __shared__ __align__(16) float part[SCORES ? RT : 1][SCORES ? KEYS : 4];
+  __shared__ float part[SCORES ? RT : 1][SCORES ? KEYS : 1];
   pdl_trigger();
   const int32_t* off = SCORES ? p.seq.score_off : p.seq.stat_off;
   const int h = blockIdx.y, b = find_sequence(off, p.seq.batch, blockIdx.x);
   const int n = p.seq.n[b], alpha = p.seq.alpha, P = p.seq.prefix[b];
   const int keys = SCORES ? P : n;
-  const int tile0 = (blockIdx.x - off[b]) * p.chunk_tiles, tile1 = min(tile0 + p.chunk_tiles, (keys + KEYS - 1) / KEYS);
+  const int tiles = (keys + KEYS - 1) / KEYS;
+  const int tile0 = (blockIdx.x - off[b]) * p.chunk_tiles, tile1 = min(tile0 + p.chunk_tiles, tiles);
+  const int64_t tile_id = (SCORES ? 0 : p.seq.tile_off[b]) + tile0;
   const T* kbase = static_cast<const T*>(p.k.ptr) + b * p.k.sb + h * p.k.sh;
   const T* qbase = static_cast<const T*>(p.q.ptr) + b * p.q.sb + static_cast<int64_t>(h * p.group) * p.q.sh;
   const int tk = threadIdx.x % KT, tr = threadIdx.x / KT;
   const int blocks = (p.rows + ROWS - 1) / ROWS;
   const int64_t head = static_cast<int64_t>(b) * p.num_kv_heads + h;
+  auto key_of = [&](int j) { return (j / 4) * (KT * 4) + tk * 4 + j % 4; };        // column of a tile
+  auto row_of = [&](int i) { return (i / 4) * (RT * 4) + tr * 4 + i % 4; };
+  const int steps = (tile1 - tile0) * SLICES;
+  GenSlice<KEYS> next;
+  auto load_slice = [&](int it) {                            // slice it of the chunk
+    const int key0 = (tile0 + it / SLICES) * KEYS;
+    const T* base = kbase + static_cast<int64_t>(key0) * p.k.st + (it % SLICES) * kGenSlice;
+    next.load(min(KEYS, n - key0), [&](int x) { return base + x * p.k.st; });
+  };
   pdl_wait();
 
-  float m[TR], z[TR];                                        // STATS: per row over this thread's keys of the chunk
+  float sum[SCORES ? TK : 1];                                // SCORES: of this thread's keys, over the row blocks
 #pragma unroll
-  for (int i = 0; i < TR; ++i) { m[i] = -INFINITY; z[i] = 0.f; }
-  for (int t = tile0; t < tile1; ++t) {
-    const int key0 = t * KEYS;
-    float sum[4] = {0.f, 0.f, 0.f, 0.f};                     // SCORES: of this thread's keys
-    for (int rb = 0; rb < blocks; ++rb) {
-      const int r0 = rb * ROWS;
-      __syncthreads();                                       // the tiles before have been read
-      if (blocks > 1 || t == tile0) {
-        gen_fill<ROWS, D>(qs, min(ROWS, p.rows - r0), [&](int x) {
-          const int r = r0 + x;
-          return qbase + (r / alpha) * p.q.sh + (r % alpha) * p.q.st;
-        });
-        if (SCORES)
-          for (int x = threadIdx.x; x < ROWS; x += kGenThreads)
-            lse_s[x] = r0 + x < p.rows ? fmaf(p.lse_in[head * p.rows + r0 + x], p.lse_scale, p.lse_add) : INFINITY;
-      }
-      if (rb == 0) gen_fill<KEYS, D>(ks, min(KEYS, n - key0), [&](int x) { return kbase + static_cast<int64_t>(key0 + x) * p.k.st; });
-      __syncthreads();
-      unsigned long long acc[TR / 2][4];                     // pairs of rows: the queries come in pairs as they are, only the
-#pragma unroll                                               // four keys have to be doubled
-      for (int i = 0; i < TR / 2; ++i)
+  for (int j = 0; j < (SCORES ? TK : 1); ++j) sum[j] = 0.f;
+  for (int rb = 0; rb < blocks; ++rb) {
+    const int r0 = rb * ROWS;
+    if (rb > 0) __syncthreads();                             // the block before has been read
+    load_slice(0);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
-#pragma unroll 32
-      for (int c = 0; c < D; ++c) {
-        const float4 kf = *reinterpret_cast<const float4*>(ks + gen_at<KEYS>(c, tk * 4));
-        const unsigned long long k2[4] = {pack2(kf.x, kf.x), pack2(kf.y, kf.y), pack2(kf.z, kf.z), pack2(kf.w, kf.w)};
+    for (int s = 0; s < SLICES; ++s) {
+      GenSlice<ROWS> q;
+      q.load(min(ROWS, p.rows - r0), [&](int x) {
+        const int r = r0 + x;
+        return qbase + (r / alpha) * p.q.sh + (r % alpha) * p.q.st + s * kGenSlice;
+      });
+      q.store(qs + s * kGenSlice * ROWS);
+    }
+    if (SCORES)
+      for (int x = threadIdx.x; x < ROWS; x += kGenThreads)
+        lse_s[x] = r0 + x < p.rows ? fmaf(p.lse_in[head * p.rows + r0 + x], p.lse_scale, p.lse_add) : INFINITY;
+    next.store(ks);
+    __syncthreads();
+    unsigned long long acc[TR / 2][TK];                      // pairs of rows: the queries come in pairs as they are, the
+#pragma unroll                                               // keys are doubled
+    for (int i = 0; i < TR / 2; ++i)
 #pragma unroll
-        for (int i = 0; i < TR; i += 4) {
-          const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(qs + gen_at<ROWS>(c, tr * TR + i));
+      for (int j = 0; j < TK; ++j) acc[i][j] = 0ull;
+    for (int it = 0; it < steps; ++it) {
+      if (it + 1 < steps) load_slice(it + 1);                // arrives under this slice's multiply-adds
+      const float* kc = ks + (it & 1) * (kGenSlice * KEYS);
+      const float* qc = qs + (it % SLICES) * (kGenSlice * ROWS);
+#pragma unroll 8
+      for (int c = 0; c < kGenSlice; ++c) {
+        ulonglong2 q[TR / 4];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            acc[i / 2][j] = fma2(q.x, k2[j], acc[i / 2][j]);
-            acc[i / 2 + 1][j] = fma2(q.y, k2[j], acc[i / 2 + 1][j]);
-          }
+        for (int i = 0; i < TR / 4; ++i) q[i] = *reinterpret_cast<const ulonglong2*>(qc + gen_at<ROWS>(c, i * RT * 4 + tr * 4));
+#pragma unroll
+        for (int g = 0; g < TK / 4; ++g) {
+          const float4 kf = *reinterpret_cast<const float4*>(kc + gen_at<KEYS>(c, g * KT * 4 + tk * 4));
+          const unsigned long long k2[4] = {pack2(kf.x, kf.x), pack2(kf.y, kf.y), pack2(kf.z, kf.z), pack2(kf.w, kf.w)};
+#pragma unroll
+          for (int i = 0; i < TR / 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              acc[2 * i][4 * g + j] = fma2(q[i].x, k2[j], acc[2 * i][4 * g + j]);
+              acc[2 * i + 1][4 * g + j] = fma2(q[i].y, k2[j], acc[2 * i + 1][4 * g + j]);
+            }
         }
       }
-      const int i0 = key0 + tk * 4;                          // this thread's keys
-#pragma unroll
-      for (int i = 0; i < TR; ++i) {
-        const int r = r0 + tr * TR + i;
-        float x[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          float even, odd;
-          unpack2(acc[i / 2][j], even, odd);
-          x[j] = (i & 1 ? odd : even) * p.scale_log2;
-        }
-        if (SCORES) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) sum[j] += exp2f(x[j] - lse_s[tr * TR + i]);
-          continue;
-        }
-        if (r >= p.rows) continue;
-        if (p.logits && i0 < P)
-          *reinterpret_cast<float4*>(p.logits + (head * p.rows + r) * p.ld_logits + i0) = make_float4(x[0], x[1], x[2], x[3]);
-        const int last = min(P + r % alpha, n - 1);          // row (g, j) sees keys 0 .. P + j that exist here
-        if (i0 + 3 > last) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) x[j] = i0 + j <= last ? x[j] : -INFINITY;
-        }
-        const float mn = fmaxf(fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3])), m[i]);
-        if (mn > -INFINITY) {
-          z[i] = z[i] * exp2f(m[i] - mn) + ((exp2f(x[0] - mn) + exp2f(x[1] - mn)) + (exp2f(x[2] - mn) + exp2f(x[3] - mn)));
-          m[i] = mn;
-        }
-      }
-      if (!SCORES && (blocks > 1 || t + 1 == tile1)) {       // the rows' statistics over the chunk: merge the threads along the keys
+      if (it % SLICES == SLICES - 1) {                       // the tile's logits are complete
+        const int t = tile0 + it / SLICES, key0 = t * KEYS;
+        const bool masked = key0 + KEYS - 1 > min(P, n - 1); // some key of the tile is hidden from some row
 #pragma unroll
         for (int i = 0; i < TR; ++i) {
+          const int r = r0 + row_of(i);
+          float x[TK];
 #pragma unroll
-          for (int o = 1; o < KT; o <<= 1) {
-            const float m2 = __shfl_xor_sync(0xffffffffu, m[i], o), z2 = __shfl_xor_sync(0xffffffffu, z[i], o);
-            const float mm = fmaxf(m[i], m2);
-            if (mm > -INFINITY) z[i] = z[i] * exp2f(m[i] - mm) + z2 * exp2f(m2 - mm);
-            m[i] = mm;
+          for (int j = 0; j < TK; ++j) {
+            float even, odd;
+            unpack2(acc[i / 2][j], even, odd);
+            x[j] = (i & 1 ? odd : even) * p.scale_log2;
           }
-          const int r = r0 + tr * TR + i;
+          if (SCORES) {
+#pragma unroll
+            for (int j = 0; j < TK; ++j) sum[SCORES ? j : 0] += exp2f(x[j] - lse_s[SCORES ? row_of(i) : 0]);
+            continue;
+          }
+          if (p.logits && r < p.rows) {
+            float* to = p.logits + (head * p.rows + r) * p.ld_logits + key0;
+#pragma unroll
+            for (int j = 0; j < TK; j += 4)                  // within the row: ld_logits is a multiple of every tile
+              *reinterpret_cast<float4*>(to + key_of(j)) = make_float4(x[j], x[j + 1], x[j + 2], x[j + 3]);
+          }
+          if (masked) {
+            const int last = min(P + r % alpha, n - 1);      // row (g, j) sees keys 0 .. P + j that exist here
+#pragma unroll
+            for (int j = 0; j < TK; ++j) x[j] = key0 + key_of(j) <= last ? x[j] : -INFINITY;
+          }
+          float m = x[0];
+#pragma unroll
+          for (int j = 1; j < TK; ++j) m = fmaxf(m, x[j]);
+#pragma unroll
+          for (int o = 1; o < KT; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+          const float ref = m == -INFINITY ? 0.f : m;        // arguments at most 0, one of them 0: what flushes to zero does
+          float z = 0.f;                                     // not count
+#pragma unroll
+          for (int j = 0; j < TK; ++j) z += ex2(x[j] - ref);
+#pragma unroll
+          for (int o = 1; o < KT; o <<= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
           if (tk == 0 && r < p.rows)
-            p.partial[(static_cast<int64_t>(blockIdx.x) * p.num_kv_heads + h) * p.rows + r] = make_float2(m[i], z[i]);
-          m[i] = -INFINITY;
-          z[i] = 0.f;
+            p.partial[((tile_id + it / SLICES) * p.num_kv_heads + h) * p.rows + r] = make_float2(m, z);
+        }
+#pragma unroll
+        for (int i = 0; i < TR / 2; ++i)
+#pragma unroll
+          for (int j = 0; j < TK; ++j) acc[i][j] = 0ull;
+        if (SCORES && rb + 1 == blocks) {                    // the rows of a key are spread over RT threads
+#pragma unroll
+          for (int j = 0; j < TK; ++j) {
+            part[SCORES ? tr : 0][SCORES ? key_of(j) : 0] = sum[SCORES ? j : 0];
+            sum[SCORES ? j : 0] = 0.f;
+          }
+          __syncthreads();
+          for (int x = threadIdx.x; x < KEYS; x += kGenThreads) {
+            float s = 0.f;
+#pragma unroll
+            for (int q = 0; q < RT; ++q) s += part[SCORES ? q : 0][SCORES ? x : 0];
+            if (key0 + x < P) p.scores[head * p.ld_scores + key0 + x] = s;
+          }
         }
       }
-    }
-    if (SCORES) {                                            // the rows of a key are spread over RT threads
-      *reinterpret_cast<float4*>(&part[tr][tk * 4]) = make_float4(sum[0], sum[1], sum[2], sum[3]);
+      if (it + 1 < steps) next.store(ks + ((it + 1) & 1) * (kGenSlice * KEYS));
       __syncthreads();
-      for (int x = threadIdx.x; x < KEYS; x += kGenThreads) {
-        float s = 0.f;
-#pragma unroll
-        for (int q = 0; q < RT; ++q) s += part[q][x];
-        if (key0 + x < P) p.scores[head * p.ld_scores + key0 + x] = s;
-      }
     }
   }
 }
@@ -242,7 +272,7 @@ __global__ void __launch_bounds__(kGenSumThreads) scores_of_logits_kernel(const 
   pdl_wait();
   if (blockIdx.x * kGenSumKeys >= P) return;
   const int64_t head = static_cast<int64_t>(b) * p.num_kv_heads + h;
-  const int t0 = p.seq.stat_off[b], t1 = p.seq.stat_off[b + 1];
+  const int t0 = p.seq.tile_off[b], t1 = p.seq.tile_off[b + 1];
   const int64_t step = static_cast<int64_t>(p.num_kv_heads) * p.rows;
   for (int r = threadIdx.x; r < p.rows; r += kGenSumThreads) {
     const float2* src = p.partial + static_cast<int64_t>(h) * p.rows + r;
@@ -311,7 +341,7 @@ __global__ void __launch_bounds__(kCombineThreads) combine_stats_kernel(const Sc
   const int h = blockIdx.y, b = blockIdx.z;
   const int rl = threadIdx.x & 31, sg = threadIdx.x >> 5;
   const int r = blockIdx.x * 32 + rl;
-  int t0 = p.seq.stat_off[b] * p.slots_per_chunk, t1 = p.seq.stat_off[b + 1] * p.slots_per_chunk;
+  int t0 = p.seq.tile_off[b], t1 = p.seq.tile_off[b + 1];   // fp32-pipe path: one slot per tile
   int64_t slot_stride = static_cast<int64_t>(p.num_kv_heads) * p.rows;
   int64_t first = static_cast<int64_t>(h) * p.rows;
   if (p.stat_grid > 0) {
