@@ -453,6 +453,7 @@ int launch_scores_tc(const pkv_config* c, const pkv_tensor& q, const pkv_tensor&
   tp.early = (c->flags & PKV_FLAG_INPUTS_FINAL) != 0 &&
              !(overlaps_recent_output(q, batch, c->num_q_heads, c->window, D, 2) ||
                overlaps_recent_output(k, batch, c->num_kv_heads, max_n, D, 2));
+  tp.prefetch_tiles = kTcPrefetchBytes / (kTcTileKeysA * D * 2);
   const long long test_wait = g_test_wait_clocks.load();
   tp.wait_clocks = test_wait > 0 ? test_wait : kTcWaitCycles;
   tp.withhold = g_test_withhold.load();
@@ -546,9 +547,11 @@ int launch_scores_tc(const pkv_config* c, const pkv_tensor& q, const pkv_tensor&
       mark(st, "combine_stats");
     } else {
       tp.merge = 1;                              // sweep B merges the partials of its heads itself
+      tp.early = 1;                              // sweep A lets B start after it has waited for Q and K
     }
   }
   if (sp.stats_only) return check_launch();
+  if (!tp.merge) tp.prefetch_tiles = kTcPrefetchBytes / (kTcTileKeysB * D * 2);
   launch_pdl(score_tc_kernel<D, 1>, grid_b, kTcThreads, TcSmem<D>::kTotal, st, q_map, k_map_b, tp);
   mark(st, "scores_tc");
   return check_launch();

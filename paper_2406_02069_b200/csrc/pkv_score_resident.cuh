@@ -122,7 +122,12 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  if (!p.early) pdl_wait();
+  if (!p.early) {                                              // meanwhile: this CTA's keys into the L2 (a prefetch hands no
+    if (threadIdx.x == 0)                                      // data to anybody, whoever may still write them)
+      for (int t = tile0; t < tile1; ++t)
+        for (int half = 0; half < kHalves; ++half) tma_prefetch_4d(&k_map, half * 64, t * kRsTileKeys, h, b);
+    pdl_wait();
+  }
 
   if (warp == 0) {
     // =========================================================== TMA producer

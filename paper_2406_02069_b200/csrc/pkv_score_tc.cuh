@@ -41,6 +41,7 @@ constexpr int kTcTileKeysA = 256;       // keys per K tile in sweep A (the N of 
 constexpr int kTcTileKeysB = 128;       // keys per K tile in sweep B (the M of its MMAs)
 constexpr int kTcKBytes = 128 * 1024;   // shared memory given to K stages (2 x 64 KB or 4 x 32 KB at d = 128)
 constexpr int kTcMaxGrid = 256;         // CTAs of a sweep at most (the workspace holds a partial segment per CTA)
+constexpr int kTcPrefetchBytes = 448 * 1024;   // of K per CTA into the L2 ahead of the wait: half the L2 in all
 constexpr int kTcMaxRows = 256;         // window rows (G * alpha) the tensor-core path takes
 constexpr long long kTcWaitCycles = 1ll << 31;   // bound of any one wait, in SM clocks
 constexpr int kTcStatSlots = 4;         // partial (reference, sum) slots per run segment and row in sweep A, at most
@@ -53,8 +54,10 @@ struct TcParams {
   int32_t num_kv_heads, group, rows;      // rows = group * alpha (R)
   int32_t rows_pad;             // R rounded up to 32
   int32_t fp16;                 // 1: Q and K hold binary16, 0: bfloat16 (both operands always share the type)
-  int32_t early;                // 1: the caller vouches for Q and K (PKV_FLAG_INPUTS_FINAL) and they are not outputs
-                                // of a library kernel that may still run: start reading them at once
+  int32_t early;                // 1: start reading Q and K at once.  Sweep A: the caller vouches for them
+                                // (PKV_FLAG_INPUTS_FINAL) and they are not outputs of a library kernel that may still
+                                // run.  Sweep B behind a sweep A of the same call: A has waited for them
+  int32_t prefetch_tiles;       // K tiles a CTA brings into the L2 while it waits for the kernels ahead
   int32_t withhold;             // test aid: CTA 0 of sweep A never loads its last K tile (its waits then run out)
   long long wait_clocks;        // bound of any one wait, in SM clocks
   int32_t row_blocks;           // ceil(R / 128): M-blocks of sweep A
@@ -135,6 +138,13 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
       "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
       ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
       : "memory");
+}
+
+// Brings a box of a tensor into the L2.
+__device__ __forceinline__ void tma_prefetch_4d(const CUtensorMap* map, int c0, int c1, int c2, int c3) {
+  asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global [%0, {%1, %2, %3, %4}];" ::"l"(reinterpret_cast<uint64_t>(map)), "r"(c0),
+               "r"(c1), "r"(c2), "r"(c3)
+               : "memory");
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -353,7 +363,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   const bool second_half = SWEEP == 0 || split_b < p.rows_pad; // do the groups 2, 3 have columns to read?
 
   // ---- set-up (shared memory and TMEM only: it may overlap the tail of the preceding kernel)
-  pdl_trigger();
+  // Sweep A lets sweep B start once it knows itself that Q and K are complete, so that B can read them at once.
+  if (SWEEP == 1 || p.early) pdl_trigger();
   if (threadIdx.x == 0) {
     for (int s = 0; s < 4; ++s) { mbar_init(k_full(s), 1); mbar_init(k_empty(s), 1); }
     const uint32_t consumers = second_half ? 8 : 4;            // epilogue warps that read one accumulator stage
@@ -377,13 +388,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  // Neither sweep waits here for the kernels ahead of it in the stream: copies and MMAs touch only the caller's Q
-  // and K, so they start at once, beside the tail of those kernels.  Sweep A waits just before its first write
-  // (its partials), sweep B's epilogue just before it reads the row normalisers; both wait again before they end.
-  // (When Q or K may be the output of a library kernel still in flight, e.g. a compact cache that is compressed
-  // again, the host clears `early` and the kernel waits here like any other.)
-  if (!p.early) pdl_wait();
-
   // ---- this CTA's contiguous range of work items
   const int32_t* off = SWEEP == 0 ? p.seq.stat_off : p.seq.score_off;
   const int chunk_tiles = SWEEP == 0 ? p.chunk_tiles_a : p.chunk_tiles_b;
@@ -393,6 +397,27 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   const int item1 = item0 + per + (static_cast<int>(blockIdx.x) < rem ? 1 : 0);
   // keys an item of sequence b spans: sweep A covers all n keys, sweep B the prefix only
   auto span_keys = [&](int b) { return SWEEP == 0 ? p.seq.n[b] : p.seq.prefix[b]; };
+
+  // Copies and MMAs touch only the caller's Q and K.  With `early` they start at once, beside the tail of the kernels
+  // ahead in the stream; then sweep A waits just before its first write (its partials), sweep B's epilogue just before
+  // it reads the row normalisers, and both wait again before they end.  Without it the kernel waits here, and spends
+  // the time on bringing its first K tiles into the L2: a prefetch hands no data to anybody, so it does not matter
+  // whether the kernels ahead still write them.
+  if (!p.early) {
+    if (warp == 0 && lane == 0) {
+      int left = p.prefetch_tiles;
+      for (int ii = 0; ii < item1 - item0 && left > 0; ++ii) {
+        const TcItem w = tc_item(off, p.seq.batch, p.num_kv_heads, kReverse ? item1 - 1 - ii : item0 + ii);
+        const int tile0 = w.c * chunk_tiles, tile1 = min(tile0 + chunk_tiles, (span_keys(w.b) + kTileKeys - 1) / kTileKeys);
+        for (int tt = 0; tt < tile1 - tile0 && left > 0; ++tt, --left) {
+          const int t = kReverse ? tile1 - 1 - tt : tile0 + tt;
+          for (int half = 0; half < L::kHalves; ++half) tma_prefetch_4d(&k_map, half * 64, t * kTileKeys, w.h, w.b);
+        }
+      }
+    }
+    pdl_wait();
+    if (SWEEP == 0) pdl_trigger();
+  }
 
   if (warp == 0) {
     // =========================================================== TMA producer
