@@ -216,8 +216,8 @@ int pyramidkv_score_window(const pkv_config* cfg, pkv_tensor q_win, pkv_tensor k
  * synchronise the whole device) is not acceptable.
  *   - Every GPU on which the library is loaded holds the 8 MiB until the process ends.
  *   - The problem must fit.  With 16-bit inputs and (H_q / H_kv) * alpha <= 256 rows per KV head the
- *     scratch is (256 + batch * H_kv) * 32 * (H_q / H_kv) * alpha bytes plus the row normalisers,
- *     whatever the context length (2.2 MB for one 8-head sequence with 256 rows); other shapes run
+ *     scratch is (256 + batch * H_kv) * 8 * (H_q / H_kv) * alpha bytes plus the row normalisers,
+ *     whatever the context length (0.6 MB for one 8-head sequence with 256 rows); other shapes run
  *     on the fp32-pipe kernels and need batch * H_kv * ceil(n_max / 128) * (H_q / H_kv) * alpha * 16
  *     bytes.  Larger problems are refused with PKV_ERR_STATIC_SCRATCH before anything is enqueued;
  *     use pyramidkv_score_window with a workspace for those.

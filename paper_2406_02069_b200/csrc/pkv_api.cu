@@ -165,10 +165,10 @@ Workspace carve(const pkv_config* c, int batch, int max_n, void* base) {
   const size_t chunks = (static_cast<size_t>(max_n) + kPartialChunk - 1) / kPartialChunk;
   w.status = reinterpret_cast<uint32_t*>(take(kAlign));
   w.lse2 = reinterpret_cast<float*>(take(heads * rows * sizeof(float)));
-  // fp32-pipe path: a slot per tile of 128 keys and head (room for two); tensor-core sweep: kTcStatSlots slots per segment, one segment
+  // fp32-pipe path: a slot per tile of 128 keys and head (room for two); tensor-core sweep: one segment
   // per run of a CTA over a head (at most CTAs + heads of them), whatever the context length
   const size_t partial_slots =
-      tc_eligible(c) ? (static_cast<size_t>(kTcMaxGrid) + heads) * kTcStatSlots : heads * chunks * 2;
+      tc_eligible(c) ? static_cast<size_t>(kTcMaxGrid) + heads : heads * chunks * 2;
   w.partial = reinterpret_cast<float2*>(take(partial_slots * rows * sizeof(float2)));
   w.score_scratch_bytes = off;
   w.ld_scores = static_cast<int64_t>((static_cast<size_t>(max_n) + 63) / 64 * 64);
@@ -434,11 +434,10 @@ int launch_scores_tc(const pkv_config* c, const pkv_tensor& q, const pkv_tensor&
       return PKV_ERR_CUDA;
     if (dev < 64) attr_done[dev] = true;
   }
-  alignas(64) CUtensorMap q_map, k_map_a, k_map_b;
+  alignas(64) CUtensorMap q_map, k_map;
   const bool fp16 = c->dtype == PKV_DTYPE_FP16;
   if (!make_map(&q_map, q, fp16, D, c->window, c->num_q_heads, batch, c->window, sp.group) ||
-      !make_map(&k_map_a, k, fp16, D, max_n, c->num_kv_heads, batch, kTcTileKeysA, 1) ||
-      !make_map(&k_map_b, k, fp16, D, max_n, c->num_kv_heads, batch, kTcTileKeysB, 1))
+      !make_map(&k_map, k, fp16, D, max_n, c->num_kv_heads, batch, kTcTileKeys, 1))
     return PKV_ERR_CUDA;
 
   TcParams tp{};
@@ -453,7 +452,7 @@ int launch_scores_tc(const pkv_config* c, const pkv_tensor& q, const pkv_tensor&
   tp.early = (c->flags & PKV_FLAG_INPUTS_FINAL) != 0 &&
              !(overlaps_recent_output(q, batch, c->num_q_heads, c->window, D, 2) ||
                overlaps_recent_output(k, batch, c->num_kv_heads, max_n, D, 2));
-  tp.prefetch_tiles = kTcPrefetchBytes / (kTcTileKeysA * D * 2);
+  tp.prefetch_tiles = kTcPrefetchBytes / (kTcTileKeys * D * 2);
   const long long test_wait = g_test_wait_clocks.load();
   tp.wait_clocks = test_wait > 0 ? test_wait : kTcWaitCycles;
   tp.withhold = g_test_withhold.load();
@@ -485,20 +484,19 @@ int launch_scores_tc(const pkv_config* c, const pkv_tensor& q, const pkv_tensor&
     }
     return ct;
   };
-  tp.chunk_tiles_a = pick(kTcTileKeysA, false);
-  tp.chunk_tiles_b = pick(kTcTileKeysB, true);
+  tp.chunk_tiles_a = pick(kTcTileKeys, false);
+  tp.chunk_tiles_b = pick(kTcTileKeys, true);
   int stat_items = 0, score_items = 0;
   for (int b = 0; b < batch; ++b) {
     tp.seq.stat_off[b] = stat_items;
     tp.seq.score_off[b] = score_items;
-    stat_items += ((sp.seq.n[b] + kTcTileKeysA - 1) / kTcTileKeysA + tp.chunk_tiles_a - 1) / tp.chunk_tiles_a;
-    score_items += ((sp.seq.prefix[b] + kTcTileKeysB - 1) / kTcTileKeysB + tp.chunk_tiles_b - 1) /
+    stat_items += ((sp.seq.n[b] + kTcTileKeys - 1) / kTcTileKeys + tp.chunk_tiles_a - 1) / tp.chunk_tiles_a;
+    score_items += ((sp.seq.prefix[b] + kTcTileKeys - 1) / kTcTileKeys + tp.chunk_tiles_b - 1) /
                    tp.chunk_tiles_b;
   }
   tp.seq.stat_off[batch] = stat_items;
   tp.seq.score_off[batch] = score_items;
   sp.seq = tp.seq;
-  sp.slots_per_chunk = tc_stat_slots(tp.row_blocks);  // partial slots each run segment of sweep A holds
 
   const int grid_a = static_cast<int>(std::min<long long>(std::min(sms, kTcMaxGrid),
                                                           static_cast<long long>(stat_items) * sp.num_kv_heads));
@@ -532,14 +530,14 @@ int launch_scores_tc(const pkv_config* c, const pkv_tensor& q, const pkv_tensor&
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if ((small ? cudaLaunchKernelEx(&cfg, score_resident_kernel<D, kRsStagesShort>, q_map, k_map_b, tp)
-               : cudaLaunchKernelEx(&cfg, score_resident_kernel<D, kRsStages>, q_map, k_map_b, tp)) != cudaSuccess)
+    if ((small ? cudaLaunchKernelEx(&cfg, score_resident_kernel<D, kRsStagesShort>, q_map, k_map, tp)
+               : cudaLaunchKernelEx(&cfg, score_resident_kernel<D, kRsStages>, q_map, k_map, tp)) != cudaSuccess)
       return PKV_ERR_CUDA;
     mark(st, "scores_resident");
     return check_launch();
   }
   if (sp.lse_in == sp.lse2) {                    // normalisers not supplied: sweep A
-    launch_pdl(score_tc_kernel<D, 0>, grid_a, kTcThreads, TcSmem<D>::kTotal, st, q_map, k_map_a, tp);
+    launch_pdl(score_tc_kernel<D, 0>, grid_a, kTcThreads, TcSmem<D>::kTotal, st, q_map, k_map, tp);
     mark(st, "rowstats_tc");
     if (sp.stats_only) {                         // the normalisers themselves are wanted: merge kernel
       launch_pdl(combine_stats_kernel, dim3((sp.rows + 31) / 32, sp.num_kv_heads, batch), kCombineThreads, 0, st, sp,
@@ -551,8 +549,7 @@ int launch_scores_tc(const pkv_config* c, const pkv_tensor& q, const pkv_tensor&
     }
   }
   if (sp.stats_only) return check_launch();
-  if (!tp.merge) tp.prefetch_tiles = kTcPrefetchBytes / (kTcTileKeysB * D * 2);
-  launch_pdl(score_tc_kernel<D, 1>, grid_b, kTcThreads, TcSmem<D>::kTotal, st, q_map, k_map_b, tp);
+  launch_pdl(score_tc_kernel<D, 1>, grid_b, kTcThreads, TcSmem<D>::kTotal, st, q_map, k_map, tp);
   mark(st, "scores_tc");
   return check_launch();
 }

@@ -258,7 +258,7 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
     }
   } else if (warp == 1) {
     // =========================================================== MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       // all window rows at once; with two halves always 256 columns, so that the second half holds zeros (Q rows
       // beyond R are zero) rather than what the stage held before
       const uint32_t idesc_s = instr_desc_16bit(kAtTileKeys, halves == 2 ? 256 : p.rows_pad, p.fp16);

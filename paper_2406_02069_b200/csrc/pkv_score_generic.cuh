@@ -35,16 +35,15 @@ struct ScoreParams {
   SeqTable seq;                          // stat_off / score_off count chunks of chunk_tiles tiles
   int32_t num_kv_heads, group, rows;     // rows = group * alpha
   float scale_log2;                      // log2(e) / sqrt(d)
-  float2* partial;                       // [sum_b chunks_b][slots_per_chunk][H_kv][rows] (max, sum)
-  int32_t slots_per_chunk;               // partial slots each chunk writes (tensor-core sweep)
+  float2* partial;                       // [sum_b tiles_b][H_kv][rows] (max, sum), or see stat_grid
   float* lse2;                           // [batch][H_kv][rows]
   const float* lse_in;                   // normalisers the score sweep reads: lse2, or the caller's
   float lse_scale, lse_add;              // applied on load: (1, 0), or (log2 e, log2 G) for natural-log input
   float* scores;                         // [batch][H_kv][ld]
   int64_t ld_scores;
   int32_t stats_only;                    // host side: stop after the row normalisers (no score sweep)
-  int32_t stat_grid;                     // 0: partial is [chunk][slot][H_kv][rows] (fp32-pipe sweep).  > 0: CTAs of
-                                         // the tensor-core sweep, which writes [segment][slot][rows] with segment =
+  int32_t stat_grid;                     // 0: partial is [tile][H_kv][rows] (fp32-pipe sweep).  > 0: CTAs of
+                                         // the tensor-core sweep, which writes [segment][rows] with segment =
                                          // CTA + head for every run of a CTA over one head's chunks
   float* logits;                         // fp32-pipe path: [batch][H_kv][rows][ld_logits] x values, or null
   int64_t ld_logits;
@@ -355,8 +354,8 @@ __global__ void __launch_bounds__(kCombineThreads) combine_stats_kernel(const Sc
     const int c0 = i0 < edge ? i0 / (per + 1) : rem + (i0 - edge) / per;
     const int c1 = i1 < edge ? i1 / (per + 1) : rem + (i1 - edge) / per;
     const int hg = b * p.num_kv_heads + h;
-    t0 = (c0 + hg) * p.slots_per_chunk;
-    t1 = (c1 + hg + 1) * p.slots_per_chunk;
+    t0 = c0 + hg;
+    t1 = c1 + hg + 1;
     slot_stride = p.rows;
     first = 0;
   }

@@ -157,7 +157,7 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
     }
   } else if (warp == 1) {
     // =========================================================== MMA issuer
-    if (lane == 0 && T > 0) {
+    if (elect_one() && T > 0) {
       const uint32_t idesc = instr_desc_16bit(kRsTileKeys, kRsRows, p.fp16);
       bool ok = mbar_wait(q_full, 0, abort_flag, p.wait_clocks);
       for (int t = 0; t < T && ok; ++t) {

@@ -3,7 +3,7 @@
 // Two sweeps over K, because the score of a key sums softmax rows that each have
 // their own normaliser (known only after a whole row has been seen):
 //
-//   sweep A  D[row r][key i] = Q K^T   (A operand = 128 window rows, B operand = 256-key tile)
+//   sweep A  D[row r][key i] = Q K^T   (A operand = 128 window rows, B operand = 128-key tile)
 //            TMEM lane = window row, so each epilogue thread owns one row and keeps its
 //            reference exponent and sum of 2^x privately: no cross-thread reduction at all.
 //   sweep B  D[key i][row r] = K Q^T   (A operand = 128-key tile, B operand = all window rows)
@@ -11,15 +11,13 @@
 //            2^(x_ri - lse2_r) over the rows r, reading lse2 from shared memory.
 //
 // x = (q . k) * log2(e) / sqrt(d).  Operands arrive by plain per-CTA TMA loads into
-// 128-byte-swizzled shared memory; tcgen05.mma accumulates in TMEM (two to four
-// accumulator stages of up to 256 columns); epilogue warps read TMEM with tcgen05.ld.
-// Warp roles: warp 0 = TMA producer, warp 1 = MMA issuer and TMEM owner, warps 4..19 =
-// epilogue.  The exponentials bound both sweeps (16 per clock per SM); four epilogue
+// 128-byte-swizzled shared memory; tcgen05.mma accumulates in TMEM (four
+// accumulator stages of up to 128 columns); epilogue warps read TMEM with tcgen05.ld.
+// Warp roles: warp 0 = TMA producer of K, warp 1 = MMA issuer and TMEM owner, warp 2 = TMA producer of Q, warp 3 = row
+// statistics on their way out of sweep A and into sweep B, warps 4..19 = epilogue.  The exponentials bound both sweeps (16 per clock per SM); four epilogue
 // warps per scheduler are what it takes to keep that unit busy.  The 16 epilogue
-// warps form four groups (TMEM lane quarter = warp % 4, group = (warp - 4) / 4).
-// Accumulator stage u % 2 is read by the two groups g with g % 2 == u % 2, each taking
-// half of its columns, so while one pair of groups works on a stage the MMAs of the
-// next stage run.  CTAs are persistent: each takes a contiguous range of (sequence,
+// warps form four groups (TMEM lane quarter = warp % 4, group = (warp - 4) / 4), each with
+// an accumulator stage of its own, refilled while the other three compute.  CTAs are persistent: each takes a contiguous range of (sequence,
 // KV head, key chunk) work items.
 //
 // Every wait on an mbarrier is bounded.  A wait that runs out sets an abort flag in
@@ -37,17 +35,14 @@ namespace pkv {
 constexpr int kTcThreads = 640;         // 20 warps: producer, MMA issuer, 2 idle, 16 epilogue
 constexpr int kTcEpiWarp0 = 4;          // first epilogue warp
 constexpr int kTcEpiWarps = 16;         // four per scheduler, which is what keeps the exp unit fed
-constexpr int kTcTileKeysA = 256;       // keys per K tile in sweep A (the N of its MMAs)
-constexpr int kTcTileKeysB = 128;       // keys per K tile in sweep B (the M of its MMAs)
-constexpr int kTcKBytes = 128 * 1024;   // shared memory given to K stages (2 x 64 KB or 4 x 32 KB at d = 128)
+constexpr int kTcTileKeys = 128;        // keys per K tile: the N of sweep A's MMAs, the M of sweep B's
+constexpr int kTcStageCols = 128;       // TMEM columns of an accumulator stage
+constexpr int kTcStages = 4;            // accumulator stages, one per group of epilogue warps
+constexpr int kTcKBytes = 128 * 1024;   // shared memory given to K stages (4 x 32 KB at d = 128)
 constexpr int kTcMaxGrid = 256;         // CTAs of a sweep at most (the workspace holds a partial segment per CTA)
 constexpr int kTcPrefetchBytes = 448 * 1024;   // of K per CTA into the L2 ahead of the wait: half the L2 in all
 constexpr int kTcMaxRows = 256;         // window rows (G * alpha) the tensor-core path takes
 constexpr long long kTcWaitCycles = 1ll << 31;   // bound of any one wait, in SM clocks
-constexpr int kTcStatSlots = 4;         // partial (reference, sum) slots per run segment and row in sweep A, at most
-// ... and how many of them a sweep with `row_blocks` blocks of 128 window rows writes (one per epilogue warp
-// group that works on a row)
-__host__ __device__ constexpr int tc_stat_slots(int row_blocks) { return row_blocks == 2 ? 2 : 4; }
 
 struct TcParams {
   SeqTable seq;                 // stat_off / score_off count CHUNKS of chunk_tiles tiles
@@ -61,12 +56,11 @@ struct TcParams {
   int32_t withhold;             // test aid: CTA 0 of sweep A never loads its last K tile (its waits then run out)
   long long wait_clocks;        // bound of any one wait, in SM clocks
   int32_t row_blocks;           // ceil(R / 128): M-blocks of sweep A
-  int32_t chunk_tiles_a;        // 256-key tiles per work item of sweep A
-  int32_t chunk_tiles_b;        // 128-key tiles per work item of sweep B
+  int32_t chunk_tiles_a;        // key tiles per work item of sweep A
+  int32_t chunk_tiles_b;        // key tiles per work item of sweep B
   float scale_log2;             // log2(e) / sqrt(d)
-  float2* partial;              // sweep A out: [segment][slots][R] (reference exponent, sum); a segment is one
-                                // CTA's run over one (sequence, head); slots = 2 with two row blocks, 4 with
-                                // one: every epilogue warp group writes its own slot
+  float2* partial;              // sweep A out: [segment][R] (reference exponent, sum); a segment is one CTA's run over one
+                                // (sequence, head)
   const float* lse2;            // sweep B in:  [batch][H_kv][R] row normalisers (log of the row's sum of exps)
   float lse_scale, lse_add;     // lse2_r = lse2[r] * lse_scale + lse_add: (1, 0) for the library's own sweep A,
                                 // (log2 e, log2 G) for natural-log normalisers handed in by the caller
@@ -147,6 +141,14 @@ __device__ __forceinline__ void tma_prefetch_4d(const CUtensorMap* map, int c0, 
                : "memory");
 }
 
+// One lane of a converged warp, the same one each time.  The role of the MMA issuer is entered through it: an MMA takes its
+// descriptors from uniform registers, and behind a test of the lane number the compiler does not know that there is one
+// thread only and wraps every MMA in a loop over the lanes (some 100 clocks an MMA: 32k-token layer 62.6 us, 59.8 with this).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
+  return ok != 0;
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
@@ -243,7 +245,7 @@ __device__ __forceinline__ float sum_pairs(const unsigned long long (&acc)[4]) {
   return ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
 }
 // Sweep A, slow path for the same 16 logits: moves the reference exponent up to a whole number at or above the
-// running maximum first (the row's first chunk, where m = -inf, or a logit some 60 binades above the reference).
+// running maximum first (a logit some 60 binades above the reference, or one that is not finite).
 // `live` is false for threads that only keep the warp's loads aligned.
 __device__ __forceinline__ void rowstats_rescue(const uint32_t (&v)[16], float c2, bool live, float& m, float& z) {
   if (!live) return;
@@ -303,6 +305,84 @@ __device__ __forceinline__ TcItem tc_item(const int32_t* off, int batch, int hea
   return TcItem{b, local / nc, local % nc, nc};
 }
 
+// Sweep A: row r of a finished run, from the (reference, sum of 2^(x - reference)) pairs that the epilogue warps hold of it
+// ([4 groups][128 lanes]; one pair per group that works on the row's block and per copy of the rows; (-inf, 0): no key).
+__device__ __forceinline__ float2 run_row(const float2* runs, int r, bool two_blocks, int copies) {
+  float m = -INFINITY, z = 0.f;
+  const int step = two_blocks ? 2 : 1, first = two_blocks ? r >> 7 : 0;
+  for (int c = 0; c < copies; ++c) {
+    const float2* at = runs + c * (128 / copies) + (r & 127);
+    float2 o[4];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) o[g] = first + g * step < 4 ? at[(first + g * step) * 128] : make_float2(-INFINITY, 0.f);
+    const float mn = fmaxf(m, fmaxf(fmaxf(o[0].x, o[1].x), fmaxf(o[2].x, o[3].x)));
+    if (mn > -INFINITY) {
+      z = z * ex2(m - mn) + ((o[0].y * ex2(o[0].x - mn) + o[1].y * ex2(o[1].x - mn)) +
+                             (o[2].y * ex2(o[2].x - mn) + o[3].y * ex2(o[3].x - mn)));
+      m = mn;
+    }
+  }
+  return make_float2(m, z);
+}
+
+// A head's negated row normalisers into dst (-inf for the padding rows), by THREADS threads: the caller's values, or sweep
+// A's partials of this head merged, 1 to 16 lanes per row, pairwise shuffles, always in the same order.
+template <int THREADS>
+__device__ __forceinline__ void tc_normalisers(const TcParams& p, int b, int h, int tid, float* dst) {
+  const int rows_p2 = p.rows_pad <= 32 ? 32 : (p.rows_pad <= 64 ? 64 : (p.rows_pad <= 128 ? 128 : 256));
+  const int per_row = THREADS > rows_p2 ? THREADS / rows_p2 : 1;
+  const int hg = b * p.num_kv_heads + h;
+  int s0 = 0, s1 = 0;
+  if (p.merge) {
+    // sweep A's CTAs took contiguous item ranges (items ordered sequence, head, chunk): the first `rem`
+    // CTAs per + 1 items, the others per; this head's items fell to CTAs c0..c1, one segment each
+    const int nc = p.seq.stat_off[b + 1] - p.seq.stat_off[b];
+    const int total_a = p.num_kv_heads * p.seq.stat_off[p.seq.batch];
+    const int per_a = total_a / p.stat_grid, rem_a = total_a % p.stat_grid, edge = rem_a * (per_a + 1);
+    const int i0 = p.num_kv_heads * p.seq.stat_off[b] + h * nc, i1 = i0 + nc - 1;
+    const int c0 = i0 < edge ? i0 / (per_a + 1) : rem_a + (i0 - edge) / per_a;
+    const int c1 = i1 < edge ? i1 / (per_a + 1) : rem_a + (i1 - edge) / per_a;
+    s0 = c0 + hg;
+    s1 = c1 + hg + 1;
+  }
+  const int part = tid % per_row;
+  pdl_wait();                                                  // normalisers and partials are written by kernels before
+  for (int r = tid / per_row; r < rows_p2; r += THREADS / per_row) {
+    float val = -INFINITY;
+    if (p.merge) {
+      float m = -INFINITY, z = 0.f;
+      if (r < p.rows) {
+        const float2* base = p.partial + r;
+        for (int t = s0 + part; t < s1; t += 10 * per_row) {   // a batch of loads in flight
+          float2 pz[10];
+          float mn = m;
+#pragma unroll
+          for (int q = 0; q < 10; ++q)
+            pz[q] = t + q * per_row < s1 ? __ldcg(base + static_cast<int64_t>(t + q * per_row) * p.rows) : make_float2(-INFINITY, 0.f);
+#pragma unroll
+          for (int q = 0; q < 10; ++q) mn = fmaxf(mn, pz[q].x);
+          if (mn > -INFINITY) {                                // (-inf, 0) marks a segment that saw no key of this row
+            z *= ex2(m - mn);
+#pragma unroll
+            for (int q = 0; q < 10; ++q) z = fmaf(pz[q].y, ex2(pz[q].x - mn), z);
+            m = mn;
+          }
+        }
+      }
+      for (int o = 1; o < per_row; o <<= 1) {                  // both partners of a pair compute the same merged value
+        const float2 other = make_float2(__shfl_xor_sync(0xffffffffu, m, o), __shfl_xor_sync(0xffffffffu, z, o));
+        const float mm = fmaxf(m, other.x);
+        z = (m > -INFINITY ? z * ex2(m - mm) : 0.f) + (other.x > -INFINITY ? other.y * ex2(other.x - mm) : 0.f);
+        m = mm;
+      }
+      if (r < p.rows) val = -(m + __log2f(z) + p.log2_group);
+    } else if (r < p.rows) {
+      val = -fmaf(p.lse2[static_cast<int64_t>(hg) * p.rows + r], p.lse_scale, p.lse_add);
+    }
+    if (part == 0) dst[r] = val;
+  }
+}
+
 // Dynamic shared memory carve-up (bytes), all regions 1024-aligned.
 template <int D>
 struct TcSmem {
@@ -321,7 +401,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                 const TcParams p) {
   using L = TcSmem<D>;
-  constexpr int kTileKeys = SWEEP == 0 ? kTcTileKeysA : kTcTileKeysB;
+  constexpr int kTileKeys = kTcTileKeys;
   // Sweep B walks each CTA's items and tiles from the last to the first: sweep A has just read the same keys in
   // ascending order, so the end of every range is what the L2 still holds.
   constexpr bool kReverse = SWEEP == 1;
@@ -333,12 +413,14 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   uint8_t* k_s = smem + L::kKOff;
   uint8_t* misc = smem + L::kMiscOff;
   uint64_t* bars = reinterpret_cast<uint64_t*>(misc);          // [0..3] k_full, [4..7] k_empty, [8..11] t_full,
-                                                               // [12..15] t_empty, [16] q_full, [17] q_empty,
-                                                               // [18..19] x_full, [20..21] x_empty, [22] lse_full
+                                                               // [12..15] t_empty, [16..17] q_full, [18..19] q_empty,
+                                                               // [20..21] x_full, [22..23] x_empty, [24..25] n_full,
+                                                               // [26..27] n_empty, [28] meet
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 260);
   float* xch = reinterpret_cast<float*>(misc + 1024);          // sweep B: [2][128] partial sums handed between groups
   float* lse_all = reinterpret_cast<float*>(misc + 4096);      // sweep B: [2][256] -lse2 of the current / next head
+  float2* run_all = reinterpret_cast<float2*>(misc + 8192);    // sweep A: [2][4 groups][128 lanes] (reference, sum) of a run
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t bar0 = smem_u32(bars);
@@ -346,33 +428,42 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   auto k_empty = [&](int s) { return bar0 + 8u * (4 + s); };
   auto t_full = [&](int s) { return bar0 + 8u * (8 + s); };
   auto t_empty = [&](int s) { return bar0 + 8u * (12 + s); };
-  const uint32_t q_full = bar0 + 8u * 16, q_empty = bar0 + 8u * 17;
-  auto x_full = [&](int s) { return bar0 + 8u * (18 + s); };
-  auto x_empty = [&](int s) { return bar0 + 8u * (20 + s); };
-  const uint32_t lse_full = bar0 + 8u * 22;
+  auto q_full = [&](int s) { return bar0 + 8u * (16 + s); };
+  auto q_empty = [&](int s) { return bar0 + 8u * (18 + s); };
+  auto x_full = [&](int s) { return bar0 + 8u * (20 + s); };
+  auto x_empty = [&](int s) { return bar0 + 8u * (22 + s); };
+  // n: the buffers that go through warp 3, the runs' statistics in sweep A, the heads' normalisers in sweep B
+  auto n_full = [&](int s) { return bar0 + 8u * (24 + s); };
+  auto n_empty = [&](int s) { return bar0 + 8u * (26 + s); };
+  const uint32_t meet = bar0 + 8u * 28;
 
-  // Accumulator stages.  Sweep A: 256 key columns per unit (one row block x one K tile): two stages.
-  // Sweep B: rows_pad columns per unit (one K tile), rounded up to a power of two: two to four stages.
-  int stage_cols = 256;
-  if (SWEEP == 1) {
-    stage_cols = p.rows_pad <= 32 ? 32 : (p.rows_pad <= 64 ? 64 : (p.rows_pad <= 128 ? 128 : 256));
-  }
-  const int t_stages = SWEEP == 0 ? 2 : min(4, 512 / stage_cols);
-  const bool two_blocks = p.row_blocks == 2;                   // sweep A: units per K tile
-  const int split_b = ((p.rows_pad / 2) + 31) & ~31;           // sweep B: columns [0, split) and [split, rows_pad)
-  const bool second_half = SWEEP == 0 || split_b < p.rows_pad; // do the groups 2, 3 have columns to read?
+  // A unit of work is an accumulator stage of up to 128 columns: one K tile and up to 128 window rows.  With more rows a
+  // tile makes two units: sweep A takes the rows in blocks of 128, sweep B in halves (columns [0, split) and [split, R)).
+  // Each of the four groups of epilogue warps owns one stage and takes every fourth unit, so that three groups compute
+  // while the stage of the fourth is filled.  (Two stages of 256 columns with a pair of groups each left a pair idle for
+  // the 1400 clocks of the refill: 75 us of sweep A for 131072 keys x 256 rows x 8 heads, 68 with these.)
+  const bool two_blocks = p.row_blocks == 2;
+  const int split_b = two_blocks ? ((p.rows_pad / 2) + 31) & ~31 : p.rows_pad;
+  // Sweep A: with 64 (32) rows or fewer the window rows stand two (four) times in the 128 rows of the Q tile, and each
+  // copy's lanes take their share of the key columns: otherwise the sub-partitions of the padding rows would idle.
+  const int copies = SWEEP == 1 || p.rows > 64 ? 1 : (p.rows > 32 ? 2 : 4);
+  const int copy_rows = 128 / copies;
+  // Up to 128 rows: Q tiles of two heads, so that a CTA's next head is in place when its turn comes.
+  const int q_slots = p.rows <= 128 ? 2 : 1;
 
   // ---- set-up (shared memory and TMEM only: it may overlap the tail of the preceding kernel)
   // Sweep A lets sweep B start once it knows itself that Q and K are complete, so that B can read them at once.
   if (SWEEP == 1 || p.early) pdl_trigger();
   if (threadIdx.x == 0) {
     for (int s = 0; s < 4; ++s) { mbar_init(k_full(s), 1); mbar_init(k_empty(s), 1); }
-    const uint32_t consumers = second_half ? 8 : 4;            // epilogue warps that read one accumulator stage
-    for (int s = 0; s < 4; ++s) { mbar_init(t_full(s), 1); mbar_init(t_empty(s), consumers); }
-    mbar_init(q_full, 1);
-    mbar_init(q_empty, 1);
+    for (int s = 0; s < kTcStages; ++s) { mbar_init(t_full(s), 1); mbar_init(t_empty(s), 4); }
+    for (int s = 0; s < 2; ++s) { mbar_init(q_full(s), 1); mbar_init(q_empty(s), 1); }
     for (int s = 0; s < 2; ++s) { mbar_init(x_full(s), 4); mbar_init(x_empty(s), 4); }
-    mbar_init(lse_full, kTcEpiWarps);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(n_full(s), SWEEP == 0 ? kTcEpiWarps : 1);
+      mbar_init(n_empty(s), SWEEP == 0 ? 1 : kTcEpiWarps);
+    }
+    mbar_init(meet, kTcEpiWarps);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -388,6 +479,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+
   // ---- this CTA's contiguous range of work items
   const int32_t* off = SWEEP == 0 ? p.seq.stat_off : p.seq.score_off;
   const int chunk_tiles = SWEEP == 0 ? p.chunk_tiles_a : p.chunk_tiles_b;
@@ -397,18 +489,24 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   const int item1 = item0 + per + (static_cast<int>(blockIdx.x) < rem ? 1 : 0);
   // keys an item of sequence b spans: sweep A covers all n keys, sweep B the prefix only
   auto span_keys = [&](int b) { return SWEEP == 0 ? p.seq.n[b] : p.seq.prefix[b]; };
+  auto item_at = [&](int ii) { return tc_item(off, p.seq.batch, p.num_kv_heads, kReverse ? item1 - 1 - ii : item0 + ii); };
+  auto last_tile = [&](const TcItem& w) { return min((w.c + 1) * chunk_tiles, (span_keys(w.b) + kTileKeys - 1) / kTileKeys); };
 
   // Copies and MMAs touch only the caller's Q and K.  With `early` they start at once, beside the tail of the kernels
-  // ahead in the stream; then sweep A waits just before its first write (its partials), sweep B's epilogue just before
-  // it reads the row normalisers, and both wait again before they end.  Without it the kernel waits here, and spends
+  // ahead in the stream; then sweep A waits just before its first write (its partials), sweep B just before it reads
+  // the row normalisers, and both wait again before they end.  Without it the kernel waits here, and spends
   // the time on bringing its first K tiles into the L2: a prefetch hands no data to anybody, so it does not matter
   // whether the kernels ahead still write them.
   if (!p.early) {
     if (warp == 0 && lane == 0) {
       int left = p.prefetch_tiles;
+      if (item0 < item1) {
+        const TcItem w = item_at(0);
+        for (int half = 0; half < L::kHalves; ++half) tma_prefetch_4d(&q_map, half * 64, 0, w.h * p.group, w.b);
+      }
       for (int ii = 0; ii < item1 - item0 && left > 0; ++ii) {
-        const TcItem w = tc_item(off, p.seq.batch, p.num_kv_heads, kReverse ? item1 - 1 - ii : item0 + ii);
-        const int tile0 = w.c * chunk_tiles, tile1 = min(tile0 + chunk_tiles, (span_keys(w.b) + kTileKeys - 1) / kTileKeys);
+        const TcItem w = item_at(ii);
+        const int tile0 = w.c * chunk_tiles, tile1 = last_tile(w);
         for (int tt = 0; tt < tile1 - tile0 && left > 0; ++tt, --left) {
           const int t = kReverse ? tile1 - 1 - tt : tile0 + tt;
           for (int half = 0; half < L::kHalves; ++half) tma_prefetch_4d(&k_map, half * 64, t * kTileKeys, w.h, w.b);
@@ -420,26 +518,13 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   }
 
   if (warp == 0) {
-    // =========================================================== TMA producer
+    // =========================================================== TMA producer of K
     if (lane == 0) {
-      uint32_t it = 0, heads_loaded = 0;                       // it counts K tiles
-      int cur_b = -1, cur_h = -1;
+      uint32_t it = 0;                                         // K tiles
       bool ok = true;
       for (int ii = 0; ii < item1 - item0 && ok; ++ii) {
-        const int id = kReverse ? item1 - 1 - ii : item0 + ii;
-        const TcItem w = tc_item(off, p.seq.batch, p.num_kv_heads, id);
-        if (w.b != cur_b || w.h != cur_h) {
-          if (heads_loaded > 0) ok = mbar_wait(q_empty, (heads_loaded - 1) & 1, abort_flag, p.wait_clocks);
-          if (!ok) break;
-          mbar_expect_tx(q_full, static_cast<uint32_t>(p.rows) * D * 2);
-          for (int half = 0; half < L::kHalves; ++half)
-            tma_load_4d(smem_u32(q_s) + half * kTcMaxRows * 128, &q_map, q_full, half * 64, 0, w.h * p.group, w.b);
-          ++heads_loaded;
-          cur_b = w.b; cur_h = w.h;
-        }
-        const int keys = span_keys(w.b);
-        const int tile0 = w.c * chunk_tiles;
-        const int tile1 = min(tile0 + chunk_tiles, (keys + kTileKeys - 1) / kTileKeys);
+        const TcItem w = item_at(ii);
+        const int tile0 = w.c * chunk_tiles, tile1 = last_tile(w);
         for (int tt = 0; tt < tile1 - tile0 && ok; ++tt, ++it) {
           const int t = kReverse ? tile1 - 1 - tt : tile0 + tt;
           const int s = it % kKStages;
@@ -459,52 +544,75 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
         for (uint32_t j = first; j < it; ++j)
           for (uint32_t spin = 0; spin < (1u << 16) && !mbar_test(k_full(j % kKStages), (j / kKStages) & 1); ++spin)
             __nanosleep(64);
-        if (heads_loaded > 0)
-          for (uint32_t spin = 0; spin < (1u << 16) && !mbar_test(q_full, (heads_loaded - 1) & 1); ++spin) __nanosleep(64);
       }
+    }
+  } else if (warp == 2) {
+    // =========================================================== TMA producer of Q, one tile per head
+    if (lane == 0) {
+      uint32_t heads = 0;
+      int cur_b = -1, cur_h = -1;
+      bool ok = true;
+      for (int ii = 0; ii < item1 - item0 && ok; ++ii) {
+        const TcItem w = item_at(ii);
+        if (w.b == cur_b && w.h == cur_h) continue;
+        cur_b = w.b; cur_h = w.h;
+        const uint32_t slot = heads % q_slots, round = heads / q_slots;
+        ok = mbar_wait(q_empty(slot), (round & 1) ^ 1, abort_flag, p.wait_clocks);
+        if (!ok) break;
+        mbar_expect_tx(q_full(slot), static_cast<uint32_t>(copies * p.rows) * D * 2);
+        for (int half = 0; half < L::kHalves; ++half)
+          for (int c = 0; c < copies; ++c)
+            tma_load_4d(smem_u32(q_s) + half * kTcMaxRows * 128 + (slot * 128 + c * copy_rows) * 128, &q_map, q_full(slot),
+                        half * 64, 0, w.h * p.group, w.b);
+        ++heads;
+      }
+      if (!ok)
+        for (uint32_t j = heads > 2 ? heads - 2 : 0; j < heads; ++j)
+          for (uint32_t spin = 0; spin < (1u << 16) && !mbar_test(q_full(j % q_slots), (j / q_slots) & 1); ++spin)
+            __nanosleep(64);
     }
   } else if (warp == 1) {
     // =========================================================== MMA issuer
-    if (lane == 0) {
-      uint32_t it = 0, u = 0, heads_seen = 0;                  // it counts K tiles, u accumulator units
+    if (elect_one()) {
+      uint32_t it = 0, u = 0, heads = 0;                       // it counts K tiles, u accumulator units
       int cur_b = -1, cur_h = -1;
       bool ok = true;
-      const uint32_t idesc = SWEEP == 0 ? instr_desc_16bit(128, kTcTileKeysA, p.fp16)
-                                        : instr_desc_16bit(kTcTileKeysB, p.rows_pad, p.fp16);
+      const uint32_t idesc0 = SWEEP == 0 ? instr_desc_16bit(128, kTileKeys, p.fp16) : instr_desc_16bit(kTileKeys, split_b, p.fp16);
+      const uint32_t idesc1 = SWEEP == 0 || !two_blocks ? idesc0 : instr_desc_16bit(kTileKeys, p.rows_pad - split_b, p.fp16);
+      uint32_t slot = 0;
       for (int ii = 0; ii < item1 - item0 && ok; ++ii) {
-        const int id = kReverse ? item1 - 1 - ii : item0 + ii;
-        const TcItem w = tc_item(off, p.seq.batch, p.num_kv_heads, id);
+        const TcItem w = item_at(ii);
         if (w.b != cur_b || w.h != cur_h) {
-          ok = mbar_wait(q_full, heads_seen & 1, abort_flag, p.wait_clocks);
+          slot = heads % q_slots;
+          ok = mbar_wait(q_full(slot), (heads / q_slots) & 1, abort_flag, p.wait_clocks);
           if (!ok) break;
-          ++heads_seen;
+          ++heads;
           cur_b = w.b; cur_h = w.h;
         }
         // does the next item belong to another head?  then Q may be overwritten after this item's MMAs
         bool last_of_head = ii + 1 >= item1 - item0;
         if (!last_of_head) {
-          const TcItem nx = tc_item(off, p.seq.batch, p.num_kv_heads, kReverse ? id - 1 : id + 1);
+          const TcItem nx = item_at(ii + 1);
           last_of_head = nx.b != w.b || nx.h != w.h;
         }
-        const int keys = span_keys(w.b);
-        const int tile0 = w.c * chunk_tiles;
-        const int tile1 = min(tile0 + chunk_tiles, (keys + kTileKeys - 1) / kTileKeys);
+        const int tile0 = w.c * chunk_tiles, tile1 = last_tile(w);
         for (int tt = 0; tt < tile1 - tile0 && ok; ++tt, ++it) {
           const int s = it % kKStages;
           ok = mbar_wait(k_full(s), (it / kKStages) & 1, abort_flag, p.wait_clocks);
           if (!ok) break;
           const uint32_t k_addr = smem_u32(k_s) + s * kStageBytes;
-          const uint32_t q_addr = smem_u32(q_s);
-          const int units = SWEEP == 0 ? p.row_blocks : 1;
-          for (int rb = 0; rb < units && ok; ++rb, ++u) {
-            const int ts = u % t_stages;
-            ok = mbar_wait(t_empty(ts), ((u / t_stages) & 1) ^ 1, abort_flag, p.wait_clocks);
+          const uint32_t q_addr = smem_u32(q_s) + slot * 128 * 128;
+          for (int rb = 0; rb < p.row_blocks && ok; ++rb, ++u) {
+            const int ts = u % kTcStages;
+            ok = mbar_wait(t_empty(ts), ((u / kTcStages) & 1) ^ 1, abort_flag, p.wait_clocks);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t d_addr = tmem_base + ts * stage_cols;
+            const uint32_t d_addr = tmem_base + ts * kTcStageCols;
+            const uint32_t idesc = rb == 0 ? idesc0 : idesc1;
+            const int row_at = SWEEP == 0 ? rb * 128 : rb * split_b;     // first window row of the unit
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
-              const uint32_t qa = q_addr + (kk / 4) * kTcMaxRows * 128 + rb * 128 * 128 + (kk % 4) * 32;
+              const uint32_t qa = q_addr + (kk / 4) * kTcMaxRows * 128 + row_at * 128 + (kk % 4) * 32;
               const uint32_t ka = k_addr + (kk / 4) * kTileKeys * 128 + (kk % 4) * 32;
               if (SWEEP == 0) tc_mma_f16kind(d_addr, smem_desc_sw128(qa), smem_desc_sw128(ka), idesc, kk > 0);
               else tc_mma_f16kind(d_addr, smem_desc_sw128(ka), smem_desc_sw128(qa), idesc, kk > 0);
@@ -513,101 +621,156 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
           }
           if (ok) tc_commit(k_empty(s));
         }
-        if (ok && last_of_head) tc_commit(q_empty);
+        if (ok && last_of_head) tc_commit(q_empty(slot));
       }
     }
-  } else if (warp >= kTcEpiWarp0) {
+  } else if (warp == 3) {
+    // =========================================================== statistics between the sweeps, off the epilogue's path
+    // Sweep A: merges what the sixteen warps hold of a finished run and writes one (reference, sum) per window row, to
+    // the segment numbered blockIdx.x + head: along the item order either the CTA or the head advances from one run to
+    // the next, so the numbers are distinct, and a head's segments follow from the CTAs its items fall to.
+    // Sweep B: the normalisers of the CTA's second and later heads, while the epilogue works on the head before.
+    uint32_t heads = 0;
+    int cur_b = -1, cur_h = -1;
+    bool ok = true;
+    if (SWEEP == 0) pdl_wait();                                // the partials of the call before have been read
+    auto finish = [&](int b, int h) {
+      if (SWEEP == 0) {
+        const uint32_t buf = heads & 1u;
+        ok = mbar_wait(n_full(buf), (heads >> 1) & 1, abort_flag, p.wait_clocks);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) return;
+        const float2* runs = run_all + buf * 512;
+        const int64_t seg = static_cast<int64_t>(blockIdx.x) + b * p.num_kv_heads + h;
+        for (int r = lane; r < p.rows; r += 32) p.partial[seg * p.rows + r] = run_row(runs, r, two_blocks, copies);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(n_empty(buf));
+      } else if (heads > 0) {
+        const uint32_t buf = heads & 1u;
+        if (heads > 1) {
+          ok = mbar_wait(n_empty(buf), ((heads >> 1) & 1) ^ 1, abort_flag, p.wait_clocks);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) return;
+        }
+        tc_normalisers<32>(p, b, h, lane, lse_all + buf * 256);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(n_full(buf));
+      }
+      ++heads;
+    };
+    for (int ii = 0; ii < item1 - item0 && ok; ++ii) {
+      const TcItem w = item_at(ii);
+      if (w.b == cur_b && w.h == cur_h) continue;
+      if (SWEEP == 0 && ii > 0) finish(cur_b, cur_h);          // a run that has ended; the last one is the epilogue's
+      cur_b = w.b; cur_h = w.h;
+      if (SWEEP == 1) finish(w.b, w.h);
+    }
+  } else {
     // =========================================================== epilogue
     const int e = warp - kTcEpiWarp0;
     const int quarter = warp & 3;               // TMEM lanes 32*quarter .. +31 are this warp's
     const int grp = e >> 2;                     // 0..3
-    const int par = grp & 1;                    // this group reads the units u with u % 2 == par
-    const int ch = grp >> 1;                    // ... and this half of their columns
+    const int blk = two_blocks ? grp & 1 : 0;   // row block (half) of its units
+    const int par = grp >> 1;                   // two blocks: parity of its K tiles
     const int lane_row = quarter * 32 + lane;   // TMEM lane of this thread
     const float c2 = p.scale_log2;
-    uint32_t u = 0, mine = 0;                   // units seen by the CTA / units this group's pair has read
-    uint32_t heads_seen = 0;                    // sweep B: (sequence, head) changes so far
+    uint32_t u = 0, mine = 0;                   // units seen by the CTA / read by this group
+    uint32_t heads = 0;                         // (sequence, head) changes so far
     const float* lse_s = lse_all;               // sweep B: the current head's -lse2
     int cur_b = -1, cur_h = -1;
     bool ok = true;
-    // Sweep A: a thread's (reference, sum) runs on over consecutive work items of one (sequence, head) and is
-    // written once per run, to the segment numbered blockIdx.x + head: along the item order either the CTA
-    // or the head advances from one run to the next, so the numbers are distinct, and the merge kernel finds
-    // a head's segments from the CTAs its items fall to.
+    // Sweep A: a thread's (reference, sum) runs on over consecutive work items of one (sequence, head), then goes to warp 3
+    // (the CTA's last one, which the end of the kernel waits for, is merged by all epilogue warps together).
     float m = -INFINITY, z = 0.f;
-    int run_b = -1, run_h = -1;
-    auto flush_run = [&]() {
-      const int r = (two_blocks ? par * 128 : 0) + lane_row;
-      if (run_b < 0 || r >= p.rows) return;
-      pdl_wait();                                             // the partials of the call before have been merged
-      const int slots = tc_stat_slots(p.row_blocks);
-      const int slot = two_blocks ? ch : grp;
-      const int64_t seg = static_cast<int64_t>(blockIdx.x) + run_b * p.num_kv_heads + run_h;
-      p.partial[(seg * slots + slot) * p.rows + r] = make_float2(m, z);
+    auto flush_run = [&]() -> bool {            // hands run number heads - 1 over
+      const uint32_t run = heads - 1, buf = run & 1u;
+      bool good = mbar_wait(n_empty(buf), ((run >> 1) & 1) ^ 1, abort_flag, p.wait_clocks);
+      good = __all_sync(0xffffffffu, good);
+      if (!good) return false;
+      run_all[buf * 512 + grp * 128 + lane_row] = make_float2(m, z);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(n_full(buf));
+      m = -INFINITY;
+      z = 0.f;
+      return true;
     };
     for (int ii = 0; ii < item1 - item0 && ok; ++ii) {
-      const int id = kReverse ? item1 - 1 - ii : item0 + ii;
-      const TcItem w = tc_item(off, p.seq.batch, p.num_kv_heads, id);
+      const TcItem w = item_at(ii);
       const int n = p.seq.n[w.b], alpha = p.seq.alpha, P = p.seq.prefix[w.b];
-      const int keys = span_keys(w.b);
-      const int tile0 = w.c * chunk_tiles;
-      const int tile1 = min(tile0 + chunk_tiles, (keys + kTileKeys - 1) / kTileKeys);
+      const int tile0 = w.c * chunk_tiles, tile1 = last_tile(w);
+      const bool new_head = w.b != cur_b || w.h != cur_h;
       if (SWEEP == 0) {
-        // thread -> window row.  With two row blocks the unit parity is the row block, so a group always
-        // works on the same block; with one, the pairs of groups take alternate K tiles.  Either way a
-        // thread keeps one (reference, sum) per run of work items and every group writes its own partial slot.
-        const int r = (two_blocks ? par * 128 : 0) + lane_row;
+        // thread -> window row (and, with copies of the rows, share of the columns), the same in all units of the group: a
+        // thread keeps one (reference, sum) per run of work items.
+        const int r = blk * 128 + lane_row % copy_rows;
         const int last_visible = min(P + (r % alpha), n - 1); // row (g, j) sees keys 0 .. P + j that exist here
-        const int units = p.row_blocks;
-        // a warp whose 32 TMEM lanes are all padding rows (R < 128) has nothing to evaluate
-        const bool warp_has_rows = (two_blocks ? par * 128 : 0) + quarter * 32 < p.rows;
-        if (w.b != run_b || w.h != run_h) {
-          flush_run();
-          m = -INFINITY;
-          z = 0.f;
-          run_b = w.b;
-          run_h = w.h;
+        const int cols = 128 / copies;                        // this thread's key columns of a unit
+        const int col0 = (lane_row / copy_rows) * cols;
+        // a warp whose 32 TMEM lanes are all padding rows has nothing to evaluate
+        const bool warp_has_rows = blk * 128 + (quarter * 32) % copy_rows < p.rows;
+        if (new_head) {
+          if (heads > 0) ok = flush_run();
+          if (!ok) break;
+          cur_b = w.b; cur_h = w.h;
+          ++heads;
         }
         for (int t = tile0; t < tile1 && ok; ++t) {
-          for (int rb = 0; rb < units && ok; ++rb, ++u) {
-            if (static_cast<int>(u & 1u) != par) continue;    // the other pair's unit
-            const int ts = u & 1;
-            ok = mbar_wait(t_full(ts), (u >> 1) & 1, abort_flag, p.wait_clocks);
+          for (int rb = 0; rb < p.row_blocks && ok; ++rb, ++u) {
+            if (static_cast<int>(u % kTcStages) != grp) continue;        // another group's unit
+            ok = mbar_wait(t_full(grp), (u / kTcStages) & 1, abort_flag, p.wait_clocks);
             ok = __all_sync(0xffffffffu, ok);                 // whole warp proceeds together or not at all
             if (!ok) break;
             tc_fence_after();
-            const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + ts * stage_cols + ch * 128;
-            const int key_base = t * kTcTileKeysA + ch * 128;
+            const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + grp * kTcStageCols + col0;
+            const int key_base = t * kTileKeys + col0;
             if (!warp_has_rows) {
               // only the hand-shake below
-            } else if (key_base + 127 <= min(P, n - 1)) {     // every key visible to every row: no mask
-              // fast path over the 128 columns; the sums are only looked at once, at the end
-              const unsigned long long cc = pack2(c2, c2), mm = pack2(-m, -m);
-              unsigned long long acc[4] = {pack2(0.f, 0.f), pack2(0.f, 0.f), pack2(0.f, 0.f), pack2(0.f, 0.f)};
+            } else if (key_base + cols - 1 <= min(P, n - 1)) {   // every key visible to every row: no mask
+              // fast path over the columns; the sums are only looked at once, at the end
               // 16-column loads, double buffered: the next load is in flight while a chunk is evaluated
               uint32_t va[16], vb[16];
               tc_ld16(taddr, va);
+              if (m == -INFINITY) {                           // a new run: any of the row's logits will do as the reference
+                tc_wait_ld();
+                float gm = __uint_as_float(va[0]);
 #pragma unroll
-              for (int cg = 0; cg < 128; cg += 32) {
-                tc_wait_ld();
-                tc_ld16(taddr + cg + 16, vb);
-                rowstats_accumulate(va, cc, mm, acc);
-                tc_wait_ld();
-                if (cg + 32 < 128) tc_ld16(taddr + cg + 32, va);
-                rowstats_accumulate(vb, cc, mm, acc);
+                for (int j = 1; j < 16; ++j) gm = fmaxf(gm, __uint_as_float(va[j]));
+                m = ceilf(gm * c2);
+              }
+              const unsigned long long cc = pack2(c2, c2), mm = pack2(-m, -m);
+              unsigned long long acc[4] = {pack2(0.f, 0.f), pack2(0.f, 0.f), pack2(0.f, 0.f), pack2(0.f, 0.f)};
+              if (copies == 1) {
+#pragma unroll
+                for (int cg = 0; cg < 128; cg += 32) {
+                  tc_wait_ld();
+                  tc_ld16(taddr + cg + 16, vb);
+                  rowstats_accumulate(va, cc, mm, acc);
+                  tc_wait_ld();
+                  if (cg + 32 < 128) tc_ld16(taddr + cg + 32, va);
+                  rowstats_accumulate(vb, cc, mm, acc);
+                }
+              } else {
+                for (int cg = 0; cg < cols; cg += 32) {
+                  tc_wait_ld();
+                  tc_ld16(taddr + cg + 16, vb);
+                  rowstats_accumulate(va, cc, mm, acc);
+                  tc_wait_ld();
+                  if (cg + 32 < cols) tc_ld16(taddr + cg + 32, va);
+                  rowstats_accumulate(vb, cc, mm, acc);
+                }
               }
               const float g = sum_pairs(acc);
               const bool good = g < 1.0e18f;                  // false for inf and NaN too
               if (good) z += g;
               if (!__all_sync(0xffffffffu, good)) {           // rare: the warp reads its columns again, slow path
-                for (int cg = 0; cg < 128; cg += 16) {
+                for (int cg = 0; cg < cols; cg += 16) {
                   tc_ld16(taddr + cg, va);
                   tc_wait_ld();
                   rowstats_rescue(va, c2, !good, m, z);
                 }
               }
             } else {
-              for (int cg = 0; cg < 128; cg += 16) {
+              for (int cg = 0; cg < cols; cg += 16) {
                 uint32_t v[16];
                 tc_ld16(taddr + cg, v);
                 tc_wait_ld();
@@ -632,108 +795,64 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(t_empty(ts));
+            if (lane == 0) mbar_arrive(t_empty(grp));
           }
         }
         if (!ok) break;
       } else {
-        // thread -> key.  The pairs of groups take alternate K tiles; inside a pair the groups split the
-        // window rows (columns) of a key and group ch = 1 hands its partial sum to group ch = 0.
-        // The head's normalisers, negated (the epilogue adds them), in one of two buffers that alternate from
-        // head to head.  The sixteen warps fill a buffer together (512 threads over the rows, 2 to 16 lanes per
-        // row), then meet at a barrier; a buffer is written again only after every warp has passed the barrier of
-        // the head in between, i.e. after all of them are done with it.  The values come either from the caller
-        // (or the merge kernel), or straight from sweep A's partial (reference, sum) pairs of this head, which
-        // every CTA that works on the head merges for itself, always in the same order.
-        if (w.b != cur_b || w.h != cur_h) {
-          pdl_wait();                                         // normalisers and partials are written by kernels before
-          float* dst = lse_all + (heads_seen & 1u) * 256;
-          const int rows_p2 = p.rows_pad <= 32 ? 32 : (p.rows_pad <= 64 ? 64 : (p.rows_pad <= 128 ? 128 : 256));
-          const int per_row = (kTcEpiWarps * 32) / rows_p2;   // lanes that share a row: 2, 4, 8 or 16
-          const int r = (e * 32 + lane) / per_row, part = (e * 32 + lane) % per_row;
-          float val = -INFINITY;
-          if (p.merge) {
-            // sweep A's CTAs took contiguous item ranges (items ordered sequence, head, chunk): the first `rem`
-            // CTAs per + 1 items, the others per; this head's items fell to CTAs c0..c1, one segment each
-            const int nc = p.seq.stat_off[w.b + 1] - p.seq.stat_off[w.b];
-            const int total_a = p.num_kv_heads * p.seq.stat_off[p.seq.batch];
-            const int per_a = total_a / p.stat_grid, rem_a = total_a % p.stat_grid, edge = rem_a * (per_a + 1);
-            const int i0 = p.num_kv_heads * p.seq.stat_off[w.b] + w.h * nc, i1 = i0 + nc - 1;
-            const int c0 = i0 < edge ? i0 / (per_a + 1) : rem_a + (i0 - edge) / per_a;
-            const int c1 = i1 < edge ? i1 / (per_a + 1) : rem_a + (i1 - edge) / per_a;
-            const int hg = w.b * p.num_kv_heads + w.h, slots = tc_stat_slots(p.row_blocks);
-            const int t0 = (c0 + hg) * slots, t1 = (c1 + hg + 1) * slots;
-            float m = -INFINITY, z = 0.f;
-            if (r < p.rows) {
-              const float2* base = p.partial + r;
-              for (int t = t0 + part; t < t1; t += 4 * per_row) {
-                float2 pz[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                  pz[q] = t + q * per_row < t1 ? __ldcg(base + static_cast<int64_t>(t + q * per_row) * p.rows)
-                                               : make_float2(-INFINITY, 0.f);
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                  if (pz[q].x > -INFINITY) {                  // (-inf, 0) marks a slot that saw no key of this row
-                    const float mn = fmaxf(m, pz[q].x);
-                    z = z * ex2(m - mn) + pz[q].y * ex2(pz[q].x - mn);
-                    m = mn;
-                  }
-              }
-            }
-            for (int o = 1; o < per_row; o <<= 1) {           // the lanes of a row meet pairwise; both partners of a
-              const float m2 = __shfl_xor_sync(0xffffffffu, m, o), z2 = __shfl_xor_sync(0xffffffffu, z, o);   // pair
-              const float mm = fmaxf(m, m2);                                        // compute the same merged value
-              z = (m > -INFINITY ? z * ex2(m - mm) : 0.f) + (m2 > -INFINITY ? z2 * ex2(m2 - mm) : 0.f);
-              m = mm;
-            }
-            if (r < p.rows) val = -(m + __log2f(z) + p.log2_group);
-          } else if (r < p.rows) {
-            const float* src = p.lse2 + (static_cast<int64_t>(w.b) * p.num_kv_heads + w.h) * p.rows;
-            val = -fmaf(src[r], p.lse_scale, p.lse_add);
+        // thread -> key.  The head's normalisers, negated (the epilogue adds them), sit in one of two buffers that alternate
+        // from head to head.  The first one is filled by the sixteen warps together, which then meet; the others by warp 3,
+        // ahead of time.  They come from the caller (or the merge kernel), or straight from sweep A's partials of the head,
+        // which every CTA that works on it merges for itself, always in the same order.
+        if (new_head) {
+          const uint32_t buf = heads & 1u;
+          if (heads == 0) {
+            tc_normalisers<kTcEpiWarps * 32>(p, w.b, w.h, e * 32 + lane, lse_all);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(meet);
+            ok = mbar_wait(meet, 0, abort_flag, p.wait_clocks);
+          } else {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(n_empty(buf ^ 1u));    // done with the head before
+            ok = mbar_wait(n_full(buf), buf == 1u ? (heads >> 1) & 1 : ((heads >> 1) & 1) ^ 1, abort_flag, p.wait_clocks);
           }
-          if (part == 0) dst[r] = val;
-          __syncwarp();
-          if (lane == 0) mbar_arrive(lse_full);
-          ok = mbar_wait(lse_full, heads_seen & 1u, abort_flag, p.wait_clocks);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
-          lse_s = dst;
-          ++heads_seen;
+          lse_s = lse_all + buf * 256;
           cur_b = w.b; cur_h = w.h;
+          ++heads;
         }
         float* srow = p.scores + (static_cast<int64_t>(w.b) * p.num_kv_heads + w.h) * p.ld_scores;
-        const int col0 = ch == 0 ? 0 : split_b, col1 = ch == 0 ? split_b : p.rows_pad;
-        for (int tt = 0; tt < tile1 - tile0 && ok; ++tt, ++u) {
+        const float* nlse = lse_s + (blk ? split_b : 0);
+        const int cols = blk ? p.rows_pad - split_b : split_b;
+        for (int tt = 0; tt < tile1 - tile0 && ok; ++tt, u += p.row_blocks) {
           const int t = kReverse ? tile1 - 1 - tt : tile0 + tt;
-          if (static_cast<int>(u & 1u) != par) continue;      // the other pair's tile
-          if (ch == 1 && !second_half) continue;              // nothing for this group to read
-          const int ts = u % t_stages;
-          ok = mbar_wait(t_full(ts), (u / t_stages) & 1, abort_flag, p.wait_clocks);
+          if ((u + blk) % kTcStages != static_cast<uint32_t>(grp)) continue;     // another group's unit
+          ok = mbar_wait(t_full(grp), (u / kTcStages) & 1, abort_flag, p.wait_clocks);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           tc_fence_after();
-          const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + ts * stage_cols;
+          const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + grp * kTcStageCols;
           unsigned long long acc[4] = {pack2(0.f, 0.f), pack2(0.f, 0.f), pack2(0.f, 0.f), pack2(0.f, 0.f)};
           const unsigned long long cc = pack2(c2, c2);
           {
             uint32_t va[16], vb[16];
-            tc_ld16(taddr + col0, va);
-            for (int cg = col0; cg < col1; cg += 32) {
+            tc_ld16(taddr, va);
+            for (int cg = 0; cg < cols; cg += 32) {
               tc_wait_ld();
               tc_ld16(taddr + cg + 16, vb);
-              score_group(va, cc, lse_s + cg, acc);
+              score_group(va, cc, nlse + cg, acc);
               tc_wait_ld();
-              if (cg + 32 < col1) tc_ld16(taddr + cg + 32, va);
-              score_group(vb, cc, lse_s + cg + 16, acc);
+              if (cg + 32 < cols) tc_ld16(taddr + cg + 32, va);
+              score_group(vb, cc, nlse + cg + 16, acc);
             }
           }
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(t_empty(ts));
+          if (lane == 0) mbar_arrive(t_empty(grp));
           float sum = sum_pairs(acc);
-          if (second_half) {
-            if (ch == 1) {
+          if (two_blocks) {                                   // the second half's group hands its partial sum to the first's
+            if (blk == 1) {
               ok = mbar_wait(x_empty(par), (mine & 1) ^ 1, abort_flag, p.wait_clocks);
               ok = __all_sync(0xffffffffu, ok);
               if (!ok) break;
@@ -750,13 +869,22 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
             }
           }
           ++mine;
-          const int i = t * kTcTileKeysB + lane_row;
-          if (ch == 0 && i < P) srow[i] = sum;
+          const int i = t * kTileKeys + lane_row;
+          if (blk == 0 && i < P) srow[i] = sum;
         }
         if (!ok) break;
       }
     }
-    if (SWEEP == 0 && ok) flush_run();                        // the CTA's last run
+    if (SWEEP == 0 && ok && heads > 0 && flush_run()) {       // the CTA's last run
+      const uint32_t run = heads - 1;
+      if (mbar_wait(n_full(run & 1u), (run >> 1) & 1, abort_flag, p.wait_clocks)) {
+        pdl_wait();                                           // the partials of the call before have been read
+        const int r = e * 32 + lane;
+        if (r < p.rows)
+          p.partial[(static_cast<int64_t>(blockIdx.x) + cur_b * p.num_kv_heads + cur_h) * p.rows + r] =
+              run_row(run_all + (run & 1u) * 512, r, two_blocks, copies);
+      }
+    }
   }
 
   // ---- teardown
