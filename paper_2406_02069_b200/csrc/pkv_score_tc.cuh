@@ -40,7 +40,7 @@ constexpr int kTcStageCols = 128;       // TMEM columns of an accumulator stage
 constexpr int kTcStages = 4;            // accumulator stages, one per group of epilogue warps
 constexpr int kTcKBytes = 128 * 1024;   // shared memory given to K stages (4 x 32 KB at d = 128)
 constexpr int kTcMaxGrid = 256;         // CTAs of a sweep at most (the workspace holds a partial segment per CTA)
-constexpr int kTcPrefetchBytes = 448 * 1024;   // of K per CTA into the L2 ahead of the wait: half the L2 in all
+constexpr int kTcPrefetchBytes = 128 * 1024;   // of K per CTA into the L2 ahead of the wait: what the start needs (more gains nothing)
 constexpr int kTcMaxRows = 256;         // window rows (G * alpha) the tensor-core path takes
 constexpr long long kTcWaitCycles = 1ll << 31;   // bound of any one wait, in SM clocks
 
