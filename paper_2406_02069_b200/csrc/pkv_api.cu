@@ -870,26 +870,21 @@ bool paged_args_ok(const int32_t* block_table, int page_size, int num_pages, con
 // SM) and every CTA keeps a step's worth of rows.
 int decode_cluster(long long units, int max_count, int sms) {
   int cluster = 1;
-  while (cluster < kDecMaxCluster && units * cluster * 2 <= 2ll * sms && max_count >= 2 * cluster * kDecMinRows) cluster *= 2;
+  while (cluster < kDecMaxCluster && units * cluster * 2 <= sms && max_count >= 2 * cluster * kDecMinRows) cluster *= 2;
   return cluster;
 }
 
 // ---------------------------------------------------------------- decode attention
-template <typename T, int D, int GT, bool PAGED>
-int launch_decode(DecodeParams& dp, int batch, int max_count, cudaStream_t st) {
+// gt: query heads per CTA of the kernel.  Measured on one B200, one token through 32 layers, 8 KV heads x 4 query heads,
+// d = 128, bf16: see the table of decode_cluster.
+int launch_decode(void (*kernel)(DecodeParams), int gt, DecodeParams& dp, int batch, int max_count, cudaStream_t st) {
   const int sms = device_sm_count();
   if (sms <= 0) return PKV_ERR_CUDA;
-  auto kernel = decode_attention_kernel<T, D, GT, PAGED>;
-  static bool attr_done[64] = {};                  // clusters of 16 CTAs are an opt-in of the kernel, per device
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return PKV_ERR_CUDA;
-  if (dev >= 64 || !attr_done[dev]) {
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return PKV_ERR_CUDA;
-    if (dev < 64) attr_done[dev] = true;
-  }
-  dp.head_blocks = (dp.group + GT - 1) / GT;
+  dp.head_blocks = (dp.group + gt - 1) / gt;
   const long long units = static_cast<long long>(dp.num_kv_heads) * dp.head_blocks * batch;
   const int cluster = decode_cluster(units, max_count, sms);
+  if (cluster > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+    return PKV_ERR_CUDA;                           // clusters of 16 CTAs are an opt-in of the kernel
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(cluster * dp.num_kv_heads * dp.head_blocks, batch);
   cfg.blockDim = dim3(kDecThreads);
@@ -903,16 +898,17 @@ int launch_decode(DecodeParams& dp, int batch, int max_count, cudaStream_t st) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (cudaLaunchKernelEx(&cfg, kernel, static_cast<const DecodeParams&>(dp)) != cudaSuccess) return PKV_ERR_CUDA;
+  void* args[1] = {&dp};
+  if (cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kernel), args) != cudaSuccess) return PKV_ERR_CUDA;
   return check_launch();
 }
 
-template <typename T, int D, bool PAGED>
-int launch_decode_group(DecodeParams& dp, int batch, int max_count, cudaStream_t st) {
-  if (dp.group == 1) return launch_decode<T, D, 1, PAGED>(dp, batch, max_count, st);
-  if (dp.group == 2) return launch_decode<T, D, 2, PAGED>(dp, batch, max_count, st);
-  if (dp.group <= 4) return launch_decode<T, D, 4, PAGED>(dp, batch, max_count, st);
-  return launch_decode<T, D, 8, PAGED>(dp, batch, max_count, st);
+template <int D, bool PAGED>
+int launch_decode_fp32(DecodeParams& dp, int batch, int max_count, cudaStream_t st) {
+  if (dp.group == 1) return launch_decode(decode_attention_kernel<D, 1, PAGED>, 1, dp, batch, max_count, st);
+  if (dp.group == 2) return launch_decode(decode_attention_kernel<D, 2, PAGED>, 2, dp, batch, max_count, st);
+  if (dp.group <= 4) return launch_decode(decode_attention_kernel<D, 4, PAGED>, 4, dp, batch, max_count, st);
+  return launch_decode(decode_attention_kernel<D, 8, PAGED>, 8, dp, batch, max_count, st);
 }
 
 template <bool PAGED>
@@ -925,14 +921,13 @@ int run_decode(const pkv_config* c, DecodeParams& dp, int batch, cudaStream_t st
   const bool wide = c->head_dim == 128;
   switch (c->dtype) {
     case PKV_DTYPE_FP32:
-      return wide ? launch_decode_group<float, 128, PAGED>(dp, batch, max_count, st)
-                  : launch_decode_group<float, 64, PAGED>(dp, batch, max_count, st);
+      return wide ? launch_decode_fp32<128, PAGED>(dp, batch, max_count, st) : launch_decode_fp32<64, PAGED>(dp, batch, max_count, st);
     case PKV_DTYPE_FP16:
-      return wide ? launch_decode_group<__half, 128, PAGED>(dp, batch, max_count, st)
-                  : launch_decode_group<__half, 64, PAGED>(dp, batch, max_count, st);
+      return launch_decode(wide ? decode_mma_kernel<__half, 128, PAGED> : decode_mma_kernel<__half, 64, PAGED>, kDecMmaHeads, dp, batch,
+                           max_count, st);
     default:
-      return wide ? launch_decode_group<__nv_bfloat16, 128, PAGED>(dp, batch, max_count, st)
-                  : launch_decode_group<__nv_bfloat16, 64, PAGED>(dp, batch, max_count, st);
+      return launch_decode(wide ? decode_mma_kernel<__nv_bfloat16, 128, PAGED> : decode_mma_kernel<__nv_bfloat16, 64, PAGED>, kDecMmaHeads,
+                           dp, batch, max_count, st);
   }
 }
 

@@ -2,19 +2,17 @@
 // inference): out[b][g] = softmax(q[b][g] . K_s^T / sqrt(d)) V_s for one new token per sequence, packed or paged rows.
 //
 // What bounds it: the cache is read once, so the floor is its bytes over the memory bandwidth (a few microseconds);
-// below that it is a chain of latencies (launch, loads, merges).  The work is therefore split for loads in flight:
-//   * one cluster of 1..16 CTAs per (sequence, KV head, block of at most 8 query heads): every K and V row is read once
-//     for all query heads of its group, and few long rows lists still spread over the chip.  No scratch memory is
-//     needed, the CTAs of a cluster merge through distributed shared memory (this call has no workspace);
-//   * inside a CTA a team of D / 8 lanes takes kDecRows rows at a time, 8 elements of a row per lane (16 bytes of a
-//     16-bit row), K and V loads of a step issued together;
-//   * the row x head dot products of a step are summed over the team's lanes by halving: every exchange also halves the
-//     number of values a lane holds, so that reducing n values over L lanes costs about n exchanges instead of
-//     n log2 L, and each softmax weight is evaluated once instead of once per lane.
-// Everything stays in fp32.  Measured on one B200, one token through 32 layers, 8 KV heads x 4 query heads, d = 128,
-// bf16: 2048 rows a head on average, one sequence (269 MB): 8.8 ms with one CTA per query head (32 CTAs, each K and V
-// row read four times, a dependent exponential and four exchanges per row), 0.37 ms now (0.46 with clusters of at most
-// 8); 512 rows on average, eight sequences, pages of 16 rows (543 MB): 3.3 ms -> 0.40 ms.
+// below that it is a chain of latencies (launch, loads, merges) and, on the fp32 pipe, the instructions per row: with one
+// warp instruction per 2 rows x 8 channels a step of 8 rows took a warp 400 of them.
+//   * One cluster of 1..16 CTAs per (sequence, KV head, block of query heads): every K and V row is read once for all
+//     query heads of its block, and few long row lists still spread over the chip.  No scratch memory is needed (this
+//     call has no workspace): the CTAs hand their sums to one another through distributed shared memory, each channel
+//     to the CTA that finishes it, with one cluster barrier.
+//   * 16-bit rows go through mma.sync (decode_mma_kernel): M = query heads, fp32 accumulation.  The softmax weights stay
+//     fp32 in effect: each is split into three 16-bit parts (hi + mid + lo carry 24 bits and more), which stand in
+//     different rows of the same M = 16 operand (4 heads x 3 parts), so that the split costs no extra products.
+//   * fp32 rows stay on the fp32 pipe (decode_attention_kernel).
+// Measured on one B200, one token through 32 layers, 8 KV heads x 4 query heads, d = 128, bf16: see launch_decode.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -42,23 +40,8 @@ struct DecodeParams {
   float scale_log2;         // log2(e) / sqrt(d)
 };
 
-// Eight consecutive elements of a row, as loaded and as four packed pairs of floats.
-template <typename T>
+// Eight consecutive floats of a row as four packed pairs.
 struct Dec8 {
-  uint4 u;
-  __device__ __forceinline__ void load(const T* p) { u = *reinterpret_cast<const uint4*>(p); }
-  __device__ __forceinline__ void zero() { u = make_uint4(0, 0, 0, 0); }
-  __device__ __forceinline__ unsigned long long pair(int i) const {
-    const uint32_t w = i == 0 ? u.x : (i == 1 ? u.y : (i == 2 ? u.z : u.w));
-    if (sizeof(T) == 2 && __is_same(T, __half)) {
-      const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w));
-      return pack2(f.x, f.y);
-    }
-    return pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));      // bfloat16: the upper half of a float
-  }
-};
-template <>
-struct Dec8<float> {
   float4 a, b;
   __device__ __forceinline__ void load(const float* p) {
     a = reinterpret_cast<const float4*>(p)[0];
@@ -70,9 +53,65 @@ struct Dec8<float> {
   }
 };
 
-// grid (cluster * H_kv * head_blocks, batch), cluster (cluster, 1, 1), block kDecThreads.  GT: query heads per CTA (a
-// power of two; heads beyond the group are computed on zeros and not written).
-template <typename T, int D, int GT, bool PAGED>
+// Shared memory in which the warps of a CTA, then the CTAs of a cluster meet.
+template <int D, int GT>
+struct DecMerge {
+  float acc[kDecWarps][GT * D];
+  float m[kDecWarps][GT], z[kDecWarps][GT];
+  float in[kDecMaxCluster * ((GT * D + kDecMaxCluster - 1) / kDecMaxCluster)];   // this CTA's channels, from every CTA
+  float2 mz[kDecMaxCluster][GT];                                                 // every CTA's (maximum, sum) per head
+};
+
+// Sums of the warps (in shared memory behind a barrier) -> output.  hq0: first query head of the block.  The cluster's
+// barrier has been arrived at once at the start of the kernel.
+template <int D, int GT>
+__device__ __forceinline__ void dec_finish(DecMerge<D, GT>& s, const DecodeParams& p, int C, int rank, int64_t hq0, int heads) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  if (C > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");        // every CTA of the cluster has started
+  const int share = (GT * D + C - 1) / C;        // channels each CTA finishes
+  for (int o = threadIdx.x; o < GT * D; o += kDecThreads) {
+    const int g = o / D;
+    float mm = -INFINITY;
+#pragma unroll
+    for (int w = 0; w < kDecWarps; ++w) mm = fmaxf(mm, s.m[w][g]);
+    float zz = 0.f, a = 0.f;
+#pragma unroll
+    for (int w = 0; w < kDecWarps; ++w) {
+      const float f = s.m[w][g] == -INFINITY ? 0.f : exp2f(s.m[w][g] - mm);      // 0: the warp saw no row
+      zz += s.z[w][g] * f;
+      a += s.acc[w][o] * f;
+    }
+    if (C == 1) {
+      if (g < heads) p.out[hq0 * D + o] = a / zz;
+    } else {
+      const int to = o / share;
+      cluster.map_shared_rank(s.in, to)[rank * share + o - to * share] = a;
+      if (o == to * share || o % D == 0) cluster.map_shared_rank(&s.mz[0][0], to)[rank * GT + g] = make_float2(mm, zz);
+    }
+  }
+  if (C == 1) return;
+  cluster.sync();
+  for (int i = threadIdx.x; i < share; i += kDecThreads) {
+    const int o = rank * share + i, g = o / D;
+    if (o >= GT * D || g >= heads) continue;
+    float mm = -INFINITY, zz = 0.f, a = 0.f;
+    for (int c = 0; c < C; ++c) mm = fmaxf(mm, s.mz[c][g].x);
+    for (int c = 0; c < C; ++c) {
+      const float f = s.mz[c][g].x == -INFINITY ? 0.f : exp2f(s.mz[c][g].x - mm);
+      zz += s.mz[c][g].y * f;
+      a += s.in[c * share + i] * f;
+    }
+    p.out[hq0 * D + o] = a / zz;
+  }
+}
+
+// fp32 rows.  grid (cluster * H_kv * head_blocks, batch), cluster (cluster, 1, 1), block kDecThreads.  GT: query heads per
+// CTA (a power of two; heads beyond the group are computed on zeros and not written).  A team of D / 8 lanes takes four
+// (eight) rows at a time, 8 channels of a row per lane.  The row x head dot products of a step are summed over the team's
+// lanes by halving: every exchange also halves the number of values a lane holds, so that reducing n values over L lanes
+// costs about n exchanges instead of n log2 L, and each softmax weight is evaluated once instead of once per lane.
+template <int D, int GT, bool PAGED>
 __global__ void __launch_bounds__(kDecThreads) decode_attention_kernel(const DecodeParams p) {
   constexpr int L = D / 8;                       // lanes per row
   constexpr int RPW = 32 / L;                    // teams per warp
@@ -82,13 +121,13 @@ __global__ void __launch_bounds__(kDecThreads) decode_attention_kernel(const Dec
   constexpr int PER = NV > L ? NV / L : 1;       // ... of which a lane ends up with this many (consecutive ones)
   constexpr int SHARE = NV < L ? L / NV : 1;     // ... or this many lanes hold the same one
   static_assert(PER <= U, "a lane's values belong to one head");
+  using T = float;
   namespace cg = cooperative_groups;
-  __shared__ float s_acc[kDecWarps][GT * D];
-  __shared__ float s_m[kDecWarps][GT], s_z[kDecWarps][GT];
-  __shared__ float s_cm[GT], s_cz[GT];
+  __shared__ DecMerge<D, GT> s_mrg;
   pdl_trigger();
   cg::cluster_group cluster = cg::this_cluster();
   const int C = cluster.dim_blocks().x, rank = cluster.block_rank();
+  if (C > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");      // this CTA's shared memory may be written
   const int unit = blockIdx.x / C, b = blockIdx.y;
   const int h = unit / p.head_blocks, g0 = (unit % p.head_blocks) * GT;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -103,7 +142,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_attention_kernel(const Dec
   unsigned long long q2[GT][4], acc[GT][4];
 #pragma unroll
   for (int g = 0; g < GT; ++g) {
-    Dec8<T> raw;
+    Dec8 raw;
     if (g0 + g < p.group) raw.load(static_cast<const T*>(p.q) + (hq0 + g) * D + sub * 8);
     else raw.zero();
 #pragma unroll
@@ -114,7 +153,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_attention_kernel(const Dec
   float m = -INFINITY, z = 0.f;                  // of head my_head: m over the team's rows, z over this lane's
 
   for (int r0 = lo; r0 < hi; r0 += U * TEAMS) {
-    Dec8<T> kr[U], vr[U];
+    Dec8 kr[U], vr[U];
     uint32_t live = 0;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -239,51 +278,196 @@ __global__ void __launch_bounds__(kDecThreads) decode_attention_kernel(const Dec
         x += __shfl_xor_sync(0xffffffffu, x, s);
         y += __shfl_xor_sync(0xffffffffu, y, s);
       }
-      if (lane < L) *reinterpret_cast<float2*>(&s_acc[warp][g * D + sub * 8 + 2 * c]) = make_float2(x, y);
+      if (lane < L) *reinterpret_cast<float2*>(&s_mrg.acc[warp][g * D + sub * 8 + 2 * c]) = make_float2(x, y);
     }
   }
   if (lane < L && sub % (L / GT) == 0) {         // one lane per head
-    s_m[warp][my_head] = mw;
-    s_z[warp][my_head] = z;
+    s_mrg.m[warp][my_head] = mw;
+    s_mrg.z[warp][my_head] = z;
   }
   __syncthreads();
-  for (int o = tid; o < GT * D; o += kDecThreads) {
-    const int g = o / D;
-    float mm = -INFINITY;
+  dec_finish<D, GT>(s_mrg, p, C, rank, hq0, p.group - g0);
+}
+
+// ------------------------------------------------------------------ 16-bit rows
+constexpr int kDecMmaHeads = 4;           // query heads per CTA: 4 heads x 3 parts of the weights in the 16 rows of an MMA
+
+template <typename T>
+struct Dec16;
+template <>
+struct Dec16<__nv_bfloat16> {
+  static constexpr float kShift = 0.f;    // bfloat16 has the range of fp32
+  __device__ __forceinline__ static uint32_t pack(float lo, float hi) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&v);
+  }
+  __device__ __forceinline__ static float2 unpack(uint32_t u) {
+    return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
+  }
+  __device__ __forceinline__ static void mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+  }
+};
+template <>
+struct Dec16<__half> {
+  static constexpr float kShift = 13.f;   // weights carry 2^13, so that the third part of small ones is not subnormal
+  __device__ __forceinline__ static uint32_t pack(float lo, float hi) {
+    const __half2 v = __floats2half2_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&v);
+  }
+  __device__ __forceinline__ static float2 unpack(uint32_t u) { return __half22float2(*reinterpret_cast<const __half2*>(&u)); }
+  __device__ __forceinline__ static void mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+  }
+};
+
+// grid, cluster and block as above, kDecMmaHeads query heads per CTA.  A warp takes tiles of 16 rows.  With g = lane / 4 and
+// c = lane % 4 the fragments of m16n8k16 are
+//   S  = Q K^T   A: row i = head i % 4 (every head four times), B: n = row g of 8, channels dealt so that a lane's B words are
+//                its own 16-byte pieces of K (the order of the contraction is free as long as Q has the same one);
+//                result: head g % 4, rows 2c, 2c + 1
+//   O += P V     A: rows 0-3 the high parts of the weights, 4-7 the middle ones, 8-11 the low ones, 12-15 zero: in the very
+//                lanes and positions where S came out; B: rows 2c, 2c + 1 (+ 8, 9) of channel 64 j + 8 g + i, from 16-byte
+//                pieces of V with the halves of two rows interleaved.
+// A lane holds sums of one head only, so rescaling needs no exchange; O is the sum over the three parts.
+template <typename T, int D, bool PAGED>
+__global__ void __launch_bounds__(kDecThreads, 1) decode_mma_kernel(const DecodeParams p) {
+  constexpr int GT = kDecMmaHeads, KC = D / 32, VC = D / 64;
+  using X = Dec16<T>;
+  namespace cg = cooperative_groups;
+  __shared__ DecMerge<D, GT> s_mrg;
+  pdl_trigger();
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = cluster.dim_blocks().x, rank = cluster.block_rank();
+  if (C > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");      // this CTA's shared memory may be written
+  const int unit = blockIdx.x / C, b = blockIdx.y;
+  const int h = unit / p.head_blocks, g0 = (unit % p.head_blocks) * GT;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, c = lane & 3;
+  const int count = p.seq.count[b];
+  const int64_t row0 = p.seq.row_off[b] + static_cast<int64_t>(h) * count;
+  const int lo = static_cast<int>(static_cast<int64_t>(count) * rank / C);
+  const int hi = static_cast<int>(static_cast<int64_t>(count) * (rank + 1) / C);
+  const int64_t hq0 = static_cast<int64_t>(b) * p.num_kv_heads * p.group + static_cast<int64_t>(h) * p.group + g0;
+  const T* kc = static_cast<const T*>(p.k_cache);
+  const T* vc = static_cast<const T*>(p.v_cache);
+  pdl_wait();
+
+  uint4 q[KC];
 #pragma unroll
-    for (int w = 0; w < kDecWarps; ++w) mm = fmaxf(mm, s_m[w][g]);
-    float zz = 0.f, a = 0.f;
+  for (int j = 0; j < KC; ++j)
+    q[j] = g0 + g % GT < p.group ? *reinterpret_cast<const uint4*>(static_cast<const T*>(p.q) + (hq0 + g % GT) * D + j * 32 + c * 8)
+                                 : make_uint4(0, 0, 0, 0);
+  float o[VC * 8][4];
 #pragma unroll
-    for (int w = 0; w < kDecWarps; ++w) {
-      if (s_m[w][g] == -INFINITY) continue;      // the warp saw no row
-      const float f = exp2f(s_m[w][g] - mm);
-      zz += s_z[w][g] * f;
-      a += s_acc[w][o] * f;
+  for (int i = 0; i < VC * 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+  float m = -INFINITY, z = 0.f;                  // of head g % 4: m over the warp's rows, z over this lane's
+  for (int t0 = lo + warp * 16; t0 < hi; t0 += kDecWarps * 16) {
+    // rows of the tile: where they lie (-1: not there)
+    auto place = [&](int r) -> int64_t {
+      if (t0 + r >= hi) return -1;
+      return PAGED ? -1 : row0 + t0 + r;
+    };
+    int64_t mine = -1;
+    if (PAGED) {
+      const int r = t0 + (lane & 15);
+      if (r < hi) {
+        mine = paged_row(p.pt, b, h, r);
+        if (mine < 0 && lane < 16) atomicOr(p.status, kStatusBadPage);
+      }
     }
-    if (C == 1) {
-      if (g0 + g < p.group) p.out[hq0 * D + o] = a / zz;
-    } else {
-      s_acc[0][o] = a;                           // only this thread reads these entries
-      if (o % D == 0) { s_cm[g] = mm; s_cz[g] = zz; }
+    auto row_at = [&](int r) -> int64_t { return PAGED ? __shfl_sync(0xffffffffu, mine, r) : place(r); };
+    uint4 k[2][KC], v[4][VC];
+    bool seen[2][2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const int64_t at = row_at(t * 8 + g);
+#pragma unroll
+      for (int j = 0; j < KC; ++j)
+        k[t][j] = at >= 0 ? *reinterpret_cast<const uint4*>(kc + at * D + j * 32 + c * 8) : make_uint4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int64_t at = row_at((t >> 1) * 8 + 2 * c + (t & 1));
+      seen[t >> 1][t & 1] = at >= 0;
+#pragma unroll
+      for (int j = 0; j < VC; ++j)
+        v[t][j] = at >= 0 ? *reinterpret_cast<const uint4*>(vc + at * D + j * 64 + g * 8) : make_uint4(0, 0, 0, 0);
+    }
+    float x[2][2];
+    float mx = -INFINITY;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int j = 0; j < KC; ++j) {
+        X::mma(s0, q[j].x, q[j].x, q[j].y, q[j].y, k[t][j].x, k[t][j].y);
+        X::mma(s1, q[j].z, q[j].z, q[j].w, q[j].w, k[t][j].z, k[t][j].w);
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        x[t][i] = seen[t][i] ? (s0[i] + s1[i]) * p.scale_log2 : -INFINITY;
+        mx = fmaxf(mx, x[t][i]);
+      }
+    }
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    const float mn = fmaxf(m, mx);
+    const float ref = mn == -INFINITY ? 0.f : mn - X::kShift;
+    if (__any_sync(0xffffffffu, mn > m)) {
+      const float corr = m == -INFINITY ? 0.f : ex2(m - mn);
+      z *= corr;
+#pragma unroll
+      for (int i = 0; i < VC * 8; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[i][e] *= corr;
+    }
+    m = mn;
+    uint32_t a[2][2];                            // [rows 2c.. / 2c + 8..][fragment row g / g + 8]
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const float w0 = ex2(x[t][0] - ref), w1 = ex2(x[t][1] - ref);
+      z += w0 + w1;
+      const uint32_t high = X::pack(w0, w1);
+      const float2 hf = X::unpack(high);
+      const uint32_t mid = X::pack(w0 - hf.x, w1 - hf.y);
+      const float2 mf = X::unpack(mid);
+      const uint32_t low = X::pack(w0 - hf.x - mf.x, w1 - hf.y - mf.y);
+      a[t][0] = g < 4 ? high : mid;
+      a[t][1] = g < 4 ? low : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < VC; ++j) {
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        const uint32_t v0 = reinterpret_cast<const uint32_t*>(&v[0][j])[w], v1 = reinterpret_cast<const uint32_t*>(&v[1][j])[w];
+        const uint32_t v2 = reinterpret_cast<const uint32_t*>(&v[2][j])[w], v3 = reinterpret_cast<const uint32_t*>(&v[3][j])[w];
+        X::mma(o[j * 8 + 2 * w], a[0][0], a[0][1], a[1][0], a[1][1], __byte_perm(v0, v1, 0x5410), __byte_perm(v2, v3, 0x5410));
+        X::mma(o[j * 8 + 2 * w + 1], a[0][0], a[0][1], a[1][0], a[1][1], __byte_perm(v0, v1, 0x7632), __byte_perm(v2, v3, 0x7632));
+      }
     }
   }
-  if (C == 1) return;
-  cluster.sync();
-  for (int o = rank * kDecThreads + tid; o < GT * D; o += C * kDecThreads) {
-    const int g = o / D;
-    if (g0 + g >= p.group) continue;
-    float mm = -INFINITY, zz = 0.f, a = 0.f;
-    for (int c = 0; c < C; ++c) mm = fmaxf(mm, *cluster.map_shared_rank(&s_cm[g], c));
-    for (int c = 0; c < C; ++c) {
-      const float mc = *cluster.map_shared_rank(&s_cm[g], c);
-      if (mc == -INFINITY) continue;
-      const float f = exp2f(mc - mm);
-      zz += *cluster.map_shared_rank(&s_cz[g], c) * f;
-      a += *cluster.map_shared_rank(&s_acc[0][o], c) * f;
+  // ---- the parts, then the warps, then the CTAs of the cluster
+  z += __shfl_xor_sync(0xffffffffu, z, 1);
+  z += __shfl_xor_sync(0xffffffffu, z, 2);
+#pragma unroll
+  for (int i = 0; i < VC * 8; ++i) {             // channels 64 j + 8 (2c + e) + i % 8 of head g % 4
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      float s = o[i][e] + o[i][2 + e];
+      s += __shfl_xor_sync(0xffffffffu, s, 16);
+      if (g < 4) s_mrg.acc[warp][g * D + (i >> 3) * 64 + (2 * c + e) * 8 + (i & 7)] = s;
     }
-    p.out[hq0 * D + o] = a / zz;
   }
-  cluster.sync();                                // nobody reads this CTA's shared memory any more
+  if (g < 4 && c == 0) {
+    s_mrg.m[warp][g] = m;
+    s_mrg.z[warp][g] = z;
+  }
+  __syncthreads();
+  dec_finish<D, GT>(s_mrg, p, C, rank, hq0, p.group - g0);
 }
 
 }  // namespace pkv
