@@ -866,8 +866,8 @@ bool paged_args_ok(const int32_t* block_table, int page_size, int num_pages, con
   return reinterpret_cast<uintptr_t>(k_pool) % 16 == 0 && reinterpret_cast<uintptr_t>(v_pool) % 16 == 0;
 }
 
-// CTAs of a decode cluster: doubled while the doubled grid still finds a place on the device at once (two CTAs to an
-// SM) and every CTA keeps a step's worth of rows.
+// CTAs of a decode cluster: doubled while every CTA of the doubled grid still has an SM to itself (the 16-bit kernel's
+// registers fill one) and keeps 64 rows (at 32 or 128 the times of 64 to 4096 rows a head are the same or worse).
 int decode_cluster(long long units, int max_count, int sms) {
   int cluster = 1;
   while (cluster < kDecMaxCluster && units * cluster * 2 <= sms && max_count >= 2 * cluster * kDecMinRows) cluster *= 2;
@@ -875,16 +875,13 @@ int decode_cluster(long long units, int max_count, int sms) {
 }
 
 // ---------------------------------------------------------------- decode attention
-// gt: query heads per CTA of the kernel.  Measured on one B200, one token through 32 layers, 8 KV heads x 4 query heads,
-// d = 128, bf16: see the table of decode_cluster.
+// gt: query heads per CTA of the kernel.
 int launch_decode(void (*kernel)(DecodeParams), int gt, DecodeParams& dp, int batch, int max_count, cudaStream_t st) {
   const int sms = device_sm_count();
   if (sms <= 0) return PKV_ERR_CUDA;
   dp.head_blocks = (dp.group + gt - 1) / gt;
   const long long units = static_cast<long long>(dp.num_kv_heads) * dp.head_blocks * batch;
   const int cluster = decode_cluster(units, max_count, sms);
-  if (cluster > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-    return PKV_ERR_CUDA;                           // clusters of 16 CTAs are an opt-in of the kernel
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(cluster * dp.num_kv_heads * dp.head_blocks, batch);
   cfg.blockDim = dim3(kDecThreads);

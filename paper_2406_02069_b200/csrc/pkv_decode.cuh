@@ -4,7 +4,7 @@
 // What bounds it: the cache is read once, so the floor is its bytes over the memory bandwidth (a few microseconds);
 // below that it is a chain of latencies (launch, loads, merges) and, on the fp32 pipe, the instructions per row: with one
 // warp instruction per 2 rows x 8 channels a step of 8 rows took a warp 400 of them.
-//   * One cluster of 1..16 CTAs per (sequence, KV head, block of query heads): every K and V row is read once for all
+//   * One cluster of 1..8 CTAs per (sequence, KV head, block of query heads): every K and V row is read once for all
 //     query heads of its block, and few long row lists still spread over the chip.  No scratch memory is needed (this
 //     call has no workspace): the CTAs hand their sums to one another through distributed shared memory, each channel
 //     to the CTA that finishes it, with one cluster barrier.
@@ -12,7 +12,10 @@
 //     fp32 in effect: each is split into three 16-bit parts (hi + mid + lo carry 24 bits and more), which stand in
 //     different rows of the same M = 16 operand (4 heads x 3 parts), so that the split costs no extra products.
 //   * fp32 rows stay on the fp32 pipe (decode_attention_kernel).
-// Measured on one B200, one token through 32 layers, 8 KV heads x 4 query heads, d = 128, bf16: see launch_decode.
+// Measured on one B200, one token through 32 layers, 8 KV heads x 4 query heads, d = 128, bf16: 2048 rows a head on
+// average, one sequence (269 MB): 8.8 ms with one CTA per query head (32 CTAs, each K and V row read four times), 365 us
+// with clusters on the fp32 pipe, 256 us on mma.sync; 512 rows, eight sequences, pages of 16 rows (543 MB): 3.3 ms, 397,
+// 330 us.  (Loads of the next tile under this one's products: 272 / 345 us, the copies cost more than they hide.)
 #pragma once
 
 #include <cooperative_groups.h>
@@ -24,7 +27,8 @@ namespace pkv {
 
 constexpr int kDecThreads = 256;
 constexpr int kDecWarps = kDecThreads / 32;
-constexpr int kDecMaxCluster = 16;
+constexpr int kDecMaxCluster = 8;         // 16 CTAs need a GPC to themselves: their launches cannot overlap (+4.5 us each)
+constexpr int kDecPrefetchRows = 512;     // rows a CTA brings into the L2 while it waits
 constexpr int kDecMinRows = 64;            // rows a CTA should have before a cluster grows: one step of its teams
 
 struct DecodeParams {
@@ -354,6 +358,20 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_mma_kernel(const Decode
   const int64_t hq0 = static_cast<int64_t>(b) * p.num_kv_heads * p.group + static_cast<int64_t>(h) * p.group + g0;
   const T* kc = static_cast<const T*>(p.k_cache);
   const T* vc = static_cast<const T*>(p.v_cache);
+  // While the kernels ahead in the stream finish, this CTA's rows come into the L2 (a prefetch hands no data to anybody, so
+  // it does not matter whether they are still being written; a page table read here is only used for it).
+  for (int i = threadIdx.x; i < min(hi - lo, kDecPrefetchRows) * 2; i += kDecThreads) {     // K and V rows in turn
+    int64_t at = row0 + lo + i / 2;
+    if (PAGED) {
+      const int r = lo + i / 2;
+      const int page = __ldcg(p.pt.table + p.pt.tab_off[b] + static_cast<int64_t>(h) * p.pt.pages[b] + r / p.pt.page_size);
+      if (page < 0 || page >= p.pt.num_pages) continue;
+      at = static_cast<int64_t>(page) * p.pt.page_size + r % p.pt.page_size;
+    }
+    const T* row = (i & 1 ? vc : kc) + at * D;
+#pragma unroll
+    for (int e = 0; e < D; e += 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + e));
+  }
   pdl_wait();
 
   uint4 q[KC];
