@@ -750,14 +750,17 @@ int run_select(const pkv_config* c, const float* scores, int64_t ld, const SeqTa
                  : (wide ? reinterpret_cast<const void*>(pool_select_kernel<false, 8>) : reinterpret_cast<const void*>(pool_select_kernel<false, 1>));
   } else {
     kernel = avg ? select_instance<true>(slice, &threads) : select_instance<false>(slice, &threads);
-    // room for the staged scores, and for the keys of all candidates (about k per CTA, or about k in all)
+    // room for the keys of the cluster's candidates: about k from each CTA, or about k in all
     int k_max = 0;
     for (int b = 0; b < batch; ++b) k_max = std::max(k_max, table.count[b] - c->window);
     sp.common_rows = kSelCommonCandidates / cluster;
-    const int expect = k_max > sp.common_rows ? k_max + k_max / 4 : cluster * (k_max + k_max / 4);
-    const int raw = static_cast<int>(sel_smem_floats(slice)), most = static_cast<int>((kSelSmemMax - static_cast<size_t>(slice) * 8) / 4);
-    sp.flat_cap = std::max(raw, std::min(std::min(max_p, expect) + 256, most)) & ~3;
-    smem = static_cast<size_t>(sp.flat_cap) * 4 + static_cast<size_t>(slice) * 8;
+    sp.max_slice = slice;
+    sp.raw_floats = static_cast<int>(sel_smem_floats(slice));
+    if (cluster > 1) {
+      const int most = static_cast<int>((kSelSmemMax - sel_smem_bytes(slice, 0, 0)) / 4) / cluster;
+      sp.inbox = std::min(std::min(slice, k_max + k_max / 4 + 64), most) & ~3;
+    }
+    smem = sel_smem_bytes(slice, cluster, sp.inbox);
   }
   static bool attr_done[64] = {};  // the attribute is per device; setting it twice is harmless
   int dev = 0;

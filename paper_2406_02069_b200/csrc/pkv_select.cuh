@@ -68,7 +68,9 @@ struct SelectParams {
   int32_t pieces;           // 16-byte pieces per row = d * elem_bytes / 16
   int32_t log_pieces;       // log2 of that
   int32_t vec;              // score rows start on 16-byte boundaries
-  int32_t flat_cap;         // floats in front of a CTA's candidate list in shared memory (a multiple of 4)
+  int32_t max_slice;        // positions of the longest slice of the launch
+  int32_t raw_floats;       // floats of the staged scores in shared memory (a multiple of 4)
+  int32_t inbox;            // keys that a CTA has room for from each CTA of its cluster (a multiple of 4)
   int32_t common_rows;      // lists of more rows than this take one bound for the whole cluster
   int32_t paged;            // kept rows go to page slots of k_out / v_out through pt instead of packed rows
   PageTable pt;
@@ -466,8 +468,8 @@ __global__ void __launch_bounds__(kSelThreads, 1) pool_select_kernel(const Selec
 //     counts with the number of its positions that hold its maximum (pooled scores come in plateaus), so that the bound
 //     lets through about k positions.  Short lists take a bound per CTA (about k candidates each); for long ones the
 //     CTAs' histograms are added up first, one cluster barrier more, and about k candidates are left in all;
-//   * every CTA of the cluster finishes on its own: it reads the candidates of all (distributed shared memory), finds
-//     the threshold, and emits and copies the rows of its own slice.  There is one full cluster barrier (up to three
+//   * every CTA of the cluster finishes on its own: it is sent the candidates of all (distributed shared memory), finds
+//     the threshold, and emits and copies the rows of its own slice, which it has brought into the L2 by then.  There is one full cluster barrier (up to three
 //     when the list is long) and no trip through global memory;
 //   * the exact threshold is searched inside [largest bound of the CTAs, largest key], ten bits a pass, and finished by
 //     a warp as soon as at most 32 candidates are left in the bin (mostly after the first pass).
@@ -571,9 +573,12 @@ __device__ __forceinline__ void sel_pool_run(const float* raw, int at, int radiu
 // Dynamic shared memory of an instance for slices of `slice` positions (a multiple of 32).
 __host__ __device__ constexpr size_t sel_smem_floats(int slice) { return static_cast<size_t>(slice + 2 * kSelHalo) * 9 / 8 + 4; }
 constexpr size_t kSelSmemMax = 208 * 1024;
+// Staged scores, the CTA's candidates (4-byte keys, 2-byte offsets in the slice), keys from the cluster.
+__host__ __device__ constexpr size_t sel_smem_bytes(int slice, int cluster, int inbox) {
+  return (sel_smem_floats(slice) + static_cast<size_t>(slice) + static_cast<size_t>(slice) / 2 + static_cast<size_t>(cluster) * inbox) * 4;
+}
 
-// grid (cluster * H_kv, batch), cluster (cluster, 1, 1), block THREADS, dynamic shared memory flat_cap floats and
-// eight bytes per position of a slice.
+// grid (cluster * H_kv, batch), cluster (cluster, 1, 1), block THREADS, dynamic shared memory sel_smem_bytes.
 // RUNS runs of eight positions per thread: a CTA takes at most THREADS * RUNS * 8 positions.
 template <int THREADS, int RUNS, bool AVG>
 __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kernel(const SelectParams p) {
@@ -584,7 +589,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
   __shared__ uint32_t rows[32];
   __shared__ uint32_t warp_a[WARPS], warp_b[WARPS], warp_c[WARPS], warp_d[WARPS];
   __shared__ uint32_t few[32], few_n;
-  __shared__ uint4 pub;                                     // candidates, bound, largest key: read by the whole cluster
+  __shared__ uint4 pub[kSelMaxCluster];                     // every CTA's number of candidates, bound, largest key
 
   pdl_trigger();
   cg::cluster_group cluster = cg::this_cluster();
@@ -601,9 +606,11 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
   const int64_t head = static_cast<int64_t>(b) * p.num_kv_heads + h;
   const int64_t row0 = p.seq.row_off[b] + static_cast<int64_t>(h) * count;
   int32_t* out = p.indices + row0;
-  float* raw = reinterpret_cast<float*>(sel_dyn);           // staged scores; later keys of all candidates, then own list
-  const int flat_cap = p.flat_cap;
-  uint2* list = reinterpret_cast<uint2*>(sel_dyn + static_cast<size_t>(flat_cap) * 4);   // own candidates (key, position)
+  float* raw = reinterpret_cast<float*>(sel_dyn);           // staged scores; later the positions this CTA keeps
+  uint32_t* list_key = reinterpret_cast<uint32_t*>(raw + p.raw_floats);                 // own candidates in position order
+  uint16_t* list_pos = reinterpret_cast<uint16_t*>(list_key + p.max_slice);                // ... offsets in the slice
+  uint32_t* inbox = list_key + p.max_slice + p.max_slice / 2;                           // [C][p.inbox] everybody's keys
+  if (C > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");              // this CTA's inbox may be written
 
   for (int i = tid; i < 2 * kSelBinsLin; i += THREADS) (&hist[0][0])[i] = 0;
   if (tid == 0) few_n = 0;
@@ -667,6 +674,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
 
     // ---- lower bound of the k-th key, candidates in position order
     const bool common = C > 1 && k > p.common_rows;         // uniform over the cluster
+    if (C > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");              // every CTA has started
     if (common) {
       cluster.sync();
       for (int i = tid; i < kSelBinsLin; i += THREADS) {
@@ -734,54 +742,54 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
         if ((c2 >> (16 * r)) & 0xffffu) {
 #pragma unroll
           for (int j = 0; j < kSelRun; ++j)
-            if (at + j < len && key[r][j] >= bound) list[to++] = make_uint2(key[r][j], static_cast<uint32_t>(lo + at + j));
+            if (at + j < len && key[r][j] >= bound) {
+              list_key[to] = key[r][j];
+              list_pos[to++] = static_cast<uint16_t>(at + j);
+            }
         }
       }
     }
     mx = __reduce_max_sync(full, warp_a[lane & (WARPS - 1)]);
-    if (tid == 0) pub = make_uint4(static_cast<uint32_t>(M), bound, mx, 0u);
     for (int i = tid; i < 2 * kSelBinsLin; i += THREADS) (&local[0][0])[i] = 0;
+    __syncthreads();
+    // every CTA gets everybody's keys: stores into the others' shared memory, which nobody waits for until the barrier
+    // (reading them there after it cost 2 to 3 us)
+    if (tid < C) {
+      const uint4 mine = make_uint4(static_cast<uint32_t>(M), bound, mx, 0u);
+      if (C == 1) pub[0] = mine; else cluster.map_shared_rank(&pub[0], tid)[rank] = mine;
+    }
+    if (C > 1)
+      for (int i = tid; i < min(M, p.inbox); i += THREADS) {
+        const uint32_t x = list_key[i];
+        for (int c = 0; c < C; ++c)
+          if (c != rank) cluster.map_shared_rank(inbox, c)[rank * p.inbox + i] = x;
+      }
     if (C == 1) __syncthreads(); else cluster.sync();       // candidates of the whole cluster are in place
 
     // ---- the threshold T (k-th largest key) and how many ties at T are taken
-    uint32_t m_c = 0, b_c = 0, x_c = 0;
-    if (lane < C) {
-      const uint4 o = C == 1 ? pub : *cluster.map_shared_rank(&pub, lane);
-      m_c = o.x; b_c = o.y; x_c = o.z;
-    }
-    uint32_t pre[kSelMaxCluster + 1];
-    pre[0] = 0;
+    uint32_t base = 0, top = 0;                             // at least k keys of some CTA, so of all, reach its bound
 #pragma unroll
-    for (int c = 0; c < kSelMaxCluster; ++c) pre[c + 1] = pre[c] + __shfl_sync(full, m_c, c);
-    const int N = static_cast<int>(pre[kSelMaxCluster]);
-    uint32_t base = __reduce_max_sync(full, b_c);           // at least k keys of some CTA, so of all, reach its bound
-    const uint32_t top = __reduce_max_sync(full, x_c);
-    uint32_t* flat = reinterpret_cast<uint32_t*>(raw);      // the raw scores are dead: keys of all candidates
-    auto remote = [&](int j) -> uint32_t {
-      if (C == 1) return list[j].x;
-      int c = 0;
-#pragma unroll
-      for (int q = 1; q < kSelMaxCluster; ++q) c += static_cast<uint32_t>(j) >= pre[q] ? 1 : 0;
-      uint32_t from = 0;
-#pragma unroll
-      for (int q = 1; q < kSelMaxCluster; ++q) from = c == q ? pre[q] : from;
-      return cluster.map_shared_rank(list, c)[j - static_cast<int>(from)].x;
+    for (int c = 0; c < kSelMaxCluster; ++c)
+      if (c < C) {
+        const uint4 o = pub[c];
+        base = max(base, o.y);
+        top = max(top, o.z);
+      }
+    // Key i of CTA c; a CTA whose candidates did not fit its place in the inbox is asked for the rest.  The warps are
+    // dealt round to the CTAs: warp w takes CTA w % C, 32 keys at a time.
+    auto key_at = [&](int c, int i) -> uint32_t {
+      if (c == rank) return list_key[i];
+      return i < p.inbox ? inbox[c * p.inbox + i] : cluster.map_shared_rank(list_key, c)[i];
     };
-    const int held = min(N, flat_cap);
-    auto at_flat = [&](int j) -> uint32_t { return j < held ? flat[j] : remote(j); };
+    const int my_c = warp & (C - 1), my_first = (warp / C) * 32 + lane, my_step = (WARPS / C) * 32;
+    const int my_n = static_cast<int>(pub[my_c].x);
     uint32_t want = static_cast<uint32_t>(k), T = 0, need_eq = 0;
     int shift = max(0, 22 - __clz(top - base));
     uint32_t span = 0xffffffffu;                            // keys base .. base + span take part
     for (int pass = 0;; ++pass) {
       uint32_t* hc = local[pass & 1];
-      for (int j = tid; j < N; j += THREADS) {
-        uint32_t x;
-        if (pass == 0) {
-          x = remote(j);
-          if (j < held) flat[j] = x;
-        } else {
-          x = at_flat(j);
-        }
+      for (int i = my_first; i < my_n; i += my_step) {
+        const uint32_t x = key_at(my_c, i);
         if (x >= base && x - base <= span) atomicAdd(&hc[(x - base) >> shift], 1u);
       }
       __syncthreads();
@@ -790,14 +798,25 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
       want -= above;
       base += digit << shift;
       const uint32_t in_bin = hc[digit];
+      if (pass == 0 && p.k_out != nullptr) {                // all but a few of the rows to copy are known: into the L2
+        const int64_t ks = p.k.st * p.elem_bytes, vs = p.v.st * p.elem_bytes;
+        const char* kb = static_cast<const char*>(p.k.ptr) + (b * p.k.sb + h * p.k.sh + static_cast<int64_t>(lo) * p.k.st) * p.elem_bytes;
+        const char* vb = static_cast<const char*>(p.v.ptr) + (b * p.v.sb + h * p.v.sh + static_cast<int64_t>(lo) * p.v.st) * p.elem_bytes;
+        for (int i = tid; i < M; i += THREADS)
+          if (list_key[i] >= base)
+            for (int c = 0; c < p.pieces * 16; c += 128) {
+              asm volatile("prefetch.global.L2 [%0];" ::"l"(kb + list_pos[i] * ks + c));
+              asm volatile("prefetch.global.L2 [%0];" ::"l"(vb + list_pos[i] * vs + c));
+            }
+      }
       if (shift == 0) {
         T = base;
         need_eq = want;
         break;
       }
       if (in_bin <= 32u) {                                  // few enough for a warp: rank them by counting
-        for (int j = tid; j < N; j += THREADS) {
-          const uint32_t x = at_flat(j);
+        for (int i = my_first; i < my_n; i += my_step) {
+          const uint32_t x = key_at(my_c, i);
           if (x >= base && ((x - base) >> shift) == 0) few[atomicAdd(&few_n, 1u)] = x;
         }
         __syncthreads();
@@ -822,15 +841,13 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
 
     // ---- emit: kept = keys above T and the leftmost need_eq of those at T.  Counted over the candidates of the CTAs
     //      before this one (where its part of the list starts) and over its own, warp by warp in contiguous chunks
-    int own_lo = 0;                                         // candidates of the CTAs before this one
-#pragma unroll
-    for (int q = 1; q < kSelMaxCluster; ++q) own_lo = rank == q ? static_cast<int>(pre[q]) : own_lo;
     uint32_t pgt = 0, peq = 0;
-    for (int j = tid; j < own_lo; j += THREADS) {
-      const uint32_t x = at_flat(j);
-      pgt += x > T ? 1u : 0u;
-      peq += x == T ? 1u : 0u;
-    }
+    if (my_c < rank)
+      for (int i = my_first; i < my_n; i += my_step) {
+        const uint32_t x = key_at(my_c, i);
+        pgt += x > T ? 1u : 0u;
+        peq += x == T ? 1u : 0u;
+      }
     pgt = __reduce_add_sync(full, pgt);
     peq = __reduce_add_sync(full, peq);
     const int chunk = (((M + WARPS - 1) / WARPS) + 31) & ~31;
@@ -838,7 +855,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
     uint32_t ngt = 0, neq = 0;
     for (int j0 = j_lo; j0 < j_hi; j0 += 32) {
       const int j = j0 + lane;
-      const uint32_t x = j < j_hi ? list[j].x : 0u;
+      const uint32_t x = j < j_hi ? list_key[j] : 0u;
       ngt += __popc(__ballot_sync(full, j < j_hi && x > T));
       neq += __popc(__ballot_sync(full, j < j_hi && x == T));
     }
@@ -856,20 +873,23 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
     if (rank == C - 1 && tid == 0 && own1 != k) atomicOr(p.status, kStatusSelectMismatch);
     for (int j0 = j_lo; j0 < j_hi; j0 += 32) {
       const int j = j0 + lane;
-      const uint2 kv = j < j_hi ? list[j] : make_uint2(0u, 0u);
+      const uint2 kv = j < j_hi ? make_uint2(list_key[j], static_cast<uint32_t>(lo) + list_pos[j]) : make_uint2(0u, 0u);
       const bool is_gt = j < j_hi && kv.x > T, is_eq = j < j_hi && kv.x == T;
       const uint32_t bg = __ballot_sync(full, is_gt), be = __ballot_sync(full, is_eq);
       const uint32_t g = gt_before + __popc(bg & lt), e = eq_before + __popc(be & lt);
       if (is_gt || (is_eq && e < need_eq)) {
         const int at = static_cast<int>(g + min(e, need_eq));
         out[at] = static_cast<int32_t>(kv.y);
-        kept[at - own0] = static_cast<int32_t>(kv.y);       // over the flat keys, which nobody reads any more
+        kept[at - own0] = static_cast<int32_t>(kv.y);       // over the scores, which nobody reads any more
       }
       gt_before += __popc(bg);
       eq_before += __popc(be);
     }
     if (C > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");   // done with the others' memory
-  } else if (k >= P) {                                      // nothing to evict: this CTA's share of the identity list
+  } else if (C > 1) {
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  }
+  if (!selecting && k >= P) {                               // nothing to evict: this CTA's share of the identity list
     own0 = lo;
     own1 = lo + len;
     for (int i = tid; i < len; i += THREADS) out[lo + i] = lo + i;
