@@ -465,34 +465,13 @@ int launch_scores_tc(const pkv_config* c, const pkv_tensor& q, const pkv_tensor&
   tp.scores = sp.scores;
   tp.ld_scores = sp.ld_scores;
   tp.status = status;
-  // Key tiles per work item: the largest power of two that still spreads the items evenly over the SMs.
-  auto items_for = [&](int ct, int tile_keys, bool prefix) {
-    long long items = 0;
-    for (int b = 0; b < batch; ++b) {
-      const int keys = prefix ? sp.seq.prefix[b] : sp.seq.n[b];
-      const int tiles = (keys + tile_keys - 1) / tile_keys;
-      items += (tiles + ct - 1) / ct;
-    }
-    return items * sp.num_kv_heads;
-  };
-  auto pick = [&](int tile_keys, bool prefix) {
-    int ct = 16;
-    for (; ct > 1; ct /= 2) {
-      const long long items = items_for(ct, tile_keys, prefix);
-      const long long waves = (items + sms - 1) / sms;
-      if (items >= sms && static_cast<double>(items) / static_cast<double>(waves * sms) >= 0.93) break;
-    }
-    return ct;
-  };
-  tp.chunk_tiles_a = pick(kTcTileKeys, false);
-  tp.chunk_tiles_b = pick(kTcTileKeys, true);
+  // Every CTA takes a contiguous range of key tiles (sequence, head, tile), a tile more or less than the others.
   int stat_items = 0, score_items = 0;
   for (int b = 0; b < batch; ++b) {
     tp.seq.stat_off[b] = stat_items;
     tp.seq.score_off[b] = score_items;
-    stat_items += ((sp.seq.n[b] + kTcTileKeys - 1) / kTcTileKeys + tp.chunk_tiles_a - 1) / tp.chunk_tiles_a;
-    score_items += ((sp.seq.prefix[b] + kTcTileKeys - 1) / kTcTileKeys + tp.chunk_tiles_b - 1) /
-                   tp.chunk_tiles_b;
+    stat_items += (sp.seq.n[b] + kTcTileKeys - 1) / kTcTileKeys;
+    score_items += (sp.seq.prefix[b] + kTcTileKeys - 1) / kTcTileKeys;
   }
   tp.seq.stat_off[batch] = stat_items;
   tp.seq.score_off[batch] = score_items;

@@ -45,7 +45,7 @@ constexpr int kTcMaxRows = 256;         // window rows (G * alpha) the tensor-co
 constexpr long long kTcWaitCycles = 1ll << 31;   // bound of any one wait, in SM clocks
 
 struct TcParams {
-  SeqTable seq;                 // stat_off / score_off count CHUNKS of chunk_tiles tiles
+  SeqTable seq;                 // stat_off / score_off count key tiles (of all keys / of the prefix)
   int32_t num_kv_heads, group, rows;      // rows = group * alpha (R)
   int32_t rows_pad;             // R rounded up to 32
   int32_t fp16;                 // 1: Q and K hold binary16, 0: bfloat16 (both operands always share the type)
@@ -56,8 +56,6 @@ struct TcParams {
   int32_t withhold;             // test aid: CTA 0 of sweep A never loads its last K tile (its waits then run out)
   long long wait_clocks;        // bound of any one wait, in SM clocks
   int32_t row_blocks;           // ceil(R / 128): M-blocks of sweep A
-  int32_t chunk_tiles_a;        // key tiles per work item of sweep A
-  int32_t chunk_tiles_b;        // key tiles per work item of sweep B
   float scale_log2;             // log2(e) / sqrt(d)
   float2* partial;              // sweep A out: [segment][R] (reference exponent, sum); a segment is one CTA's run over one
                                 // (sequence, head)
@@ -134,6 +132,19 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
+// The same with a cache policy for the lines it brings into the L2.
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2, int c3,
+                                            uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5, %6}], [%2], %7;"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "l"(policy)
+      : "memory");
+}
+__device__ __forceinline__ uint64_t l2_evict_first() {
+  uint64_t policy;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  return policy;
+}
 // Brings a box of a tensor into the L2.
 __device__ __forceinline__ void tma_prefetch_4d(const CUtensorMap* map, int c0, int c1, int c2, int c3) {
   asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global [%0, {%1, %2, %3, %4}];" ::"l"(reinterpret_cast<uint64_t>(map)), "r"(c0),
@@ -177,9 +188,11 @@ __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sy
 // The special-function unit evaluates 16 exponentials per clock per SM, which is what bounds both
 // sweeps when every 2^x goes through it.  A fixed share of the exponentials is therefore evaluated on
 // the FMA pipe instead, two at a time with the packed fp32 instructions.  Of every eight consecutive
-// pairs of values (16 accumulator columns), kTcPolyPairs go this way, spread evenly over the eight.
+// pairs of values (16 accumulator columns), kTcPolyPairs go this way, spread evenly over the eight.  Measured at 0 / 1 / 2 /
+// 3 / 4 of 8: one layer of 131072 tokens (at the board's power cap) 211 / 206 / 209 / 213 / 223 us, 32768 tokens 54.8 / 53.6
+// / 54.0 / 53.5 / 55.1 us, 32 ragged layers 2.71 / 2.70 / 2.76 / 2.82 / 2.87 ms.
 #ifndef PKV_POLY_PAIRS
-#define PKV_POLY_PAIRS 2
+#define PKV_POLY_PAIRS 1
 #endif
 constexpr int kTcPolyPairs = PKV_POLY_PAIRS;    // 0 = every exponential on the special-function unit
 __host__ __device__ constexpr bool tc_pair_is_poly(int pair) {
@@ -295,7 +308,7 @@ __device__ __forceinline__ uint32_t instr_desc_16bit(int M, int N, int fp16) {
          (static_cast<uint32_t>(M >> 4) << 24);
 }
 
-// Work item -> (sequence, head, chunk).  Items are ordered sequence, head, chunk.
+// Work item -> (sequence, head, chunk).  Items are ordered sequence, head, chunk (in the sweeps a chunk is a key tile).
 struct TcItem { int b, h, c, nchunks; };
 __device__ __forceinline__ TcItem tc_item(const int32_t* off, int batch, int heads, int id) {
   int b = 0;
@@ -380,6 +393,26 @@ __device__ __forceinline__ void tc_normalisers(const TcParams& p, int b, int h, 
       val = -fmaf(p.lse2[static_cast<int64_t>(hg) * p.rows + r], p.lse_scale, p.lse_add);
     }
     if (part == 0) dst[r] = val;
+  }
+}
+
+// The item behind (REVERSE: before) w; behind the last one w stays on its sequence.
+template <bool REVERSE>
+__device__ __forceinline__ void tc_next(const int32_t* off, int batch, int heads, TcItem& w) {
+  if (REVERSE) {
+    if (--w.c >= 0) return;
+    if (--w.h < 0) {
+      w.h = heads - 1;
+      if (w.b > 0) { --w.b; w.nchunks = off[w.b + 1] - off[w.b]; }
+    }
+    w.c = w.nchunks - 1;
+  } else {
+    if (++w.c < w.nchunks) return;
+    w.c = 0;
+    if (++w.h == heads) {
+      w.h = 0;
+      if (w.b + 1 < batch) { ++w.b; w.nchunks = off[w.b + 1] - off[w.b]; }
+    }
   }
 }
 
@@ -480,17 +513,15 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  // ---- this CTA's contiguous range of work items
+  // ---- this CTA's contiguous range of key tiles
   const int32_t* off = SWEEP == 0 ? p.seq.stat_off : p.seq.score_off;
-  const int chunk_tiles = SWEEP == 0 ? p.chunk_tiles_a : p.chunk_tiles_b;
   const int total = p.num_kv_heads * off[p.seq.batch];
   const int per = total / gridDim.x, rem = total % gridDim.x;
   const int item0 = blockIdx.x * per + min(static_cast<int>(blockIdx.x), rem);
   const int item1 = item0 + per + (static_cast<int>(blockIdx.x) < rem ? 1 : 0);
-  // keys an item of sequence b spans: sweep A covers all n keys, sweep B the prefix only
-  auto span_keys = [&](int b) { return SWEEP == 0 ? p.seq.n[b] : p.seq.prefix[b]; };
-  auto item_at = [&](int ii) { return tc_item(off, p.seq.batch, p.num_kv_heads, kReverse ? item1 - 1 - ii : item0 + ii); };
-  auto last_tile = [&](const TcItem& w) { return min((w.c + 1) * chunk_tiles, (span_keys(w.b) + kTileKeys - 1) / kTileKeys); };
+  const int ntiles = item1 - item0;
+  auto first_tile = [&]() { return tc_item(off, p.seq.batch, p.num_kv_heads, kReverse ? item1 - 1 : item0); };
+  auto next_tile = [&](TcItem& w) { tc_next<kReverse>(off, p.seq.batch, p.num_kv_heads, w); };
 
   // Copies and MMAs touch only the caller's Q and K.  With `early` they start at once, beside the tail of the kernels
   // ahead in the stream; then sweep A waits just before its first write (its partials), sweep B just before it reads
@@ -499,19 +530,10 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
   // whether the kernels ahead still write them.
   if (!p.early) {
     if (warp == 0 && lane == 0) {
-      int left = p.prefetch_tiles;
-      if (item0 < item1) {
-        const TcItem w = item_at(0);
-        for (int half = 0; half < L::kHalves; ++half) tma_prefetch_4d(&q_map, half * 64, 0, w.h * p.group, w.b);
-      }
-      for (int ii = 0; ii < item1 - item0 && left > 0; ++ii) {
-        const TcItem w = item_at(ii);
-        const int tile0 = w.c * chunk_tiles, tile1 = last_tile(w);
-        for (int tt = 0; tt < tile1 - tile0 && left > 0; ++tt, --left) {
-          const int t = kReverse ? tile1 - 1 - tt : tile0 + tt;
-          for (int half = 0; half < L::kHalves; ++half) tma_prefetch_4d(&k_map, half * 64, t * kTileKeys, w.h, w.b);
-        }
-      }
+      TcItem w = first_tile();
+      for (int half = 0; half < L::kHalves; ++half) tma_prefetch_4d(&q_map, half * 64, 0, w.h * p.group, w.b);
+      for (int it = 0; it < min(ntiles, p.prefetch_tiles); ++it, next_tile(w))
+        for (int half = 0; half < L::kHalves; ++half) tma_prefetch_4d(&k_map, half * 64, w.c * kTileKeys, w.h, w.b);
     }
     pdl_wait();
     if (SWEEP == 0) pdl_trigger();
@@ -521,21 +543,20 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
     // =========================================================== TMA producer of K
     if (lane == 0) {
       uint32_t it = 0;                                         // K tiles
+      // behind a sweep A this is the last time a tile is read
+      const uint64_t policy = l2_evict_first();
       bool ok = true;
-      for (int ii = 0; ii < item1 - item0 && ok; ++ii) {
-        const TcItem w = item_at(ii);
-        const int tile0 = w.c * chunk_tiles, tile1 = last_tile(w);
-        for (int tt = 0; tt < tile1 - tile0 && ok; ++tt, ++it) {
-          const int t = kReverse ? tile1 - 1 - tt : tile0 + tt;
-          const int s = it % kKStages;
-          ok = mbar_wait(k_empty(s), ((it / kKStages) & 1) ^ 1, abort_flag, p.wait_clocks);
-          if (!ok) break;
-          if (SWEEP == 0 && p.withhold && blockIdx.x == 0 && ii + 1 == item1 - item0 && tt + 1 == tile1 - tile0)
-            continue;                                       // test aid: this tile never arrives
-          mbar_expect_tx(k_full(s), kStageBytes);
-          for (int half = 0; half < L::kHalves; ++half)
-            tma_load_4d(smem_u32(k_s) + s * kStageBytes + half * kTileKeys * 128, &k_map, k_full(s), half * 64,
-                        t * kTileKeys, w.h, w.b);
+      TcItem w = first_tile();
+      for (; static_cast<int>(it) < ntiles; ++it, next_tile(w)) {
+        const int s = it % kKStages;
+        ok = mbar_wait(k_empty(s), ((it / kKStages) & 1) ^ 1, abort_flag, p.wait_clocks);
+        if (!ok) break;
+        if (SWEEP == 0 && p.withhold && blockIdx.x == 0 && static_cast<int>(it) + 1 == ntiles) continue;   // test aid: never arrives
+        mbar_expect_tx(k_full(s), kStageBytes);
+        for (int half = 0; half < L::kHalves; ++half) {
+          const uint32_t dst = smem_u32(k_s) + s * kStageBytes + half * kTileKeys * 128;
+          if (SWEEP == 1 && p.merge) tma_load_4d(dst, &k_map, k_full(s), half * 64, w.c * kTileKeys, w.h, w.b, policy);
+          else tma_load_4d(dst, &k_map, k_full(s), half * 64, w.c * kTileKeys, w.h, w.b);
         }
       }
       if (!ok) {
@@ -552,8 +573,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
       uint32_t heads = 0;
       int cur_b = -1, cur_h = -1;
       bool ok = true;
-      for (int ii = 0; ii < item1 - item0 && ok; ++ii) {
-        const TcItem w = item_at(ii);
+      TcItem w = first_tile();
+      for (int ii = 0; ii < ntiles; ++ii, next_tile(w)) {
         if (w.b == cur_b && w.h == cur_h) continue;
         cur_b = w.b; cur_h = w.h;
         const uint32_t slot = heads % q_slots, round = heads / q_slots;
@@ -580,8 +601,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
       const uint32_t idesc0 = SWEEP == 0 ? instr_desc_16bit(128, kTileKeys, p.fp16) : instr_desc_16bit(kTileKeys, split_b, p.fp16);
       const uint32_t idesc1 = SWEEP == 0 || !two_blocks ? idesc0 : instr_desc_16bit(kTileKeys, p.rows_pad - split_b, p.fp16);
       uint32_t slot = 0;
-      for (int ii = 0; ii < item1 - item0 && ok; ++ii) {
-        const TcItem w = item_at(ii);
+      TcItem w = first_tile();
+      for (; static_cast<int>(it) < ntiles && ok; ++it) {
         if (w.b != cur_b || w.h != cur_h) {
           slot = heads % q_slots;
           ok = mbar_wait(q_full(slot), (heads / q_slots) & 1, abort_flag, p.wait_clocks);
@@ -589,14 +610,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
           ++heads;
           cur_b = w.b; cur_h = w.h;
         }
-        // does the next item belong to another head?  then Q may be overwritten after this item's MMAs
-        bool last_of_head = ii + 1 >= item1 - item0;
-        if (!last_of_head) {
-          const TcItem nx = item_at(ii + 1);
-          last_of_head = nx.b != w.b || nx.h != w.h;
-        }
-        const int tile0 = w.c * chunk_tiles, tile1 = last_tile(w);
-        for (int tt = 0; tt < tile1 - tile0 && ok; ++tt, ++it) {
+        {
           const int s = it % kKStages;
           ok = mbar_wait(k_full(s), (it / kKStages) & 1, abort_flag, p.wait_clocks);
           if (!ok) break;
@@ -621,7 +635,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
           }
           if (ok) tc_commit(k_empty(s));
         }
-        if (ok && last_of_head) tc_commit(q_empty(slot));
+        // does the next tile belong to another head?  then Q may be overwritten after these MMAs
+        next_tile(w);
+        if (ok && (w.b != cur_b || w.h != cur_h || static_cast<int>(it) + 1 == ntiles)) tc_commit(q_empty(slot));
       }
     }
   } else if (warp == 3) {
@@ -658,8 +674,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
       }
       ++heads;
     };
-    for (int ii = 0; ii < item1 - item0 && ok; ++ii) {
-      const TcItem w = item_at(ii);
+    TcItem w = first_tile();
+    for (int ii = 0; ii < ntiles && ok; ++ii, next_tile(w)) {
       if (w.b == cur_b && w.h == cur_h) continue;
       if (SWEEP == 0 && ii > 0) finish(cur_b, cur_h);          // a run that has ended; the last one is the epilogue's
       cur_b = w.b; cur_h = w.h;
@@ -694,11 +710,13 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
       z = 0.f;
       return true;
     };
-    for (int ii = 0; ii < item1 - item0 && ok; ++ii) {
-      const TcItem w = item_at(ii);
-      const int n = p.seq.n[w.b], alpha = p.seq.alpha, P = p.seq.prefix[w.b];
-      const int tile0 = w.c * chunk_tiles, tile1 = last_tile(w);
+    TcItem w = first_tile();
+    int n = 0, P = 0;
+    const int alpha = p.seq.alpha;
+    float* srow = nullptr;                      // sweep B: the head's scores
+    for (int ii = 0; ii < ntiles && ok; ++ii, next_tile(w)) {
       const bool new_head = w.b != cur_b || w.h != cur_h;
+      if (new_head) { n = p.seq.n[w.b]; P = p.seq.prefix[w.b]; }
       if (SWEEP == 0) {
         // thread -> window row (and, with copies of the rows, share of the columns), the same in all units of the group: a
         // thread keeps one (reference, sum) per run of work items.
@@ -714,7 +732,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
           cur_b = w.b; cur_h = w.h;
           ++heads;
         }
-        for (int t = tile0; t < tile1 && ok; ++t) {
+        {
           for (int rb = 0; rb < p.row_blocks && ok; ++rb, ++u) {
             if (static_cast<int>(u % kTcStages) != grp) continue;        // another group's unit
             ok = mbar_wait(t_full(grp), (u / kTcStages) & 1, abort_flag, p.wait_clocks);
@@ -722,7 +740,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
             if (!ok) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + grp * kTcStageCols + col0;
-            const int key_base = t * kTileKeys + col0;
+            const int key_base = w.c * kTileKeys + col0;
             if (!warp_has_rows) {
               // only the hand-shake below
             } else if (key_base + cols - 1 <= min(P, n - 1)) {   // every key visible to every row: no mask
@@ -820,15 +838,16 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
           if (!ok) break;
           lse_s = lse_all + buf * 256;
           cur_b = w.b; cur_h = w.h;
+          srow = p.scores + (static_cast<int64_t>(w.b) * p.num_kv_heads + w.h) * p.ld_scores;
           ++heads;
         }
-        float* srow = p.scores + (static_cast<int64_t>(w.b) * p.num_kv_heads + w.h) * p.ld_scores;
         const float* nlse = lse_s + (blk ? split_b : 0);
         const int cols = blk ? p.rows_pad - split_b : split_b;
-        for (int tt = 0; tt < tile1 - tile0 && ok; ++tt, u += p.row_blocks) {
-          const int t = kReverse ? tile1 - 1 - tt : tile0 + tt;
-          if ((u + blk) % kTcStages != static_cast<uint32_t>(grp)) continue;     // another group's unit
-          ok = mbar_wait(t_full(grp), (u / kTcStages) & 1, abort_flag, p.wait_clocks);
+        const bool ours = (u + blk) % kTcStages == static_cast<uint32_t>(grp);   // or another group's unit
+        const uint32_t phase = (u / kTcStages) & 1;
+        u += p.row_blocks;
+        if (ours) {
+          ok = mbar_wait(t_full(grp), phase, abort_flag, p.wait_clocks);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           tc_fence_after();
@@ -869,10 +888,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
             }
           }
           ++mine;
-          const int i = t * kTileKeys + lane_row;
+          const int i = w.c * kTileKeys + lane_row;
           if (blk == 0 && i < P) srow[i] = sum;
         }
-        if (!ok) break;
       }
     }
     if (SWEEP == 0 && ok && heads > 0 && flush_run()) {       // the CTA's last run
