@@ -413,9 +413,15 @@ bool make_map(CUtensorMap* map, const pkv_tensor& t, bool fp16, int d, uint64_t 
 }
 
 
+// Where the tensor-core row-statistics sweep left its partials, for a kernel that merges them itself.
+struct TcStats {
+  SeqTable seq;
+  int grid, early;
+};
+
 template <int D>
 int launch_scores_tc(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, ScoreParams& sp, int batch,
-                     int max_n, uint32_t* status, cudaStream_t st) {
+                     int max_n, uint32_t* status, cudaStream_t st, TcStats* stats) {
   int sms = device_sm_count();
   if (sms <= 0) return PKV_ERR_CUDA;
   if (c->sweep_ctas > 0) sms = std::min(sms, static_cast<int>(c->sweep_ctas));   // the caller's share of the SMs
@@ -518,7 +524,11 @@ int launch_scores_tc(const pkv_config* c, const pkv_tensor& q, const pkv_tensor&
   if (sp.lse_in == sp.lse2) {                    // normalisers not supplied: sweep A
     launch_pdl(score_tc_kernel<D, 0>, grid_a, kTcThreads, TcSmem<D>::kTotal, st, q_map, k_map, tp);
     mark(st, "rowstats_tc");
-    if (sp.stats_only) {                         // the normalisers themselves are wanted: merge kernel
+    if (stats) {
+      stats->seq = tp.seq;
+      stats->grid = grid_a;
+      stats->early = tp.early;
+    } else if (sp.stats_only) {                  // the normalisers themselves are wanted: merge kernel
       launch_pdl(combine_stats_kernel, dim3((sp.rows + 31) / 32, sp.num_kv_heads, batch), kCombineThreads, 0, st, sp,
                  tp.log2_group);
       mark(st, "combine_stats");
@@ -536,7 +546,7 @@ int launch_scores_tc(const pkv_config* c, const pkv_tensor& q, const pkv_tensor&
 // window_lse: null, or the caller's natural-log row normalisers [batch][H_q][alpha] (then sweep A is skipped).
 int run_scores(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, const SeqTable& table, int batch,
                float* scores, int64_t ld, const Workspace& w, cudaStream_t st, const float* window_lse = nullptr,
-               bool stats_only = false) {
+               bool stats_only = false, TcStats* stats = nullptr) {
   ScoreParams sp{};
   sp.stats_only = stats_only ? 1 : 0;
   sp.q = view(q);
@@ -558,8 +568,8 @@ int run_scores(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, co
   if (tc_eligible(c)) {
     int max_n = 0;
     for (int b = 0; b < batch; ++b) max_n = std::max(max_n, table.n[b]);
-    return c->head_dim == 64 ? launch_scores_tc<64>(c, q, k, sp, batch, max_n, w.status, st)
-                             : launch_scores_tc<128>(c, q, k, sp, batch, max_n, w.status, st);
+    return c->head_dim == 64 ? launch_scores_tc<64>(c, q, k, sp, batch, max_n, w.status, st, stats)
+                             : launch_scores_tc<128>(c, q, k, sp, batch, max_n, w.status, st, stats);
   }
   if (c->dtype == PKV_DTYPE_FP32)
     return c->head_dim == 64 ? launch_scores_generic<float, 64>(sp, batch, st)
@@ -572,10 +582,11 @@ int run_scores(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, co
 }
 
 // ---------------------------------------------------------------- window attention fused with the scores
-// Needs the row normalisers in w.lse2 (run_scores with stats_only).  Writes the scores of the prefix positions and
+// Needs the partials of the row-statistics sweep (run_scores with stats).  Writes the scores of the prefix positions and
 // attn_out[batch][H_q][alpha][d].
-int run_attend(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, const pkv_tensor& v, const SeqTable& table,
-               int batch, int max_n, float* scores, int64_t ld, float* attn_out, const Workspace& w, cudaStream_t st) {
+int run_attend(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, const pkv_tensor& v, int batch,
+               int max_n, float* scores, int64_t ld, float* attn_out, const Workspace& w, const TcStats& stats,
+               cudaStream_t st) {
   const int sms = device_sm_count();
   if (sms <= 0) return PKV_ERR_CUDA;
   static bool attr_done[64] = {};
@@ -595,7 +606,7 @@ int run_attend(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, co
       !make_map(&v_map, v, fp16, kAtD, max_n, c->num_kv_heads, batch, kAtTileKeys, 1))
     return PKV_ERR_CUDA;
   AtParams ap{};
-  ap.seq = table;
+  ap.seq = stats.seq;
   ap.num_kv_heads = c->num_kv_heads;
   ap.group = group;
   ap.rows = group * c->window;
@@ -605,31 +616,19 @@ int run_attend(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, co
   ap.wait_clocks = test_wait > 0 ? test_wait : kTcWaitCycles;
   ap.withhold = g_test_withhold_attend.load();
   ap.scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(c->head_dim)));
-  ap.lse2 = w.lse2;
+  ap.partial = w.partial;
+  ap.merge = 1;
+  ap.stat_grid = stats.grid;
+  ap.wait_v = stats.early;
+  ap.log2_group = std::log2(static_cast<float>(group)) - kAtShift;
   ap.scores = scores;
   ap.ld_scores = ld;
   ap.o_partial = w.o_partial;
   ap.out = attn_out;
   ap.status = w.status;
   const int grid_cap = std::min(c->sweep_ctas > 0 ? std::min(sms, static_cast<int>(c->sweep_ctas)) : sms, kAtMaxGrid);
-  // Key tiles per work item: the largest power of two that still spreads the items evenly over the SMs.
-  auto items_for = [&](int ct) {
-    long long items = 0;
-    for (int b = 0; b < batch; ++b) items += ((table.n[b] + kAtTileKeys - 1) / kAtTileKeys + ct - 1) / ct;
-    return items * c->num_kv_heads;
-  };
-  int ct = 16;
-  for (; ct > 1; ct /= 2) {
-    const long long items = items_for(ct), waves = (items + grid_cap - 1) / grid_cap;
-    if (items >= grid_cap && static_cast<double>(items) / static_cast<double>(waves * grid_cap) >= 0.93) break;
-  }
-  ap.chunk_tiles = ct;
-  int items = 0;
-  for (int b = 0; b < batch; ++b) {
-    ap.seq.score_off[b] = items;
-    items += ((table.n[b] + kAtTileKeys - 1) / kAtTileKeys + ct - 1) / ct;
-  }
-  ap.seq.score_off[batch] = items;
+  static_assert(kAtTileKeys == kTcTileKeys, "the sweep's tiles");
+  const int items = stats.seq.stat_off[batch];
   ap.grid = static_cast<int>(std::min<long long>(grid_cap, static_cast<long long>(items) * c->num_kv_heads));
   launch_pdl(window_attend_kernel, ap.grid, kAtThreads, kAtSmemBytes, st, q_map, k_map, v_map, ap);
   mark(st, "window_attend");
@@ -1152,8 +1151,9 @@ static int attend_impl(const pkv_config* cfg, int32_t layer, pkv_tensor q_win, p
   const int64_t ld = scores_or_null ? ld_scores : w.ld_scores;
   if (ld < max_n - cfg->window) return PKV_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (int rc = run_scores(cfg, q_win, k, table, batch, scores, ld, w, st, nullptr, /*stats_only=*/true)) return rc;
-  if (int rc = run_attend(cfg, q_win, k, v, table, batch, max_n, scores, ld, attn_out, w, st)) return rc;
+  TcStats stats;
+  if (int rc = run_scores(cfg, q_win, k, table, batch, scores, ld, w, st, nullptr, /*stats_only=*/true, &stats)) return rc;
+  if (int rc = run_attend(cfg, q_win, k, v, batch, max_n, scores, ld, attn_out, w, stats, st)) return rc;
   if (!compress) return PKV_OK;
   return run_select(cfg, scores, ld, table, batch, max_n, indices, w, st, &k, &v, k_out, v_out);
 }

@@ -53,13 +53,17 @@ constexpr int kAtSmemBytes = kAtMiscOff + kAtMiscBytes;     // 227 KB: all a CTA
 static_assert(kAtSmemBytes <= 232448, "shared memory of the window-attention kernel");
 
 struct AtParams {
-  SeqTable seq;                 // score_off counts this kernel's work items: chunks of chunk_tiles tiles over ALL n keys
+  SeqTable seq;                 // stat_off counts the key tiles over ALL n keys, here and in the row-statistics sweep
   int32_t num_kv_heads, group, rows, rows_pad, fp16;
-  int32_t chunk_tiles;
   int32_t withhold;             // test aid: CTA 0 never loads its last K tile (its waits then run out)
   long long wait_clocks;
   float scale_log2;             // log2(e) / sqrt(d)
-  const float* lse2;            // [batch][H_kv][R]: log2 of the row's sum of 2^x, plus log2 G
+  // the row normalisers come from the partials of the row-statistics sweep, as in the score sweep (tc_normalisers)
+  const float2* partial;
+  const float* lse2;
+  float lse_scale, lse_add, log2_group;      // log2 G - kAtShift
+  int32_t merge, stat_grid;
+  int32_t wait_v;               // 1: the sweep ahead started on the caller's word for Q and K alone: V waits for it to end
   float* scores;                // [batch][H_kv][ld]: the prefix positions are written
   int64_t ld_scores;
   float* o_partial;             // [segment][R][d]: a segment is one CTA's run over one (sequence, head)
@@ -184,17 +188,17 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  pdl_wait();                                                  // the normalisers come from the kernels before
+  // No wait here: Q, K and V are the caller's and the row-statistics sweep ahead has waited for them before it let this
+  // kernel start (or see wait_v); the epilogue waits before it reads the sweep's partials and before its first write.
 
-  const int32_t* off = p.seq.score_off;
+  const int32_t* off = p.seq.stat_off;
   const int total = p.num_kv_heads * off[p.seq.batch];
   const int per = total / gridDim.x, rem = total % gridDim.x;
   const int item0 = blockIdx.x * per + min(static_cast<int>(blockIdx.x), rem);
   const int item1 = item0 + per + (static_cast<int>(blockIdx.x) < rem ? 1 : 0);
-  auto tiles_of = [&](const TcItem& w, int& tile0, int& tile1) {
-    tile0 = w.c * p.chunk_tiles;
-    tile1 = min(tile0 + p.chunk_tiles, (p.seq.n[w.b] + kAtTileKeys - 1) / kAtTileKeys);
-  };
+  const int ntiles = item1 - item0;
+  auto first_tile = [&]() { return tc_item(off, p.seq.batch, p.num_kv_heads, item0); };
+  auto next_tile = [&](TcItem& w) { tc_next<false>(off, p.seq.batch, p.num_kv_heads, w); };
 
   if (warp == 0) {
     // =========================================================== TMA producer: Q per head, K per tile
@@ -202,8 +206,8 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
       uint32_t it = 0, heads_loaded = 0;
       int cur_b = -1, cur_h = -1;
       bool ok = true;
-      for (int id = item0; id < item1 && ok; ++id) {
-        const TcItem w = tc_item(off, p.seq.batch, p.num_kv_heads, id);
+      TcItem w = first_tile();
+      for (; static_cast<int>(it) < ntiles; ++it, next_tile(w)) {
         if (w.b != cur_b || w.h != cur_h) {
           if (heads_loaded > 0) ok = mbar_wait(q_empty, (heads_loaded - 1) & 1, abort_flag, p.wait_clocks);
           if (!ok) break;
@@ -213,16 +217,12 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
           ++heads_loaded;
           cur_b = w.b; cur_h = w.h;
         }
-        int tile0, tile1;
-        tiles_of(w, tile0, tile1);
-        for (int t = tile0; t < tile1 && ok; ++t, ++it) {
-          ok = mbar_wait(k_empty, (it & 1) ^ 1, abort_flag, p.wait_clocks);
-          if (!ok) break;
-          if (p.withhold && blockIdx.x == 0 && id + 1 == item1 && t + 1 == tile1) continue;   // test aid: never arrives
-          mbar_expect_tx(k_full, kAtTileBytes);
-          for (int half = 0; half < 2; ++half)
-            tma_load_4d(smem_u32(k_s) + half * kAtTileKeys * 128, &k_map, k_full, half * 64, t * kAtTileKeys, w.h, w.b);
-        }
+        ok = mbar_wait(k_empty, (it & 1) ^ 1, abort_flag, p.wait_clocks);
+        if (!ok) break;
+        if (p.withhold && blockIdx.x == 0 && static_cast<int>(it) + 1 == ntiles) continue;   // test aid: never arrives
+        mbar_expect_tx(k_full, kAtTileBytes);
+        for (int half = 0; half < 2; ++half)
+          tma_load_4d(smem_u32(k_s) + half * kAtTileKeys * 128, &k_map, k_full, half * 64, w.c * kAtTileKeys, w.h, w.b);
       }
       if (!ok) {
         if (it > 0)
@@ -236,19 +236,16 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
-      for (int id = item0; id < item1 && ok; ++id) {
-        const TcItem w = tc_item(off, p.seq.batch, p.num_kv_heads, id);
-        int tile0, tile1;
-        tiles_of(w, tile0, tile1);
-        for (int t = tile0; t < tile1 && ok; ++t, ++it) {
-          const int s = it & 1;
-          ok = mbar_wait(v_empty(s), ((it >> 1) & 1) ^ 1, abort_flag, p.wait_clocks);
-          if (!ok) break;
-          mbar_expect_tx(v_full(s), kAtTileBytes);
-          for (int half = 0; half < 2; ++half)
-            tma_load_4d(smem_u32(v_s) + s * kAtTileBytes + half * kAtTileKeys * 128, &v_map, v_full(s), half * 64,
-                        t * kAtTileKeys, w.h, w.b);
-        }
+      if (p.wait_v) pdl_wait();
+      TcItem w = first_tile();
+      for (; static_cast<int>(it) < ntiles; ++it, next_tile(w)) {
+        const int s = it & 1;
+        ok = mbar_wait(v_empty(s), ((it >> 1) & 1) ^ 1, abort_flag, p.wait_clocks);
+        if (!ok) break;
+        mbar_expect_tx(v_full(s), kAtTileBytes);
+        for (int half = 0; half < 2; ++half)
+          tma_load_4d(smem_u32(v_s) + s * kAtTileBytes + half * kAtTileKeys * 128, &v_map, v_full(s), half * 64,
+                      w.c * kAtTileKeys, w.h, w.b);
       }
       if (!ok) {
         const uint32_t first = it > 2 ? it - 2 : 0;
@@ -300,8 +297,8 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
         fresh = true;
         return true;
       };
-      for (int id = item0; id < item1 && ok; ++id) {
-        const TcItem w = tc_item(off, p.seq.batch, p.num_kv_heads, id);
+      TcItem w = first_tile();
+      for (; static_cast<int>(it) < ntiles && ok; ++it) {
         if (w.b != cur_b || w.h != cur_h) {
           if (cur_b >= 0) ok = end_run();
           if (!ok) break;
@@ -310,14 +307,7 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
           ++heads_seen;
           cur_b = w.b; cur_h = w.h;
         }
-        bool last_of_head = id + 1 >= item1;
-        if (!last_of_head) {
-          const TcItem nx = tc_item(off, p.seq.batch, p.num_kv_heads, id + 1);
-          last_of_head = nx.b != w.b || nx.h != w.h;
-        }
-        int tile0, tile1;
-        tiles_of(w, tile0, tile1);
-        for (int t = tile0; t < tile1 && ok; ++t, ++it) {
+        {
           ok = mbar_wait(k_full, it & 1, abort_flag, p.wait_clocks);
           if (!ok) break;
           ok = mbar_wait(s_empty, (it & 1) ^ 1, abort_flag, p.wait_clocks);   // the tile before is in registers
@@ -338,7 +328,8 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
           if (pend) ok = issue_pv(it - 1);
           pend = true;
         }
-        if (ok && last_of_head) tc_commit(q_empty);
+        next_tile(w);
+        if (ok && (w.b != cur_b || w.h != cur_h || static_cast<int>(it) + 1 == ntiles)) tc_commit(q_empty);
       }
       if (ok && cur_b >= 0) end_run();
     }
@@ -389,9 +380,10 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
       ++lse_rounds;
       return __all_sync(0xffffffffu, good);
     };
-    for (int id = item0; id < item1 && ok; ++id) {
-      const TcItem w = tc_item(off, p.seq.batch, p.num_kv_heads, id);
-      const int n = p.seq.n[w.b], alpha = p.seq.alpha, P = p.seq.prefix[w.b];
+    TcItem w = first_tile();
+    int n = 0, P = 0;
+    const int alpha = p.seq.alpha;
+    for (; static_cast<int>(it) < ntiles && ok; ++it, next_tile(w)) {
       if (w.b != cur_b || w.h != cur_h) {
         if (cur_b >= 0) ok = flush_o();
         if (!ok) break;
@@ -399,19 +391,16 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
         // once everybody has written
         ok = meet();
         if (!ok) break;
-        const int r = e * 32 + lane;
-        if (r < kTcMaxRows) {
-          const float* src = p.lse2 + (static_cast<int64_t>(w.b) * p.num_kv_heads + w.h) * p.rows;
-          lse_all[r] = r < p.rows ? static_cast<float>(kAtShift) - src[r] : -INFINITY;
-        }
+        tc_normalisers<kAtEpiWarps * 32>(p, w.b, w.h, e * 32 + lane, lse_all);
         ok = meet();
         if (!ok) break;
         cur_b = w.b; cur_h = w.h;
+        n = p.seq.n[w.b];
+        P = p.seq.prefix[w.b];
       }
       float* srow = p.scores + (static_cast<int64_t>(w.b) * p.num_kv_heads + w.h) * p.ld_scores;
-      int tile0, tile1;
-      tiles_of(w, tile0, tile1);
-      for (int t = tile0; t < tile1 && ok; ++t, ++it) {
+      {
+        const int t = w.c;
         const int i = t * kAtTileKeys + lane_row;
         const bool in_seq = i < n;
         const int jp = i - P;                                  // window key P + jp is seen by rows j >= jp
@@ -532,10 +521,10 @@ __global__ void __launch_bounds__(kAtD) window_attend_reduce_kernel(const AtPara
   pdl_trigger();
   pdl_wait();
   const int r = blockIdx.x, h = blockIdx.y, b = blockIdx.z, c = threadIdx.x;
-  const int nc = p.seq.score_off[b + 1] - p.seq.score_off[b];
-  const int total = p.num_kv_heads * p.seq.score_off[p.seq.batch];
+  const int nc = p.seq.stat_off[b + 1] - p.seq.stat_off[b];
+  const int total = p.num_kv_heads * p.seq.stat_off[p.seq.batch];
   const int per = total / p.grid, rem = total % p.grid, edge = rem * (per + 1);
-  const int i0 = p.num_kv_heads * p.seq.score_off[b] + h * nc, i1 = i0 + nc - 1;
+  const int i0 = p.num_kv_heads * p.seq.stat_off[b] + h * nc, i1 = i0 + nc - 1;
   const int c0 = i0 < edge ? i0 / (per + 1) : rem + (i0 - edge) / per;
   const int c1 = i1 < edge ? i1 / (per + 1) : rem + (i1 - edge) / per;
   const int hg = b * p.num_kv_heads + h;

@@ -340,8 +340,8 @@ __device__ __forceinline__ float2 run_row(const float2* runs, int r, bool two_bl
 
 // A head's negated row normalisers into dst (-inf for the padding rows), by THREADS threads: the caller's values, or sweep
 // A's partials of this head merged, 1 to 16 lanes per row, pairwise shuffles, always in the same order.
-template <int THREADS>
-__device__ __forceinline__ void tc_normalisers(const TcParams& p, int b, int h, int tid, float* dst) {
+template <int THREADS, typename Params>
+__device__ __forceinline__ void tc_normalisers(const Params& p, int b, int h, int tid, float* dst) {
   const int rows_p2 = p.rows_pad <= 32 ? 32 : (p.rows_pad <= 64 ? 64 : (p.rows_pad <= 128 ? 128 : 256));
   const int per_row = THREADS > rows_p2 ? THREADS / rows_p2 : 1;
   const int hg = b * p.num_kv_heads + h;
