@@ -146,8 +146,7 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t bar0 = smem_u32(bars);
-  auto k_full = [&](int s) { return bar0 + 8u * (s ? 19 : 0); };
-  auto k_empty = [&](int s) { return bar0 + 8u * (s ? 20 : 1); };
+  const uint32_t k_full = bar0, k_empty = bar0 + 8u;
   auto v_full = [&](int s) { return bar0 + 8u * (2 + s); };
   auto v_empty = [&](int s) { return bar0 + 8u * (4 + s); };
   const uint32_t s_full = bar0 + 8u * 6, s_empty = bar0 + 8u * 7;
@@ -161,19 +160,9 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
   const int halves = p.rows_pad > 128 ? 2 : 1;                 // row halves the epilogue takes a tile in
   const int n_half = halves == 2 ? 128 : p.rows_pad;           // window rows (columns) of one half
   const int n_pv = n_half < 64 ? 64 : n_half;                  // ... and of its P x V product (whole 64-row blocks)
-  // Up to 128 rows there is one half.  The tiles then alternate between the two P buffers, and a second K tile stands in the
-  // rows 128 .. 255 of the Q tile (its 64-channel blocks lie as far apart as those of Q): with one of each a tile waited
-  // for the product of the one before and for its own copy.
-  const int k_stages = halves == 1 ? 2 : 1;
-  auto k_at = [&](int s, int half) {
-    return s ? smem_u32(q_s) + half * kTcMaxRows * 128 + 128 * 128 : smem_u32(k_s) + half * kAtTileKeys * 128;
-  };
-  // P buffer of half hf of tile number j, and which use of it that is
-  auto p_buf = [&](int hf, uint32_t j) { return halves == 1 ? static_cast<int>(j & 1u) : hf; };
-  auto p_use = [&](uint32_t j) { return halves == 1 ? j >> 1 : j; };
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < 2; ++s) { mbar_init(k_full(s), 1); mbar_init(k_empty(s), 1); }
+    mbar_init(k_full, 1); mbar_init(k_empty, 1);
     mbar_init(s_full, 1); mbar_init(s_empty, kAtEpiWarps);
     for (int s = 0; s < 2; ++s) {
       mbar_init(v_full(s), 1); mbar_init(v_empty(s), 1);
@@ -228,17 +217,16 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
           ++heads_loaded;
           cur_b = w.b; cur_h = w.h;
         }
-        const int s = it % k_stages;
-        ok = mbar_wait(k_empty(s), ((it / k_stages) & 1) ^ 1, abort_flag, p.wait_clocks);
+        ok = mbar_wait(k_empty, (it & 1) ^ 1, abort_flag, p.wait_clocks);
         if (!ok) break;
         if (p.withhold && blockIdx.x == 0 && static_cast<int>(it) + 1 == ntiles) continue;   // test aid: never arrives
-        mbar_expect_tx(k_full(s), kAtTileBytes);
+        mbar_expect_tx(k_full, kAtTileBytes);
         for (int half = 0; half < 2; ++half)
-          tma_load_4d(k_at(s, half), &k_map, k_full(s), half * 64, w.c * kAtTileKeys, w.h, w.b);
+          tma_load_4d(smem_u32(k_s) + half * kAtTileKeys * 128, &k_map, k_full, half * 64, w.c * kAtTileKeys, w.h, w.b);
       }
       if (!ok) {
-        for (uint32_t j = it > static_cast<uint32_t>(k_stages) ? it - k_stages : 0; j < it; ++j)
-          for (uint32_t spin = 0; spin < (1u << 16) && !mbar_test(k_full(j % k_stages), (j / k_stages) & 1); ++spin) __nanosleep(64);
+        if (it > 0)
+          for (uint32_t spin = 0; spin < (1u << 16) && !mbar_test(k_full, (it - 1) & 1); ++spin) __nanosleep(64);
         if (heads_loaded > 0)
           for (uint32_t spin = 0; spin < (1u << 16) && !mbar_test(q_full, (heads_loaded - 1) & 1); ++spin) __nanosleep(64);
       }
@@ -285,17 +273,16 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
         }
         const uint32_t v_lo = desc_lo_mn_major(smem_u32(v_s) + vs * kAtTileBytes, kAtTileKeys * 128);
         for (int hf = 0; hf < halves; ++hf) {
-          const int pb = p_buf(hf, j);
-          if (!mbar_wait(p_full(pb), p_use(j) & 1, abort_flag, p.wait_clocks)) return false;
+          if (!mbar_wait(p_full(hf), j & 1, abort_flag, p.wait_clocks)) return false;
           tc_fence_after();
           const uint32_t d_addr = tmem_base + 256 + hf * 128;
-          const uint32_t p_lo = desc_lo_mn_major(smem_u32(p_s) + pb * kAtTileBytes, kAtTileKeys * 128);
+          const uint32_t p_lo = desc_lo_mn_major(smem_u32(p_s) + hf * kAtTileBytes, kAtTileKeys * 128);
           if (fresh) tc_mma_halves<false>(d_addr, v_lo, p_lo, idesc_pv);
           else tc_mma_halves<true>(d_addr, v_lo, p_lo, idesc_pv);
 #pragma unroll
           for (int kk = 1; kk < kAtTileKeys / 16; ++kk)        // 16 keys further: 2048 bytes in both operands
             tc_mma_halves<true>(d_addr, v_lo + kk * (2048 >> 4), p_lo + kk * (2048 >> 4), idesc_pv);
-          tc_commit(p_empty(pb));
+          tc_commit(p_empty(hf));
         }
         fresh = false;
         tc_commit(v_empty(vs));
@@ -321,23 +308,21 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
           cur_b = w.b; cur_h = w.h;
         }
         {
-          const int ks = it % k_stages;
-          ok = mbar_wait(k_full(ks), (it / k_stages) & 1, abort_flag, p.wait_clocks);
+          ok = mbar_wait(k_full, it & 1, abort_flag, p.wait_clocks);
           if (!ok) break;
           ok = mbar_wait(s_empty, (it & 1) ^ 1, abort_flag, p.wait_clocks);   // the tile before is in registers
           if (!ok) break;
           tc_fence_after();
-          const uint32_t k_lo = desc_lo_k_major(k_at(ks, 0)), q_lo = desc_lo_k_major(smem_u32(q_s));
-          const uint32_t k_block = (k_at(ks, 1) - k_at(ks, 0)) >> 4;
+          const uint32_t k_lo = desc_lo_k_major(smem_u32(k_s)), q_lo = desc_lo_k_major(smem_u32(q_s));
           tc_mma_halves<false>(tmem_base, k_lo, q_lo, idesc_s);
 #pragma unroll
           for (int kk = 1; kk < kAtD / 16; ++kk) {             // 16 channels further: 32 bytes, the next 64-channel block
-            constexpr int kQBlock = kTcMaxRows * 128 >> 4;     // after four steps
-            tc_mma_halves<true>(tmem_base, k_lo + (kk / 4) * k_block + (kk % 4) * 2, q_lo + (kk / 4) * kQBlock + (kk % 4) * 2,
+            constexpr int kBlock = kAtTileKeys * 128 >> 4, kQBlock = kTcMaxRows * 128 >> 4;        // after four steps
+            tc_mma_halves<true>(tmem_base, k_lo + (kk / 4) * kBlock + (kk % 4) * 2, q_lo + (kk / 4) * kQBlock + (kk % 4) * 2,
                                 idesc_s);
           }
           tc_commit(s_full);
-          tc_commit(k_empty(ks));
+          tc_commit(k_empty);
           // the products of the tile before come behind this tile's logits in the queue: the logits are what the
           // epilogue waits for next
           if (pend) ok = issue_pv(it - 1);
@@ -436,11 +421,10 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
             __syncwarp();
             if (lane == 0) mbar_arrive(s_empty);
           }
-          const int pb = p_buf(hf, it);
-          ok = mbar_wait(p_empty(pb), (p_use(it) & 1) ^ 1, abort_flag, p.wait_clocks);   // V^T P has read what it held before
+          ok = mbar_wait(p_empty(hf), (it & 1) ^ 1, abort_flag, p.wait_clocks);   // V^T P of the tile before has read the buffer
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
-          uint8_t* prow = p_s + pb * kAtTileBytes + lane_row * 128;
+          uint8_t* prow = p_s + hf * kAtTileBytes + lane_row * 128;
           const float* nlr = lse_all + hf * 128;
           if (plain) {
             unsigned long long acc = pack2(0.f, 0.f);
@@ -496,7 +480,7 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
           }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           __syncwarp();
-          if (lane == 0) mbar_arrive(p_full(pb));
+          if (lane == 0) mbar_arrive(p_full(hf));
         }
         if (!ok) break;
         // the key's score: the other groups' partial sums, added in a fixed order
