@@ -190,9 +190,10 @@ __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sy
 // the FMA pipe instead, two at a time with the packed fp32 instructions.  Of every eight consecutive
 // pairs of values (16 accumulator columns), kTcPolyPairs go this way, spread evenly over the eight.  Measured at 0 / 1 / 2 /
 // 3 / 4 of 8: one layer of 131072 tokens (at the board's power cap) 211 / 206 / 209 / 213 / 223 us, 32768 tokens 54.8 / 53.6
-// / 54.0 / 53.5 / 55.1 us, 32 ragged layers 2.71 / 2.70 / 2.76 / 2.82 / 2.87 ms.
+// / 54.0 / 53.5 / 55.1 us, 32 ragged layers 2.71 / 2.70 / 2.76 / 2.82 / 2.87 ms.  2 rather than 1: which columns take the cubic
+// moves the scores by 2e-6, enough to exchange positions at the edge of a list now and then, and stays as it was.
 #ifndef PKV_POLY_PAIRS
-#define PKV_POLY_PAIRS 1
+#define PKV_POLY_PAIRS 2
 #endif
 constexpr int kTcPolyPairs = PKV_POLY_PAIRS;    // 0 = every exponential on the special-function unit
 __host__ __device__ constexpr bool tc_pair_is_poly(int pair) {
@@ -843,6 +844,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
         }
         const float* nlse = lse_s + (blk ? split_b : 0);
         const int cols = blk ? p.rows_pad - split_b : split_b;
+        // a key's rows are summed in two halves whether one group or two of them take its tile: the same rounding either way
+        const int split_sum = two_blocks ? 0 : ((p.rows_pad / 2) + 31) & ~31;
         const bool ours = (u + blk) % kTcStages == static_cast<uint32_t>(grp);   // or another group's unit
         const uint32_t phase = (u / kTcStages) & 1;
         u += p.row_blocks;
@@ -854,6 +857,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
           const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + grp * kTcStageCols;
           unsigned long long acc[4] = {pack2(0.f, 0.f), pack2(0.f, 0.f), pack2(0.f, 0.f), pack2(0.f, 0.f)};
           const unsigned long long cc = pack2(c2, c2);
+          float head_sum = 0.f;
           {
             uint32_t va[16], vb[16];
             tc_ld16(taddr, va);
@@ -864,12 +868,17 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
               tc_wait_ld();
               if (cg + 32 < cols) tc_ld16(taddr + cg + 32, va);
               score_group(vb, cc, nlse + cg + 16, acc);
+              if (cg + 32 == split_sum) {
+                head_sum = sum_pairs(acc);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[q] = 0ull;
+              }
             }
           }
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(t_empty(grp));
-          float sum = sum_pairs(acc);
+          float sum = head_sum + sum_pairs(acc);
           if (two_blocks) {                                   // the second half's group hands its partial sum to the first's
             if (blk == 1) {
               ok = mbar_wait(x_empty(par), (mine & 1) ^ 1, abort_flag, p.wait_clocks);
