@@ -1,0 +1,50 @@
+"""The two-sweep score kernels at the edges of their split: window rows around the copies in the padding rows (32, 64), the
+row blocks (128) and uneven halves, key tiles around 128 keys, and CTAs that go through many heads (one to three CTAs for all
+of them), with the library's own normalisers and with the caller's."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2406_02069_b200 as pkv
+from paper_2406_02069_b200 import binding
+from helpers import assert_scores_close
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+# (query heads per KV head, KV heads, window, head size, dtype, CTAs of a sweep or 0, lengths)
+CASES = [
+    (1, 3, 17, 128, "bf16", 1, [129, 128, 700]), (1, 2, 32, 64, "fp16", 2, [2000]), (3, 2, 11, 128, "bf16", 0, [500, 12]),
+    (4, 2, 16, 64, "fp16", 3, [255, 256, 257, 18]), (5, 5, 13, 128, "bf16", 1, [400, 300]), (2, 8, 48, 128, "fp16", 3, [130, 1000, 600]),
+    (4, 2, 32, 128, "bf16", 0, [3000]), (4, 3, 33, 128, "bf16", 1, [385, 90]), (8, 2, 23, 64, "fp16", 2, [640, 641]),
+    (8, 4, 32, 128, "bf16", 3, [200, 1025, 129]),
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: "g%d_h%d_a%d_d%d_%s_c%d" % c[:6])
+def test_scores_against_the_oracle(case):
+    group, heads, window, d, dtype, ctas, lens = case
+    cfg = pkv.make_config(num_layers=1, num_q_heads=group * heads, num_kv_heads=heads, head_dim=d, window=window, pool_kernel=1,
+                          dtype=dtype, avg_budget=window, sweep_ctas=ctas)
+    t = {"bf16": torch.bfloat16, "fp16": torch.float16}[dtype]
+    g = torch.Generator().manual_seed(31)
+    q = (2.0 * torch.randn(len(lens), group * heads, window, d, generator=g)).to(t)
+    k = torch.randn(len(lens), heads, max(lens), d, generator=g).to(t)
+    qd, kd = q.to(DEV), k.to(DEV)
+    ws = pkv.new_workspace(cfg, len(lens), max(lens), DEV)
+    own, handed = (torch.full((len(lens), heads, max(lens)), -1.0, device=DEV) for _ in range(2))
+    lse = torch.from_numpy(np.stack([oracle.window_lse(q[b], k[b, :, :n]) for b, n in enumerate(lens)]).astype(np.float32))
+    binding.test_hooks(two_sweeps=True)
+    try:
+        pkv.score_window(cfg, qd, kd, lens, own, ws)
+        pkv.score_window(cfg, qd, kd, lens, handed, ws, window_lse=lse.reshape(len(lens), group * heads, window).to(DEV))
+        pkv.check_status(ws)
+    finally:
+        binding.test_hooks()
+    for b, n in enumerate(lens):
+        want, _ = oracle.window_scores(q[b], k[b, :, :n])
+        for got, what in ((own, "own"), (handed, "handed")):
+            # exponentials to 7.5e-5 relative at most, fp32 sums: far inside the 2e-3 of the helper
+            assert_scores_close(got[b, :, : n - window].cpu().numpy(), want, "%s sequence %d" % (what, b))
+            assert torch.all(got[b, :, n - window:] == -1.0)
