@@ -41,13 +41,24 @@ CASES = [
 
 
 @pytest.mark.parametrize("case", CASES, ids=lambda c: "P%d_k%d_w%d_%s_%s" % (c[0], c[1], c[2], "avg" if c[3] else "max", c[4]))
-def test_selection_and_placement_are_exact(case):
+def test_selection_is_exact(case):
+    check_selection(case, 0)
+
+
+# slices of 4097 .. 8192 positions by half-size CTAs, where the configuration caps the sweeps' CTAs
+@pytest.mark.parametrize("case", [c for c in CASES if c[0] in (4096, 4097, 8191, 8192, 8193, 20001, 32736, 40000)],
+                         ids=lambda c: "P%d_k%d_%s" % (c[0], c[1], c[4]))
+def test_selection_beside_other_layers_is_exact(case):
+    check_selection(case, 74)
+
+
+def check_selection(case, sweep_ctas):
     P, k, w, avg, kind, slack = case
     heads, d = 2, 64
     short = max(1, P // 3)                                   # a second, shorter sequence in the same launch
     lens = [P + ALPHA, short + ALPHA]
     cfg = pkv.make_config(num_layers=1, num_q_heads=heads, num_kv_heads=heads, head_dim=d, window=ALPHA, pool_kernel=w, dtype="bf16",
-                          avg_budget=ALPHA, pool_kind=avg)
+                          avg_budget=ALPHA, pool_kind=avg, sweep_ctas=sweep_ctas)
     s = torch.zeros(2, heads, P + slack)
     s[0, :, :P] = scores_of(kind, heads, P, 3)
     s[1, :, :short] = scores_of(kind, heads, short, 4)
