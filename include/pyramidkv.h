@@ -177,6 +177,9 @@ int pyramidkv_kept_count(const pkv_config* cfg, int32_t k_layer, int32_t seq_len
 /*
  * Bytes of device scratch that any call below needs for up to `batch` sequences
  * of at most `max_seq_len` tokens.  Host only.  Returns 0 for an invalid config.
+ * Grows with both, so that one workspace serves every smaller call.  (Inputs that
+ * the fp32-pipe score kernels take get up to 256 MiB in it for logits; those
+ * calls also run in a workspace without that room, and then form them twice.)
  * The workspace must be 256-byte aligned.  Its first 256 bytes hold a status
  * word that kernels only ever set to non-zero; the caller zeroes those bytes once
  * after allocation (the rest needs no initialisation).  Calls that share a

@@ -138,9 +138,10 @@ struct Workspace {
   uint32_t* sel_cnt;         // selection: pairs per cluster rank, [heads][kSelMaxCluster]
   float* logits;             // fp32-pipe path: [heads][rows][ld_logits] logits between its two passes, or null
   int64_t ld_logits;
+  size_t logit_bytes;        // what they take; 0: a path that never stores them
   float* o_partial;          // window attention: per-segment accumulators [kAtMaxGrid + heads][R][d], or null
   size_t score_scratch_bytes;   // bytes of the leading regions that the score kernels alone need
-  size_t bytes;
+  size_t bytes;                 // what a call cannot do without; stored logits come behind it, where there is room
 };
 
 // Which configurations the tensor-core score kernels take (the others go to the fp32-pipe kernels).
@@ -176,14 +177,13 @@ Workspace carve(const pkv_config* c, int batch, int max_n, void* base) {
   w.sel_cand_stride = static_cast<int64_t>(max_n) + 32 * kSelMaxCluster;   // cluster * slice never exceeds this
   w.sel_cand = reinterpret_cast<uint2*>(take(heads * w.sel_cand_stride * sizeof(uint2)));
   w.sel_cnt = reinterpret_cast<uint32_t*>(take(heads * kSelMaxCluster * sizeof(uint32_t)));
-  if (!tc_eligible(c)) {
-    w.ld_logits = static_cast<int64_t>((static_cast<size_t>(max_n) + 127) / 128 * 128);
-    const size_t bytes = heads * rows * static_cast<size_t>(w.ld_logits) * sizeof(float);
-    if (bytes <= kMaxLogitBytes) w.logits = reinterpret_cast<float*>(take(bytes));
-  }
   if (attend_eligible(c))
     w.o_partial = reinterpret_cast<float*>(take((static_cast<size_t>(kAtMaxGrid) + heads) * rows * kAtD * sizeof(float)));
   w.bytes = off;
+  if (!tc_eligible(c)) {
+    w.ld_logits = static_cast<int64_t>((static_cast<size_t>(max_n) + 127) / 128 * 128);
+    w.logit_bytes = align_up(heads * rows * static_cast<size_t>(w.ld_logits) * sizeof(float));
+  }
   return w;
 }
 
@@ -938,7 +938,12 @@ int build_shard_table(const pkv_config* c, const int32_t* shard_keys, const int3
 int workspace_check(const pkv_config* c, int batch, int max_n, void* ws, size_t ws_bytes, Workspace* out) {
   if (!ws || reinterpret_cast<uintptr_t>(ws) % kAlign) return PKV_ERR_WORKSPACE;
   *out = carve(c, batch, max_n, ws);
-  return out->bytes <= ws_bytes ? PKV_OK : PKV_ERR_WORKSPACE;
+  if (out->bytes > ws_bytes) return PKV_ERR_WORKSPACE;
+  // Logits are stored where the workspace has room for them and formed a second time otherwise: a workspace sized for a
+  // longer context or a larger batch, which never stored any, serves a smaller call too.
+  if (out->logit_bytes > 0 && out->logit_bytes <= kMaxLogitBytes && out->logit_bytes <= ws_bytes - out->bytes)
+    out->logits = reinterpret_cast<float*>(static_cast<char*>(ws) + out->bytes);
+  return PKV_OK;
 }
 
 }  // namespace
@@ -989,7 +994,10 @@ int pyramidkv_kept_count(const pkv_config* cfg, int32_t k_layer, int32_t seq_len
 
 size_t pyramidkv_workspace_bytes(const pkv_config* cfg, int32_t batch, int32_t max_seq_len) {
   if (!config_ok(cfg) || batch < 1 || batch > PKV_MAX_BATCH || max_seq_len < cfg->window + 1) return 0;
-  return carve(cfg, batch, max_seq_len, nullptr).bytes;
+  // Grows with the batch and the length: a call that is too large to store its logits still reserves the room that the
+  // smaller ones made on the same workspace use.
+  const Workspace w = carve(cfg, batch, max_seq_len, nullptr);
+  return w.bytes + std::min(w.logit_bytes, kMaxLogitBytes);
 }
 
 static int score_window_impl(const pkv_config* cfg, pkv_tensor q_win, pkv_tensor k, const float* window_lse,
@@ -1721,8 +1729,7 @@ extern "C" int pyramidkv_score_window_static(const pkv_config* cfg, pkv_tensor q
   if (need > PKV_STATIC_SCRATCH_BYTES) return PKV_ERR_STATIC_SCRATCH;
   void* base = static_scratch_address();
   if (!base) return PKV_ERR_CUDA;
-  Workspace w = carve(cfg, batch, max_n, base);
-  w.logits = nullptr;                              // no room for logits here: they are formed again instead
+  const Workspace w = carve(cfg, batch, max_n, base);   // no room for logits here: they are formed again instead
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // The array keeps whatever the previous call left.  Only the status word has to start from zero;
   // statistics and normalisers are fully rewritten before they are read.

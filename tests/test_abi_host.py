@@ -154,6 +154,57 @@ def test_workspace_grows_with_the_problem():
     assert pkv.workspace_bytes(cfg, 65, 4096) == 0
 
 
+# (dtype, query heads, KV heads, window, head size): the fp32-pipe kernels keep logits in the workspace up to a limit
+LOGIT_CONFIGS = [("fp32", 32, 8, 32, 128), ("fp32", 4, 2, 8, 64), ("bf16", 64, 8, 64, 128), ("fp16", 40, 8, 64, 64)]
+
+
+@pytest.mark.parametrize("dtype,hq,hkv,window,d", LOGIT_CONFIGS)
+def test_a_larger_problem_never_needs_a_smaller_workspace(dtype, hq, hkv, window, d):
+    cfg = pkv.make_config(num_layers=1, num_q_heads=hq, num_kv_heads=hkv, head_dim=d, window=window, pool_kernel=7, dtype=dtype,
+                          avg_budget=128)
+    lengths = sorted({n + e for n in [2 ** i for i in range(8, 21)] for e in (-1, 0, 1)})
+    for batch in range(1, 65):
+        sizes = [pkv.workspace_bytes(cfg, batch, n) for n in lengths]
+        assert sizes == sorted(sizes) and sizes[0] > 0, batch
+    for n in lengths:
+        sizes = [pkv.workspace_bytes(cfg, batch, n) for batch in range(1, 65)]
+        assert sizes == sorted(sizes), n
+
+
+_ACCEPTED = r'''
+import ctypes, sys
+import paper_2406_02069_b200 as pkv
+from paper_2406_02069_b200 import binding
+
+lib, fake, base = binding._lib, binding.PkvTensor(4096, 1 << 40, 1 << 30, 128), 4096
+for dtype, hq, hkv, window, d in eval(sys.argv[1]):
+    cfg = pkv.make_config(num_layers=1, num_q_heads=hq, num_kv_heads=hkv, head_dim=d, window=window, pool_kernel=7, dtype=dtype, avg_budget=128)
+    ref = ctypes.byref(cfg)
+    for big_batch, big_n in ((1, 131072), (8, 65536), (64, 16384), (1, 4096)):
+        size = pkv.workspace_bytes(cfg, big_batch, big_n)
+        for batch, n in ((1, 200), (1, 8192), (1, 16384), (4, 16384), (8, 4096), (big_batch, big_n)):
+            if batch > big_batch or n > big_n:
+                continue
+            lens = (ctypes.c_int32 * batch)(*[n] * batch)
+            calls = {
+                "score": lib.pyramidkv_score_window(ref, fake, fake, lens, batch, base, n, base, size, None),
+                "select": lib.pyramidkv_select_topk(ref, base, n, lens, batch, 4, base, base, size, None),
+                "shard": lib.pyramidkv_shard_window_lse(ref, fake, fake, (ctypes.c_int32 * batch)(*[n - window] * batch),
+                                                        (ctypes.c_int32 * batch)(*[0] * batch), batch, base, base, size, None)}
+            for name, st in calls.items():               # no device here: whatever passes the checks ends in a CUDA error
+                assert st == binding.PKV_ERR_CUDA, (name, dtype, big_batch, big_n, batch, n, st)
+print("accepted")
+'''
+
+
+def test_a_workspace_for_a_larger_problem_serves_the_smaller_ones():
+    """In a child process that sees no GPU (the pointers are invented): every call gets past the workspace check."""
+    env = dict(os.environ, CUDA_VISIBLE_DEVICES="")
+    out = subprocess.run([sys.executable, "-c", _ACCEPTED, repr(LOGIT_CONFIGS)], cwd=ROOT, env=env, capture_output=True, text=True,
+                         timeout=600)
+    assert out.returncode == 0 and "accepted" in out.stdout, out.stdout[-2000:] + out.stderr[-4000:]
+
+
 def test_workload_generator_is_seeded_and_shaped():
     w = workloads.scaled(workloads.MISTRAL_RAGGED, num_layers=2, batch=3)
     lens = w.seq_lens()

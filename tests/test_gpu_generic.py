@@ -48,3 +48,25 @@ def test_scores_against_the_oracle(case):
             # 2e-3 relative bound covers it with the exponentials
             assert_scores_close(got[b, :, :P].cpu().numpy(), want, "%s sequence %d" % (what, b))
             assert torch.all(got[b, :, P:] == -1.0)          # nothing is written behind the prefix
+
+
+def test_a_workspace_of_a_longer_context_serves_a_short_call():
+    """Sized for a context whose logits are not kept, and cut down to what that call itself needs: with room for the short
+    call's logits and without."""
+    heads, group, window, d, n = 2, 4, 32, 128, 700
+    cfg = pkv.make_config(num_layers=1, num_q_heads=group * heads, num_kv_heads=heads, head_dim=d, window=window, pool_kernel=1,
+                          dtype="fp32", avg_budget=window)
+    g = torch.Generator().manual_seed(22)
+    q = 1.5 * torch.randn(1, group * heads, window, d, generator=g)
+    k = torch.randn(1, heads, n, d, generator=g)
+    want, _ = oracle.window_scores(q[0], k[0])
+    ws = pkv.new_workspace(cfg, 1, 400000, DEV)
+    assert ws.numel() > 256 << 20
+    own = pkv.workspace_bytes(cfg, 1, n)
+    for size in (ws.numel(), own, own - heads * group * window * 768 * 4):   # 768: n rounded up to whole tiles
+        got = torch.full((1, heads, n), -1.0, device=DEV)
+        pkv.score_window(cfg, q.to(DEV), k.to(DEV), [n], got, ws[:size])
+        pkv.check_status(ws)
+        assert_scores_close(got[0, :, : n - window].cpu().numpy(), want, "workspace of %d bytes" % size)
+    with pytest.raises(pkv.PkvError):
+        pkv.score_window(cfg, q.to(DEV), k.to(DEV), [n], got, ws[: own - heads * group * window * 768 * 4 - 256])
