@@ -28,6 +28,8 @@
 
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "pkv_common.cuh"
 
 namespace pkv {
@@ -339,12 +341,81 @@ __device__ __forceinline__ float2 run_row(const float2* runs, int r, bool two_bl
   return make_float2(m, z);
 }
 
-// A head's negated row normalisers into dst (-inf for the padding rows), by THREADS threads: the caller's values, or sweep
-// A's partials of this head merged, 1 to 16 lanes per row, pairwise shuffles, always in the same order.
+// Segments t, t + per_row, ... < s1 of sweep A's partials, of U rows from r on, r_step apart, in batches of Q loads:
+// (reference, sum) added to m, z.  How many are loaded at a time does not change a bit of the result as long as one batch
+// holds them all, or Q is the same.  The loads are unconditional (of the last row and segment where there is none), so
+// that all of a batch are in flight.
+template <int U, int Q>
+__device__ __forceinline__ void tc_fold_segments(const float2* partial, int r, int r_step, int rows, int t, int s1, int per_row,
+                                                 float* m, float* z) {
+  for (; t < s1; t += Q * per_row) {
+    float2 pz[U][Q];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int q = 0; q < Q; ++q)
+        pz[u][q] = __ldcg(partial + static_cast<int64_t>(min(t + q * per_row, s1 - 1)) * rows + min(r + u * r_step, rows - 1));
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      float mn = m[u];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        if (q > 0 && t + q * per_row >= s1) pz[u][q] = make_float2(-INFINITY, 0.f);
+        mn = fmaxf(mn, pz[u][q].x);
+      }
+      if (mn > -INFINITY) {                                    // (-inf, 0) marks a segment that saw no key of this row
+        z[u] = __fmul_rn(z[u], ex2(m[u] - mn));
+#pragma unroll
+        for (int q = 0; q < Q; ++q) z[u] = fmaf(pz[u][q].y, ex2(pz[u][q].x - mn), z[u]);
+        m[u] = mn;
+      }
+    }
+  }
+}
+
+// Two lanes' (reference, sum) of one row; the first operand is the one of the lower lane.
+__device__ __forceinline__ float2 tc_merge_pair(float2 a, float2 b) {
+  const float mm = fmaxf(a.x, b.x);
+  return make_float2(mm, __fadd_rn(a.x > -INFINITY ? __fmul_rn(a.y, ex2(a.x - mm)) : 0.f,
+                                   b.x > -INFINITY ? __fmul_rn(b.y, ex2(b.x - mm)) : 0.f));
+}
+
+// What PER_ROW lanes with at most Q segments each make of a row, by one lane.
+template <int PER_ROW, int Q>
+__device__ __forceinline__ float2 tc_merge_row(const float2* row, int rows, int s0, int s1) {
+  float2 pz[Q][PER_ROW];
+#pragma unroll
+  for (int q = 0; q < Q; ++q)
+#pragma unroll
+    for (int i = 0; i < PER_ROW; ++i) pz[q][i] = __ldcg(row + static_cast<int64_t>(min(s0 + q * PER_ROW + i, s1 - 1)) * rows);
+  float2 lane[PER_ROW];
+#pragma unroll
+  for (int i = 0; i < PER_ROW; ++i) {
+    lane[i] = s0 + i < s1 ? pz[0][i] : make_float2(-INFINITY, 0.f);
+    if (Q == 2 && s0 + PER_ROW + i < s1) {
+      const float mn = fmaxf(lane[i].x, pz[Q - 1][i].x);
+      if (mn > -INFINITY)
+        lane[i] = make_float2(mn, fmaf(pz[Q - 1][i].y, ex2(pz[Q - 1][i].x - mn), __fmul_rn(lane[i].y, ex2(lane[i].x - mn))));
+    }
+  }
+#pragma unroll
+  for (int o = 1; o < PER_ROW; o <<= 1)
+#pragma unroll
+    for (int i = 0; i < PER_ROW; i += 2 * o) lane[i] = tc_merge_pair(lane[i], lane[i + o]);
+  return lane[0];
+}
+
+// A head's negated row normalisers into dst (-inf for the padding rows), by THREADS threads (the sixteen epilogue warps or one
+// warp): the caller's values, or sweep A's partials of this head merged.  Every CTA that works on a head merges it for
+// itself, and equal keys must get equal scores whichever CTA has them, so the additions come in the same order whoever does
+// it: 2 to 16 lanes per row by the number of rows alone, each with every per_row-th segment, then pairwise.  A single warp
+// does the same with a lane per row where the head has few segments (what it has to save there are instructions, beside
+// four warps of the epilogue on its scheduler), else in sixteen steps, four at a time if it can (L2 latencies).
 template <int THREADS, typename Params>
 __device__ __forceinline__ void tc_normalisers(const Params& p, int b, int h, int tid, float* dst) {
+  constexpr int kSteps = kTcEpiWarps * 32 / THREADS;           // of THREADS / per_row rows
   const int rows_p2 = p.rows_pad <= 32 ? 32 : (p.rows_pad <= 64 ? 64 : (p.rows_pad <= 128 ? 128 : 256));
-  const int per_row = THREADS > rows_p2 ? THREADS / rows_p2 : 1;
+  const int per_row = kTcEpiWarps * 32 / rows_p2, r_step = THREADS / per_row;
   const int hg = b * p.num_kv_heads + h;
   int s0 = 0, s1 = 0;
   if (p.merge) {
@@ -361,39 +432,58 @@ __device__ __forceinline__ void tc_normalisers(const Params& p, int b, int h, in
   }
   const int part = tid % per_row;
   pdl_wait();                                                  // normalisers and partials are written by kernels before
-  for (int r = tid / per_row; r < rows_p2; r += THREADS / per_row) {
-    float val = -INFINITY;
+  // U steps from `step` on, segments in batches of Q
+  auto some = [&](int step, auto u_const, auto q_const) {
+    constexpr int U = decltype(u_const)::value, Q = decltype(q_const)::value;
+    const int r0 = step * r_step + tid / per_row;
+    float m[U], z[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) { m[u] = -INFINITY; z[u] = 0.f; }
     if (p.merge) {
-      float m = -INFINITY, z = 0.f;
-      if (r < p.rows) {
-        const float2* base = p.partial + r;
-        for (int t = s0 + part; t < s1; t += 10 * per_row) {   // a batch of loads in flight
-          float2 pz[10];
-          float mn = m;
+      tc_fold_segments<U, Q>(p.partial, r0, r_step, p.rows, s0 + part, s1, per_row, m, z);
+      for (int o = 1; o < per_row; o <<= 1) {
 #pragma unroll
-          for (int q = 0; q < 10; ++q)
-            pz[q] = t + q * per_row < s1 ? __ldcg(base + static_cast<int64_t>(t + q * per_row) * p.rows) : make_float2(-INFINITY, 0.f);
-#pragma unroll
-          for (int q = 0; q < 10; ++q) mn = fmaxf(mn, pz[q].x);
-          if (mn > -INFINITY) {                                // (-inf, 0) marks a segment that saw no key of this row
-            z *= ex2(m - mn);
-#pragma unroll
-            for (int q = 0; q < 10; ++q) z = fmaf(pz[q].y, ex2(pz[q].x - mn), z);
-            m = mn;
-          }
+        for (int u = 0; u < U; ++u) {                          // both partners of a pair compute the same merged value
+          const float2 both = tc_merge_pair(make_float2(m[u], z[u]), make_float2(__shfl_xor_sync(0xffffffffu, m[u], o),
+                                                                                 __shfl_xor_sync(0xffffffffu, z[u], o)));
+          m[u] = both.x;
+          z[u] = both.y;
         }
       }
-      for (int o = 1; o < per_row; o <<= 1) {                  // both partners of a pair compute the same merged value
-        const float2 other = make_float2(__shfl_xor_sync(0xffffffffu, m, o), __shfl_xor_sync(0xffffffffu, z, o));
-        const float mm = fmaxf(m, other.x);
-        z = (m > -INFINITY ? z * ex2(m - mm) : 0.f) + (other.x > -INFINITY ? other.y * ex2(other.x - mm) : 0.f);
-        m = mm;
-      }
-      if (r < p.rows) val = -(m + __log2f(z) + p.log2_group);
-    } else if (r < p.rows) {
-      val = -fmaf(p.lse2[static_cast<int64_t>(hg) * p.rows + r], p.lse_scale, p.lse_add);
     }
-    if (part == 0) dst[r] = val;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int r = r0 + u * r_step;
+      float val = -INFINITY;
+      if (r < p.rows)
+        val = p.merge ? -(m[u] + __log2f(z[u]) + p.log2_group)
+                      : -fmaf(p.lse2[static_cast<int64_t>(hg) * p.rows + r], p.lse_scale, p.lse_add);
+      if (part == 0) dst[r] = val;
+    }
+  };
+  using std::integral_constant;
+  if constexpr (kSteps == 1) {
+    some(0, integral_constant<int, 1>{}, integral_constant<int, 10>{});
+  } else {
+    auto lane_a_row = [&](auto lanes, auto q_const) {
+#pragma unroll 1
+      for (int r = tid; r < rows_p2; r += THREADS) {
+        const float2 mz = tc_merge_row<decltype(lanes)::value, decltype(q_const)::value>(p.partial + min(r, p.rows - 1), p.rows, s0, s1);
+        dst[r] = r < p.rows ? -(mz.x + __log2f(mz.y) + p.log2_group) : -INFINITY;
+      }
+    };
+    if (p.merge && s1 - s0 <= min(2 * per_row, 16)) {
+      if (per_row == 2) lane_a_row(integral_constant<int, 2>{}, integral_constant<int, 2>{});
+      else if (per_row == 4) lane_a_row(integral_constant<int, 4>{}, integral_constant<int, 2>{});
+      else if (per_row == 8) lane_a_row(integral_constant<int, 8>{}, integral_constant<int, 2>{});
+      else lane_a_row(integral_constant<int, 16>{}, integral_constant<int, 1>{});
+    } else if (s1 - s0 <= 5 * per_row) {
+#pragma unroll 1
+      for (int step = 0; step < kSteps; step += 4) some(step, integral_constant<int, 4>{}, integral_constant<int, 5>{});
+    } else {
+#pragma unroll 1
+      for (int step = 0; step < kSteps; ++step) some(step, integral_constant<int, 1>{}, integral_constant<int, 10>{});
+    }
   }
 }
 
@@ -822,7 +912,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
         // thread -> key.  The head's normalisers, negated (the epilogue adds them), sit in one of two buffers that alternate
         // from head to head.  The first one is filled by the sixteen warps together, which then meet; the others by warp 3,
         // ahead of time.  They come from the caller (or the merge kernel), or straight from sweep A's partials of the head,
-        // which every CTA that works on it merges for itself, always in the same order.
+        // which every CTA that works on it merges for itself, always in the same order (see tc_normalisers).
         if (new_head) {
           const uint32_t buf = heads & 1u;
           if (heads == 0) {

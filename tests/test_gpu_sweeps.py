@@ -48,3 +48,30 @@ def test_scores_against_the_oracle(case):
             # exponentials to 7.5e-5 relative at most, fp32 sums: far inside the 2e-3 of the helper
             assert_scores_close(got[b, :, : n - window].cpu().numpy(), want, "%s sequence %d" % (what, b))
             assert torch.all(got[b, :, n - window:] == -1.0)
+
+
+# (query heads per KV head, window, head size, dtype): 32, 64, 128 and 256 window rows
+@pytest.mark.parametrize("ctas", [7, 20, 41, 0])
+@pytest.mark.parametrize("group,window,d,dtype", [(4, 8, 128, "bf16"), (8, 8, 64, "fp16"), (4, 32, 128, "bf16"), (8, 32, 128, "fp16")])
+def test_equal_keys_get_equal_scores_whichever_cta_has_them(group, window, d, dtype, ctas):
+    """The same key in every tile of heads that many CTAs share, some of them as their second or third head: a head's row
+    normalisers are the same bits in every CTA, so its equal keys tie exactly."""
+    heads, lens = 5, [5000, 2100]
+    cfg = pkv.make_config(num_layers=1, num_q_heads=group * heads, num_kv_heads=heads, head_dim=d, window=window, pool_kernel=1,
+                          dtype=dtype, avg_budget=window, sweep_ctas=ctas)
+    t = {"bf16": torch.bfloat16, "fp16": torch.float16}[dtype]
+    g = torch.Generator().manual_seed(7)
+    q = (2.0 * torch.randn(len(lens), group * heads, window, d, generator=g)).to(t)
+    k = torch.randn(len(lens), heads, max(lens), d, generator=g).to(t)
+    k[:, :, 5::128] = k[:, :, 5:6]
+    ws = pkv.new_workspace(cfg, len(lens), max(lens), DEV)
+    scores = torch.zeros(len(lens), heads, max(lens), device=DEV)
+    binding.test_hooks(two_sweeps=True)
+    try:
+        pkv.score_window(cfg, q.to(DEV), k.to(DEV), lens, scores, ws)
+        pkv.check_status(ws)
+    finally:
+        binding.test_hooks()
+    for b, n in enumerate(lens):
+        same = scores[b, :, 5: n - window: 128]
+        assert torch.equal(same, same[:, :1].expand_as(same)), [int((row != row[0]).sum()) for row in same]
