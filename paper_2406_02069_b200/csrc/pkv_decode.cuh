@@ -329,6 +329,42 @@ struct Dec16<__half> {
   }
 };
 
+// One head's sums over a warp's rows on the fp32 pipe, D / 32 channels per lane: for rows that hold infinities or NaN.  In the
+// matrix product every part of a weight meets every value, and a part that is zero or negative makes NaN of an infinity;
+// one weight, one product gives what the sum says (an infinity of the value's sign, NaN where both signs or NaN are
+// summed).  ref: the exponent that the warp's weights are relative to.
+template <typename T, int D, bool PAGED>
+__device__ __forceinline__ void dec_sum_special(const DecodeParams& p, int b, int h, const T* q, int64_t row0, int first, int hi,
+                                                float ref, float* acc) {
+  constexpr int PER = D / 32;
+  const int lane = threadIdx.x & 31;
+  float qv[PER], a[PER];
+#pragma unroll
+  for (int c = 0; c < PER; ++c) {
+    qv[c] = to_float(q[lane * PER + c]);
+    a[c] = 0.f;
+  }
+#pragma unroll 1
+  for (int t0 = first; t0 < hi; t0 += kDecWarps * 16)
+#pragma unroll 1
+    for (int r = t0; r < min(t0 + 16, hi); ++r) {
+      const int64_t at = PAGED ? paged_row(p.pt, b, h, r) : row0 + r;
+      if (at < 0) continue;
+      const T* k = static_cast<const T*>(p.k_cache) + at * D + lane * PER;
+      const T* v = static_cast<const T*>(p.v_cache) + at * D + lane * PER;
+      float dot = 0.f;
+#pragma unroll
+      for (int c = 0; c < PER; ++c) dot = fmaf(qv[c], to_float(k[c]), dot);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+      const float w = exp2f(dot * p.scale_log2 - ref);
+#pragma unroll
+      for (int c = 0; c < PER; ++c) a[c] = fmaf(w, to_float(v[c]), a[c]);
+    }
+#pragma unroll
+  for (int c = 0; c < PER; ++c) acc[lane * PER + c] = a[c];
+}
+
 // grid, cluster and block as above, kDecMmaHeads query heads per CTA.  A warp takes tiles of 16 rows.  With g = lane / 4 and
 // c = lane % 4 the fragments of m16n8k16 are
 //   S  = Q K^T   A: row i = head i % 4 (every head four times), B: n = row g of 8, channels dealt so that a lane's B words are
@@ -471,13 +507,24 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_mma_kernel(const Decode
   // ---- the parts, then the warps, then the CTAs of the cluster
   z += __shfl_xor_sync(0xffffffffu, z, 1);
   z += __shfl_xor_sync(0xffffffffu, z, 2);
+  float special[4] = {0.f, 0.f, 0.f, 0.f};       // NaN once a sum is not finite
 #pragma unroll
   for (int i = 0; i < VC * 8; ++i) {             // channels 64 j + 8 (2c + e) + i % 8 of head g % 4
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       float s = o[i][e] + o[i][2 + e];
       s += __shfl_xor_sync(0xffffffffu, s, 16);
+      special[i & 3] = fmaf(s, 0.f, special[i & 3]);
       if (g < 4) s_mrg.acc[warp][g * D + (i >> 3) * 64 + (2 * c + e) * 8 + (i & 7)] = s;
+    }
+  }
+  if (__any_sync(0xffffffffu, (special[0] + special[1]) + (special[2] + special[3]) != 0.f)) {
+    __syncwarp();
+#pragma unroll 1
+    for (int j = 0; j < min(GT, p.group - g0); ++j) {
+      const float mj = __shfl_sync(0xffffffffu, m, j * 4);
+      dec_sum_special<T, D, PAGED>(p, b, h, static_cast<const T*>(p.q) + (hq0 + j) * D, row0, lo + warp * 16, hi,
+                                   mj == -INFINITY ? 0.f : mj - X::kShift, &s_mrg.acc[warp][j * D]);
     }
   }
   if (g < 4 && c == 0) {

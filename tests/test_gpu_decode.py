@@ -67,3 +67,39 @@ def test_decode_against_the_oracle(case):
             # than 1e-5: 7e-5 of the output over |V|
             bound = oracle.decode_attention(q[b, hq], k[sl], v[sl].abs())
             assert np.all(np.abs(got[b, hq] - want) <= 7e-5 * bound + 1e-7), (b, hq)
+
+
+@pytest.mark.parametrize("what", ["inf", "-inf", "both signs", "nan", "small weight", "last row"])
+@pytest.mark.parametrize("dtype,d,group", [("fp32", 128, 4), ("bf16", 128, 4), ("fp16", 128, 5), ("bf16", 64, 1), ("fp16", 64, 2)])
+def test_infinities_and_nan_in_the_values_stay_in_their_channel(dtype, d, group, what):
+    heads, window, kl, lens = 2, 4, 296, [700, 90]
+    cfg = pkv.make_config(num_layers=1, num_q_heads=group * heads, num_kv_heads=heads, head_dim=d, window=window, pool_kernel=1,
+                          dtype=dtype, avg_budget=window)
+    t = {"fp32": torch.float32, "bf16": torch.bfloat16, "fp16": torch.float16}[dtype]
+    g = torch.Generator().manual_seed(17)
+    rows = pkv.total_rows(cfg, kl, lens)
+    k, v = (torch.randn(rows, d, generator=g).to(t) for _ in range(2))
+    q = (1.5 * torch.randn(len(lens), group * heads, d, generator=g)).to(t)
+    inf = float("inf")
+    if what == "both signs":
+        v[10, 3], v[200, 3], v[10, 40] = inf, -inf, -inf
+    elif what == "small weight":                             # another row's logit some 40 binades above
+        v[10, 3] = inf
+        k[20] = (q[0, 0].float() * (40.0 / 1.4427 * d ** 0.5 / q[0, 0].float().square().sum())).to(t)
+    elif what == "last row":
+        v[rows - 1, d - 1], v[299, 0] = -inf, inf
+    else:
+        v[10, 3] = float(what)
+    out = torch.zeros(len(lens), group * heads, d, device=DEV)
+    pkv.decode_attention(cfg, q.to(DEV), k.to(DEV), v.to(DEV), lens, kl, out)
+    counts, got = [pkv.kept_count(cfg, kl, n) for n in lens], out.cpu().double()
+    for b, h, sl in packed_rows(counts, heads):
+        for j in range(group):
+            hq = h * group + j
+            w = torch.softmax(k[sl].double() @ q[b, hq].double() / d ** 0.5, 0)[:, None]
+            want = (w * v[sl].double()).sum(0)
+            assert torch.equal(torch.isnan(got[b, hq]), torch.isnan(want)), (b, hq)
+            special = ~torch.isfinite(want)
+            assert torch.equal(got[b, hq][special & ~torch.isnan(want)], want[special & ~torch.isnan(want)]), (b, hq)
+            bound = (w * v[sl].double().abs()).sum(0)        # as in the test above
+            assert torch.all((got[b, hq] - want).abs()[~special] <= 7e-5 * bound[~special] + 1e-7), (b, hq)
