@@ -432,6 +432,11 @@ __device__ __forceinline__ void tc_normalisers(const Params& p, int b, int h, in
   }
   const int part = tid % per_row;
   pdl_wait();                                                  // normalisers and partials are written by kernels before
+  if (!p.merge) {
+    for (int r = tid; r < rows_p2; r += THREADS)
+      dst[r] = r < p.rows ? -fmaf(p.lse2[static_cast<int64_t>(hg) * p.rows + r], p.lse_scale, p.lse_add) : -INFINITY;
+    return;
+  }
   // U steps from `step` on, segments in batches of Q
   auto some = [&](int step, auto u_const, auto q_const) {
     constexpr int U = decltype(u_const)::value, Q = decltype(q_const)::value;
@@ -439,26 +444,20 @@ __device__ __forceinline__ void tc_normalisers(const Params& p, int b, int h, in
     float m[U], z[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) { m[u] = -INFINITY; z[u] = 0.f; }
-    if (p.merge) {
-      tc_fold_segments<U, Q>(p.partial, r0, r_step, p.rows, s0 + part, s1, per_row, m, z);
-      for (int o = 1; o < per_row; o <<= 1) {
+    tc_fold_segments<U, Q>(p.partial, r0, r_step, p.rows, s0 + part, s1, per_row, m, z);
+    for (int o = 1; o < per_row; o <<= 1) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {                          // both partners of a pair compute the same merged value
-          const float2 both = tc_merge_pair(make_float2(m[u], z[u]), make_float2(__shfl_xor_sync(0xffffffffu, m[u], o),
-                                                                                 __shfl_xor_sync(0xffffffffu, z[u], o)));
-          m[u] = both.x;
-          z[u] = both.y;
-        }
+      for (int u = 0; u < U; ++u) {                            // both partners of a pair compute the same merged value
+        const float2 both = tc_merge_pair(make_float2(m[u], z[u]), make_float2(__shfl_xor_sync(0xffffffffu, m[u], o),
+                                                                               __shfl_xor_sync(0xffffffffu, z[u], o)));
+        m[u] = both.x;
+        z[u] = both.y;
       }
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int r = r0 + u * r_step;
-      float val = -INFINITY;
-      if (r < p.rows)
-        val = p.merge ? -(m[u] + __log2f(z[u]) + p.log2_group)
-                      : -fmaf(p.lse2[static_cast<int64_t>(hg) * p.rows + r], p.lse_scale, p.lse_add);
-      if (part == 0) dst[r] = val;
+      if (part == 0) dst[r] = r < p.rows ? -(m[u] + __log2f(z[u]) + p.log2_group) : -INFINITY;
     }
   };
   using std::integral_constant;
@@ -472,7 +471,7 @@ __device__ __forceinline__ void tc_normalisers(const Params& p, int b, int h, in
         dst[r] = r < p.rows ? -(mz.x + __log2f(mz.y) + p.log2_group) : -INFINITY;
       }
     };
-    if (p.merge && s1 - s0 <= min(2 * per_row, 16)) {
+    if (s1 - s0 <= min(2 * per_row, 16)) {
       if (per_row == 2) lane_a_row(integral_constant<int, 2>{}, integral_constant<int, 2>{});
       else if (per_row == 4) lane_a_row(integral_constant<int, 4>{}, integral_constant<int, 2>{});
       else if (per_row == 8) lane_a_row(integral_constant<int, 8>{}, integral_constant<int, 2>{});
