@@ -478,6 +478,7 @@ constexpr int kSelRun = 8;                 // consecutive positions of a thread
 constexpr int kSelClusterSlice = 8192;     // a cluster doubles (up to 8 CTAs) while its slices are longer than this
 constexpr int kSelCopyBytes = 128 << 10;   // ... or while a CTA would copy more than this and SMs are idle
 constexpr int kSelCommonCandidates = 4096; // more expected candidates (k per CTA) than this: one bound for the cluster
+constexpr int kSelCrowd = 1024;            // candidates of a CTA beyond 2 k that its bound may let through before it is refined
 constexpr int kSelEvenRows = 1024;         // lists of at least this many rows are copied by the whole cluster evenly
 
 // Position i of the staged scores in shared memory: four floats of padding after every 32.
@@ -568,6 +569,97 @@ __device__ __forceinline__ void sel_pool_run(const float* raw, int at, int radiu
     if (AVG) best = __fdiv_rn(best, static_cast<float>(2 * radius + 1));
     key[j] = ordered_key(best);
   }
+}
+
+// Candidates beyond all use: the scale of sel_bin has 32 bins an octave between 2^-26 and 2^6, so a flat row (its keys share a
+// few bins) or scores on another scale (which share the first or last one) can have every position above the bound.  Every
+// candidate is sent to and ranked by all CTAs of the cluster, some 2 us per 1000 of them.  Here the range from the smallest
+// to the largest candidate is divided, ten bits at a time, until the bound lets through little more than k, and the list
+// is closed up.  131040 positions, k = 96: flat rows 93 -> 20 us, scores near 1e-12 147 -> 22 us
+// (rows spread over the scale: 12).
+// Called by the whole block (common: by the whole cluster) behind a barrier; ends with one.  Out of line: the registers of
+// the ordinary way are not to be shared with it.  minima: scratch, a word per warp; maxima: the warps' largest keys.
+// Returns the number of candidates left and the new bound.
+template <int THREADS, int RUNS>
+__device__ __noinline__ uint2 sel_refine(uint32_t* list_key, uint16_t* list_pos, int M, uint32_t k, uint32_t* hist, uint32_t* rows,
+                                         uint32_t* minima, uint32_t* maxima, bool common) {
+  constexpr int WARPS = THREADS / 32, E = RUNS * kSelRun;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = cluster.dim_blocks().x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t full = 0xffffffffu, lt = (1u << lane) - 1u;
+  // a warp takes consecutive entries, 32 * per of them; entry j * 32 + lane of these is this lane's j-th
+  const int per = (M + THREADS - 1) / THREADS, first = warp * per * 32 + lane;
+  auto mine = [&](int j) { return j < per && first + j * 32 < M; };
+  uint32_t key[E], least = 0xffffffffu;
+#pragma unroll
+  for (int j = 0; j < E; ++j) {
+    key[j] = mine(j) ? list_key[first + j * 32] : 0u;
+    if (mine(j)) least = min(least, key[j]);
+  }
+  least = __reduce_min_sync(full, least);
+  if (lane == 0) minima[warp] = least;
+  if (common) cluster.sync(); else __syncthreads();         // (and everybody has read the counts before)
+  uint32_t bound = 0xffffffffu, top = 0;                    // the smallest and the largest candidate
+  for (int c = 0; c < (common ? C : 1); ++c)
+    if (lane < WARPS) {
+      bound = min(bound, common ? cluster.map_shared_rank(minima, c)[lane] : minima[lane]);
+      top = max(top, common ? cluster.map_shared_rank(maxima, c)[lane] : maxima[lane]);
+    }
+  bound = __reduce_min_sync(full, bound);
+  top = __reduce_max_sync(full, top);
+  uint32_t span = 0xffffffffu, want = k;
+  int shift = max(0, 22 - __clz(top - bound));
+  uint32_t* counts = hist + (common ? kSelBinsLin : 0);
+  for (;;) {
+    for (int i = tid; i < 2 * kSelBinsLin; i += THREADS) hist[i] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < E; ++j)
+      if (mine(j) && key[j] >= bound && key[j] - bound <= span) atomicAdd(&hist[(key[j] - bound) >> shift], 1u);
+    if (common) {
+      cluster.sync();
+      for (int i = tid; i < kSelBinsLin; i += THREADS) {
+        uint32_t sum = 0;
+        for (int c = 0; c < C; ++c) sum += cluster.map_shared_rank(hist, c)[i];
+        counts[i] = sum;
+      }
+    }
+    __syncthreads();
+    uint32_t digit = 0, above = 0;
+    sel_find_from_top<THREADS>(counts, rows, want, digit, above);
+    bound += digit << shift;
+    want -= above;
+    if (shift == 0 || k - want + counts[digit] <= k + k / 4 + 128) break;
+    span = (1u << shift) - 1u;
+    shift = max(0, shift - 10);
+    if (common) cluster.sync(); else __syncthreads();       // everybody has read the counts
+  }
+  uint32_t left = 0;
+#pragma unroll
+  for (int j = 0; j < E; ++j) left += __popc(__ballot_sync(full, mine(j) && key[j] >= bound));
+  uint32_t pos[E / 2];                                      // (read before anybody writes)
+#pragma unroll
+  for (int j = 0; j < E; ++j) {
+    const uint32_t x = mine(j) ? list_pos[first + j * 32] : 0u;
+    pos[j / 2] = j & 1 ? pos[j / 2] | x << 16 : x;
+  }
+  if (common) cluster.sync(); else __syncthreads();         // the others have read this CTA's minima
+  if (lane == 0) minima[warp] = left;
+  __syncthreads();
+  const uint32_t sum = lane < WARPS ? minima[lane] : 0u;
+  uint32_t to = __reduce_add_sync(full, lane < warp ? sum : 0u);
+#pragma unroll
+  for (int j = 0; j < E; ++j) {
+    const bool stays = mine(j) && key[j] >= bound;
+    const uint32_t all = __ballot_sync(full, stays);
+    if (stays) {
+      list_key[to + __popc(all & lt)] = key[j];
+      list_pos[to + __popc(all & lt)] = static_cast<uint16_t>(pos[j / 2] >> (16 * (j & 1)));
+    }
+    to += __popc(all);
+  }
+  __syncthreads();
+  return make_uint2(__reduce_add_sync(full, sum), bound);
 }
 
 // Dynamic shared memory of an instance for slices of `slice` positions (a multiple of 32).
@@ -686,10 +778,12 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
     }
     __syncthreads();
     uint32_t bound = 0;
-    {
+    bool crowded = false;                                   // common bound: many more candidates than wanted (the runs stand for
+    {                                                       // them; without one the CTA counts them below)
       uint32_t digit, above;
       if (sel_find_from_top<THREADS>(hist[common ? 1 : 0], rows, static_cast<uint32_t>(k), digit, above)) {
         bound = sel_bin_edge(digit);
+        crowded = common && above + hist[1][digit] > 2u * k + kSelCrowd / 2 * C;
       } else if (common || k < len) {                       // the plateaus do not add up to k: count every position
         if (common) cluster.sync(); else __syncthreads();   // everybody has read the first counts
         for (int i = tid; i < 2 * kSelBinsLin; i += THREADS) (&hist[0][0])[i] = 0;
@@ -732,7 +826,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
     __syncthreads();
     uint32_t wsum = lane < WARPS ? warp_c[lane] : 0u;
     const uint32_t before = __reduce_add_sync(full, lane < warp ? wsum : 0u), all = __reduce_add_sync(full, wsum);
-    const int M = static_cast<int>((all & 0xffffu) + (all >> 16));
+    int M = static_cast<int>((all & 0xffffu) + (all >> 16));
     {
       const uint32_t base2 = before + incl - c2;
 #pragma unroll
@@ -752,6 +846,14 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
     mx = __reduce_max_sync(full, warp_a[lane & (WARPS - 1)]);
     for (int i = tid; i < 2 * kSelBinsLin; i += THREADS) (&local[0][0])[i] = 0;
     __syncthreads();
+    if constexpr (THREADS * RUNS > 512) {                   // (up to 4096 candidates of one CTA are ranked in 10 us all the same)
+      if (!common) crowded = k < len && M > 2 * k + kSelCrowd;
+      if (crowded) {
+        const uint2 refined = sel_refine<THREADS, RUNS>(list_key, list_pos, M, k, &hist[0][0], rows, warp_c, warp_a, common);
+        M = static_cast<int>(refined.x);
+        bound = refined.y;
+      }
+    }
     // every CTA gets everybody's keys: stores into the others' shared memory, which nobody waits for until the barrier
     // (reading them there after it cost 2 to 3 us)
     if (tid < C) {

@@ -21,6 +21,14 @@ def scores_of(kind, heads, P, seed):
         return torch.randint(0, 3, (heads, P), generator=g).float()
     if kind == "equal":
         return torch.full((heads, P), 0.25)
+    if kind == "tiny":                                       # scales off the kernel's absolute bins, and rows within one bin
+        return (torch.rand(heads, P, generator=g) ** 8) * 1e-12
+    if kind == "negative":
+        return torch.rand(heads, P, generator=g) - 2
+    if kind == "huge":
+        return (torch.rand(heads, P, generator=g) ** 8) * 1e6
+    if kind == "flat":
+        return (1 + 0.02 * torch.rand(heads, P, generator=g)) / P
     s = torch.rand(heads, P, generator=g) * 1e-6             # "crowd": the winners sit in one stretch, with one huge score
     at = (P * 5) // 7
     s[:, at: at + P // 16 + 2] += 1.0 + torch.rand(heads, min(P // 16 + 2, P - at), generator=g)
@@ -75,6 +83,41 @@ def check_selection(case, sweep_ctas):
             want = np.concatenate([want, np.arange(prefix, n)])
             assert np.array_equal(got[at: at + len(want)], want), (b, h)
             at += len(want)
+
+
+SCALES = ["tiny", "negative", "huge", "flat"]
+
+
+# one CTA, two, eight; bounds per CTA and for the cluster; more rows than runs; all but a few
+@pytest.mark.parametrize("kind", SCALES)
+@pytest.mark.parametrize("P,k,w,avg", [(1500, 40, 1, 0), (4000, 96, 7, 0), (8190, 3000, 3, 0), (12000, 480, 7, 1), (20000, 1100, 5, 0),
+                                       (33000, 3000, 1, 0), (100000, 64, 21, 0), (131040, 96, 7, 0), (131001, 5000, 1, 0), (131072, 130000, 3, 1)])
+def test_selection_is_exact_on_any_scale(P, k, w, avg, kind):
+    check_selection((P, k, w, avg, kind, 3), 0)
+
+
+@pytest.mark.parametrize("kind", SCALES)
+def test_the_time_of_a_selection_does_not_depend_on_the_scale(kind):
+    P, heads, k = 131040, 8, 96
+    cfg = pkv.make_config(num_layers=1, num_q_heads=heads, num_kv_heads=heads, head_dim=64, window=ALPHA, pool_kernel=7, dtype="bf16",
+                          avg_budget=ALPHA)
+    ws = pkv.new_workspace(cfg, 1, P + ALPHA, DEV)
+    idx = torch.empty(pkv.total_rows(cfg, k, [P + ALPHA]), dtype=torch.int32, device=DEV)
+
+    def fastest(s):
+        s, times = s[None].to(DEV), []
+        for _ in range(20):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(10):
+                pkv.select_topk(cfg, s, [P + ALPHA], k, idx, ws)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b))
+        return min(times)
+
+    # a pass or two more over the candidates; with every position a candidate to the end it is 8 to 13 times as long
+    assert fastest(scores_of(kind, heads, P, 3)) < 4 * fastest(scores_of("normal", heads, P, 3))
 
 
 @pytest.mark.parametrize("P,budget", [(3000, 96), (9001, 2048), (40000, 1500)])
