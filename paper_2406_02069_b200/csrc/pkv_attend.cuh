@@ -130,6 +130,7 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
   uint8_t* smem = at_smem;
   pdl_trigger();
   if (smem_u32(smem) & 1023u) {                                // the carve-up below needs this; never seen otherwise
+    pdl_wait();                                                // (as below: never before the sweep ahead)
     if (threadIdx.x == 0) atomicOr(p.status, kStatusWaitExpired);
     return;
   }
@@ -506,6 +507,7 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
   }
 
   // ---- teardown
+  pdl_wait();                                                  // never finish before the sweep ahead, also when a wait ran out early
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && *abort_flag) atomicOr(p.status, kStatusWaitExpired);
