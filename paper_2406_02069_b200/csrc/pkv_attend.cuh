@@ -26,8 +26,9 @@
 // TMEM: columns 0..255 the S stage, 256..511 O^T (lane = channel c, column = window row).
 // Shared memory: Q 64 KB, one K tile, two V tiles, two P buffers of 32 KB each (128 keys x 128 rows).
 //
-// Every wait on an mbarrier is bounded, as in the score sweeps: a wait that runs out sets the abort
-// flag, all roles leave their loops, copies in flight are drained, TMEM is released.
+// Every wait on an mbarrier is bounded, as in the score sweeps, and the roles that wait for the epilogue wait for the sweep
+// ahead first: a wait that runs out sets the abort flag, all roles leave their loops, copies in flight are drained, TMEM is
+// released.
 #pragma once
 
 #include "pkv_score_tc.cuh"
@@ -210,7 +211,10 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
       TcItem w = first_tile();
       for (; static_cast<int>(it) < ntiles; ++it, next_tile(w)) {
         if (w.b != cur_b || w.h != cur_h) {
-          if (heads_loaded > 0) ok = mbar_wait(q_empty, (heads_loaded - 1) & 1, abort_flag, p.wait_clocks);
+          if (heads_loaded > 0) {
+            pdl_wait();
+            ok = mbar_wait(q_empty, (heads_loaded - 1) & 1, abort_flag, p.wait_clocks);
+          }
           if (!ok) break;
           mbar_expect_tx(q_full, static_cast<uint32_t>(p.rows) * kAtD * 2);
           for (int half = 0; half < 2; ++half)
@@ -218,6 +222,7 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
           ++heads_loaded;
           cur_b = w.b; cur_h = w.h;
         }
+        if (it == 2) pdl_wait();                               // (from here on it waits for the epilogue)
         ok = mbar_wait(k_empty, (it & 1) ^ 1, abort_flag, p.wait_clocks);
         if (!ok) break;
         if (p.withhold && blockIdx.x == 0 && static_cast<int>(it) + 1 == ntiles) continue;   // test aid: never arrives
@@ -241,6 +246,7 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
       TcItem w = first_tile();
       for (; static_cast<int>(it) < ntiles; ++it, next_tile(w)) {
         const int s = it & 1;
+        if (it == 2) pdl_wait();
         ok = mbar_wait(v_empty(s), ((it >> 1) & 1) ^ 1, abort_flag, p.wait_clocks);
         if (!ok) break;
         mbar_expect_tx(v_full(s), kAtTileBytes);
@@ -267,6 +273,7 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
       // V^T P of both row halves of tile j, each as soon as its P buffer is full
       auto issue_pv = [&](uint32_t j) -> bool {
         const int vs = j & 1;
+        if (j == 0) pdl_wait();                                // V and P come behind the sweep ahead
         if (!mbar_wait(v_full(vs), (j >> 1) & 1, abort_flag, p.wait_clocks)) return false;
         if (wait_o) {                                          // the epilogue has read the accumulators of the run before
           if (!mbar_wait(o_empty, (runs - 1) & 1, abort_flag, p.wait_clocks)) return false;
@@ -311,6 +318,7 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
         {
           ok = mbar_wait(k_full, it & 1, abort_flag, p.wait_clocks);
           if (!ok) break;
+          if (it == 1) pdl_wait();
           ok = mbar_wait(s_empty, (it & 1) ^ 1, abort_flag, p.wait_clocks);   // the tile before is in registers
           if (!ok) break;
           tc_fence_after();

@@ -20,7 +20,8 @@
 // an accumulator stage of its own, refilled while the other three compute.  CTAs are persistent: each takes a contiguous range of (sequence,
 // KV head, key chunk) work items.
 //
-// Every wait on an mbarrier is bounded.  A wait that runs out sets an abort flag in
+// Every wait on an mbarrier is bounded.  Sweep B's epilogue waits for sweep A, whose time that bound says nothing about, so
+// the roles that wait for the epilogue wait for sweep A first (pdl_wait).  A wait that runs out sets an abort flag in
 // shared memory and a status bit in the workspace; all roles then leave their loops,
 // the producer drains the copies it still has in flight, TMEM is released and the
 // kernel returns.
@@ -639,6 +640,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
       TcItem w = first_tile();
       for (; static_cast<int>(it) < ntiles; ++it, next_tile(w)) {
         const int s = it % kKStages;
+        if (SWEEP == 1 && it == static_cast<uint32_t>(kKStages + kTcStages / p.row_blocks)) pdl_wait();
         ok = mbar_wait(k_empty(s), ((it / kKStages) & 1) ^ 1, abort_flag, p.wait_clocks);
         if (!ok) break;
         if (SWEEP == 0 && p.withhold && blockIdx.x == 0 && static_cast<int>(it) + 1 == ntiles) continue;   // test aid: never arrives
@@ -668,6 +670,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
         if (w.b == cur_b && w.h == cur_h) continue;
         cur_b = w.b; cur_h = w.h;
         const uint32_t slot = heads % q_slots, round = heads / q_slots;
+        if (SWEEP == 1 && heads == static_cast<uint32_t>(q_slots)) pdl_wait();
         ok = mbar_wait(q_empty(slot), (round & 1) ^ 1, abort_flag, p.wait_clocks);
         if (!ok) break;
         mbar_expect_tx(q_full(slot), static_cast<uint32_t>(copies * p.rows) * D * 2);
@@ -708,6 +711,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
           const uint32_t q_addr = smem_u32(q_s) + slot * 128 * 128;
           for (int rb = 0; rb < p.row_blocks && ok; ++rb, ++u) {
             const int ts = u % kTcStages;
+            if (SWEEP == 1 && u == kTcStages) pdl_wait();
             ok = mbar_wait(t_empty(ts), ((u / kTcStages) & 1) ^ 1, abort_flag, p.wait_clocks);
             if (!ok) break;
             tc_fence_after();

@@ -75,3 +75,33 @@ def test_equal_keys_get_equal_scores_whichever_cta_has_them(group, window, d, dt
     for b, n in enumerate(lens):
         same = scores[b, :, 5: n - window: 128]
         assert torch.equal(same, same[:, :1].expand_as(same)), [int((row != row[0]).sum()) for row in same]
+
+
+def test_a_long_sweep_ahead_is_not_a_wait_that_ran_out():
+    """One CTA takes milliseconds for the row statistics of sixteen heads; the window-attention kernel behind it is on the
+    device all that time, with the bound of its waits at about one millisecond (one head takes it less than half of that).
+    Three attempts: a hiccup of the device may use up so short a bound, the sweep would do it every time."""
+    heads, group, window, n = 16, 8, 32, 16384 + 32
+    cfg = pkv.make_config(num_layers=1, num_q_heads=group * heads, num_kv_heads=heads, head_dim=128, window=window, pool_kernel=1,
+                          dtype="bf16", avg_budget=window, sweep_ctas=1)
+    g = torch.Generator(device=DEV).manual_seed(3)
+    q = torch.randn(1, group * heads, window, 128, generator=g, device=DEV).bfloat16()
+    k, v = (torch.randn(1, heads, n, 128, generator=g, device=DEV).bfloat16() for _ in range(2))
+
+    def attend(bound):
+        ws = pkv.new_workspace(cfg, 1, n, DEV)
+        scores, out = torch.zeros(1, heads, n, device=DEV), torch.zeros(1, group * heads, window, 128, device=DEV)
+        binding.test_hooks(wait_clocks=bound)
+        try:
+            pkv.attend_window(cfg, q, k, v, [n], out, scores, ws)
+            pkv.check_status(ws)
+        except pkv.PkvError:
+            return None
+        finally:
+            binding.test_hooks()
+        return scores, out
+
+    want = attend(0)
+    got = next((r for r in (attend(1 << 21) for _ in range(3)) if r is not None), None)
+    assert got is not None, "the time of the sweep ahead counts as a wait"
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
