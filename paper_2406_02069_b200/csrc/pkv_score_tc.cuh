@@ -458,7 +458,7 @@ __device__ __forceinline__ void tc_normalisers(const Params& p, int b, int h, in
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int r = r0 + u * r_step;
-      if (part == 0) dst[r] = r < p.rows ? -(m[u] + __log2f(z[u]) + p.log2_group) : -INFINITY;
+      if (part == 0) dst[r] = r < p.rows ? -(m[u] + log2f(z[u]) + p.log2_group) : -INFINITY;
     }
   };
   using std::integral_constant;
@@ -469,7 +469,7 @@ __device__ __forceinline__ void tc_normalisers(const Params& p, int b, int h, in
 #pragma unroll 1
       for (int r = tid; r < rows_p2; r += THREADS) {
         const float2 mz = tc_merge_row<decltype(lanes)::value, decltype(q_const)::value>(p.partial + min(r, p.rows - 1), p.rows, s0, s1);
-        dst[r] = r < p.rows ? -(mz.x + __log2f(mz.y) + p.log2_group) : -INFINITY;
+        dst[r] = r < p.rows ? -(mz.x + log2f(mz.y) + p.log2_group) : -INFINITY;
       }
     };
     if (s1 - s0 <= min(2 * per_row, 16)) {
