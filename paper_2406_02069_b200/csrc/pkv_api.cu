@@ -617,7 +617,6 @@ int run_attend(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, co
   ap.withhold = g_test_withhold_attend.load();
   ap.scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(c->head_dim)));
   ap.partial = w.partial;
-  ap.merge = 1;
   ap.stat_grid = stats.grid;
   ap.wait_v = stats.early;
   ap.log2_group = std::log2(static_cast<float>(group)) - kAtShift;

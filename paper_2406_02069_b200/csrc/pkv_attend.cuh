@@ -59,11 +59,10 @@ struct AtParams {
   int32_t withhold;             // test aid: CTA 0 never loads its last K tile (its waits then run out)
   long long wait_clocks;
   float scale_log2;             // log2(e) / sqrt(d)
-  // the row normalisers come from the partials of the row-statistics sweep, as in the score sweep (tc_normalisers)
+  // the row normalisers come from the partials of the row-statistics sweep, as in the score sweep (tc_merge_head)
   const float2* partial;
-  const float* lse2;
-  float lse_scale, lse_add, log2_group;      // log2 G - kAtShift
-  int32_t merge, stat_grid;
+  float log2_group;             // log2 G - kAtShift
+  int32_t stat_grid;
   int32_t wait_v;               // 1: the sweep ahead started on the caller's word for Q and K alone: V waits for it to end
   float* scores;                // [batch][H_kv][ld]: the prefix positions are written
   int64_t ld_scores;
@@ -400,7 +399,7 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
         // once everybody has written
         ok = meet();
         if (!ok) break;
-        tc_normalisers<kAtEpiWarps * 32>(p, w.b, w.h, e * 32 + lane, lse_all);
+        tc_merge_head<kAtEpiWarps * 32, true>(p, w.b, w.h, e * 32 + lane, lse_all);
         ok = meet();
         if (!ok) break;
         cur_b = w.b; cur_h = w.h;

@@ -35,7 +35,7 @@
 
 namespace pkv {
 
-constexpr int kTcThreads = 640;         // 20 warps: producer, MMA issuer, 2 idle, 16 epilogue
+constexpr int kTcThreads = 640;         // 20 warps: producer of K, MMA issuer, producer of Q, statistics, 16 epilogue
 constexpr int kTcEpiWarp0 = 4;          // first epilogue warp
 constexpr int kTcEpiWarps = 16;         // four per scheduler, which is what keeps the exp unit fed
 constexpr int kTcTileKeys = 128;        // keys per K tile: the N of sweep A's MMAs, the M of sweep B's
@@ -406,38 +406,31 @@ __device__ __forceinline__ float2 tc_merge_row(const float2* row, int rows, int 
   return lane[0];
 }
 
-// A head's negated row normalisers into dst (-inf for the padding rows), by THREADS threads (the sixteen epilogue warps or one
-// warp): the caller's values, or sweep A's partials of this head merged.  Every CTA that works on a head merges it for
-// itself, and equal keys must get equal scores whichever CTA has them, so the additions come in the same order whoever does
+// Sweep A's partials of a head -> its negated row normalisers in dst (-inf for the padding rows), by THREADS threads (the sixteen
+// epilogue warps or one warp).  Every CTA that works on a head merges it for itself, and equal keys must get equal scores whichever CTA has them, so the additions come in the same order whoever does
 // it: 2 to 16 lanes per row by the number of rows alone, each with every per_row-th segment, then pairwise.  A single warp
 // does the same with a lane per row where the head has few segments (what it has to save there are instructions, beside
 // four warps of the epilogue on its scheduler), else in sixteen steps, four at a time if it can (L2 latencies).
-template <int THREADS, typename Params>
-__device__ __forceinline__ void tc_normalisers(const Params& p, int b, int h, int tid, float* dst) {
+template <int THREADS, bool ACCURATE, typename Params>
+__device__ __forceinline__ void tc_merge_head(const Params& p, int b, int h, int tid, float* dst) {
   constexpr int kSteps = kTcEpiWarps * 32 / THREADS;           // of THREADS / per_row rows
   const int rows_p2 = p.rows_pad <= 32 ? 32 : (p.rows_pad <= 64 ? 64 : (p.rows_pad <= 128 ? 128 : 256));
   const int per_row = kTcEpiWarps * 32 / rows_p2, r_step = THREADS / per_row;
   const int hg = b * p.num_kv_heads + h;
-  int s0 = 0, s1 = 0;
-  if (p.merge) {
-    // sweep A's CTAs took contiguous item ranges (items ordered sequence, head, chunk): the first `rem`
-    // CTAs per + 1 items, the others per; this head's items fell to CTAs c0..c1, one segment each
-    const int nc = p.seq.stat_off[b + 1] - p.seq.stat_off[b];
-    const int total_a = p.num_kv_heads * p.seq.stat_off[p.seq.batch];
-    const int per_a = total_a / p.stat_grid, rem_a = total_a % p.stat_grid, edge = rem_a * (per_a + 1);
-    const int i0 = p.num_kv_heads * p.seq.stat_off[b] + h * nc, i1 = i0 + nc - 1;
-    const int c0 = i0 < edge ? i0 / (per_a + 1) : rem_a + (i0 - edge) / per_a;
-    const int c1 = i1 < edge ? i1 / (per_a + 1) : rem_a + (i1 - edge) / per_a;
-    s0 = c0 + hg;
-    s1 = c1 + hg + 1;
-  }
+  // sweep A's CTAs took contiguous item ranges (items ordered sequence, head, chunk): the first `rem`
+  // CTAs per + 1 items, the others per; this head's items fell to CTAs c0..c1, one segment each
+  const int nc = p.seq.stat_off[b + 1] - p.seq.stat_off[b];
+  const int total_a = p.num_kv_heads * p.seq.stat_off[p.seq.batch];
+  const int per_a = total_a / p.stat_grid, rem_a = total_a % p.stat_grid, edge = rem_a * (per_a + 1);
+  const int i0 = p.num_kv_heads * p.seq.stat_off[b] + h * nc, i1 = i0 + nc - 1;
+  const int c0 = i0 < edge ? i0 / (per_a + 1) : rem_a + (i0 - edge) / per_a;
+  const int c1 = i1 < edge ? i1 / (per_a + 1) : rem_a + (i1 - edge) / per_a;
+  const int s0 = c0 + hg, s1 = c1 + hg + 1;
   const int part = tid % per_row;
-  pdl_wait();                                                  // normalisers and partials are written by kernels before
-  if (!p.merge) {
-    for (int r = tid; r < rows_p2; r += THREADS)
-      dst[r] = r < p.rows ? -fmaf(p.lse2[static_cast<int64_t>(hg) * p.rows + r], p.lse_scale, p.lse_add) : -INFINITY;
-    return;
-  }
+  pdl_wait();                                                  // the partials are written by the kernel before
+  // log2f costs the warp that merges ahead of sweep B's epilogue some instructions (three steps of two sequences at head size
+  // 64: 33.7 -> 34.2 us); the exponentials of the score sweeps are not as exact as __log2f
+  auto log_of = [](float x) { return ACCURATE ? log2f(x) : __log2f(x); };
   // U steps from `step` on, segments in batches of Q
   auto some = [&](int step, auto u_const, auto q_const) {
     constexpr int U = decltype(u_const)::value, Q = decltype(q_const)::value;
@@ -458,7 +451,7 @@ __device__ __forceinline__ void tc_normalisers(const Params& p, int b, int h, in
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int r = r0 + u * r_step;
-      if (part == 0) dst[r] = r < p.rows ? -(m[u] + log2f(z[u]) + p.log2_group) : -INFINITY;
+      if (part == 0) dst[r] = r < p.rows ? -(m[u] + log_of(z[u]) + p.log2_group) : -INFINITY;
     }
   };
   using std::integral_constant;
@@ -469,7 +462,7 @@ __device__ __forceinline__ void tc_normalisers(const Params& p, int b, int h, in
 #pragma unroll 1
       for (int r = tid; r < rows_p2; r += THREADS) {
         const float2 mz = tc_merge_row<decltype(lanes)::value, decltype(q_const)::value>(p.partial + min(r, p.rows - 1), p.rows, s0, s1);
-        dst[r] = r < p.rows ? -(mz.x + log2f(mz.y) + p.log2_group) : -INFINITY;
+        dst[r] = r < p.rows ? -(mz.x + log_of(mz.y) + p.log2_group) : -INFINITY;
       }
     };
     if (s1 - s0 <= min(2 * per_row, 16)) {
@@ -485,6 +478,19 @@ __device__ __forceinline__ void tc_normalisers(const Params& p, int b, int h, in
       for (int step = 0; step < kSteps; ++step) some(step, integral_constant<int, 1>{}, integral_constant<int, 10>{});
     }
   }
+}
+
+// Sweep B: the same from the caller's values (or the merge kernel's), or from sweep A's partials.
+template <int THREADS>
+__device__ __forceinline__ void tc_normalisers(const TcParams& p, int b, int h, int tid, float* dst) {
+  if (p.merge) {
+    tc_merge_head<THREADS, false>(p, b, h, tid, dst);
+    return;
+  }
+  const int rows_p2 = p.rows_pad <= 32 ? 32 : (p.rows_pad <= 64 ? 64 : (p.rows_pad <= 128 ? 128 : 256));
+  const float* lse2 = p.lse2 + (static_cast<int64_t>(b) * p.num_kv_heads + h) * p.rows;
+  pdl_wait();                                                  // normalisers may be written by a kernel before
+  for (int r = tid; r < rows_p2; r += THREADS) dst[r] = r < p.rows ? -fmaf(lse2[r], p.lse_scale, p.lse_add) : -INFINITY;
 }
 
 // The item behind (REVERSE: before) w; behind the last one w stays on its sequence.
@@ -915,7 +921,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant
         // thread -> key.  The head's normalisers, negated (the epilogue adds them), sit in one of two buffers that alternate
         // from head to head.  The first one is filled by the sixteen warps together, which then meet; the others by warp 3,
         // ahead of time.  They come from the caller (or the merge kernel), or straight from sweep A's partials of the head,
-        // which every CTA that works on it merges for itself, always in the same order (see tc_normalisers).
+        // which every CTA that works on it merges for itself, always in the same order (see tc_merge_head).
         if (new_head) {
           const uint32_t buf = heads & 1u;
           if (heads == 0) {
