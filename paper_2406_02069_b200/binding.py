@@ -17,6 +17,8 @@ from __future__ import annotations
 import ctypes
 import importlib.machinery
 import importlib.util
+import subprocess
+import warnings
 from typing import List, Optional, Sequence
 
 import torch
@@ -137,22 +139,32 @@ _lib = _LazyLibrary()
 
 class _LazyNative:
     """The functions of _pkv_native.so, loaded on first use (after libpyramidkv.so, which it is linked against) and
-    kept as attributes."""
+    kept as attributes.  Where it cannot be built or loaded (no compiler, no Python or torch headers) every function
+    takes nothing, and the calls go through ctypes: one warning says so."""
 
     def __getattr__(self, name):
         if name.startswith("__"):
             raise AttributeError(name)
         _lib.pyramidkv_strerror                     # loads libpyramidkv.so
-        path = _build.build_binding()
-        spec = importlib.util.spec_from_loader("_pkv_native", importlib.machinery.ExtensionFileLoader("_pkv_native", path))
-        module = importlib.util.module_from_spec(spec)
-        spec.loader.exec_module(module)
+        try:
+            path = _build.build_binding()
+            spec = importlib.util.spec_from_loader("_pkv_native", importlib.machinery.ExtensionFileLoader("_pkv_native", path))
+            module = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(module)
+        except (OSError, subprocess.CalledProcessError, ImportError) as e:
+            warnings.warn("the native half of the binding is not available (%s): calls take some 20 us more of host time" % e,
+                          RuntimeWarning, stacklevel=3)
+            for f in _NATIVE_CALLS:
+                setattr(self, f, lambda *args: _NOT_TAKEN)
+            return self.__dict__[name]
         for f in dir(module):
             if not f.startswith("__"):
                 setattr(self, f, getattr(module, f))
         return self.__dict__[name]
 
 
+_NATIVE_CALLS = ("compress_layer", "attend_compress_layer", "compress_layer_paged", "score_window", "select_topk", "gather_compact",
+                 "decode_attention", "decode_attention_paged")
 _native = _LazyNative()
 _NOT_TAKEN = -1        # the native call left the arguments to the checks here; nothing was enqueued
 

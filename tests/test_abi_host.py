@@ -205,6 +205,36 @@ def test_a_workspace_for_a_larger_problem_serves_the_smaller_ones():
     assert out.returncode == 0 and "accepted" in out.stdout, out.stdout[-2000:] + out.stderr[-4000:]
 
 
+_NO_COMPILER = r'''
+import warnings
+import torch
+import paper_2406_02069_b200 as pkv
+from paper_2406_02069_b200 import binding, build
+
+build.BINDING = build.BINDING + ".absent.so"              # as in an installation that ships libpyramidkv.so alone
+cfg = pkv.make_config(num_layers=1, num_q_heads=2, num_kv_heads=2, head_dim=64, window=4, pool_kernel=1, dtype="bf16", avg_budget=4)
+scores, idx, ws = torch.zeros(1, 2, 96), torch.zeros(64, dtype=torch.int32), torch.zeros(1 << 20, dtype=torch.uint8)
+with warnings.catch_warnings(record=True) as seen:
+    warnings.simplefilter("always")
+    for _ in range(2):
+        try:
+            pkv.select_topk(cfg, scores, [100], 4, idx, ws)
+        except ValueError as e:                              # the Python checks: no device tensors here
+            assert "device tensor" in str(e)
+        else:
+            raise AssertionError("not refused")
+assert [w.category for w in seen] == [RuntimeWarning], seen
+assert set(binding._NATIVE_CALLS) <= set(vars(binding._native))
+print("ctypes path")
+'''
+
+
+def test_a_library_without_the_native_binding_works_through_ctypes():
+    env = dict(os.environ, CUDA_VISIBLE_DEVICES="", CXX="/nonexistent/compiler")
+    out = subprocess.run([sys.executable, "-c", _NO_COMPILER], cwd=ROOT, env=env, capture_output=True, text=True, timeout=600)
+    assert out.returncode == 0 and "ctypes path" in out.stdout, out.stdout[-2000:] + out.stderr[-4000:]
+
+
 def test_workload_generator_is_seeded_and_shaped():
     w = workloads.scaled(workloads.MISTRAL_RAGGED, num_layers=2, batch=3)
     lens = w.seq_lens()
