@@ -151,6 +151,7 @@ class _LazyNative:
             spec = importlib.util.spec_from_loader("_pkv_native", importlib.machinery.ExtensionFileLoader("_pkv_native", path))
             module = importlib.util.module_from_spec(spec)
             spec.loader.exec_module(module)
+            module.set_config_type(PkvConfig)
         except (OSError, subprocess.CalledProcessError, ImportError) as e:
             warnings.warn("the native half of the binding is not available (%s): calls take some 20 us more of host time" % e,
                           RuntimeWarning, stacklevel=3)

@@ -26,6 +26,7 @@
 namespace {
 
 constexpr int kNotTaken = -1;
+PyObject* g_config_type = nullptr;       // PkvConfig: other objects that expose a buffer of its size are not configurations
 
 // A tensor argument as the checks need it (borrowed: the arguments outlive the call).
 struct View {
@@ -61,6 +62,7 @@ struct Call {
   ~Call() { if (cfg) PyBuffer_Release(&buf); }
 
   bool open(PyObject* config, PyObject* seq_lens) {
+    if (!g_config_type || PyObject_IsInstance(config, g_config_type) != 1) { PyErr_Clear(); return false; }
     if (PyObject_GetBuffer(config, &buf, PyBUF_SIMPLE) != 0) { PyErr_Clear(); return false; }
     cfg = static_cast<const pkv_config*>(buf.buf);               // released by the destructor from here on
     if (buf.len != static_cast<Py_ssize_t>(sizeof(pkv_config))) return false;
@@ -73,7 +75,7 @@ struct Call {
       PyObject* o = list ? PyList_GET_ITEM(seq_lens, i) : PyTuple_GET_ITEM(seq_lens, i);
       if (!PyLong_CheckExact(o)) return false;
       const long v = PyLong_AsLong(o);
-      if (v < cfg->window + 1l || v > INT32_MAX) { PyErr_Clear(); return false; }
+      if ((v == -1 && PyErr_Occurred()) || v < cfg->window + 1l || v > INT32_MAX) { PyErr_Clear(); return false; }
       lens[i] = static_cast<int32_t>(v);
       longest = std::max(longest, lens[i]);
     }
@@ -335,10 +337,18 @@ PyObject* guarded(PyObject* self, PyObject* const* a, Py_ssize_t n) {
   }
 }
 
+// (type): the class of the configurations.
+PyObject* set_config_type(PyObject*, PyObject* type) {
+  Py_INCREF(type);
+  Py_XDECREF(g_config_type);
+  g_config_type = type;
+  Py_RETURN_NONE;
+}
+
 #define PKV_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(guarded<name>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {PKV_METHOD(compress_layer), PKV_METHOD(attend_compress_layer), PKV_METHOD(compress_layer_paged),
                          PKV_METHOD(score_window), PKV_METHOD(select_topk), PKV_METHOD(gather_compact), PKV_METHOD(decode_attention),
-                         PKV_METHOD(decode_attention_paged), {nullptr, nullptr, 0, nullptr}};
+                         PKV_METHOD(decode_attention_paged), {"set_config_type", set_config_type, METH_O, nullptr}, {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_pkv_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace

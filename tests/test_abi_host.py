@@ -235,6 +235,18 @@ def test_a_library_without_the_native_binding_works_through_ctypes():
     assert out.returncode == 0 and "ctypes path" in out.stdout, out.stdout[-2000:] + out.stderr[-4000:]
 
 
+def test_the_native_binding_leaves_odd_arguments_to_the_checks():
+    """Another object with a configuration's bytes, and a length that no integer type holds beside a window that admits
+    every length: not taken, and no error left behind."""
+    cfg = pkv.make_config(num_layers=1, num_q_heads=2, num_kv_heads=2, head_dim=64, window=4, pool_kernel=1, dtype="bf16", avg_budget=4)
+    t = [None] * 5
+    assert binding._native.select_topk(bytes(cfg), t[0], [100], 4, t[1], t[2], None) == -1
+    cfg.window = -5
+    assert binding._native.select_topk(cfg, t[0], [2 ** 70], 4, t[1], t[2], None) == -1
+    with pytest.raises(AttributeError):
+        pkv.select_topk(bytes(cfg), t[0], [100], 4, t[1], t[2])
+
+
 def test_workload_generator_is_seeded_and_shaped():
     w = workloads.scaled(workloads.MISTRAL_RAGGED, num_layers=2, batch=3)
     lens = w.seq_lens()
