@@ -110,7 +110,10 @@ typedef struct pkv_config {
   uint32_t sweep_ctas;   /* CTAs the persistent score sweeps of a call launch: 0 = one per SM (default), else at
                             most this many (<= 1024).  A caller that runs independent layers on several streams
                             gives each call a share of the SMs this way, so that two layers' sweeps run side by
-                            side instead of one after the other; results do not depend on it beyond rounding. */
+                            side instead of one after the other; results do not depend on it beyond rounding.
+                            A cap below the device's SMs also says that other layers run beside this call: the
+                            selection then takes half-size CTAs for slices of 4097 to 8192 positions (two to an SM,
+                            more work in the same time; the same lists). */
 } pkv_config;
 
 typedef struct pkv_tensor {

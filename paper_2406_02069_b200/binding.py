@@ -195,7 +195,8 @@ def make_config(*, num_layers: int, num_q_heads: int, num_kv_heads: int, head_di
                 schedule: str = "linear", inputs_final: bool = False, sweep_ctas: int = 0) -> PkvConfig:
     """inputs_final sets PKV_FLAG_INPUTS_FINAL: nothing still running on the stream writes q_win or k when a call is
     enqueued, so the score kernels may read them before the kernels ahead of them have finished.  sweep_ctas > 0
-    caps the CTAs of the persistent score sweeps (a share of the SMs for callers that run layers on several streams)."""
+    caps the CTAs of the persistent score sweeps (a share of the SMs for callers that run layers on several streams; the
+    selection then takes its CTAs for calls beside other layers too)."""
     code = {"fp32": 0, "bf16": 1, "fp16": 2, torch.float32: 0, torch.bfloat16: 1, torch.float16: 2}[dtype]
     return PkvConfig(num_layers, num_q_heads, num_kv_heads, head_dim, window, pool_kernel, pool_kind, code,
                      avg_budget, {"linear": 0, "geometric": 1}[schedule], float(beta), 1 if inputs_final else 0, int(sweep_ctas))

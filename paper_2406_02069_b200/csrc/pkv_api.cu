@@ -33,7 +33,11 @@ std::atomic<int> g_test_two_sweeps{0};     // 1: never take the single-sweep ker
 constexpr size_t kAlign = 256;
 constexpr int kPartialChunk = 128;   // keys per partial slot of the fp32-pipe path (sizes the workspace)
 static_assert(kPartialChunk == kGenTile, "one partial per tile");
-constexpr size_t kMaxLogitBytes = size_t{256} << 20;   // fp32-pipe path: logits are kept between its passes up to this size
+// fp32-pipe path: logits are kept between its passes up to this size.  Scores of 32 / 8 heads, d = 128, 32 window rows, kept
+// against formed again: 8192 tokens 79 / 125 us, 32768 281 / 413, 65536 (256 MB) 626 / 807; 64 / 8 heads x 64 rows in bf16,
+// 16384 tokens (256 MB) 567 / 916.  With few rows and long contexts it is the other way round, because every CTA of the sums
+// merges all partials: 8 rows x 4 heads, 65536 tokens (64 MB) 289 / 266, 131072 715 / 524; d = 64, 32768 85 / 78.
+constexpr size_t kMaxLogitBytes = size_t{256} << 20;
 
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
@@ -166,7 +170,8 @@ Workspace carve(const pkv_config* c, int batch, int max_n, void* base) {
   const size_t chunks = (static_cast<size_t>(max_n) + kPartialChunk - 1) / kPartialChunk;
   w.status = reinterpret_cast<uint32_t*>(take(kAlign));
   w.lse2 = reinterpret_cast<float*>(take(heads * rows * sizeof(float)));
-  // fp32-pipe path: a slot per tile of 128 keys and head (room for two); tensor-core sweep: one segment
+  // fp32-pipe path: a slot per tile of 128 keys and head (room for two, which is what decides what the call without a
+  // workspace takes); tensor-core sweep: one segment
   // per run of a CTA over a head (at most CTAs + heads of them), whatever the context length
   const size_t partial_slots =
       tc_eligible(c) ? static_cast<size_t>(kTcMaxGrid) + heads : heads * chunks * 2;

@@ -14,8 +14,9 @@
 // 128-byte-swizzled shared memory; tcgen05.mma accumulates in TMEM (four
 // accumulator stages of up to 128 columns); epilogue warps read TMEM with tcgen05.ld.
 // Warp roles: warp 0 = TMA producer of K, warp 1 = MMA issuer and TMEM owner, warp 2 = TMA producer of Q, warp 3 = row
-// statistics on their way out of sweep A and into sweep B, warps 4..19 = epilogue.  The exponentials bound both sweeps (16 per clock per SM); four epilogue
-// warps per scheduler are what it takes to keep that unit busy.  The 16 epilogue
+// statistics on their way out of sweep A and into sweep B, warps 4..19 = epilogue, four per scheduler: the exponentials (16 per
+// clock per SM on their unit, a quarter of them on the FMA pipe) are the longest of the resources a tile needs, but no unit
+// is the bound (see the split below: 0 to 4 pairs of eight make a few per cent).  The 16 epilogue
 // warps form four groups (TMEM lane quarter = warp % 4, group = (warp - 4) / 4), each with
 // an accumulator stage of its own, refilled while the other three compute.  CTAs are persistent: each takes a contiguous range of (sequence,
 // KV head, key chunk) work items.

@@ -1,5 +1,6 @@
-"""Decode attention over the compact cache at the edges of its split: query heads per KV head around the block of
-eight, head sizes, types, and row counts around a team's step, a cluster's slices and a single row."""
+"""Decode attention over the compact cache at the edges of its split: query heads per KV head around the blocks (of four
+with 16-bit rows, of up to eight in fp32), head sizes, types, and row counts around a step, a cluster's slices and a single
+row."""
 import numpy as np
 import pytest
 import torch
@@ -19,10 +20,13 @@ CASES = [
     (2, 2, 128, "fp16", 4, 60, [500]),               # 64 rows
     (3, 2, 128, "bf16", 5, 60, [500]),               # 65 rows, a group padded to four heads
     (4, 2, 64, "fp32", 8, 505, [2000, 700]),
-    (4, 8, 128, "bf16", 32, 3900, [5000]),           # long lists over clusters of sixteen
-    (7, 1, 128, "bf16", 8, 1017, [1500]),            # 1025 rows over sixteen CTAs of one head
+    (4, 8, 128, "bf16", 32, 3900, [5000]),           # long lists over clusters of eight
+    (7, 1, 128, "bf16", 8, 1017, [1500]),            # 1025 rows over eight CTAs of one head, two blocks of query heads
     (8, 2, 64, "bf16", 8, 200, [300, 5000, 301]),
-    (12, 1, 128, "fp16", 8, 120, [4000]),            # two blocks of query heads, the second half full
+    (12, 1, 128, "fp16", 8, 120, [4000]),            # three blocks of query heads
+    (5, 2, 128, "bf16", 8, 120, [4000, 90]),         # two, one head in the second
+    (6, 1, 64, "fp16", 8, 700, [4000]),              # ... two heads
+    (12, 2, 128, "fp32", 8, 120, [4000, 90]),        # fp32: a block of eight and half a one
     (8, 40, 128, "fp32", 2, 30, [100, 101, 102, 103]),   # enough heads that no cluster forms
 ]
 
