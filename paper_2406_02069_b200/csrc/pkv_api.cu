@@ -17,6 +17,7 @@
 #include "pkv_score_generic.cuh"
 #include "pkv_score_tc.cuh"
 #include "pkv_score_resident.cuh"
+#include "pkv_score_split.cuh"
 #include "pkv_attend.cuh"
 #include "pkv_select.cuh"
 #include "pkv_shard.cuh"
@@ -371,10 +372,57 @@ int launch_logit_tiles(ScoreParams& sp, int batch, cudaStream_t st) {
   return check_launch();
 }
 
+// fp32 rows as triples of bfloat16 on the tensor cores (pkv_score_split.cuh).  Returns the CTAs to take, 0: not for this call.
+// From 33 window rows on; with up to 32 the fp32 pipe is faster (scores, fp32 pipe / split: 32 rows, 32 heads, 2000 keys,
+// d = 128 28.6 / 30.3 us; 32 rows, 8 heads, 1000 keys 14.0 / 17.9; 16 rows, 2 heads, 512 keys, d = 64 8.8 / 11.2; 64 rows, 2 heads, 8000
+// keys, d = 64 20.5 / 19.8; 64 rows, 8 heads, 4001 keys, d = 128 27.3 / 25.6; 384 rows, 8 heads, 3000 keys 121 / 47).
+constexpr int kSplitMinRows = 32;
+int split_grid(const ScoreParams& sp, int batch, int max_n, int sms) {
+  if (!sp.logits || sp.stats_only || sp.lse_in != sp.lse2 || sp.rows <= kSplitMinRows || sp.rows > 8192) return 0;
+  const long long blocks = (sp.rows + kSpRows - 1) / kSpRows, units = sp.num_kv_heads * blocks * batch;
+  long long tiles = 0;
+  for (int b = 0; b < batch; ++b) tiles += (sp.seq.n[b] + kSpKeys - 1) / kSpKeys;
+  tiles *= sp.num_kv_heads * blocks;
+  // a segment of row statistics per CTA and unit: the workspace has room for two per 128 keys of a head
+  const long long room = 2ll * batch * sp.num_kv_heads * ((max_n + kPartialChunk - 1) / kPartialChunk) - units;
+  return static_cast<int>(std::max<long long>(0, std::min(std::min<long long>(std::min(sms, kSpMaxGrid), tiles), room)));
+}
+
+template <int D>
+int launch_scores_split(ScoreParams& sp, int batch, int max_n, int grid, cudaStream_t st) {
+  static bool attr_done[64] = {};  // the attribute is per device; setting it twice is harmless
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return PKV_ERR_CUDA;
+  if (dev >= 64 || !attr_done[dev]) {
+    if (cudaFuncSetAttribute(split_logits_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SpSmem<D>::kTotal) != cudaSuccess)
+      return PKV_ERR_CUDA;
+    if (dev < 64) attr_done[dev] = true;
+  }
+  int tiles = 0;
+  for (int b = 0; b < batch; ++b) {
+    sp.seq.stat_off[b] = tiles;
+    tiles += (sp.seq.n[b] + kSpKeys - 1) / kSpKeys;
+  }
+  sp.seq.stat_off[batch] = tiles;
+  sp.stat_grid = grid;
+  sp.log2_group = std::log2(static_cast<float>(sp.group));
+  launch_pdl(split_logits_kernel<D>, dim3(grid), kSpThreads, SpSmem<D>::kTotal, st, sp);
+  mark(st, "logits_split");
+  launch_pdl(split_scores_kernel, dim3((max_n - sp.seq.alpha + kSpSumKeys - 1) / kSpSumKeys, sp.num_kv_heads, batch), kSpSumThreads,
+             static_cast<size_t>(sp.rows) * sizeof(float), st, sp);
+  mark(st, "scores_split");
+  return check_launch();
+}
+
 // Row blocks as large as the window rows need (16-bit inputs only come here with more than 256 rows).
 template <typename T, int D>
 int launch_scores_generic(ScoreParams& sp, int batch, cudaStream_t st) {
   if constexpr (sizeof(T) == 4) {
+    int max_n = 0;
+    for (int b = 0; b < batch; ++b) max_n = std::max(max_n, sp.seq.n[b]);
+    const int sms = device_sm_count();
+    if (sms <= 0) return PKV_ERR_CUDA;
+    if (const int grid = split_grid(sp, batch, max_n, sms)) return launch_scores_split<D>(sp, batch, max_n, grid, st);
     if (sp.rows <= 32) return launch_logit_tiles<T, D, 32, 4, 4>(sp, batch, st);
     if (sp.rows <= 64) return launch_logit_tiles<T, D, 64, 4, 8>(sp, batch, st);
   }
@@ -570,6 +618,7 @@ int run_scores(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, co
   sp.ld_scores = ld;
   sp.logits = w.logits;
   sp.ld_logits = w.ld_logits;
+  sp.status = w.status;
   if (tc_eligible(c)) {
     int max_n = 0;
     for (int b = 0; b < batch; ++b) max_n = std::max(max_n, table.n[b]);

@@ -49,6 +49,7 @@ struct ScoreParams {
   int64_t ld_logits;
   int32_t chunk_tiles;                   // tiles per CTA (1 when there are several row blocks)
   float log2_group;
+  uint32_t* status;
 };
 
 // Four consecutive channels of a row as floats.
