@@ -906,25 +906,20 @@ bool paged_args_ok(const int32_t* block_table, int page_size, int num_pages, con
   return reinterpret_cast<uintptr_t>(k_pool) % 16 == 0 && reinterpret_cast<uintptr_t>(v_pool) % 16 == 0;
 }
 
-// CTAs of a decode cluster: doubled while every CTA of the doubled grid still has an SM to itself (the 16-bit kernel's
-// registers fill one) and keeps 64 rows (at 32 or 128 the times of 64 to 4096 rows a head are the same or worse).
-int decode_cluster(long long units, int max_count, int sms) {
+// CTAs of a decode cluster: doubled while the doubled grid still has `slots` places (CTAs at a time) and every CTA keeps
+// `rows` rows.
+int decode_cluster(long long units, int max_count, long long slots, int rows) {
   int cluster = 1;
-  while (cluster < kDecMaxCluster && units * cluster * 2 <= sms && max_count >= 2 * cluster * kDecMinRows) cluster *= 2;
+  while (cluster < kDecMaxCluster && units * cluster * 2 <= slots && max_count >= 2 * cluster * rows) cluster *= 2;
   return cluster;
 }
 
 // ---------------------------------------------------------------- decode attention
-// gt: query heads per CTA of the kernel.
-int launch_decode(void (*kernel)(DecodeParams), int gt, DecodeParams& dp, int batch, int max_count, cudaStream_t st) {
-  const int sms = device_sm_count();
-  if (sms <= 0) return PKV_ERR_CUDA;
-  dp.head_blocks = (dp.group + gt - 1) / gt;
-  const long long units = static_cast<long long>(dp.num_kv_heads) * dp.head_blocks * batch;
-  const int cluster = decode_cluster(units, max_count, sms);
+int launch_decode(void (*kernel)(DecodeParams), const DecodeParams& dp, int batch, int cluster, int threads, int smem, cudaStream_t st) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(cluster * dp.num_kv_heads * dp.head_blocks, batch);
-  cfg.blockDim = dim3(kDecThreads);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -935,17 +930,45 @@ int launch_decode(void (*kernel)(DecodeParams), int gt, DecodeParams& dp, int ba
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  void* args[1] = {&dp};
+  void* args[1] = {const_cast<DecodeParams*>(&dp)};
   if (cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kernel), args) != cudaSuccess) return PKV_ERR_CUDA;
   return check_launch();
 }
 
 template <int D, bool PAGED>
-int launch_decode_fp32(DecodeParams& dp, int batch, int max_count, cudaStream_t st) {
-  if (dp.group == 1) return launch_decode(decode_attention_kernel<D, 1, PAGED>, 1, dp, batch, max_count, st);
-  if (dp.group == 2) return launch_decode(decode_attention_kernel<D, 2, PAGED>, 2, dp, batch, max_count, st);
-  if (dp.group <= 4) return launch_decode(decode_attention_kernel<D, 4, PAGED>, 4, dp, batch, max_count, st);
-  return launch_decode(decode_attention_kernel<D, 8, PAGED>, 8, dp, batch, max_count, st);
+int launch_decode_fp32(DecodeParams& dp, int batch, int max_count, int sms, cudaStream_t st) {
+  const int gt = dp.group >= 5 ? 8 : (dp.group >= 3 ? 4 : dp.group);   // query heads per CTA of the kernel
+  dp.head_blocks = (dp.group + gt - 1) / gt;
+  const int cluster = decode_cluster(static_cast<long long>(dp.num_kv_heads) * dp.head_blocks * batch, max_count, sms, kDecMinRows);
+  if (gt == 1) return launch_decode(decode_attention_kernel<D, 1, PAGED>, dp, batch, cluster, kDecThreads, 0, st);
+  if (gt == 2) return launch_decode(decode_attention_kernel<D, 2, PAGED>, dp, batch, cluster, kDecThreads, 0, st);
+  if (gt == 4) return launch_decode(decode_attention_kernel<D, 4, PAGED>, dp, batch, cluster, kDecThreads, 0, st);
+  return launch_decode(decode_attention_kernel<D, 8, PAGED>, dp, batch, cluster, kDecThreads, 0, st);
+}
+
+// 16-bit rows.  Eight warps to a CTA where clusters of eight such CTAs (the largest) leave SMs free: few lists, as many warps on
+// each as can be.  Else four, two CTAs to an SM: the next call's CTAs then start, and bring their rows into the L2, as
+// soon as there is half an SM for them (32 layers, 8 sequences x 8 KV heads, 347 to 937 rows a head in pages of 16: 247 us;
+// 291 with grids of one such CTA per SM, 303 with eight warps and rows in registers, one CTA per SM).
+template <typename T, int D, bool PAGED>
+int launch_decode_16bit(DecodeParams& dp, int batch, int max_count, int sms, cudaStream_t st) {
+  constexpr int kSmem8 = 8 * kDecStages * 64 * D, kSmem4 = 4 * kDecStages * 64 * D;
+  static bool attr_done[64] = {};  // the attribute is per device; setting it twice is harmless
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return PKV_ERR_CUDA;
+  if (dev >= 64 || !attr_done[dev]) {
+    if (cudaFuncSetAttribute(decode_mma_kernel<T, D, PAGED, 8, kDecStages>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem8) != cudaSuccess ||
+        cudaFuncSetAttribute(decode_mma_kernel<T, D, PAGED, 4, kDecStages>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem4) != cudaSuccess)
+      return PKV_ERR_CUDA;
+    if (dev < 64) attr_done[dev] = true;
+  }
+  dp.head_blocks = (dp.group + kDecMmaHeads - 1) / kDecMmaHeads;
+  const long long units = static_cast<long long>(dp.num_kv_heads) * dp.head_blocks * batch;
+  if (units * kDecMaxCluster <= sms)
+    return launch_decode(decode_mma_kernel<T, D, PAGED, 8, kDecStages>, dp, batch, decode_cluster(units, max_count, sms, kDecMinRows), 8 * 32,
+                         kSmem8, st);
+  return launch_decode(decode_mma_kernel<T, D, PAGED, 4, kDecStages>, dp, batch, decode_cluster(units, max_count, 2ll * sms, kDecMinRows),
+                       4 * 32, kSmem4, st);
 }
 
 template <bool PAGED>
@@ -955,16 +978,18 @@ int run_decode(const pkv_config* c, DecodeParams& dp, int batch, cudaStream_t st
   dp.scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(c->head_dim)));
   int max_count = 0;
   for (int b = 0; b < batch; ++b) max_count = std::max(max_count, dp.seq.count[b]);
+  const int sms = device_sm_count();
+  if (sms <= 0) return PKV_ERR_CUDA;
   const bool wide = c->head_dim == 128;
   switch (c->dtype) {
     case PKV_DTYPE_FP32:
-      return wide ? launch_decode_fp32<128, PAGED>(dp, batch, max_count, st) : launch_decode_fp32<64, PAGED>(dp, batch, max_count, st);
+      return wide ? launch_decode_fp32<128, PAGED>(dp, batch, max_count, sms, st) : launch_decode_fp32<64, PAGED>(dp, batch, max_count, sms, st);
     case PKV_DTYPE_FP16:
-      return launch_decode(wide ? decode_mma_kernel<__half, 128, PAGED> : decode_mma_kernel<__half, 64, PAGED>, kDecMmaHeads, dp, batch,
-                           max_count, st);
+      return wide ? launch_decode_16bit<__half, 128, PAGED>(dp, batch, max_count, sms, st)
+                  : launch_decode_16bit<__half, 64, PAGED>(dp, batch, max_count, sms, st);
     default:
-      return launch_decode(wide ? decode_mma_kernel<__nv_bfloat16, 128, PAGED> : decode_mma_kernel<__nv_bfloat16, 64, PAGED>, kDecMmaHeads,
-                           dp, batch, max_count, st);
+      return wide ? launch_decode_16bit<__nv_bfloat16, 128, PAGED>(dp, batch, max_count, sms, st)
+                  : launch_decode_16bit<__nv_bfloat16, 64, PAGED>(dp, batch, max_count, sms, st);
   }
 }
 

@@ -11,11 +11,14 @@
 //   * 16-bit rows go through mma.sync (decode_mma_kernel): M = query heads, fp32 accumulation.  The softmax weights stay
 //     fp32 in effect: each is split into three 16-bit parts (hi + mid + lo carry 24 bits and more), which stand in
 //     different rows of the same M = 16 operand (4 heads x 3 parts), so that the split costs no extra products.
+//     Rows come by asynchronous copies into a ring in shared memory, three tiles of 16 rows per warp: a tile in registers
+//     at a time left the warp waiting some 1.1 us for every tile, and took the registers that a second CTA on the SM needs.
 //   * fp32 rows stay on the fp32 pipe (decode_attention_kernel).
 // Measured on one B200, one token through 32 layers, 8 KV heads x 4 query heads, d = 128, bf16: 2048 rows a head on
 // average, one sequence (269 MB): 8.8 ms with one CTA per query head (32 CTAs, each K and V row read four times), 365 us
-// with clusters on the fp32 pipe, 256 us on mma.sync; 512 rows, eight sequences, pages of 16 rows (543 MB): 3.3 ms, 397,
-// 330 us.  (Loads of the next tile under this one's products: 272 / 345 us, the copies cost more than they hide.)
+// with clusters on the fp32 pipe, 258 on mma.sync with rows in registers, 197 with the ring; 512 rows, eight sequences, pages
+// of 16 rows (543 MB): 3.3 ms, 397, 319, 247 us.  A call of few rows takes 5 us from one wait for the kernels ahead to the
+// next: rows out of the L2 1.2, products and merges of the warps 0.7, the cluster's exchange 1.2, end of the grid 1.7.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -28,6 +31,7 @@ namespace pkv {
 constexpr int kDecThreads = 256;
 constexpr int kDecWarps = kDecThreads / 32;
 constexpr int kDecMaxCluster = 8;         // 16 CTAs need a GPC to themselves: their launches cannot overlap (+4.5 us each)
+constexpr int kDecStages = 3;             // tiles of a warp in shared memory or on their way
 constexpr int kDecPrefetchRows = 512;     // rows a CTA brings into the L2 while it waits
 constexpr int kDecMinRows = 64;            // rows a CTA should have before a cluster grows: one step of its teams
 
@@ -58,53 +62,68 @@ struct Dec8 {
 };
 
 // Shared memory in which the warps of a CTA, then the CTAs of a cluster meet.
-template <int D, int GT>
+template <int D, int GT, int WARPS>
 struct DecMerge {
-  float acc[kDecWarps][GT * D];
-  float m[kDecWarps][GT], z[kDecWarps][GT];
-  float in[kDecMaxCluster * ((GT * D + kDecMaxCluster - 1) / kDecMaxCluster)];   // this CTA's channels, from every CTA
+  static constexpr int kHead = D + 4;            // floats from a head's sums to the next one's: other banks
+  float acc[WARPS][GT * kHead];
+  float m[WARPS][GT], z[WARPS][GT];
+  float in[GT * D];                                                              // this CTA's channels, from every CTA
   float2 mz[kDecMaxCluster][GT];                                                 // every CTA's (maximum, sum) per head
 };
 
 // Sums of the warps (in shared memory behind a barrier) -> output.  hq0: first query head of the block.  The cluster's
-// barrier has been arrived at once at the start of the kernel.
-template <int D, int GT>
-__device__ __forceinline__ void dec_finish(DecMerge<D, GT>& s, const DecodeParams& p, int C, int rank, int64_t hq0, int heads) {
+// barrier has been arrived at once at the start of the kernel.  C is a power of two, so every CTA finishes GT * D / C channels.
+template <int D, int GT, int WARPS>
+__device__ __forceinline__ void dec_finish(DecMerge<D, GT, WARPS>& s, const DecodeParams& p, int C, int rank, int64_t hq0, int heads) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   if (C > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");        // every CTA of the cluster has started
-  const int share = (GT * D + C - 1) / C;        // channels each CTA finishes
-  for (int o = threadIdx.x; o < GT * D; o += kDecThreads) {
+  const int share = GT * D / C;                  // channels each CTA finishes
+  for (int o = threadIdx.x * 2; o < GT * D; o += WARPS * 64) {                   // two channels of a head
     const int g = o / D;
     float mm = -INFINITY;
 #pragma unroll
-    for (int w = 0; w < kDecWarps; ++w) mm = fmaxf(mm, s.m[w][g]);
-    float zz = 0.f, a = 0.f;
+    for (int w = 0; w < WARPS; ++w) mm = fmaxf(mm, s.m[w][g]);
+    float zz = 0.f;
+    float2 a = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int w = 0; w < kDecWarps; ++w) {
-      const float f = s.m[w][g] == -INFINITY ? 0.f : exp2f(s.m[w][g] - mm);      // 0: the warp saw no row
+    for (int w = 0; w < WARPS; ++w) {
+      const float f = s.m[w][g] == -INFINITY ? 0.f : ex2(s.m[w][g] - mm);        // 0: the warp saw no row
+      const float2 v = *reinterpret_cast<const float2*>(&s.acc[w][g * DecMerge<D, GT, WARPS>::kHead + o % D]);
       zz += s.z[w][g] * f;
-      a += s.acc[w][o] * f;
+      a.x += v.x * f;
+      a.y += v.y * f;
     }
     if (C == 1) {
-      if (g < heads) p.out[hq0 * D + o] = a / zz;
+      if (g < heads) {                           // (the output is as aligned as a float)
+        p.out[hq0 * D + o] = a.x / zz;
+        p.out[hq0 * D + o + 1] = a.y / zz;
+      }
     } else {
       const int to = o / share;
-      cluster.map_shared_rank(s.in, to)[rank * share + o - to * share] = a;
+      *reinterpret_cast<float2*>(cluster.map_shared_rank(s.in, to) + rank * share + o - to * share) = a;
       if (o == to * share || o % D == 0) cluster.map_shared_rank(&s.mz[0][0], to)[rank * GT + g] = make_float2(mm, zz);
     }
   }
   if (C == 1) return;
   cluster.sync();
-  for (int i = threadIdx.x; i < share; i += kDecThreads) {
+  for (int i = threadIdx.x; i < share; i += WARPS * 32) {
     const int o = rank * share + i, g = o / D;
-    if (o >= GT * D || g >= heads) continue;
+    if (g >= heads) continue;
+    float2 mz[kDecMaxCluster];
+    float in[kDecMaxCluster];
     float mm = -INFINITY, zz = 0.f, a = 0.f;
-    for (int c = 0; c < C; ++c) mm = fmaxf(mm, s.mz[c][g].x);
-    for (int c = 0; c < C; ++c) {
-      const float f = s.mz[c][g].x == -INFINITY ? 0.f : exp2f(s.mz[c][g].x - mm);
-      zz += s.mz[c][g].y * f;
-      a += s.in[c * share + i] * f;
+#pragma unroll
+    for (int c = 0; c < kDecMaxCluster; ++c) {
+      mz[c] = c < C ? s.mz[c][g] : make_float2(-INFINITY, 0.f);
+      in[c] = c < C ? s.in[c * share + i] : 0.f;
+      mm = fmaxf(mm, mz[c].x);
+    }
+#pragma unroll
+    for (int c = 0; c < kDecMaxCluster; ++c) {
+      const float f = mz[c].x == -INFINITY ? 0.f : ex2(mz[c].x - mm);
+      zz += mz[c].y * f;
+      a += in[c] * f;
     }
     p.out[hq0 * D + o] = a / zz;
   }
@@ -127,7 +146,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_attention_kernel(const Dec
   static_assert(PER <= U, "a lane's values belong to one head");
   using T = float;
   namespace cg = cooperative_groups;
-  __shared__ DecMerge<D, GT> s_mrg;
+  __shared__ DecMerge<D, GT, kDecWarps> s_mrg;
   pdl_trigger();
   cg::cluster_group cluster = cg::this_cluster();
   const int C = cluster.dim_blocks().x, rank = cluster.block_rank();
@@ -282,7 +301,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_attention_kernel(const Dec
         x += __shfl_xor_sync(0xffffffffu, x, s);
         y += __shfl_xor_sync(0xffffffffu, y, s);
       }
-      if (lane < L) *reinterpret_cast<float2*>(&s_mrg.acc[warp][g * D + sub * 8 + 2 * c]) = make_float2(x, y);
+      if (lane < L) *reinterpret_cast<float2*>(&s_mrg.acc[warp][g * (D + 4) + sub * 8 + 2 * c]) = make_float2(x, y);
     }
   }
   if (lane < L && sub % (L / GT) == 0) {         // one lane per head
@@ -290,7 +309,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_attention_kernel(const Dec
     s_mrg.z[warp][my_head] = z;
   }
   __syncthreads();
-  dec_finish<D, GT>(s_mrg, p, C, rank, hq0, p.group - g0);
+  dec_finish<D, GT, kDecWarps>(s_mrg, p, C, rank, hq0, p.group - g0);
 }
 
 // ------------------------------------------------------------------ 16-bit rows
@@ -333,7 +352,7 @@ struct Dec16<__half> {
 // matrix product every part of a weight meets every value, and a part that is zero or negative makes NaN of an infinity;
 // one weight, one product gives what the sum says (an infinity of the value's sign, NaN where both signs or NaN are
 // summed).  ref: the exponent that the warp's weights are relative to.
-template <typename T, int D, bool PAGED>
+template <typename T, int D, bool PAGED, int WARPS>
 __device__ __forceinline__ void dec_sum_special(const DecodeParams& p, int b, int h, const T* q, int64_t row0, int first, int hi,
                                                 float ref, float* acc) {
   constexpr int PER = D / 32;
@@ -345,7 +364,7 @@ __device__ __forceinline__ void dec_sum_special(const DecodeParams& p, int b, in
     a[c] = 0.f;
   }
 #pragma unroll 1
-  for (int t0 = first; t0 < hi; t0 += kDecWarps * 16)
+  for (int t0 = first; t0 < hi; t0 += WARPS * 16)
 #pragma unroll 1
     for (int r = t0; r < min(t0 + 16, hi); ++r) {
       const int64_t at = PAGED ? paged_row(p.pt, b, h, r) : row0 + r;
@@ -365,8 +384,19 @@ __device__ __forceinline__ void dec_sum_special(const DecodeParams& p, int b, in
   for (int c = 0; c < PER; ++c) acc[lane * PER + c] = a[c];
 }
 
-// grid, cluster and block as above, kDecMmaHeads query heads per CTA.  A warp takes tiles of 16 rows.  With g = lane / 4 and
-// c = lane % 4 the fragments of m16n8k16 are
+// Bytes from global to shared memory past the registers, zeros where `there` is false.
+__device__ __forceinline__ void dec_copy16(uint32_t to, const void* from, bool there) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(from), "r"(there ? 16u : 0u) : "memory");
+}
+__device__ __forceinline__ uint4 dec_lds16(uint32_t at) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
+  return v;
+}
+
+// grid, cluster as above, WARPS warps, kDecMmaHeads query heads per CTA.  A warp takes tiles of 16 rows, STAGES of them in
+// shared memory or on their way there (dynamic, WARPS * STAGES * 64 * D bytes).  With g = lane / 4 and c = lane % 4 the
+// fragments of m16n8k16 are
 //   S  = Q K^T   A: row i = head i % 4 (every head four times), B: n = row g of 8, channels dealt so that a lane's B words are
 //                its own 16-byte pieces of K (the order of the contraction is free as long as Q has the same one);
 //                result: head g % 4, rows 2c, 2c + 1
@@ -374,12 +404,17 @@ __device__ __forceinline__ void dec_sum_special(const DecodeParams& p, int b, in
 //                lanes and positions where S came out; B: rows 2c, 2c + 1 (+ 8, 9) of channel 64 j + 8 g + i, from 16-byte
 //                pieces of V with the halves of two rows interleaved.
 // A lane holds sums of one head only, so rescaling needs no exchange; O is the sum over the three parts.
-template <typename T, int D, bool PAGED>
-__global__ void __launch_bounds__(kDecThreads, 1) decode_mma_kernel(const DecodeParams p) {
-  constexpr int GT = kDecMmaHeads, KC = D / 32, VC = D / 64;
+// In shared memory the 16-byte pieces of a row are exchanged (K: by the row's lowest bit, V: by the next two), so that eight
+// lanes that read together touch every bank once.
+template <typename T, int D, bool PAGED, int WARPS, int STAGES>
+__global__ void __launch_bounds__(WARPS * 32, WARPS == 8 ? 1 : 2) decode_mma_kernel(const DecodeParams p) {
+  constexpr int GT = kDecMmaHeads, KC = D / 32, VC = D / 64, THREADS = WARPS * 32;
+  constexpr int PIECES = D / 8, ROWS_AT_ONCE = 32 / PIECES;    // 16-byte pieces of a row; rows that a warp copies per step
+  constexpr uint32_t ROW = D * 2, TILE = 16 * ROW;
   using X = Dec16<T>;
   namespace cg = cooperative_groups;
-  __shared__ DecMerge<D, GT> s_mrg;
+  extern __shared__ __align__(128) uint8_t dec_smem[];
+  __shared__ __align__(16) DecMerge<D, GT, WARPS> s_mrg;
   pdl_trigger();
   cg::cluster_group cluster = cg::this_cluster();
   const int C = cluster.dim_blocks().x, rank = cluster.block_rank();
@@ -394,9 +429,11 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_mma_kernel(const Decode
   const int64_t hq0 = static_cast<int64_t>(b) * p.num_kv_heads * p.group + static_cast<int64_t>(h) * p.group + g0;
   const T* kc = static_cast<const T*>(p.k_cache);
   const T* vc = static_cast<const T*>(p.v_cache);
+  const T* q_head = static_cast<const T*>(p.q) + (hq0 + min(g % GT, p.group - g0 - 1)) * D;
   // While the kernels ahead in the stream finish, this CTA's rows come into the L2 (a prefetch hands no data to anybody, so
   // it does not matter whether they are still being written; a page table read here is only used for it).
-  for (int i = threadIdx.x; i < min(hi - lo, kDecPrefetchRows) * 2; i += kDecThreads) {     // K and V rows in turn
+  if (warp == 0 && c < KC / 2) asm volatile("prefetch.global.L2 [%0];" ::"l"(q_head + c * 64));
+  for (int i = threadIdx.x; i < min(hi - lo, kDecPrefetchRows) * 2; i += THREADS) {         // K and V rows in turn
     int64_t at = row0 + lo + i / 2;
     if (PAGED) {
       const int r = lo + i / 2;
@@ -410,121 +447,151 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_mma_kernel(const Decode
   }
   pdl_wait();
 
+  // Rows of a tile: lane l (and l + 16) looks up where row l lies (-1: not there).
+  auto look_up = [&](int t0) -> int64_t {
+    const int r = t0 + (lane & 15);
+    if (r >= hi) return -1;
+    if (!PAGED) return row0 + r;
+    const int64_t at = paged_row(p.pt, b, h, r);
+    if (at < 0 && lane < 16) atomicOr(p.status, kStatusBadPage);
+    return at;
+  };
+  const uint32_t ring = static_cast<uint32_t>(__cvta_generic_to_shared(dec_smem)) + warp * (STAGES * 2 * TILE);
+  // One group of copies per tile, empty behind the last one.
+  auto copy_tile = [&](int t0, int slot, int64_t mine) {
+    if (t0 < hi) {
+#pragma unroll
+      for (int s = 0; s < 16 / ROWS_AT_ONCE; ++s) {
+        const int r = s * ROWS_AT_ONCE + lane / PIECES, piece = lane % PIECES;
+        const int64_t at = __shfl_sync(0xffffffffu, mine, r);
+        const int64_t from = (at >= 0 ? at : 0) * D + piece * 8;
+        const uint32_t to = ring + slot * (2 * TILE) + r * ROW;
+        dec_copy16(to + ((piece ^ ((r & 1) << 2)) << 4), kc + from, at >= 0);
+        dec_copy16(to + TILE + ((piece ^ (((r >> 1) & 3) << 1)) << 4), vc + from, at >= 0);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const int first = lo + warp * 16;
+  constexpr int STEP = WARPS * 16;
+  uint32_t there[STAGES];                        // rows of the tiles in the ring
+  {
+    int64_t mine[STAGES];
+#pragma unroll
+    for (int s = 0; s < STAGES; ++s) mine[s] = look_up(first + s * STEP);
+#pragma unroll
+    for (int s = 0; s < STAGES; ++s) {
+      copy_tile(first + s * STEP, s, mine[s]);
+      there[s] = __ballot_sync(0xffffffffu, mine[s] >= 0);
+    }
+  }
+  int64_t mine = look_up(first + STAGES * STEP);                // of the tile that is copied next
   uint4 q[KC];
 #pragma unroll
   for (int j = 0; j < KC; ++j)
-    q[j] = g0 + g % GT < p.group ? *reinterpret_cast<const uint4*>(static_cast<const T*>(p.q) + (hq0 + g % GT) * D + j * 32 + c * 8)
-                                 : make_uint4(0, 0, 0, 0);
+    q[j] = g0 + g % GT < p.group ? *reinterpret_cast<const uint4*>(q_head + j * 32 + c * 8) : make_uint4(0, 0, 0, 0);
   float o[VC * 8][4];
 #pragma unroll
   for (int i = 0; i < VC * 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
   float m = -INFINITY, z = 0.f;                  // of head g % 4: m over the warp's rows, z over this lane's
-  for (int t0 = lo + warp * 16; t0 < hi; t0 += kDecWarps * 16) {
-    // rows of the tile: where they lie (-1: not there)
-    auto place = [&](int r) -> int64_t {
-      if (t0 + r >= hi) return -1;
-      return PAGED ? -1 : row0 + t0 + r;
-    };
-    int64_t mine = -1;
-    if (PAGED) {
-      const int r = t0 + (lane & 15);
-      if (r < hi) {
-        mine = paged_row(p.pt, b, h, r);
-        if (mine < 0 && lane < 16) atomicOr(p.status, kStatusBadPage);
+  for (int t0 = first; t0 < hi;) {
+#pragma unroll
+    for (int slot = 0; slot < STAGES; ++slot) {
+      if (t0 >= hi) break;                       // (uniform over the warp)
+      asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 1) : "memory");
+      __syncwarp();
+      const uint32_t k_at = ring + slot * (2 * TILE), v_at = k_at + TILE;
+      float x[2][2];
+      float mx = -INFINITY;
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int j = 0; j < KC; ++j) {
+          const uint4 k = dec_lds16(k_at + (t * 8 + g) * ROW + (((j * 4 + c) ^ ((g & 1) << 2)) << 4));
+          X::mma(s0, q[j].x, q[j].x, q[j].y, q[j].y, k.x, k.y);
+          X::mma(s1, q[j].z, q[j].z, q[j].w, q[j].w, k.z, k.w);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          x[t][i] = (there[slot] >> (t * 8 + 2 * c + i)) & 1u ? (s0[i] + s1[i]) * p.scale_log2 : -INFINITY;
+          mx = fmaxf(mx, x[t][i]);
+        }
       }
-    }
-    auto row_at = [&](int r) -> int64_t { return PAGED ? __shfl_sync(0xffffffffu, mine, r) : place(r); };
-    uint4 k[2][KC], v[4][VC];
-    bool seen[2][2];
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+      const float mn = fmaxf(m, mx);
+      const float ref = mn == -INFINITY ? 0.f : mn - X::kShift;
+      if (__any_sync(0xffffffffu, mn > m)) {
+        const float corr = m == -INFINITY ? 0.f : ex2(m - mn);
+        z *= corr;
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const int64_t at = row_at(t * 8 + g);
+        for (int i = 0; i < VC * 8; ++i)
 #pragma unroll
-      for (int j = 0; j < KC; ++j)
-        k[t][j] = at >= 0 ? *reinterpret_cast<const uint4*>(kc + at * D + j * 32 + c * 8) : make_uint4(0, 0, 0, 0);
-    }
+          for (int e = 0; e < 4; ++e) o[i][e] *= corr;
+      }
+      m = mn;
+      uint32_t a[2][2];                          // [rows 2c.. / 2c + 8..][fragment row g / g + 8]
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int64_t at = row_at((t >> 1) * 8 + 2 * c + (t & 1));
-      seen[t >> 1][t & 1] = at >= 0;
-#pragma unroll
-      for (int j = 0; j < VC; ++j)
-        v[t][j] = at >= 0 ? *reinterpret_cast<const uint4*>(vc + at * D + j * 64 + g * 8) : make_uint4(0, 0, 0, 0);
-    }
-    float x[2][2];
-    float mx = -INFINITY;
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int j = 0; j < KC; ++j) {
-        X::mma(s0, q[j].x, q[j].x, q[j].y, q[j].y, k[t][j].x, k[t][j].y);
-        X::mma(s1, q[j].z, q[j].z, q[j].w, q[j].w, k[t][j].z, k[t][j].w);
+      for (int t = 0; t < 2; ++t) {
+        const float w0 = ex2(x[t][0] - ref), w1 = ex2(x[t][1] - ref);
+        z += w0 + w1;
+        const uint32_t high = X::pack(w0, w1);
+        const float2 hf = X::unpack(high);
+        const uint32_t mid = X::pack(w0 - hf.x, w1 - hf.y);
+        const float2 mf = X::unpack(mid);
+        const uint32_t low = X::pack(w0 - hf.x - mf.x, w1 - hf.y - mf.y);
+        a[t][0] = g < 4 ? high : mid;
+        a[t][1] = g < 4 ? low : 0u;
       }
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        x[t][i] = seen[t][i] ? (s0[i] + s1[i]) * p.scale_log2 : -INFINITY;
-        mx = fmaxf(mx, x[t][i]);
+      for (int j = 0; j < VC; ++j) {
+        uint4 v[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t)              // row (t / 2) * 8 + 2c + t % 2
+          v[t] = dec_lds16(v_at + ((t >> 1) * 8 + 2 * c + (t & 1)) * ROW + (((j * 8 + g) ^ (c << 1)) << 4));
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          const uint32_t v0 = reinterpret_cast<const uint32_t*>(&v[0])[w], v1 = reinterpret_cast<const uint32_t*>(&v[1])[w];
+          const uint32_t v2 = reinterpret_cast<const uint32_t*>(&v[2])[w], v3 = reinterpret_cast<const uint32_t*>(&v[3])[w];
+          X::mma(o[j * 8 + 2 * w], a[0][0], a[0][1], a[1][0], a[1][1], __byte_perm(v0, v1, 0x5410), __byte_perm(v2, v3, 0x5410));
+          X::mma(o[j * 8 + 2 * w + 1], a[0][0], a[0][1], a[1][0], a[1][1], __byte_perm(v0, v1, 0x7632), __byte_perm(v2, v3, 0x7632));
+        }
       }
-    }
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    const float mn = fmaxf(m, mx);
-    const float ref = mn == -INFINITY ? 0.f : mn - X::kShift;
-    if (__any_sync(0xffffffffu, mn > m)) {
-      const float corr = m == -INFINITY ? 0.f : ex2(m - mn);
-      z *= corr;
-#pragma unroll
-      for (int i = 0; i < VC * 8; ++i)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) o[i][e] *= corr;
-    }
-    m = mn;
-    uint32_t a[2][2];                            // [rows 2c.. / 2c + 8..][fragment row g / g + 8]
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const float w0 = ex2(x[t][0] - ref), w1 = ex2(x[t][1] - ref);
-      z += w0 + w1;
-      const uint32_t high = X::pack(w0, w1);
-      const float2 hf = X::unpack(high);
-      const uint32_t mid = X::pack(w0 - hf.x, w1 - hf.y);
-      const float2 mf = X::unpack(mid);
-      const uint32_t low = X::pack(w0 - hf.x - mf.x, w1 - hf.y - mf.y);
-      a[t][0] = g < 4 ? high : mid;
-      a[t][1] = g < 4 ? low : 0u;
-    }
-#pragma unroll
-    for (int j = 0; j < VC; ++j) {
-#pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        const uint32_t v0 = reinterpret_cast<const uint32_t*>(&v[0][j])[w], v1 = reinterpret_cast<const uint32_t*>(&v[1][j])[w];
-        const uint32_t v2 = reinterpret_cast<const uint32_t*>(&v[2][j])[w], v3 = reinterpret_cast<const uint32_t*>(&v[3][j])[w];
-        X::mma(o[j * 8 + 2 * w], a[0][0], a[0][1], a[1][0], a[1][1], __byte_perm(v0, v1, 0x5410), __byte_perm(v2, v3, 0x5410));
-        X::mma(o[j * 8 + 2 * w + 1], a[0][0], a[0][1], a[1][0], a[1][1], __byte_perm(v0, v1, 0x7632), __byte_perm(v2, v3, 0x7632));
-      }
+      __syncwarp();                              // the tile has been read
+      copy_tile(t0 + STAGES * STEP, slot, mine);
+      there[slot] = __ballot_sync(0xffffffffu, mine >= 0);
+      t0 += STEP;
+      mine = look_up(t0 + STAGES * STEP);
     }
   }
   // ---- the parts, then the warps, then the CTAs of the cluster
   z += __shfl_xor_sync(0xffffffffu, z, 1);
   z += __shfl_xor_sync(0xffffffffu, z, 2);
   float special[4] = {0.f, 0.f, 0.f, 0.f};       // NaN once a sum is not finite
+  // Lanes g and g + 4 hold parts of the same sums: each keeps one of the two channel octets 64 j + 8 (2c + e) + 0 .. 7 of head
+  // g % 4, the lower one e = 0.  (Sixteen-byte stores; scalar ones met in two banks, eight lanes each, 0.7 us.)
+  const bool upper = g >= 4;
 #pragma unroll
-  for (int i = 0; i < VC * 8; ++i) {             // channels 64 j + 8 (2c + e) + i % 8 of head g % 4
+  for (int j = 0; j < VC; ++j) {
+    float s[8];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      float s = o[i][e] + o[i][2 + e];
-      s += __shfl_xor_sync(0xffffffffu, s, 16);
-      special[i & 3] = fmaf(s, 0.f, special[i & 3]);
-      if (g < 4) s_mrg.acc[warp][g * D + (i >> 3) * 64 + (2 * c + e) * 8 + (i & 7)] = s;
+    for (int i = 0; i < 8; ++i) {
+      const float s0 = o[j * 8 + i][0] + o[j * 8 + i][2], s1 = o[j * 8 + i][1] + o[j * 8 + i][3];
+      s[i] = (upper ? s1 : s0) + __shfl_xor_sync(0xffffffffu, upper ? s0 : s1, 16);
+      special[i & 3] = fmaf(s[i], 0.f, special[i & 3]);
     }
+    float4* to = reinterpret_cast<float4*>(&s_mrg.acc[warp][(g & 3) * (D + 4) + j * 64 + (2 * c + (upper ? 1 : 0)) * 8]);
+    to[0] = make_float4(s[0], s[1], s[2], s[3]);
+    to[1] = make_float4(s[4], s[5], s[6], s[7]);
   }
   if (__any_sync(0xffffffffu, (special[0] + special[1]) + (special[2] + special[3]) != 0.f)) {
     __syncwarp();
 #pragma unroll 1
     for (int j = 0; j < min(GT, p.group - g0); ++j) {
       const float mj = __shfl_sync(0xffffffffu, m, j * 4);
-      dec_sum_special<T, D, PAGED>(p, b, h, static_cast<const T*>(p.q) + (hq0 + j) * D, row0, lo + warp * 16, hi,
-                                   mj == -INFINITY ? 0.f : mj - X::kShift, &s_mrg.acc[warp][j * D]);
+      dec_sum_special<T, D, PAGED, WARPS>(p, b, h, static_cast<const T*>(p.q) + (hq0 + j) * D, row0, lo + warp * 16, hi,
+                                   mj == -INFINITY ? 0.f : mj - X::kShift, &s_mrg.acc[warp][j * (D + 4)]);
     }
   }
   if (g < 4 && c == 0) {
@@ -532,7 +599,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_mma_kernel(const Decode
     s_mrg.z[warp][g] = z;
   }
   __syncthreads();
-  dec_finish<D, GT>(s_mrg, p, C, rank, hq0, p.group - g0);
+  dec_finish<D, GT, WARPS>(s_mrg, p, C, rank, hq0, p.group - g0);
 }
 
 }  // namespace pkv
