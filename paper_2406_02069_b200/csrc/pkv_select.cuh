@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) pool_select_kernel(const Selec
 //     lets through about k positions.  Short lists take a bound per CTA (about k candidates each); for long ones the
 //     CTAs' histograms are added up first, one cluster barrier more, and about k candidates are left in all;
 //   * every CTA of the cluster finishes on its own: it is sent the candidates of all (distributed shared memory), finds
-//     the threshold, and emits and copies the rows of its own slice, which it has brought into the L2 by then.  There is one full cluster barrier (up to three
+//     the threshold, and emits and copies the rows of its own slice.  There is one full cluster barrier (up to three
 //     when the list is long) and no trip through global memory;
 //   * the exact threshold is searched inside [largest bound of the CTAs, largest key], ten bits a pass, and finished by
 //     a warp as soon as at most 32 candidates are left in the bin (mostly after the first pass).
@@ -479,6 +479,7 @@ constexpr int kSelClusterSlice = 8192;     // a cluster doubles (up to 8 CTAs) w
 constexpr int kSelCopyBytes = 128 << 10;   // ... or while a CTA would copy more than this and SMs are idle
 constexpr int kSelCommonCandidates = 4096; // more expected candidates (k per CTA) than this: one bound for the cluster
 constexpr int kSelCrowd = 1024;            // candidates of a CTA beyond 2 k that its bound may let through before it is refined
+constexpr int kSelPrefetchPieces = 32;     // rows of at least this many 16-byte pieces are prefetched once they are known
 constexpr int kSelEvenRows = 1024;         // lists of at least this many rows are copied by the whole cluster evenly
 
 // Position i of the staged scores in shared memory: four floats of padding after every 32.
@@ -676,11 +677,13 @@ template <int THREADS, int RUNS, bool AVG>
 __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kernel(const SelectParams p) {
   constexpr int WARPS = THREADS / 32;
   extern __shared__ __align__(16) uint8_t sel_dyn[];
-  __shared__ uint32_t hist[2][kSelBinsLin];                 // [0]: read by the whole cluster when the bound is a common one
-  __shared__ uint32_t local[2][kSelBinsLin];                // threshold search
+  __shared__ __align__(16) uint32_t hist[2][kSelBinsLin];                 // [0]: read by the whole cluster when the bound is a common one
+  __shared__ __align__(16) uint32_t local[2][kSelBinsLin];  // threshold search
   __shared__ uint32_t rows[32];
   __shared__ uint32_t warp_a[WARPS], warp_b[WARPS], warp_c[WARPS], warp_d[WARPS];
-  __shared__ uint32_t few[32], few_n;
+  __shared__ __align__(16) uint32_t few[32];
+  __shared__ uint32_t few_n;
+  __shared__ uint2 found;                                   // threshold, ties at it that are taken
   __shared__ uint4 pub[kSelMaxCluster];                     // every CTA's number of candidates, bound, largest key
 
   pdl_trigger();
@@ -704,7 +707,11 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
   uint32_t* inbox = list_key + p.max_slice + p.max_slice / 2;                           // [C][p.inbox] everybody's keys
   if (C > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");              // this CTA's inbox may be written
 
-  for (int i = tid; i < 2 * kSelBinsLin; i += THREADS) (&hist[0][0])[i] = 0;
+  for (int i = tid; i < kSelBinsLin / 4; i += THREADS) {    // (hist[1] is written before it is read)
+    reinterpret_cast<uint4*>(hist[0])[i] = make_uint4(0, 0, 0, 0);
+    reinterpret_cast<uint4*>(local[0])[i] = make_uint4(0, 0, 0, 0);
+  }
+  if (tid < 32) few[tid] = 0;
   if (tid == 0) few_n = 0;
   pdl_wait();
 
@@ -844,7 +851,6 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
       }
     }
     mx = __reduce_max_sync(full, warp_a[lane & (WARPS - 1)]);
-    for (int i = tid; i < 2 * kSelBinsLin; i += THREADS) (&local[0][0])[i] = 0;
     __syncthreads();
     if constexpr (THREADS * RUNS > 512) {                   // (up to 4096 candidates of one CTA are ranked in 10 us all the same)
       if (!common) crowded = k < len && M > 2 * k + kSelCrowd;
@@ -885,58 +891,73 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
     };
     const int my_c = warp & (C - 1), my_first = (warp / C) * 32 + lane, my_step = (WARPS / C) * 32;
     const int my_n = static_cast<int>(pub[my_c].x);
+    // Most candidates lie within an octave of the bound and a few far above it: the first pass divides the lowest eighth of
+    // the range, what lies above counts in its last bin.  (Over the whole range a bin held some 50 of 3600 candidates, and
+    // a second pass followed.)
     uint32_t want = static_cast<uint32_t>(k), T = 0, need_eq = 0;
-    int shift = max(0, 22 - __clz(top - base));
+    int shift = max(0, 22 - 3 - __clz(top - base));
     uint32_t span = 0xffffffffu;                            // keys base .. base + span take part
     for (int pass = 0;; ++pass) {
       uint32_t* hc = local[pass & 1];
       for (int i = my_first; i < my_n; i += my_step) {
         const uint32_t x = key_at(my_c, i);
-        if (x >= base && x - base <= span) atomicAdd(&hc[(x - base) >> shift], 1u);
+        if (x >= base && x - base <= span) atomicAdd(&hc[min((x - base) >> shift, kSelBinsLin - 1u)], 1u);
       }
       __syncthreads();
       uint32_t digit = 0, above = 0;
       sel_find_from_top<THREADS>(hc, rows, want, digit, above);
+      const bool beyond = digit == kSelBinsLin - 1u && min(span, top - base) >> shift > digit;      // in what was put together
       want -= above;
       base += digit << shift;
       const uint32_t in_bin = hc[digit];
-      if (pass == 0 && p.k_out != nullptr) {                // all but a few of the rows to copy are known: into the L2
-        const int64_t ks = p.k.st * p.elem_bytes, vs = p.v.st * p.elem_bytes;
-        const char* kb = static_cast<const char*>(p.k.ptr) + (b * p.k.sb + h * p.k.sh + static_cast<int64_t>(lo) * p.k.st) * p.elem_bytes;
-        const char* vb = static_cast<const char*>(p.v.ptr) + (b * p.v.sb + h * p.v.sh + static_cast<int64_t>(lo) * p.v.st) * p.elem_bytes;
-        for (int i = tid; i < M; i += THREADS)
-          if (list_key[i] >= base)
-            for (int c = 0; c < p.pieces * 16; c += 128) {
-              asm volatile("prefetch.global.L2 [%0];" ::"l"(kb + list_pos[i] * ks + c));
-              asm volatile("prefetch.global.L2 [%0];" ::"l"(vb + list_pos[i] * vs + c));
-            }
+      // All but a few of the rows to copy are known.  Short slices' rows of 512 bytes go into the L2 ahead of the copy (8101 fp32
+      // keys, d = 128, 700 rows a head: 58.0 us, 61.2 without).  Not in the other instances, where the prefetches cost more
+      // than they save, the search's own accesses queueing behind them: 4096 keys 28.8 us, 28.1 without; 32768 keys 51.6, 50.9;
+      // three steps of 2 x 10000 keys 32.9, 32.2.
+      if constexpr (THREADS == 256) {
+        if (pass == 0 && p.k_out != nullptr && p.pieces >= kSelPrefetchPieces) {
+          const int64_t ks = p.k.st * p.elem_bytes, vs = p.v.st * p.elem_bytes;
+          const char* kb = static_cast<const char*>(p.k.ptr) + (b * p.k.sb + h * p.k.sh + static_cast<int64_t>(lo) * p.k.st) * p.elem_bytes;
+          const char* vb = static_cast<const char*>(p.v.ptr) + (b * p.v.sb + h * p.v.sh + static_cast<int64_t>(lo) * p.v.st) * p.elem_bytes;
+          for (int i = tid; i < M; i += THREADS)
+            if (list_key[i] >= base)
+              for (int c = 0; c < p.pieces * 16; c += 128) {
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(kb + list_pos[i] * ks + c));
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(vb + list_pos[i] * vs + c));
+              }
+        }
       }
-      if (shift == 0) {
+      if (shift == 0 && !beyond) {
         T = base;
         need_eq = want;
         break;
       }
       if (in_bin <= 32u) {                                  // few enough for a warp: rank them by counting
+        const uint32_t width = beyond ? 0xffffffffu : (1u << shift) - 1u;
         for (int i = my_first; i < my_n; i += my_step) {
           const uint32_t x = key_at(my_c, i);
-          if (x >= base && ((x - base) >> shift) == 0) few[atomicAdd(&few_n, 1u)] = x;
+          if (x >= base && x - base <= width) few[atomicAdd(&few_n, 1u)] = x;
         }
         __syncthreads();
-        const uint32_t x = lane < static_cast<int>(in_bin) ? few[lane] : 0u;
-        uint32_t gt = 0, ge = 0;
-        for (int q = 0; q < static_cast<int>(in_bin); ++q) {
-          const uint32_t o = __shfl_sync(full, x, q);
-          gt += o > x ? 1u : 0u;
-          ge += o >= x ? 1u : 0u;
+        if (warp == 0) {                                    // (all for themselves with shuffles: 0.5 us more at 1024 threads)
+          const uint32_t x = few[lane];                     // (zeros behind the last one)
+          uint32_t gt = 0, ge = 0;
+#pragma unroll
+          for (int q = 0; q < 32; q += 4) {
+            const uint4 o = *reinterpret_cast<const uint4*>(few + q);
+            gt += (o.x > x ? 1u : 0u) + (o.y > x ? 1u : 0u) + (o.z > x ? 1u : 0u) + (o.w > x ? 1u : 0u);
+            ge += (o.x >= x ? 1u : 0u) + (o.y >= x ? 1u : 0u) + (o.z >= x ? 1u : 0u) + (o.w >= x ? 1u : 0u);
+          }
+          const uint32_t hit = __ballot_sync(full, lane < static_cast<int>(in_bin) && gt < want && want <= ge);
+          if (lane == __ffs(hit) - 1) found = make_uint2(x, want - gt);
         }
-        const uint32_t hit = __ballot_sync(full, lane < static_cast<int>(in_bin) && gt < want && want <= ge);
-        const int src = __ffs(hit) - 1;
-        T = __shfl_sync(full, x, src);
-        need_eq = want - __shfl_sync(full, gt, src);
+        __syncthreads();
+        T = found.x;
+        need_eq = found.y;
         break;
       }
-      span = (1u << shift) - 1u;
-      shift = max(0, shift - 10);
+      span = beyond ? 0xffffffffu : (1u << shift) - 1u;
+      shift = beyond ? max(0, 22 - __clz(top - base)) : max(0, shift - 10);
       for (int i = tid; i < kSelBinsLin; i += THREADS) local[(pass + 1) & 1][i] = 0;
       __syncthreads();
     }
