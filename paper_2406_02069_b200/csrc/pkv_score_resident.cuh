@@ -15,7 +15,9 @@
 // K is read once, the contraction runs once, and one launch replaces two.  Taken for R = G * alpha <= 32 window
 // rows per KV head (multi-head attention with the usual windows) and contexts of at most 8 x 2048 keys; everything
 // else goes to the two-sweep kernels.  Warp roles: warp 0 = TMA producer, warp 1 = MMA issuer and TMEM owner,
-// warps 2..5 = epilogue (one per quarter of the TMEM lanes).  Every wait on an mbarrier is bounded as in the
+// warps 2..9 = epilogue (two per quarter of the TMEM lanes, each for half of the window rows: with one for all rows, a layer
+// call at 4096 keys x 32 heads took 28.1 us, 27.0 now; 32 such layers on four streams 324, 314; and a thread's pairs of half the rows
+// fit 96 registers, so that two such CTAs still share an SM).  Every wait on an mbarrier is bounded as in the
 // two-sweep kernels; a CTA that gave up still walks through the two cluster barriers, so its peers are never
 // left waiting, and the status word gets kStatusWaitExpired.
 #pragma once
@@ -26,7 +28,7 @@
 
 namespace pkv {
 
-constexpr int kRsThreads = 192;
+constexpr int kRsThreads = 320;             // producer, MMA issuer, eight epilogue warps
 constexpr int kRsRows = 32;                 // window rows (columns of a tile's accumulator)
 constexpr int kRsTileKeys = 128;
 constexpr int kRsMaxTiles = 512 / kRsRows;  // tiles a CTA keeps in its 512 TMEM columns
@@ -63,7 +65,7 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&v)[32]) {
 // Uses of TcParams: seq (n, prefix, alpha), num_kv_heads, group, rows (<= 32), fp16, early, scale_log2, log2_group,
 // scores, ld_scores, status, wait_clocks.
 template <int D, int STAGES>
-__global__ void __launch_bounds__(kRsThreads, 1)
+__global__ void __launch_bounds__(kRsThreads, STAGES == kRsStagesShort ? 2 : 1)
 score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                       const TcParams p) {
   namespace cg = cooperative_groups;
@@ -77,7 +79,7 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
   uint64_t* bars = reinterpret_cast<uint64_t*>(misc);          // [0..5] k_full, [6..11] k_empty, [12] q_full, [13..28] t_full
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 260);
-  float2* warp_stat = reinterpret_cast<float2*>(misc + 512);   // [4 epilogue warps][32 rows] (maximum, sum)
+  float2* warp_stat = reinterpret_cast<float2*>(misc + 512);   // [8 epilogue warps][16 rows] (maximum, sum)
   float2* cta_stat = reinterpret_cast<float2*>(misc + 1536);   // [32]: read by the other CTAs of the cluster
 
   cg::cluster_group cluster = cg::this_cluster();
@@ -179,9 +181,10 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
     }
   }
 
-  // =========================================================== epilogue (warps 2..5), in step with the cluster
+  // =========================================================== epilogue (warps 2..9), in step with the cluster
   const bool epi = warp >= 2;
   const int quarter = warp & 3;                               // TMEM lanes 32 * quarter .. + 31 are this warp's
+  const int rh = (warp - 2) >> 2;                             // ... and window rows 16 * rh .. + 15
   const int lane_row = quarter * 32 + lane;
   const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
   const float c2 = p.scale_log2;
@@ -199,46 +202,51 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
   //      2^(x - maximum) over the thread's own keys (x = logit in log2 units; a row (g, jj) sees keys 0 .. P + jj)
   float lse2 = 0.f;                                            // of row `lane`, after the cluster barrier
   if (epi) {
-    float m[kRsRows], z[kRsRows];
+    constexpr int kHalf = kRsRows / 2;
+    float m[kHalf], z[kHalf];
 #pragma unroll
-    for (int j = 0; j < kRsRows; ++j) { m[j] = -INFINITY; z[j] = 0.f; }
+    for (int j = 0; j < kHalf; ++j) { m[j] = -INFINITY; z[j] = 0.f; }
     for (int t = 0; t < T && ok; ++t) {
       ok = mbar_wait(t_full(t), 0, abort_flag, p.wait_clocks);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
-      uint32_t v[32];
-      tc_ld32(lane_addr + t * kRsRows, v);
+      uint32_t v[kHalf];
+      tc_ld16(lane_addr + t * kRsRows + rh * kHalf, v);
       tc_wait_ld();
       if (whole(t)) {
 #pragma unroll
-        for (int j = 0; j < kRsRows; ++j) {
+        for (int j = 0; j < kHalf; ++j) {
           const float x = __uint_as_float(v[j]) * c2, mn = fmaxf(m[j], x);
           z[j] = z[j] * ex2(m[j] - mn) + ex2(x - mn);          // m = -inf the first time: 0 * 0 + 1
           m[j] = mn;
         }
       } else {
         const int i = (tile0 + t) * kRsTileKeys + lane_row;
+        int jr = (rh * kHalf) % alpha;                         // window index of the row, counted up (no division per row)
 #pragma unroll
-        for (int j = 0; j < kRsRows; ++j)
-          if (i <= min(P + (j % alpha), n - 1)) {
+        for (int j = 0; j < kHalf; ++j) {
+          if (i <= min(P + jr, n - 1)) {
             const float x = __uint_as_float(v[j]) * c2, mn = fmaxf(m[j], x);
             z[j] = z[j] * ex2(m[j] - mn) + ex2(x - mn);
             m[j] = mn;
           }
+          jr = jr + 1 == alpha ? 0 : jr + 1;
+        }
       }
     }
     // lanes, then the four warps, then (behind the cluster barrier) the CTAs.  Over the lanes by halving: lane bit s picks
-    // the half of the rows a lane keeps, so that after five exchanges lane r holds row r (31 merges per thread; a
-    // butterfly over all rows takes 160 and took 5.4 us of the 28 us that scores and selection of 4096 keys need)
+    // the half of the rows a lane keeps, so that after four exchanges lanes 2r and 2r + 1 hold row r, after a fifth both
+    // of it (a butterfly over all rows takes ten times the merges and took 5.4 us of the 28 us that scores and selection
+    // of 4096 keys needed)
     {
-      int cnt = kRsRows;
+      int cnt = kHalf;
 #pragma unroll
-      for (int s = 16; s >= 1; s >>= 1) {
+      for (int s = 16; s >= 2; s >>= 1) {
         const int half = cnt / 2;
         const bool upper = (lane & s) != 0;
 #pragma unroll
-        for (int j = 0; j < kRsRows / 2; ++j)
+        for (int j = 0; j < kHalf / 2; ++j)
           if (j < half) {
             const float m_send = upper ? m[j] : m[j + half], z_send = upper ? z[j] : z[j + half];
             m[j] = upper ? m[j + half] : m[j];
@@ -247,14 +255,15 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
           }
         cnt = half;
       }
+      merge(m[0], z[0], __shfl_xor_sync(0xffffffffu, m[0], 1), __shfl_xor_sync(0xffffffffu, z[0], 1));
     }
-    const float2 mine = make_float2(m[0], z[0]);
-    warp_stat[(warp - 2) * kRsRows + lane] = mine;
-    asm volatile("bar.sync 1, 128;" ::: "memory");             // the four epilogue warps
+    if (!(lane & 1)) warp_stat[(warp - 2) * kHalf + (lane >> 1)] = make_float2(m[0], z[0]);
+    asm volatile("bar.sync 1, 256;" ::: "memory");             // the eight epilogue warps
     if (warp == 2) {
-      float2 r = warp_stat[lane];
+      const float2* of_row = warp_stat + (lane / kHalf) * 4 * kHalf + lane % kHalf;
+      float2 r = of_row[0];
 #pragma unroll
-      for (int w2 = 1; w2 < 4; ++w2) merge(r.x, r.y, warp_stat[w2 * kRsRows + lane].x, warp_stat[w2 * kRsRows + lane].y);
+      for (int w2 = 1; w2 < 4; ++w2) merge(r.x, r.y, of_row[w2 * kHalf].x, of_row[w2 * kHalf].y);
       cta_stat[lane] = r;
     }
   }
@@ -271,36 +280,44 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
   // ---- scores of the prefix keys, from the logits still in TMEM (loads double buffered)
   if (epi) {
     pdl_wait();                                                // the score buffer may still be read by the call before
-    float nl[kRsRows];
+    constexpr int kHalf = kRsRows / 2;
+    float nl[kHalf];
 #pragma unroll
-    for (int j = 0; j < kRsRows; ++j) {
-      const float l = __shfl_sync(0xffffffffu, lse2, j);
-      nl[j] = j < p.rows ? -l : -INFINITY;
+    for (int j = 0; j < kHalf; ++j) {
+      const float l = __shfl_sync(0xffffffffu, lse2, rh * kHalf + j);
+      nl[j] = rh * kHalf + j < p.rows ? -l : -INFINITY;
     }
-    float* srow = p.scores + (static_cast<int64_t>(b) * p.num_kv_heads + h) * p.ld_scores;
-    auto score_tile = [&](int t, const uint32_t (&v)[32]) {
+    // each half of the rows into its place over the K tiles, which nobody reads any more; then the halves meet
+    float* part = reinterpret_cast<float*>(k_s);               // [2][tiles][128]
+    auto half_sum = [&](int t, const uint32_t (&v)[kHalf]) {
       float s0 = 0.f, s1 = 0.f;
 #pragma unroll
-      for (int j = 0; j < kRsRows; j += 2) {                   // a prefix key is seen by every row: no mask
+      for (int j = 0; j < kHalf; j += 2) {                     // a prefix key is seen by every row: no mask
         s0 += ex2(fmaf(__uint_as_float(v[j]), c2, nl[j]));
         s1 += ex2(fmaf(__uint_as_float(v[j + 1]), c2, nl[j + 1]));
       }
-      const int i = (tile0 + t) * kRsTileKeys + lane_row;
-      if (i < P) srow[i] = s0 + s1;
+      part[(rh * kRsMaxTiles + t) * kRsTileKeys + lane_row] = s0 + s1;
     };
     if (ok && T > 0) {
-      uint32_t va[32], vb[32];
-      tc_ld32(lane_addr, va);
+      const uint32_t from = lane_addr + rh * kHalf;
+      uint32_t va[kHalf], vb[kHalf];
+      tc_ld16(from, va);
       for (int t = 0; t < T; t += 2) {
         tc_wait_ld();
-        if (t + 1 < T) tc_ld32(lane_addr + (t + 1) * kRsRows, vb);
-        score_tile(t, va);
+        if (t + 1 < T) tc_ld16(from + (t + 1) * kRsRows, vb);
+        half_sum(t, va);
         if (t + 1 < T) {
           tc_wait_ld();
-          if (t + 2 < T) tc_ld32(lane_addr + (t + 2) * kRsRows, va);
-          score_tile(t + 1, vb);
+          if (t + 2 < T) tc_ld16(from + (t + 2) * kRsRows, va);
+          half_sum(t + 1, vb);
         }
       }
+    }
+    asm volatile("bar.sync %0, 64;" ::"r"(2 + quarter) : "memory");            // (reached whether a wait ran out or not)
+    float* srow = p.scores + (static_cast<int64_t>(b) * p.num_kv_heads + h) * p.ld_scores;
+    for (int t = rh; t < T && ok; t += 2) {
+      const int i = (tile0 + t) * kRsTileKeys + lane_row;
+      if (i < P) srow[i] = part[t * kRsTileKeys + lane_row] + part[(kRsMaxTiles + t) * kRsTileKeys + lane_row];
     }
   }
   cluster.sync();                                              // barrier 2: nobody reads this CTA's shared memory any more
