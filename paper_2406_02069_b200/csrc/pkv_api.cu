@@ -158,6 +158,7 @@ bool tc_eligible(const pkv_config* c) {
 
 // Which configurations the fused window-attention kernel takes.
 bool attend_eligible(const pkv_config* c) { return tc_eligible(c) && c->head_dim == kAtD; }
+constexpr int kAtHeadTiles = 4;      // what a change of heads costs a CTA of the window-attention kernel, in tiles
 constexpr int kAtMaxGrid = 160;      // CTAs of the window-attention kernel at most (sizes its partial accumulators)
 
 // Carves the workspace for `batch` sequences of at most max_n tokens.  base may be null (sizing only).
@@ -647,9 +648,8 @@ int run_attend(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, co
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return PKV_ERR_CUDA;
   if (dev >= 64 || !attr_done[dev]) {
-    if (cudaFuncSetAttribute(window_attend_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAtSmemBytes) !=
-        cudaSuccess)
-      return PKV_ERR_CUDA;
+    for (auto f : {window_attend_kernel, window_attend_narrow_kernel})
+      if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kAtSmemBytes) != cudaSuccess) return PKV_ERR_CUDA;
     if (dev < 64) attr_done[dev] = true;
   }
   const bool fp16 = c->dtype == PKV_DTYPE_FP16;
@@ -683,7 +683,20 @@ int run_attend(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, co
   static_assert(kAtTileKeys == kTcTileKeys, "the sweep's tiles");
   const int items = stats.seq.stat_off[batch];
   ap.grid = static_cast<int>(std::min<long long>(grid_cap, static_cast<long long>(items) * c->num_kv_heads));
-  launch_pdl(window_attend_kernel, ap.grid, kAtThreads, kAtSmemBytes, st, q_map, k_map, v_map, ap);
+  // A CTA that goes from one head to the next in the middle of its range hands its accumulators over and merges the next
+  // head's normalisers, some five tiles' time that all others wait for in the end.  Where all heads are of one length,
+  // each gets the same number of CTAs, unless that makes the longest range longer by more.
+  const int heads = batch * c->num_kv_heads, tiles = stats.seq.stat_off[1];
+  bool even = heads <= grid_cap;
+  for (int b = 1; b < batch; ++b) even = even && stats.seq.stat_off[b + 1] - stats.seq.stat_off[b] == tiles;
+  if (even) {
+    const int cut = std::min(grid_cap / heads, tiles);
+    if ((tiles + cut - 1) / cut <= (items * c->num_kv_heads + ap.grid - 1) / ap.grid + kAtHeadTiles) {
+      ap.per_head = cut;
+      ap.grid = heads * cut;
+    }
+  }
+  launch_pdl(ap.rows <= 128 ? window_attend_narrow_kernel : window_attend_kernel, ap.grid, kAtThreads, kAtSmemBytes, st, q_map, k_map, v_map, ap);
   mark(st, "window_attend");
   launch_pdl(window_attend_reduce_kernel, dim3(ap.rows, c->num_kv_heads, batch), kAtD, 0, st, ap);
   mark(st, "window_attend_reduce");

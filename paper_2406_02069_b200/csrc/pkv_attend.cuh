@@ -69,6 +69,8 @@ struct AtParams {
   float* o_partial;             // [segment][R][d]: a segment is one CTA's run over one (sequence, head)
   float* out;                   // reduce kernel: [batch][H_q][alpha][d]
   int32_t grid;                 // CTAs the attention kernel runs with (the reduce kernel finds a head's segments from it)
+  int32_t per_head;             // > 0: so many CTAs to every (sequence, head), which all have the same number of tiles;
+                                // 0: equal ranges of tiles over all of them
   uint32_t* status;
 };
 
@@ -100,6 +102,21 @@ __device__ __forceinline__ uint32_t pack_16bit(float lo, float hi, int fp16) {
   }
   const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// This CTA's tiles: ntiles from number item0 on.
+__device__ __forceinline__ void at_range(const AtParams& p, int& item0, int& ntiles) {
+  const int32_t* off = p.seq.stat_off;
+  if (p.per_head > 0) {
+    const int nc = off[1], part = blockIdx.x % p.per_head, first = part * nc / p.per_head;
+    item0 = blockIdx.x / p.per_head * nc + first;
+    ntiles = (part + 1) * nc / p.per_head - first;
+  } else {
+    const int total = p.num_kv_heads * off[p.seq.batch];
+    const int per = total / gridDim.x, rem = total % gridDim.x;
+    item0 = blockIdx.x * per + min(static_cast<int>(blockIdx.x), rem);
+    ntiles = per + (static_cast<int>(blockIdx.x) < rem ? 1 : 0);
+  }
 }
 
 // 16 window rows of one key, all visible: e = 2^(v * c2 + nl), summed into acc (a packed pair of partial sums)
@@ -193,11 +210,8 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
   // kernel start (or see wait_v); the epilogue waits before it reads the sweep's partials and before its first write.
 
   const int32_t* off = p.seq.stat_off;
-  const int total = p.num_kv_heads * off[p.seq.batch];
-  const int per = total / gridDim.x, rem = total % gridDim.x;
-  const int item0 = blockIdx.x * per + min(static_cast<int>(blockIdx.x), rem);
-  const int item1 = item0 + per + (static_cast<int>(blockIdx.x) < rem ? 1 : 0);
-  const int ntiles = item1 - item0;
+  int item0, ntiles;
+  at_range(p, item0, ntiles);
   auto first_tile = [&]() { return tc_item(off, p.seq.batch, p.num_kv_heads, item0); };
   auto next_tile = [&](TcItem& w) { tc_next<false>(off, p.seq.batch, p.num_kv_heads, w); };
 
@@ -456,11 +470,12 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
               const int cg = piece == 0 ? cg_a : cg_b;
               const uint32_t (&v)[16] = piece == 0 ? va : vb;
               float ev[16];
-#pragma unroll
+              int jr = (hf * 128 + cg) % alpha;                // window index of the row: counted up, a division per row takes
+#pragma unroll                                                 // the CTA 10 us for the tile
               for (int j = 0; j < 16; ++j) {
                 const float x = ex2(fmaf(__uint_as_float(v[j]), c2, nlr[cg + j]));
-                const bool vis = in_seq && (jp <= 0 || (hf * 128 + cg + j) % alpha >= jp);
-                ev[j] = vis ? x : 0.f;
+                ev[j] = in_seq && jr >= jp ? x : 0.f;          // (jp <= 0: seen by all)
+                jr = jr + 1 == alpha ? 0 : jr + 1;
               }
               uint32_t pk[8];
 #pragma unroll
@@ -524,6 +539,404 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
   }
 }
 
+// Up to 128 window rows: two tiles in work at a time.  The sixteen epilogue warps form two teams of eight, each with an S stage (128
+// columns) and a P buffer of its own, which take the tiles in turn; in a team two warps share a quarter of the keys, each
+// with half of the window rows.  The issuer queues K Q^T of a tile as soon as the team has the logits of its last one in
+// registers, and V^T P two tiles behind, so that neither team waits for the other's exponentials.
+// Shared memory: Q 32 KB, two K tiles, two V tiles, two P buffers.  TMEM: columns 0..255 the S stages, 256..383 O^T.
+// What bounds it: a tile takes a CTA 1.3 us (64 KB of K and V, the memory's rate), behind a start of 5 us of which 4 are
+// the merge of the normalisers.  32768 keys x 8 heads x 128 rows, the whole call: 87.4 us with one team (the kernel above),
+// 79.4 with the window index counted instead of divided (the last tile of a head took its CTA 14 us), 77.3 with two teams,
+// 70.7 with the CTAs dealt out to the heads so that none goes from one head to the next (7 us).
+constexpr int kAnKOff = 128 * kAtD * 2;
+constexpr int kAnVOff = kAnKOff + 2 * kAtTileBytes;
+constexpr int kAnPOff = kAnVOff + 2 * kAtTileBytes;
+static_assert(kAnPOff + 2 * kAtTileBytes == kAtMiscOff, "the carve-up of the kernel above, Q's second half for a K tile");
+
+__global__ void __launch_bounds__(kAtThreads, 1)
+window_attend_narrow_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
+                            const __grid_constant__ CUtensorMap v_map, const AtParams p) {
+  extern __shared__ __align__(1024) uint8_t at_smem[];
+  uint8_t* smem = at_smem;
+  pdl_trigger();
+  if (smem_u32(smem) & 1023u) {                                // the carve-up below needs this; never seen otherwise
+    pdl_wait();
+    if (threadIdx.x == 0) atomicOr(p.status, kStatusWaitExpired);
+    return;
+  }
+  uint8_t* misc = smem + kAtMiscOff;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 320);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 324);
+  float* xch = reinterpret_cast<float*>(misc + 512);           // [2 teams][128] partial score sums of the second half of the rows
+  float* lse_all = reinterpret_cast<float*>(misc + 2048);      // [2 teams][128] shifted -lse2 of the team's head
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t bar0 = smem_u32(misc), smem0 = smem_u32(smem);
+  auto k_full = [&](int s) { return bar0 + 8u * s; };
+  auto k_empty = [&](int s) { return bar0 + 8u * (2 + s); };
+  auto v_full = [&](int s) { return bar0 + 8u * (4 + s); };
+  auto v_empty = [&](int s) { return bar0 + 8u * (6 + s); };
+  auto s_full = [&](int s) { return bar0 + 8u * (8 + s); };
+  auto s_empty = [&](int s) { return bar0 + 8u * (10 + s); };
+  auto p_full = [&](int s) { return bar0 + 8u * (12 + s); };
+  auto p_empty = [&](int s) { return bar0 + 8u * (14 + s); };
+  const uint32_t q_full = bar0 + 8u * 16, q_empty = bar0 + 8u * 17, o_full = bar0 + 8u * 18, o_empty = bar0 + 8u * 19;
+  auto lse_full = [&](int team) { return bar0 + 8u * (20 + team); };
+  auto x_full = [&](int team, int quarter) { return bar0 + 8u * (22 + team * 4 + quarter); };
+  auto x_empty = [&](int team, int quarter) { return bar0 + 8u * (30 + team * 4 + quarter); };
+  const int n_pv = p.rows_pad < 64 ? 64 : p.rows_pad;          // window rows of V^T P (whole 64-row blocks)
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(k_full(s), 1); mbar_init(k_empty(s), 1);
+      mbar_init(v_full(s), 1); mbar_init(v_empty(s), 1);
+      mbar_init(s_full(s), 1); mbar_init(s_empty(s), 8);
+      mbar_init(p_full(s), 8); mbar_init(p_empty(s), 1);
+      mbar_init(lse_full(s), 8);
+      for (int q = 0; q < 4; ++q) { mbar_init(x_full(s, q), 1); mbar_init(x_empty(s, q), 1); }
+    }
+    mbar_init(q_full, 1); mbar_init(q_empty, 1);
+    mbar_init(o_full, 1); mbar_init(o_empty, kAtEpiWarps);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  // Q rows beyond R and P rows beyond rows_pad stay zero for the whole kernel
+  for (int i = threadIdx.x; i < kAnKOff / 16; i += kAtThreads) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
+  for (int i = threadIdx.x; i < 2 * kAtTileBytes / 16; i += kAtThreads) reinterpret_cast<uint4*>(smem + kAnPOff)[i] = make_uint4(0, 0, 0, 0);
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  // No wait here: as in the kernel above.
+
+  const int32_t* off = p.seq.stat_off;
+  int item0, ntiles;
+  at_range(p, item0, ntiles);
+  auto first_tile = [&]() { return tc_item(off, p.seq.batch, p.num_kv_heads, item0); };
+  auto next_tile = [&](TcItem& w) { tc_next<false>(off, p.seq.batch, p.num_kv_heads, w); };
+
+  if (warp == 0) {
+    // =========================================================== TMA producer: Q per head, K per tile
+    if (lane == 0) {
+      int it = 0;
+      uint32_t heads_loaded = 0;
+      int cur_b = -1, cur_h = -1;
+      bool ok = true;
+      TcItem w = first_tile();
+      for (; it < ntiles; ++it, next_tile(w)) {
+        if (w.b != cur_b || w.h != cur_h) {
+          if (heads_loaded > 0) {
+            pdl_wait();
+            ok = mbar_wait(q_empty, (heads_loaded - 1) & 1, abort_flag, p.wait_clocks);
+          }
+          if (!ok) break;
+          mbar_expect_tx(q_full, static_cast<uint32_t>(p.rows) * kAtD * 2);
+          for (int half = 0; half < 2; ++half)
+            tma_load_4d(smem0 + half * 128 * 128, &q_map, q_full, half * 64, 0, w.h * p.group, w.b);
+          ++heads_loaded;
+          cur_b = w.b; cur_h = w.h;
+        }
+        const int s = it & 1;
+        if (it == 4) pdl_wait();                               // (from here on it waits for the epilogue)
+        ok = mbar_wait(k_empty(s), ((it >> 1) & 1) ^ 1, abort_flag, p.wait_clocks);
+        if (!ok) break;
+        if (p.withhold && blockIdx.x == 0 && it + 1 == ntiles) continue;   // test aid: never arrives
+        mbar_expect_tx(k_full(s), kAtTileBytes);
+        for (int half = 0; half < 2; ++half)
+          tma_load_4d(smem0 + kAnKOff + s * kAtTileBytes + half * kAtTileKeys * 128, &k_map, k_full(s), half * 64, w.c * kAtTileKeys,
+                      w.h, w.b);
+      }
+      if (!ok) {
+        for (int j = max(0, it - 2); j < it; ++j)
+          for (uint32_t spin = 0; spin < (1u << 16) && !mbar_test(k_full(j & 1), (j >> 1) & 1); ++spin) __nanosleep(64);
+        if (heads_loaded > 0)
+          for (uint32_t spin = 0; spin < (1u << 16) && !mbar_test(q_full, (heads_loaded - 1) & 1); ++spin) __nanosleep(64);
+      }
+    }
+  } else if (warp == 2) {
+    // =========================================================== TMA producer: V per tile
+    if (lane == 0) {
+      int it = 0;
+      bool ok = true;
+      if (p.wait_v) pdl_wait();
+      TcItem w = first_tile();
+      for (; it < ntiles; ++it, next_tile(w)) {
+        const int s = it & 1;
+        if (it == 2) pdl_wait();
+        ok = mbar_wait(v_empty(s), ((it >> 1) & 1) ^ 1, abort_flag, p.wait_clocks);
+        if (!ok) break;
+        mbar_expect_tx(v_full(s), kAtTileBytes);
+        for (int half = 0; half < 2; ++half)
+          tma_load_4d(smem0 + kAnVOff + s * kAtTileBytes + half * kAtTileKeys * 128, &v_map, v_full(s), half * 64, w.c * kAtTileKeys,
+                      w.h, w.b);
+      }
+      if (!ok)
+        for (int j = max(0, it - 2); j < it; ++j)
+          for (uint32_t spin = 0; spin < (1u << 16) && !mbar_test(v_full(j & 1), (j >> 1) & 1); ++spin) __nanosleep(64);
+    }
+  } else if (warp == 1) {
+    // =========================================================== MMA issuer
+    if (elect_one()) {
+      const uint32_t idesc_s = instr_desc_16bit(kAtTileKeys, p.rows_pad, p.fp16);
+      const uint32_t idesc_pv = instr_desc_16bit(kAtD, n_pv, p.fp16) | (1u << 15) | (1u << 16);   // A and B M/N-major
+      int it = 0, behind = 0;                                  // tile of the next K Q^T, of the next V^T P
+      uint32_t heads_seen = 0, runs = 0;
+      int cur_b = -1, cur_h = -1;
+      bool ok = true, fresh = true, wait_o = false;
+      auto issue_pv = [&]() -> bool {
+        const int s = behind & 1;
+        if (behind == 0) pdl_wait();                           // V and P come behind the sweep ahead
+        if (!mbar_wait(v_full(s), (behind >> 1) & 1, abort_flag, p.wait_clocks)) return false;
+        if (wait_o) {                                          // the epilogue has read the accumulators of the run before
+          if (!mbar_wait(o_empty, (runs - 1) & 1, abort_flag, p.wait_clocks)) return false;
+          wait_o = false;
+        }
+        if (!mbar_wait(p_full(s), (behind >> 1) & 1, abort_flag, p.wait_clocks)) return false;
+        tc_fence_after();
+        const uint32_t v_lo = desc_lo_mn_major(smem0 + kAnVOff + s * kAtTileBytes, kAtTileKeys * 128);
+        const uint32_t p_lo = desc_lo_mn_major(smem0 + kAnPOff + s * kAtTileBytes, kAtTileKeys * 128);
+        if (fresh) tc_mma_halves<false>(tmem_base + 256, v_lo, p_lo, idesc_pv);
+        else tc_mma_halves<true>(tmem_base + 256, v_lo, p_lo, idesc_pv);
+#pragma unroll
+        for (int kk = 1; kk < kAtTileKeys / 16; ++kk)          // 16 keys further: 2048 bytes in both operands
+          tc_mma_halves<true>(tmem_base + 256, v_lo + kk * (2048 >> 4), p_lo + kk * (2048 >> 4), idesc_pv);
+        tc_commit(p_empty(s));
+        tc_commit(v_empty(s));
+        fresh = false;
+        ++behind;
+        return true;
+      };
+      auto end_run = [&]() -> bool {
+        while (behind < it)
+          if (!issue_pv()) return false;
+        tc_commit(o_full);
+        ++runs;
+        wait_o = true;
+        fresh = true;
+        return true;
+      };
+      TcItem w = first_tile();
+      for (; it < ntiles && ok; ++it) {
+        if (w.b != cur_b || w.h != cur_h) {
+          if (cur_b >= 0) ok = end_run();
+          if (!ok) break;
+          ok = mbar_wait(q_full, heads_seen & 1, abort_flag, p.wait_clocks);
+          if (!ok) break;
+          ++heads_seen;
+          cur_b = w.b; cur_h = w.h;
+        }
+        const int s = it & 1;
+        ok = mbar_wait(k_full(s), (it >> 1) & 1, abort_flag, p.wait_clocks);
+        if (!ok) break;
+        if (it == 2) pdl_wait();
+        ok = mbar_wait(s_empty(s), ((it >> 1) & 1) ^ 1, abort_flag, p.wait_clocks);   // the team's last tile is in registers
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t k_lo = desc_lo_k_major(smem0 + kAnKOff + s * kAtTileBytes), q_lo = desc_lo_k_major(smem0);
+        const uint32_t d_addr = tmem_base + s * 128;
+        tc_mma_halves<false>(d_addr, k_lo, q_lo, idesc_s);
+#pragma unroll
+        for (int kk = 1; kk < kAtD / 16; ++kk) {               // 16 channels further: 32 bytes, the next 64-channel block
+          constexpr int kBlock = 128 * 128 >> 4;               // after four steps
+          tc_mma_halves<true>(d_addr, k_lo + (kk / 4) * kBlock + (kk % 4) * 2, q_lo + (kk / 4) * kBlock + (kk % 4) * 2, idesc_s);
+        }
+        tc_commit(s_full(s));
+        tc_commit(k_empty(s));
+        if (it - behind >= 2) ok = issue_pv();
+        next_tile(w);
+        if (ok && (w.b != cur_b || w.h != cur_h || it + 1 == ntiles)) tc_commit(q_empty);
+      }
+      if (ok && cur_b >= 0) end_run();
+    }
+  } else if (warp >= kAtEpiWarp0) {
+    // =========================================================== epilogue
+    const int e = warp - kAtEpiWarp0;
+    const int team = e >> 3, part = (e >> 2) & 1, quarter = warp & 3;
+    const int lane_row = quarter * 32 + lane;                  // TMEM lane: key of a tile in S, channel in O^T
+    const uint32_t lanes = static_cast<uint32_t>(quarter * 32) << 16;
+    const float c2 = p.scale_log2;
+    const float unshift = 1.0f / static_cast<float>(1 << kAtShift);
+    const int cols = p.rows_pad / 2, col0 = part * cols;       // this warp's window rows (a multiple of 16)
+    float* lse_s = lse_all + team * 128;
+    uint32_t lse_rounds = 0, runs = 0;
+    int it = 0;
+    int cur_b = -1, cur_h = -1;
+    bool ok = true;
+    // Hands the accumulators of the run that ends to global memory (raw: the reduce kernel scales).
+    auto flush_o = [&]() -> bool {
+      bool good = mbar_wait(o_full, runs & 1, abort_flag, p.wait_clocks);
+      good = __all_sync(0xffffffffu, good);
+      if (!good) return false;
+      tc_fence_after();
+      const int64_t seg = static_cast<int64_t>(blockIdx.x) + cur_b * p.num_kv_heads + cur_h;
+      float* dst = p.o_partial + seg * p.rows * kAtD + lane_row;
+      for (int cg = (e >> 2) * 16; cg < n_pv; cg += 64) {      // 16-column pieces dealt round to the four groups of warps
+        uint32_t v[16];
+        tc_ld16(tmem_base + lanes + 256 + cg, v);
+        tc_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          if (cg + j < p.rows) dst[static_cast<int64_t>(cg + j) * kAtD] = __uint_as_float(v[j]);
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(o_empty);
+      ++runs;
+      return true;
+    };
+    // One meeting of the team.
+    auto meet = [&]() -> bool {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(lse_full(team));
+      bool good = mbar_wait(lse_full(team), lse_rounds & 1u, abort_flag, p.wait_clocks);
+      ++lse_rounds;
+      return __all_sync(0xffffffffu, good);
+    };
+    TcItem w = first_tile();
+    int n = 0, P = 0;
+    const int alpha = p.seq.alpha;
+    for (; it < ntiles && ok; ++it, next_tile(w)) {
+      if (w.b != cur_b || w.h != cur_h) {
+        if (cur_b >= 0) ok = flush_o();
+        if (!ok) break;
+        // the head's normalisers, negated and shifted: written once the team is done with the old ones, read once it
+        // has written
+        ok = meet();
+        if (!ok) break;
+        tc_merge_head<8 * 32, true>(p, w.b, w.h, (e & 7) * 32 + lane, lse_s);
+        ok = meet();
+        if (!ok) break;
+        cur_b = w.b; cur_h = w.h;
+        n = p.seq.n[w.b];
+        P = p.seq.prefix[w.b];
+      }
+      if ((it & 1) != team) continue;
+      const uint32_t phase = (it >> 1) & 1;
+      const int i = w.c * kAtTileKeys + lane_row;
+      const bool in_seq = i < n;
+      const int jp = i - P;                                    // window key P + jp is seen by rows j >= jp
+      const bool plain = __all_sync(0xffffffffu, in_seq && jp <= 0);   // no mask anywhere in this warp's keys
+      ok = mbar_wait(s_full(team), phase, abort_flag, p.wait_clocks);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t taddr = tmem_base + lanes + team * 128;
+      uint8_t* prow = smem + kAnPOff + team * kAtTileBytes + lane_row * 128;
+      unsigned long long acc = pack2(0.f, 0.f);
+      float sum = 0.f;
+      for (int c = 0; c < cols && ok; c += 32) {               // pieces of 16 rows, two at a time
+        const int ca = col0 + c, cb = ca + 16;
+        const bool two = c + 16 < cols;
+        uint32_t va[16], vb[16];
+        tc_ld16(taddr + ca, va);
+        if (two) tc_ld16(taddr + cb, vb);
+        tc_wait_ld();
+        if (c + 32 >= cols) {                                  // the tile's logits are in registers: the stage is free
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(s_empty(team));
+        }
+        if (c == 0) {                                          // V^T P of the team's last tile has read the buffer
+          ok = mbar_wait(p_empty(team), phase ^ 1, abort_flag, p.wait_clocks);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+        }
+        uint8_t* pa = prow + (ca >> 6) * (kAtTileKeys * 128);
+        uint8_t* pb = prow + (cb >> 6) * (kAtTileKeys * 128);
+        if (plain) {
+          const unsigned long long cc = pack2(c2, c2);
+          const int sw = lane_row & 7;
+          if (p.fp16) {
+            at_chunk<true>(va, cc, lse_s + ca, pa, (ca & 63) >> 3, sw, acc);
+            if (two) at_chunk<true>(vb, cc, lse_s + cb, pb, (cb & 63) >> 3, sw, acc);
+          } else {
+            at_chunk<false>(va, cc, lse_s + ca, pa, (ca & 63) >> 3, sw, acc);
+            if (two) at_chunk<false>(vb, cc, lse_s + cb, pb, (cb & 63) >> 3, sw, acc);
+          }
+        } else {
+#pragma unroll
+          for (int piece = 0; piece < 2; ++piece) {
+            if (piece == 1 && !two) continue;
+            const int cg = piece == 0 ? ca : cb;
+            const uint32_t (&v)[16] = piece == 0 ? va : vb;
+            uint32_t pk[8];
+            int jr = cg % alpha;                               // window index of the row, counted up
+#pragma unroll
+            for (int j = 0; j < 16; j += 2) {
+              float ev[2];
+#pragma unroll
+              for (int u = 0; u < 2; ++u) {
+                const float x = ex2(fmaf(__uint_as_float(v[j + u]), c2, lse_s[cg + j + u]));
+                ev[u] = in_seq && jr >= jp ? x : 0.f;          // (jp <= 0: seen by all)
+                jr = jr + 1 == alpha ? 0 : jr + 1;
+              }
+              sum += ev[0] + ev[1];
+              pk[j >> 1] = pack_16bit(ev[0], ev[1], p.fp16);
+            }
+            uint8_t* blk = piece == 0 ? pa : pb;
+            const int c0 = (cg & 63) >> 3;
+            *reinterpret_cast<uint4*>(blk + ((c0 ^ (lane_row & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            *reinterpret_cast<uint4*>(blk + (((c0 + 1) ^ (lane_row & 7)) << 4)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+          }
+        }
+      }
+      if (!ok) break;
+      if (part == 0 && (w.c + 1) * kAtTileKeys > n) {
+        // last tile of a sequence: what lies behind the sequence in V may be anything, and 0 x NaN is NaN
+        ok = mbar_wait(v_full(team), phase, abort_flag, p.wait_clocks);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        if (!in_seq)
+          for (int half = 0; half < 2; ++half)
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+              reinterpret_cast<uint4*>(smem + kAnVOff + team * kAtTileBytes + half * kAtTileKeys * 128 + lane_row * 128)[c] =
+                  make_uint4(0, 0, 0, 0);
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(p_full(team));
+      // the key's score: the sums over the two halves of the rows
+      float lo, hi;
+      unpack2(acc, lo, hi);
+      sum += lo + hi;
+      if (part == 0) {
+        ok = mbar_wait(x_full(team, quarter), phase, abort_flag, p.wait_clocks);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        sum += xch[team * 128 + lane_row];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(x_empty(team, quarter));
+        if (i < P) p.scores[(static_cast<int64_t>(w.b) * p.num_kv_heads + w.h) * p.ld_scores + i] = sum * unshift;
+      } else {
+        ok = mbar_wait(x_empty(team, quarter), phase ^ 1, abort_flag, p.wait_clocks);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        xch[team * 128 + lane_row] = sum;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(x_full(team, quarter));
+      }
+    }
+    if (ok && cur_b >= 0) flush_o();
+  }
+
+  // ---- teardown
+  pdl_wait();                                                  // never finish before the sweep ahead, also when a wait ran out early
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && *abort_flag) atomicOr(p.status, kStatusWaitExpired);
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
+  }
+}
+
 // out[b][h * G + g][j][c] = G * 2^-15 * sum over the head's segments of o_partial[segment][g * alpha + j][c].
 // grid (R, H_kv, batch), block d.
 __global__ void __launch_bounds__(kAtD) window_attend_reduce_kernel(const AtParams p) {
@@ -534,9 +947,13 @@ __global__ void __launch_bounds__(kAtD) window_attend_reduce_kernel(const AtPara
   const int total = p.num_kv_heads * p.seq.stat_off[p.seq.batch];
   const int per = total / p.grid, rem = total % p.grid, edge = rem * (per + 1);
   const int i0 = p.num_kv_heads * p.seq.stat_off[b] + h * nc, i1 = i0 + nc - 1;
-  const int c0 = i0 < edge ? i0 / (per + 1) : rem + (i0 - edge) / per;
-  const int c1 = i1 < edge ? i1 / (per + 1) : rem + (i1 - edge) / per;
   const int hg = b * p.num_kv_heads + h;
+  int c0 = i0 < edge ? i0 / (per + 1) : rem + (i0 - edge) / per;
+  int c1 = i1 < edge ? i1 / (per + 1) : rem + (i1 - edge) / per;
+  if (p.per_head > 0) {
+    c0 = hg * p.per_head;
+    c1 = c0 + p.per_head - 1;
+  }
   float acc = 0.f;
   for (int s = c0 + hg; s <= c1 + hg; ++s) acc += __ldcg(p.o_partial + (static_cast<int64_t>(s) * p.rows + r) * kAtD + c);
   const int alpha = p.seq.alpha, g = r / alpha, j = r % alpha;

@@ -408,7 +408,7 @@ __device__ __forceinline__ float2 tc_merge_row(const float2* row, int rows, int 
 }
 
 // Sweep A's partials of a head -> its negated row normalisers in dst (-inf for the padding rows), by THREADS threads (the sixteen
-// epilogue warps or one warp).  Every CTA that works on a head merges it for itself, and equal keys must get equal scores whichever CTA has them, so the additions come in the same order whoever does
+// epilogue warps, eight or one).  Every CTA that works on a head merges it for itself, and equal keys must get equal scores whichever CTA has them, so the additions come in the same order whoever does
 // it: 2 to 16 lanes per row by the number of rows alone, each with every per_row-th segment, then pairwise.  A single warp
 // does the same with a lane per row where the head has few segments (what it has to save there are instructions, beside
 // four warps of the epilogue on its scheduler), else in sixteen steps, four at a time if it can (L2 latencies).
@@ -472,8 +472,9 @@ __device__ __forceinline__ void tc_merge_head(const Params& p, int b, int h, int
       else if (per_row == 8) lane_a_row(integral_constant<int, 8>{}, integral_constant<int, 2>{});
       else lane_a_row(integral_constant<int, 16>{}, integral_constant<int, 1>{});
     } else if (s1 - s0 <= 5 * per_row) {
+      constexpr int kAtOnce = kSteps < 4 ? kSteps : 4;
 #pragma unroll 1
-      for (int step = 0; step < kSteps; step += 4) some(step, integral_constant<int, 4>{}, integral_constant<int, 5>{});
+      for (int step = 0; step < kSteps; step += kAtOnce) some(step, integral_constant<int, kAtOnce>{}, integral_constant<int, 5>{});
     } else {
 #pragma unroll 1
       for (int step = 0; step < kSteps; ++step) some(step, integral_constant<int, 1>{}, integral_constant<int, 10>{});
