@@ -72,7 +72,7 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
   using L = RsSmem<D, STAGES>;
   constexpr int kHalves = D / 64;
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = smem_raw + (-smem_u32(smem_raw) & 1023u);   // (an offset, so that accesses stay known as shared memory)
   uint8_t* q_s = smem + L::kQOff;
   uint8_t* k_s = smem + L::kKOff;
   uint8_t* misc = smem + L::kMiscOff;

@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
   constexpr int kChunks = D / 8;                               // 16-byte chunks of a part's row
   constexpr int kSteps = kSpKeys * kChunks / kSpConverters;    // chunks of a K tile per converter thread
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = smem_raw + (-smem_u32(smem_raw) & 1023u);   // (an offset, so that accesses stay known as shared memory)
   uint8_t* misc = smem + L::kMiscOff;
   uint64_t* bars = reinterpret_cast<uint64_t*>(misc);          // k_full, k_empty, t_full, t_empty (two of each), x_full, x_empty
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 192);                                      // (one a quarter)
