@@ -405,6 +405,18 @@ int launch_scores_split(ScoreParams& sp, int batch, int max_n, int grid, cudaStr
     tiles += (sp.seq.n[b] + kSpKeys - 1) / kSpKeys;
   }
   sp.seq.stat_off[batch] = tiles;
+  // Units of one length each get the same number of CTAs, unless that makes the longest range longer by more than a change
+  // of units costs (the next one's window rows are split while the MMAs wait: 5 us, a tile takes 1.2 to 1.8).
+  const int blocks = (sp.rows + kSpRows - 1) / kSpRows, units = sp.num_kv_heads * blocks * batch, each = sp.seq.stat_off[1];
+  bool even = units <= grid;
+  for (int b = 1; b < batch; ++b) even = even && sp.seq.stat_off[b + 1] - sp.seq.stat_off[b] == each;
+  if (even) {
+    const int cut = std::min(grid / units, each);
+    if ((each + cut - 1) / cut <= (each * units + grid - 1) / grid + 3) {
+      sp.per_unit = cut;
+      grid = units * cut;
+    }
+  }
   sp.stat_grid = grid;
   sp.log2_group = std::log2(static_cast<float>(sp.group));
   launch_pdl(split_logits_kernel<D>, dim3(grid), kSpThreads, SpSmem<D>::kTotal, st, sp);

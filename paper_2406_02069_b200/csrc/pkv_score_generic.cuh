@@ -49,6 +49,7 @@ struct ScoreParams {
   int64_t ld_logits;
   int32_t chunk_tiles;                   // tiles per CTA (1 when there are several row blocks)
   float log2_group;
+  int32_t per_unit;                      // pkv_score_split.cuh: CTAs per unit of one length, or 0
   uint32_t* status;
 };
 

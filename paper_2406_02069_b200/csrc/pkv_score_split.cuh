@@ -20,7 +20,7 @@
 //
 // Warps 0..7 load a tile of 64 keys into registers, split it and store the parts swizzled as the MMAs want them (the loads of the next
 // tile are under way while they wait for room); warp 16 issues the MMAs; warps 8..15 take the logits out of TMEM, a
-// thread per window row and half of the keys.  Tiles of 64 keys and not 128: two stages of parts fit beside Q's, and the
+// thread per window row, in two teams that take the tiles in turn.  Tiles of 64 keys and not 128: two stages of parts fit beside Q's, and the
 // tiles spread more evenly over the CTAs.
 //
 // Infinities, NaN and magnitudes of 2^90 or more raise a flag for their tile, whose logits are then formed by plain fp32
@@ -58,6 +58,11 @@ struct SpSmem {
 
 // Where the runs of the CTAs over unit (sequence, head, row block) number `unit` went: segments [s0, s1).
 __device__ __forceinline__ void sp_segments(const ScoreParams& p, int b, int unit_in_seq, int units, int& s0, int& s1) {
+  if (p.per_unit > 0) {
+    s0 = (b * units + unit_in_seq) * (p.per_unit + 1);
+    s1 = s0 + p.per_unit;
+    return;
+  }
   const int nc = p.seq.stat_off[b + 1] - p.seq.stat_off[b];
   const int total = units * p.seq.stat_off[p.seq.batch];
   const int per = total / p.stat_grid, rem = total % p.stat_grid, edge = rem * (per + 1);
@@ -125,7 +130,7 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 196);
   volatile int* special = reinterpret_cast<volatile int*>(misc + 256);         // [8]: tiles with values that are not split
   volatile int* q_special = reinterpret_cast<volatile int*>(misc + 288);       // [8]: the same of the units' window rows
-  float2* halves = reinterpret_cast<float2*>(misc + 1024);                     // [128] statistics of the second half's threads
+  float2* halves = reinterpret_cast<float2*>(misc + 1024);                     // [128] statistics of the second team
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t bar0 = smem_u32(bars), smem0 = smem_u32(smem);
   auto k_full = [&](int s) { return bar0 + 8u * s; };
@@ -142,10 +147,10 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
       mbar_init(k_full(s), kSpConverters / 32);
       mbar_init(k_empty(s), 1);
       mbar_init(t_full(s), 1);
-      mbar_init(t_empty(s), 8);
+      mbar_init(t_empty(s), 4);
     }
     for (int q = 0; q < 4; ++q) { mbar_init(x_full(q), 1); mbar_init(x_empty(q), 1); }
-    mbar_init(q_full, kSpConverters / 32);
+    mbar_init(q_full, 2 * kSpConverters / 32);
     *abort_flag = 0;
     for (int i = 0; i < 8; ++i) special[i] = q_special[i] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -165,8 +170,13 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
   const int32_t* off = p.seq.stat_off;
   const int total = units * off[p.seq.batch];
   const int per = total / gridDim.x, rem = total % gridDim.x;
-  const int item0 = blockIdx.x * per + min(static_cast<int>(blockIdx.x), rem);
-  const int ntiles = per + (static_cast<int>(blockIdx.x) < rem ? 1 : 0);
+  int item0 = blockIdx.x * per + min(static_cast<int>(blockIdx.x), rem);
+  int ntiles = per + (static_cast<int>(blockIdx.x) < rem ? 1 : 0);
+  if (p.per_unit > 0) {
+    const int nc = off[1], part = blockIdx.x % p.per_unit, first = part * nc / p.per_unit;
+    item0 = blockIdx.x / p.per_unit * nc + first;
+    ntiles = (part + 1) * nc / p.per_unit - first;
+  }
   const int alpha = p.seq.alpha;
   const float* kptr = static_cast<const float*>(p.k.ptr);
   const float* qptr = static_cast<const float*>(p.q.ptr);
@@ -176,13 +186,14 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
   };
   // Chunk c of row x of a part of `rows` rows: 64 channels to a row of 128 bytes, its 16-byte chunks exchanged by the row.
   auto place = [](int rows, int x, int c) { return (c >> 3) * rows * 128 + x * 128 + (((c & 7) ^ (x & 7)) << 4); };
-  // The window rows of w's unit, by 256 threads; returns whether this thread saw a value that is not split.
-  auto convert_q = [&](const TcItem& w, int tid) -> bool {
-    constexpr int kBatch = D == 128 ? 2 : 4;
+  // Chunks [begin, end) of the window rows of w's unit, by 256 threads; returns whether this thread saw a value that is not split.
+  auto convert_q = [&](const TcItem& w, int tid, int begin, int end) -> bool {
+    constexpr int kBatch = 2;
+    static_assert(kSpRows * kChunks / 2 % (kBatch * kSpConverters) == 0, "halves in whole steps");
     const int r0 = (w.h % blocks) * kSpRows;
     SpSeen seen;
 #pragma unroll 1
-    for (int i0 = tid; i0 < kSpRows * kChunks; i0 += kBatch * kSpConverters) {
+    for (int i0 = begin + tid; i0 < end; i0 += kBatch * kSpConverters) {
       float4 f[kBatch][2];
 #pragma unroll
       for (int u = 0; u < kBatch; ++u) {
@@ -215,6 +226,11 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
   };
   static_assert(kSpKeys * (D / 32) <= kSpConverters, "a line per thread");
   TcItem ahead = tc_item(off, p.seq.batch, units, item0);
+  if (warp >= 8 && warp < 16)
+    for (int i = threadIdx.x - kSpConverters; i < kSpRows * (D / 32); i += kSpConverters) {
+      const int r = (ahead.h % blocks) * kSpRows + i / (D / 32);
+      if (r < p.rows) asm volatile("prefetch.global.L2 [%0];" ::"l"(q_row(ahead, r) + i % (D / 32) * 32));
+    }
   if (warp < 8)
     for (int it = 0; it < min(ntiles, kSpPrefetch); ++it, tc_next<false>(off, p.seq.batch, units, ahead)) prefetch_tile(ahead);
   pdl_wait();
@@ -240,8 +256,18 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
       }
     };
     if (ntiles > 0) load_tile(w);
-    int cur_b = w.b, cur_h = w.h, runs = 0;                    // (the first unit's rows are the epilogue's, which has time then)
+    int cur_b = w.b, cur_h = w.h, runs = 0;
     bool ok = true;
+    auto have_q = [&](int parts) {                             // of the sixteen arrivals that a unit's rows take
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0)
+        for (int i = 0; i < parts; ++i) mbar_arrive(q_full);
+    };
+    if (ntiles > 0) {                                          // the first unit's rows: half of them the epilogue's, which has time then
+      if (convert_q(w, threadIdx.x, kSpRows * kChunks / 2, kSpRows * kChunks)) q_special[0] = 1;
+      have_q(1);
+    }
     for (int it = 0; it < ntiles; ++it) {
       const int s = it % kSpStages;
       if (w.b != cur_b || w.h != cur_h) {                      // another unit: its window rows, once the MMAs of the last are done
@@ -252,10 +278,8 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
         ++runs;
         // (the epilogue is at most three tiles behind)
         if (threadIdx.x == 0) q_special[(runs + 4) & 7] = 0;
-        if (convert_q(w, threadIdx.x)) q_special[runs & 7] = 1;
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) mbar_arrive(q_full);
+        if (convert_q(w, threadIdx.x, 0, kSpRows * kChunks)) q_special[runs & 7] = 1;
+        have_q(2);
       }
       ok = mbar_wait(k_empty(s), ((it / kSpStages) & 1) ^ 1, abort_flag, limit);
       ok = __all_sync(0xffffffffu, ok);
@@ -326,15 +350,16 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
       }
     }
   } else {
-    // =========================================================== epilogue: thread = (window row, half of the tile's keys)
-    const int quarter = warp & 3, half = (warp - 8) >> 2;
+    // =========================================================== epilogue: two teams of four warps, each with an accumulator stage,
+    // take the tiles in turn; thread = window row
+    const int quarter = warp & 3, team = (warp - 8) >> 2;
     const int lane_row = quarter * 32 + lane;
     float m = -INFINITY, z = 0.f;
     uint32_t runs = 0;                                         // over units so far
     TcItem w = tc_item(off, p.seq.batch, units, item0);
     bool ok = true;
     if (ntiles > 0) {
-      if (convert_q(w, threadIdx.x - kSpConverters)) q_special[0] = 1;
+      if (convert_q(w, threadIdx.x - kSpConverters, 0, kSpRows * kChunks / 2)) q_special[0] = 1;
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(q_full);
@@ -352,79 +377,84 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
         lrow = p.logits + (static_cast<int64_t>(w.b) * p.num_kv_heads + h) * p.ld_logits * p.rows + r;
       }
       const bool live = r < p.rows;
-      const int s = it % kSpStages;
-      ok = mbar_wait(t_full(s), (it / kSpStages) & 1, abort_flag, limit);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) break;
-      tc_fence_after();
-      const int key0 = w.c * kSpKeys + half * 32;
-      const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + s * kSpAccs * kSpKeys + half * 32;
-      unsigned long long x2[16];
-#pragma unroll
-      for (int a = 0; a < kSpAccs; ++a) {
-        uint32_t v0[16], v1[16];
-        tc_ld16(taddr + a * kSpKeys, v0);
-        tc_ld16(taddr + a * kSpKeys + 16, v1);
-        tc_wait_ld();
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const unsigned long long y0 = pack2(__uint_as_float(v0[2 * j]), __uint_as_float(v0[2 * j + 1]));
-          const unsigned long long y1 = pack2(__uint_as_float(v1[2 * j]), __uint_as_float(v1[2 * j + 1]));
-          x2[j] = a == 0 ? y0 : add2(x2[j], y0);
-          x2[8 + j] = a == 0 ? y1 : add2(x2[8 + j], y1);
-        }
-      }
-      tc_fence_before();
-      float x[32];
-#pragma unroll
-      for (int j = 0; j < 16; ++j) unpack2(mul2(x2[j], scale), x[2 * j], x[2 * j + 1]);
-      if (special[it & 7] | q_special[runs & 7]) {             // the whole tile on the fp32 pipe
-        const float* q = q_row(w, min(r, p.rows - 1));
+      if (it % kSpStages == team) {
+        ok = mbar_wait(t_full(team), (it / kSpStages) & 1, abort_flag, limit);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
+        const bool on_pipe = special[it & 7] | q_special[runs & 7];            // the whole tile on the fp32 pipe
 #pragma unroll 1
-        for (int j = 0; j < 32; ++j) {
-          float dot = 0.f;
-          if (key0 + j < n) {
-            const float* k = head_keys(w) + (key0 + j) * p.k.st;
-#pragma unroll 4
-            for (int c = 0; c < D; ++c) dot = fmaf(q[c], k[c], dot);
+        for (int half = 0; half < 2; ++half) {
+          const int key0 = w.c * kSpKeys + half * 32;
+          const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + team * kSpAccs * kSpKeys + half * 32;
+          unsigned long long x2[16];
+#pragma unroll
+          for (int a = 0; a < kSpAccs; ++a) {
+            uint32_t v0[16], v1[16];
+            tc_ld16(taddr + a * kSpKeys, v0);
+            tc_ld16(taddr + a * kSpKeys + 16, v1);
+            tc_wait_ld();
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const unsigned long long y0 = pack2(__uint_as_float(v0[2 * j]), __uint_as_float(v0[2 * j + 1]));
+              const unsigned long long y1 = pack2(__uint_as_float(v1[2 * j]), __uint_as_float(v1[2 * j + 1]));
+              x2[j] = a == 0 ? y0 : add2(x2[j], y0);
+              x2[8 + j] = a == 0 ? y1 : add2(x2[8 + j], y1);
+            }
           }
-          dot *= p.scale_log2;
+          float x[32];
 #pragma unroll
-          for (int i = 0; i < 32; ++i) x[i] = i == j ? dot : x[i];
+          for (int j = 0; j < 16; ++j) unpack2(mul2(x2[j], scale), x[2 * j], x[2 * j + 1]);
+          if (on_pipe) {
+            const float* q = q_row(w, min(r, p.rows - 1));
+#pragma unroll 1
+            for (int j = 0; j < 32; ++j) {
+              float dot = 0.f;
+              if (key0 + j < n) {
+                const float* k = head_keys(w) + (key0 + j) * p.k.st;
+#pragma unroll 4
+                for (int c = 0; c < D; ++c) dot = fmaf(q[c], k[c], dot);
+              }
+              dot *= p.scale_log2;
+#pragma unroll
+              for (int i = 0; i < 32; ++i) x[i] = i == j ? dot : x[i];
+            }
+          }
+          if (half == 1) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(t_empty(team));
+          }
+          if (live) {                                          // (within the padded length)
+            float* to = lrow + static_cast<int64_t>(key0) * p.rows;
+#pragma unroll
+            for (int j = 0; j < 32; ++j, to += p.rows) *to = x[j];
+          }
+          if (key0 + 31 > min(p.seq.prefix[w.b], n - 1)) {     // some key is hidden from some row
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (key0 + j > last) x[j] = -INFINITY;
+          }
+          float gm = x[0];
+#pragma unroll
+          for (int j = 1; j < 32; ++j) gm = fmaxf(gm, x[j]);
+          const float mn = fmaxf(m, gm), ref = mn == -INFINITY ? 0.f : mn;     // (a NaN among the logits shows in z)
+          const unsigned long long minus = pack2(-ref, -ref);
+          unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            float d0, d1;
+            unpack2(add2(pack2(x[2 * j], x[2 * j + 1]), minus), d0, d1);
+            acc[j & 3] = add2(acc[j & 3], pack2(ex2(d0), ex2(d1)));
+          }
+          z = z * ex2(m - ref) + sum_pairs(acc);
+          m = mn;
         }
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(t_empty(s));
-      if (live) {                                              // (within the padded length)
-        float* to = lrow + static_cast<int64_t>(key0) * p.rows;
-#pragma unroll
-        for (int j = 0; j < 32; ++j, to += p.rows) *to = x[j];
-      }
-      if (key0 + 31 > min(p.seq.prefix[w.b], n - 1)) {                     // some key is hidden from some row
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (key0 + j > last) x[j] = -INFINITY;
-      }
-      {
-        float gm = x[0];
-#pragma unroll
-        for (int j = 1; j < 32; ++j) gm = fmaxf(gm, x[j]);
-        const float mn = fmaxf(m, gm), ref = mn == -INFINITY ? 0.f : mn;       // (a NaN among the logits shows in z)
-        const unsigned long long minus = pack2(-ref, -ref);
-        unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          float d0, d1;
-          unpack2(add2(pack2(x[2 * j], x[2 * j + 1]), minus), d0, d1);
-          acc[j & 3] = add2(acc[j & 3], pack2(ex2(d0), ex2(d1)));
-        }
-        z = z * ex2(m - ref) + sum_pairs(acc);
-        m = mn;
       }
       const TcItem was = w;
       tc_next<false>(off, p.seq.batch, units, w);
-      if (it + 1 == ntiles || w.b != was.b || w.h != was.h) {  // the run is over: the two halves of a row meet
-        if (half == 1) {
+      if (it + 1 == ntiles || w.b != was.b || w.h != was.h) {  // the run is over: the two teams meet
+        if (team == 1) {
           ok = mbar_wait(x_empty(quarter), (runs & 1) ^ 1, abort_flag, limit);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
