@@ -497,10 +497,25 @@ __global__ void __launch_bounds__(kSpSumThreads, 4) split_scores_kernel(const Sc
   const int h = blockIdx.y, b = blockIdx.z, P = p.seq.prefix[b];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int blocks = (p.rows + kSpRows - 1) / kSpRows;
+  // 1, 2, 4 or 8 adjacent lanes share a row's segments; where they lie is worked out ahead of the wait
+  const int per_row = p.rows > 128 ? 1 : (p.rows > 64 ? 2 : (p.rows > 32 ? 4 : 8)), part = threadIdx.x % per_row;
+  auto segments = [&](int r, int& s0, int& s1) {
+    s0 = s1 = 0;
+    if (r < p.rows) sp_segments(p, b, h * blocks + r / kSpRows, p.num_kv_heads * blocks, s0, s1);
+  };
+  int s0, s1;
+  segments(threadIdx.x / per_row, s0, s1);
   pdl_wait();
   if (blockIdx.x * kSpSumKeys >= P) return;
   const int64_t head = static_cast<int64_t>(b) * p.num_kv_heads + h;
-  // the first eight keys' logits are on their way while the segments are merged
+  auto load_segments = [&](int r, int t, float2 (&pz)[8]) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      pz[u] = t + u * per_row < s1 ? __ldcg(p.partial + static_cast<int64_t>(t + u * per_row) * p.rows + r) : make_float2(-INFINITY, 0.f);
+  };
+  // the segments first, then, on their way while those are merged, the first eight keys' logits
+  float2 pz[8];
+  load_segments(threadIdx.x / per_row, s0 + part, pz);
   float v[8][4];
   auto load = [&](const float* x, int r0) {
 #pragma unroll
@@ -511,28 +526,24 @@ __global__ void __launch_bounds__(kSpSumThreads, 4) split_scores_kernel(const Sc
   bool first = true;
   if (blockIdx.x * kSpSumKeys + warp * 8 >= P) first = false;
   else load(p.logits + (head * p.ld_logits + blockIdx.x * kSpSumKeys + warp * 8) * p.rows, lane);
-  // 1, 2, 4 or 8 adjacent lanes share a row's segments
-  const int per_row = p.rows > 128 ? 1 : (p.rows > 64 ? 2 : (p.rows > 32 ? 4 : 8));
   for (int r0 = 0; r0 < p.rows; r0 += kSpSumThreads / per_row) {
     const int r = r0 + threadIdx.x / per_row;
     float m = -INFINITY, z = 0.f;
-    if (r < p.rows) {
-      int s0, s1;
-      sp_segments(p, b, h * blocks + r / kSpRows, p.num_kv_heads * blocks, s0, s1);
-      for (int t = s0 + threadIdx.x % per_row; t < s1; t += 8 * per_row) {
-        float2 pz[8];
-        float mn = m;
+    if (r0 > 0) {
+      segments(r, s0, s1);
+      load_segments(r, s0 + part, pz);
+    }
+    for (int t = s0 + part; t < s1;) {
+      float mn = m;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          pz[u] = t + u * per_row < s1 ? __ldcg(p.partial + static_cast<int64_t>(t + u * per_row) * p.rows + r) : make_float2(-INFINITY, 0.f);
-          mn = fmaxf(mn, pz[u].x);
-        }
-        const float ref = mn == -INFINITY ? 0.f : mn;
-        z *= exp2f(m - ref);
+      for (int u = 0; u < 8; ++u) mn = fmaxf(mn, pz[u].x);
+      const float ref = mn == -INFINITY ? 0.f : mn;
+      z *= exp2f(m - ref);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) z += pz[u].y * exp2f(pz[u].x - ref);
-        m = mn;
-      }
+      for (int u = 0; u < 8; ++u) z += pz[u].y * exp2f(pz[u].x - ref);
+      m = mn;
+      t += 8 * per_row;
+      if (t < s1) load_segments(r, t, pz);
     }
     for (int o = 1; o < per_row; o <<= 1) {
       const float m2 = __shfl_xor_sync(0xffffffffu, m, o), z2 = __shfl_xor_sync(0xffffffffu, z, o);
@@ -540,7 +551,7 @@ __global__ void __launch_bounds__(kSpSumThreads, 4) split_scores_kernel(const Sc
       z = z * exp2f(m - ref) + z2 * exp2f(m2 - ref);
       m = mn;
     }
-    if (r < p.rows && threadIdx.x % per_row == 0) lse_all[r] = m + log2f(z) + p.log2_group;
+    if (r < p.rows && part == 0) lse_all[r] = m + log2f(z) + p.log2_group;
   }
   __syncthreads();
   for (int i0 = blockIdx.x * kSpSumKeys + warp * 8; i0 < min(P, static_cast<int>(blockIdx.x + 1) * kSpSumKeys);
