@@ -34,9 +34,9 @@ std::atomic<int> g_test_two_sweeps{0};     // 1: never take the single-sweep ker
 constexpr size_t kAlign = 256;
 constexpr int kPartialChunk = 128;   // keys per partial slot of the fp32-pipe path (sizes the workspace)
 static_assert(kPartialChunk == kGenTile, "one partial per tile");
-// fp32-pipe path: logits are kept between its passes up to this size.  Scores of 32 / 8 heads, d = 128, 32 window rows, kept
-// against formed again: 8192 tokens 79 / 125 us, 32768 281 / 413, 65536 (256 MB) 626 / 807; 64 / 8 heads x 64 rows in bf16,
-// 16384 tokens (256 MB) 567 / 916.  With few rows and long contexts it is the other way round, because every CTA of the sums
+// fp32 scores: logits are kept between the passes up to this size.  Scores of 32 / 8 heads, d = 128, 32 window rows, kept
+// (then on the tensor cores) against formed again: 8192 tokens 33 / 125 us, 32768 107 / 413, 65536 (256 MB) 202 / 807; on the fp32
+// pipe, 64 / 8 heads x 64 rows in bf16, 16384 tokens (256 MB) 567 / 916.  With few rows and long contexts it is the other way round, because every CTA of the sums
 // merges all partials: 8 rows x 4 heads, 65536 tokens (64 MB) 289 / 266, 131072 715 / 524; d = 64, 32768 85 / 78.
 constexpr size_t kMaxLogitBytes = size_t{256} << 20;
 
@@ -376,7 +376,7 @@ int launch_logit_tiles(ScoreParams& sp, int batch, cudaStream_t st) {
 // fp32 rows as triples of bfloat16 on the tensor cores (pkv_score_split.cuh).  Returns the CTAs to take, 0: not for this call.
 // From 33 window rows on; with up to 32 the fp32 pipe is faster (scores, fp32 pipe / split: 32 rows, 32 heads, 2000 keys,
 // d = 128 28.6 / 30.3 us; 32 rows, 8 heads, 1000 keys 14.0 / 17.9; 16 rows, 2 heads, 512 keys, d = 64 8.8 / 11.2; 64 rows, 2 heads, 8000
-// keys, d = 64 20.5 / 19.8; 64 rows, 8 heads, 4001 keys, d = 128 27.3 / 25.6; 384 rows, 8 heads, 3000 keys 121 / 47).
+// keys, d = 64 20.5 / 18.1; 64 rows, 8 heads, 4001 keys, d = 128 27.3 / 22.6; 384 rows, 8 heads, 3000 keys 121 / 40).
 constexpr int kSplitMinRows = 32;
 int split_grid(const ScoreParams& sp, int batch, int max_n, int sms) {
   if (!sp.logits || sp.stats_only || sp.lse_in != sp.lse2 || sp.rows <= kSplitMinRows || sp.rows > 8192) return 0;
@@ -495,9 +495,11 @@ int launch_scores_tc(const pkv_config* c, const pkv_tensor& q, const pkv_tensor&
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return PKV_ERR_CUDA;
   if (dev >= 64 || !attr_done[dev]) {
-    if (cudaFuncSetAttribute(score_resident_kernel<D, kRsStages>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(score_resident_kernel<D, kRsStages, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              RsSmem<D, kRsStages>::kTotal) != cudaSuccess ||
-        cudaFuncSetAttribute(score_resident_kernel<D, kRsStagesShort>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(score_resident_kernel<D, kRsStagesShort, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             RsSmem<D, kRsStagesShort>::kTotal) != cudaSuccess ||
+        cudaFuncSetAttribute(score_resident_kernel<D, kRsStagesShort, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              RsSmem<D, kRsStagesShort>::kTotal) != cudaSuccess ||
         cudaFuncSetAttribute(score_tc_kernel<D, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcSmem<D>::kTotal) !=
             cudaSuccess ||
@@ -567,9 +569,10 @@ int launch_scores_tc(const pkv_config* c, const pkv_tensor& q, const pkv_tensor&
       cluster *= 2;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(cluster * sp.num_kv_heads, batch);
-    cfg.blockDim = dim3(kRsThreads);
     // at most 8 tiles per CTA: three K stages and 256 TMEM columns do, and two such CTAs fit on an SM
-    const bool small = (tiles_max + cluster - 1) / cluster <= 8;
+    const int per_cta = (tiles_max + cluster - 1) / cluster;
+    const bool small = per_cta <= 8, one = per_cta < kRsSplitTiles;
+    cfg.blockDim = dim3(rs_threads(one ? 1 : 2));
     cfg.dynamicSmemBytes = small ? RsSmem<D, kRsStagesShort>::kTotal : RsSmem<D, kRsStages>::kTotal;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -581,8 +584,9 @@ int launch_scores_tc(const pkv_config* c, const pkv_tensor& q, const pkv_tensor&
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if ((small ? cudaLaunchKernelEx(&cfg, score_resident_kernel<D, kRsStagesShort>, q_map, k_map, tp)
-               : cudaLaunchKernelEx(&cfg, score_resident_kernel<D, kRsStages>, q_map, k_map, tp)) != cudaSuccess)
+    if ((one ? cudaLaunchKernelEx(&cfg, score_resident_kernel<D, kRsStagesShort, 1>, q_map, k_map, tp)
+             : small ? cudaLaunchKernelEx(&cfg, score_resident_kernel<D, kRsStagesShort, 2>, q_map, k_map, tp)
+                     : cudaLaunchKernelEx(&cfg, score_resident_kernel<D, kRsStages, 2>, q_map, k_map, tp)) != cudaSuccess)
       return PKV_ERR_CUDA;
     mark(st, "scores_resident");
     return check_launch();

@@ -15,9 +15,10 @@
 // K is read once, the contraction runs once, and one launch replaces two.  Taken for R = G * alpha <= 32 window
 // rows per KV head (multi-head attention with the usual windows) and contexts of at most 8 x 2048 keys; everything
 // else goes to the two-sweep kernels.  Warp roles: warp 0 = TMA producer, warp 1 = MMA issuer and TMEM owner,
-// warps 2..9 = epilogue (two per quarter of the TMEM lanes, each for half of the window rows: with one for all rows, a layer
-// call at 4096 keys x 32 heads took 28.1 us, 27.0 now; 32 such layers on four streams 324, 314; and a thread's pairs of half the rows
-// fit 96 registers, so that two such CTAs still share an SM).  Every wait on an mbarrier is bounded as in the
+// warps 2.. = epilogue, one or two per quarter of the TMEM lanes; two take half of the window rows each, from kRsSplitTiles tiles
+// a CTA on (4096 keys x 32 heads, 8 tiles a CTA: layer call 28.1 us with one, 27.0 with two, 32 layers on four streams 324, 314; 1673
+// keys, 4 tiles: 18.3, 19.2, the halves' meeting costs more than they save.  A thread's pairs of half the rows fit 96
+// registers, so that two such CTAs still share an SM).  Every wait on an mbarrier is bounded as in the
 // two-sweep kernels; a CTA that gave up still walks through the two cluster barriers, so its peers are never
 // left waiting, and the status word gets kStatusWaitExpired.
 #pragma once
@@ -28,7 +29,8 @@
 
 namespace pkv {
 
-constexpr int kRsThreads = 320;             // producer, MMA issuer, eight epilogue warps
+constexpr int kRsSplitTiles = 6;            // tiles a CTA from which two epilogue warps share a quarter of the TMEM lanes
+__host__ __device__ constexpr int rs_threads(int halves) { return 64 + 128 * halves; }   // producer, MMA issuer, epilogue
 constexpr int kRsRows = 32;                 // window rows (columns of a tile's accumulator)
 constexpr int kRsTileKeys = 128;
 constexpr int kRsMaxTiles = 512 / kRsRows;  // tiles a CTA keeps in its 512 TMEM columns
@@ -61,16 +63,20 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&v)[32]) {
       : "memory");
 }
 
-// grid (cluster * H_kv, batch), cluster (cluster, 1, 1), block kRsThreads, dynamic shared memory RsSmem<D, STAGES>::kTotal.
+__device__ __forceinline__ void rs_load(uint32_t taddr, uint32_t (&v)[16]) { tc_ld16(taddr, v); }
+__device__ __forceinline__ void rs_load(uint32_t taddr, uint32_t (&v)[32]) { tc_ld32(taddr, v); }
+
+// grid (cluster * H_kv, batch), cluster (cluster, 1, 1), block rs_threads(HALVES), dynamic shared memory RsSmem<D, STAGES>::kTotal.
 // Uses of TcParams: seq (n, prefix, alpha), num_kv_heads, group, rows (<= 32), fp16, early, scale_log2, log2_group,
 // scores, ld_scores, status, wait_clocks.
-template <int D, int STAGES>
-__global__ void __launch_bounds__(kRsThreads, STAGES == kRsStagesShort ? 2 : 1)
+// HALVES: epilogue warps per quarter of the TMEM lanes.
+template <int D, int STAGES, int HALVES>
+__global__ void __launch_bounds__(rs_threads(HALVES), STAGES == kRsStagesShort ? 2 : 1)
 score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                       const TcParams p) {
   namespace cg = cooperative_groups;
   using L = RsSmem<D, STAGES>;
-  constexpr int kHalves = D / 64;
+  constexpr int kHalves = D / 64, kThreads = rs_threads(HALVES);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + (-smem_u32(smem_raw) & 1023u);   // (an offset, so that accesses stay known as shared memory)
   uint8_t* q_s = smem + L::kQOff;
@@ -79,7 +85,7 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
   uint64_t* bars = reinterpret_cast<uint64_t*>(misc);          // [0..5] k_full, [6..11] k_empty, [12] q_full, [13..28] t_full
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 260);
-  float2* warp_stat = reinterpret_cast<float2*>(misc + 512);   // [8 epilogue warps][16 rows] (maximum, sum)
+  float2* warp_stat = reinterpret_cast<float2*>(misc + 512);   // [epilogue warps][their rows] (maximum, sum)
   float2* cta_stat = reinterpret_cast<float2*>(misc + 1536);   // [32]: read by the other CTAs of the cluster
 
   cg::cluster_group cluster = cg::this_cluster();
@@ -113,7 +119,7 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // rows of the Q tile beyond R stay zero (TMA only ever writes R rows)
-  for (int i = threadIdx.x; i < L::kQBytes / 16; i += kRsThreads) reinterpret_cast<uint4*>(q_s)[i] = make_uint4(0, 0, 0, 0);
+  for (int i = threadIdx.x; i < L::kQBytes / 16; i += kThreads) reinterpret_cast<uint4*>(q_s)[i] = make_uint4(0, 0, 0, 0);
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(tmem_cols)
@@ -202,7 +208,7 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
   //      2^(x - maximum) over the thread's own keys (x = logit in log2 units; a row (g, jj) sees keys 0 .. P + jj)
   float lse2 = 0.f;                                            // of row `lane`, after the cluster barrier
   if (epi) {
-    constexpr int kHalf = kRsRows / 2;
+    constexpr int kHalf = kRsRows / HALVES;                    // window rows of this warp
     float m[kHalf], z[kHalf];
 #pragma unroll
     for (int j = 0; j < kHalf; ++j) { m[j] = -INFINITY; z[j] = 0.f; }
@@ -212,7 +218,7 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
       if (!ok) break;
       tc_fence_after();
       uint32_t v[kHalf];
-      tc_ld16(lane_addr + t * kRsRows + rh * kHalf, v);
+      rs_load(lane_addr + t * kRsRows + rh * kHalf, v);
       tc_wait_ld();
       if (whole(t)) {
 #pragma unroll
@@ -236,13 +242,13 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
       }
     }
     // lanes, then the four warps, then (behind the cluster barrier) the CTAs.  Over the lanes by halving: lane bit s picks
-    // the half of the rows a lane keeps, so that after four exchanges lanes 2r and 2r + 1 hold row r, after a fifth both
-    // of it (a butterfly over all rows takes ten times the merges and took 5.4 us of the 28 us that scores and selection
+    // the half of the rows a lane keeps, so that after five exchanges lane r holds row r (with half of the rows lanes 2r and
+    // 2r + 1 after four, and the fifth merges these; a butterfly over all rows takes ten times the merges and took 5.4 us of the 28 us that scores and selection
     // of 4096 keys needed)
     {
       int cnt = kHalf;
 #pragma unroll
-      for (int s = 16; s >= 2; s >>= 1) {
+      for (int s = 16; s >= HALVES; s >>= 1) {
         const int half = cnt / 2;
         const bool upper = (lane & s) != 0;
 #pragma unroll
@@ -255,10 +261,10 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
           }
         cnt = half;
       }
-      merge(m[0], z[0], __shfl_xor_sync(0xffffffffu, m[0], 1), __shfl_xor_sync(0xffffffffu, z[0], 1));
+      if (HALVES == 2) merge(m[0], z[0], __shfl_xor_sync(0xffffffffu, m[0], 1), __shfl_xor_sync(0xffffffffu, z[0], 1));
     }
-    if (!(lane & 1)) warp_stat[(warp - 2) * kHalf + (lane >> 1)] = make_float2(m[0], z[0]);
-    asm volatile("bar.sync 1, 256;" ::: "memory");             // the eight epilogue warps
+    if (lane % HALVES == 0) warp_stat[(warp - 2) * kHalf + lane / HALVES] = make_float2(m[0], z[0]);
+    asm volatile("bar.sync 1, %0;" ::"n"(HALVES * 128) : "memory");           // the epilogue warps
     if (warp == 2) {
       const float2* of_row = warp_stat + (lane / kHalf) * 4 * kHalf + lane % kHalf;
       float2 r = of_row[0];
@@ -280,44 +286,48 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
   // ---- scores of the prefix keys, from the logits still in TMEM (loads double buffered)
   if (epi) {
     pdl_wait();                                                // the score buffer may still be read by the call before
-    constexpr int kHalf = kRsRows / 2;
+    constexpr int kHalf = kRsRows / HALVES;
     float nl[kHalf];
 #pragma unroll
     for (int j = 0; j < kHalf; ++j) {
       const float l = __shfl_sync(0xffffffffu, lse2, rh * kHalf + j);
       nl[j] = rh * kHalf + j < p.rows ? -l : -INFINITY;
     }
-    // each half of the rows into its place over the K tiles, which nobody reads any more; then the halves meet
+    float* srow = p.scores + (static_cast<int64_t>(b) * p.num_kv_heads + h) * p.ld_scores;
+    // with two warps, each half of the rows goes to its place over the K tiles, which nobody reads any more; then the halves meet
     float* part = reinterpret_cast<float*>(k_s);               // [2][tiles][128]
-    auto half_sum = [&](int t, const uint32_t (&v)[kHalf]) {
+    auto sum_rows = [&](int t, const uint32_t (&v)[kHalf]) {
       float s0 = 0.f, s1 = 0.f;
 #pragma unroll
       for (int j = 0; j < kHalf; j += 2) {                     // a prefix key is seen by every row: no mask
         s0 += ex2(fmaf(__uint_as_float(v[j]), c2, nl[j]));
         s1 += ex2(fmaf(__uint_as_float(v[j + 1]), c2, nl[j + 1]));
       }
-      part[(rh * kRsMaxTiles + t) * kRsTileKeys + lane_row] = s0 + s1;
+      const int i = (tile0 + t) * kRsTileKeys + lane_row;
+      if (HALVES == 2) part[(rh * kRsMaxTiles + t) * kRsTileKeys + lane_row] = s0 + s1;
+      else if (i < P) srow[i] = s0 + s1;
     };
     if (ok && T > 0) {
       const uint32_t from = lane_addr + rh * kHalf;
       uint32_t va[kHalf], vb[kHalf];
-      tc_ld16(from, va);
+      rs_load(from, va);
       for (int t = 0; t < T; t += 2) {
         tc_wait_ld();
-        if (t + 1 < T) tc_ld16(from + (t + 1) * kRsRows, vb);
-        half_sum(t, va);
+        if (t + 1 < T) rs_load(from + (t + 1) * kRsRows, vb);
+        sum_rows(t, va);
         if (t + 1 < T) {
           tc_wait_ld();
-          if (t + 2 < T) tc_ld16(from + (t + 2) * kRsRows, va);
-          half_sum(t + 1, vb);
+          if (t + 2 < T) rs_load(from + (t + 2) * kRsRows, va);
+          sum_rows(t + 1, vb);
         }
       }
     }
-    asm volatile("bar.sync %0, 64;" ::"r"(2 + quarter) : "memory");            // (reached whether a wait ran out or not)
-    float* srow = p.scores + (static_cast<int64_t>(b) * p.num_kv_heads + h) * p.ld_scores;
-    for (int t = rh; t < T && ok; t += 2) {
-      const int i = (tile0 + t) * kRsTileKeys + lane_row;
-      if (i < P) srow[i] = part[t * kRsTileKeys + lane_row] + part[(kRsMaxTiles + t) * kRsTileKeys + lane_row];
+    if constexpr (HALVES == 2) {
+      asm volatile("bar.sync %0, 64;" ::"r"(2 + quarter) : "memory");          // (reached whether a wait ran out or not)
+      for (int t = rh; t < T && ok; t += 2) {
+        const int i = (tile0 + t) * kRsTileKeys + lane_row;
+        if (i < P) srow[i] = part[t * kRsTileKeys + lane_row] + part[(kRsMaxTiles + t) * kRsTileKeys + lane_row];
+      }
     }
   }
   cluster.sync();                                              // barrier 2: nobody reads this CTA's shared memory any more

@@ -479,7 +479,6 @@ constexpr int kSelClusterSlice = 8192;     // a cluster doubles (up to 8 CTAs) w
 constexpr int kSelCopyBytes = 128 << 10;   // ... or while a CTA would copy more than this and SMs are idle
 constexpr int kSelCommonCandidates = 4096; // more expected candidates (k per CTA) than this: one bound for the cluster
 constexpr int kSelCrowd = 1024;            // candidates of a CTA beyond 2 k that its bound may let through before it is refined
-constexpr int kSelPrefetchPieces = 32;     // rows of at least this many 16-byte pieces are prefetched once they are known
 constexpr int kSelEvenRows = 1024;         // lists of at least this many rows are copied by the whole cluster evenly
 
 // Position i of the staged scores in shared memory: four floats of padding after every 32.
@@ -894,28 +893,30 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
     // Most candidates lie within an octave of the bound and a few far above it: the first pass divides the lowest eighth of
     // the range, what lies above counts in its last bin.  (Over the whole range a bin held some 50 of 3600 candidates, and
     // a second pass followed.)
+    // In short slices the whole range is divided and every warp ranks the last ones for itself, two barriers less (1146 to 1989
+    // positions: layer calls of 20.5 to 24.2 us take 0.7 to 0.9 more the other way).
+    constexpr bool kLong = THREADS > 256;
     uint32_t want = static_cast<uint32_t>(k), T = 0, need_eq = 0;
-    int shift = max(0, 22 - 3 - __clz(top - base));
+    int shift = max(0, 22 - (kLong ? 3 : 0) - __clz(top - base));
     uint32_t span = 0xffffffffu;                            // keys base .. base + span take part
     for (int pass = 0;; ++pass) {
       uint32_t* hc = local[pass & 1];
       for (int i = my_first; i < my_n; i += my_step) {
         const uint32_t x = key_at(my_c, i);
-        if (x >= base && x - base <= span) atomicAdd(&hc[min((x - base) >> shift, kSelBinsLin - 1u)], 1u);
+        if (x >= base && x - base <= span) atomicAdd(&hc[kLong ? min((x - base) >> shift, kSelBinsLin - 1u) : (x - base) >> shift], 1u);
       }
       __syncthreads();
       uint32_t digit = 0, above = 0;
       sel_find_from_top<THREADS>(hc, rows, want, digit, above);
-      const bool beyond = digit == kSelBinsLin - 1u && min(span, top - base) >> shift > digit;      // in what was put together
+      const bool beyond = kLong && digit == kSelBinsLin - 1u && min(span, top - base) >> shift > digit;      // in what was put together
       want -= above;
       base += digit << shift;
       const uint32_t in_bin = hc[digit];
-      // All but a few of the rows to copy are known.  Short slices' rows of 512 bytes go into the L2 ahead of the copy (8101 fp32
-      // keys, d = 128, 700 rows a head: 58.0 us, 61.2 without).  Not in the other instances, where the prefetches cost more
-      // than they save, the search's own accesses queueing behind them: 4096 keys 28.8 us, 28.1 without; 32768 keys 51.6, 50.9;
-      // three steps of 2 x 10000 keys 32.9, 32.2.
-      if constexpr (THREADS == 256) {
-        if (pass == 0 && p.k_out != nullptr && p.pieces >= kSelPrefetchPieces) {
+      // All but a few of the rows to copy are known: in short slices they go into the L2 ahead of the copy.  Not in the other
+      // instances, where the prefetches cost more than they save, the search's own accesses queueing behind them: 4096 keys 28.8 us,
+      // 28.1 without; 32768 keys 51.6, 50.9; three steps of 2 x 10000 keys 32.9, 32.2.
+      if constexpr (!kLong) {
+        if (pass == 0 && p.k_out != nullptr) {
           const int64_t ks = p.k.st * p.elem_bytes, vs = p.v.st * p.elem_bytes;
           const char* kb = static_cast<const char*>(p.k.ptr) + (b * p.k.sb + h * p.k.sh + static_cast<int64_t>(lo) * p.k.st) * p.elem_bytes;
           const char* vb = static_cast<const char*>(p.v.ptr) + (b * p.v.sb + h * p.v.sh + static_cast<int64_t>(lo) * p.v.st) * p.elem_bytes;
@@ -939,6 +940,19 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 2) select_kerne
           if (x >= base && x - base <= width) few[atomicAdd(&few_n, 1u)] = x;
         }
         __syncthreads();
+        if constexpr (!kLong) {
+          const uint32_t x = lane < static_cast<int>(in_bin) ? few[lane] : 0u;
+          uint32_t gt = 0, ge = 0;
+          for (int q = 0; q < static_cast<int>(in_bin); ++q) {
+            const uint32_t o = __shfl_sync(full, x, q);
+            gt += o > x ? 1u : 0u;
+            ge += o >= x ? 1u : 0u;
+          }
+          const uint32_t hit = __ballot_sync(full, lane < static_cast<int>(in_bin) && gt < want && want <= ge);
+          T = __shfl_sync(full, x, __ffs(hit) - 1);
+          need_eq = want - __shfl_sync(full, gt, __ffs(hit) - 1);
+          break;
+        }
         if (warp == 0) {                                    // (all for themselves with shuffles: 0.5 us more at 1024 threads)
           const uint32_t x = few[lane];                     // (zeros behind the last one)
           uint32_t gt = 0, ge = 0;
