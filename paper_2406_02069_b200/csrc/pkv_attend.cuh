@@ -15,6 +15,8 @@
 // The normalisers are final before the pass starts, so the accumulators are never rescaled.  The factor
 // 2^15 keeps binary16 probabilities of long contexts out of the subnormal range; it is exact.
 //
+// Two kernels: window_attend_kernel, described here, for more than 128 window rows, and window_attend_narrow_kernel for up to 128.
+//
 // Warp roles: 0 = TMA producer of Q and K, 1 = MMA issuer and TMEM owner, 2 = TMA producer of V,
 // 4..19 = epilogue in four groups of four warps (TMEM lane quarter = warp % 4), all on the same K tile.
 // Per tile the issuer queues ONE product K Q^T over all window rows (N up to 256: an MMA costs the issuing

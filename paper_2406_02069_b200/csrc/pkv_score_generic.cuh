@@ -1,8 +1,9 @@
 // Window-score kernels on the plain fp32 pipes (Section 4.2.2, Eq. 2 and Eq. 3).
 //
 // These cover every dtype / shape the boundary admits (fp32 inputs, any window, any group size) and are the path of
-// small fp32 problems.  The tensor-core kernels in pkv_score_tc.cuh take over for 16-bit inputs when their shape rules
-// hold.
+// fp32 problems of few window rows, of calls without room for the logits and of handed-in normalisers.  The tensor-core kernels in
+// pkv_score_tc.cuh take over for 16-bit inputs when their shape rules hold, those in pkv_score_split.cuh for fp32 ones of more
+// than 32 window rows.
 //
 // The score of a key mixes softmax rows that each have their own normaliser, so the normalisers must be known before
 // any score can be formed:

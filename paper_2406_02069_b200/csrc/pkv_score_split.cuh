@@ -14,14 +14,15 @@
 //
 // Why: 2 R n d flops per KV head are the bound of the fp32 pipe (8101 keys x 8 heads x 128 rows x 128 channels: 34 us at the
 // 63 TFLOP/s that it reaches); six products on the tensor cores take 8 us.  Scores of that shape, both kernels: 79 us on
-// the fp32 pipe, 36 here; the layer call 101 -> 58.  Error of the scores against 64 bits (2-norm / largest, relative): 2.1e-7 /
-// 8.6e-7 on the fp32 pipe, 1.8e-7 / 5.4e-7 here, and no larger at ten other shapes (16 to 384 rows, d = 64 and 128).
-// What is left is latency: the first tile waits for Q's parts, a tile takes twice the 1536 clocks of its MMAs.
+// the fp32 pipe, 33 here; the layer call 101 -> 54.  Error of the scores against 64 bits (2-norm / largest, relative): 2.1e-7 /
+// 8.6e-7 on the fp32 pipe, 1.5e-7 / 5.4e-7 here, and no larger at ten other shapes (16 to 384 rows, d = 64 and 128).
+// What is left: the first tile waits some 4 us for Q's parts, a tile takes some 2300 clocks where its MMAs take 1536, and the second
+// kernel reads the logits at 3.3 TB/s out of the L2 (10 us).
 //
-// Warps 0..7 load a tile of 64 keys into registers, split it and store the parts swizzled as the MMAs want them (the loads of the next
-// tile are under way while they wait for room); warp 16 issues the MMAs; warps 8..15 take the logits out of TMEM, a
-// thread per window row, in two teams that take the tiles in turn.  Tiles of 64 keys and not 128: two stages of parts fit beside Q's, and the
-// tiles spread more evenly over the CTAs.
+// Warps 0..7 load a tile of 64 keys into registers, split it and store the parts swizzled as the MMAs want them (the loads of
+// the next tile are under way while they wait for room); warp 16 issues the MMAs; warps 8..15 take the logits out of TMEM, a
+// thread per window row, in two teams that take the tiles in turn (all of them on every tile: 1.8 us a tile, not 1.2).
+// Tiles of 64 keys and not 128: two stages of parts fit beside Q's, and the tiles spread more evenly over the CTAs.
 //
 // Infinities, NaN and magnitudes of 2^90 or more raise a flag for their tile, whose logits are then formed by plain fp32
 // multiply-adds.  (Below that, parts that are subnormal and lost change no logit by more than 2^-28.)
