@@ -24,8 +24,10 @@
 // thread per window row, in two teams that take the tiles in turn (all of them on every tile: 1.8 us a tile, not 1.2).
 // Tiles of 64 keys and not 128: two stages of parts fit beside Q's, and the tiles spread more evenly over the CTAs.
 //
-// Infinities, NaN and magnitudes of 2^90 or more raise a flag for their tile, whose logits are then formed by plain fp32
-// multiply-adds.  (Below that, parts that are subnormal and lost change no logit by more than 2^-28.)
+// Infinities, NaN and magnitudes of 2^59 or more raise a flag for their tile, whose logits are then formed by plain fp32
+// multiply-adds.  Below that nothing overflows that the multiply-adds would not: the parts of 128 products add up to less
+// than 2^126 in magnitude.  (Parts have either sign: of products near 2^128 some would become infinities of opposite
+// signs, and NaN of a logit that is -inf.)  And parts that are subnormal and lost change no logit by more than 2^-59.
 #pragma once
 
 #include "pkv_score_generic.cuh"
@@ -41,7 +43,7 @@ constexpr int kSpStages = 2;                // of K parts, and of accumulators
 constexpr int kSpAccs = 2;                  // accumulators of a tile, each for its share of the channels
 constexpr int kSpMaxGrid = 256;
 constexpr int kSpPrefetch = 8;              // K tiles (32 KB each at d = 128) on their way into the L2 ahead of their use
-constexpr float kSpMost = 1.2379400392853803e27f;              // 2^90
+constexpr float kSpMost = 5.7646075230342349e17f;              // 2^59
 constexpr int kSpSumKeys = 128;             // split_scores_kernel: keys per CTA
 constexpr int kSpSumThreads = 256;
 
