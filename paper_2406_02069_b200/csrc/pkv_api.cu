@@ -386,7 +386,8 @@ int split_grid(const ScoreParams& sp, int batch, int max_n, int sms) {
   tiles *= sp.num_kv_heads * blocks;
   // a segment of row statistics per CTA and unit: the workspace has room for two per 128 keys of a head
   const long long room = 2ll * batch * sp.num_kv_heads * ((max_n + kPartialChunk - 1) / kPartialChunk) - units;
-  return static_cast<int>(std::max<long long>(0, std::min(std::min<long long>(std::min(sms, kSpMaxGrid), tiles), room)));
+  const long long grid = std::max<long long>(0, std::min(std::min<long long>(std::min(sms, kSpMaxGrid), tiles), room));
+  return grid * (kSpMaxTiles - 1) >= tiles ? static_cast<int>(grid) : 0;
 }
 
 template <int D>

@@ -25,7 +25,7 @@
 // Tiles of 64 keys and not 128: two stages of parts fit beside Q's, and the tiles spread more evenly over the CTAs.
 //
 // Infinities, NaN and magnitudes of 2^59 or more raise a flag for their tile, whose logits are then formed by plain fp32
-// multiply-adds.  Below that nothing overflows that the multiply-adds would not: the parts of 128 products add up to less
+// multiply-adds, once the CTA is through with the others (sp_plain_tiles).  Below that nothing overflows that the multiply-adds would not: the parts of 128 products add up to less
 // than 2^126 in magnitude.  (Parts have either sign: of products near 2^128 some would become infinities of opposite
 // signs, and NaN of a logit that is -inf.)  And parts that are subnormal and lost change no logit by more than 2^-59.
 #pragma once
@@ -43,6 +43,7 @@ constexpr int kSpStages = 2;                // of K parts, and of accumulators
 constexpr int kSpAccs = 2;                  // accumulators of a tile, each for its share of the channels
 constexpr int kSpMaxGrid = 256;
 constexpr int kSpPrefetch = 8;              // K tiles (32 KB each at d = 128) on their way into the L2 ahead of their use
+constexpr int kSpMaxTiles = 32768;          // of a CTA: a bit for each (with one CTA 256 MB of logits take at most 31800, of 33 rows each)
 constexpr float kSpMost = 5.7646075230342349e17f;              // 2^59
 constexpr int kSpSumKeys = 128;             // split_scores_kernel: keys per CTA
 constexpr int kSpSumThreads = 256;
@@ -55,7 +56,7 @@ struct SpSmem {
   static constexpr int kQOff = 0;
   static constexpr int kKOff = 3 * kQPart;
   static constexpr int kMiscOff = kKOff + kSpStages * 3 * kKPart;
-  static constexpr int kMiscBytes = 4096;
+  static constexpr int kMiscBytes = 2048 + kSpMaxTiles / 8;
   static constexpr int kTotal = kMiscOff + kMiscBytes + 1024;  // + slack for manual 1024-byte alignment
 };
 
@@ -119,9 +120,110 @@ __device__ __forceinline__ void sp_store16(uint32_t to, const uint4& v) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(to), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
+// Keys of a unit's head; window row r of it (of its KV head, over all blocks).
+__device__ __forceinline__ const float* sp_keys(const ScoreParams& p, const TcItem& w, int blocks) {
+  return static_cast<const float*>(p.k.ptr) + w.b * p.k.sb + (w.h / blocks) * p.k.sh;
+}
+__device__ __forceinline__ const float* sp_q_row(const ScoreParams& p, const TcItem& w, int blocks, int r) {
+  const int alpha = p.seq.alpha;
+  return static_cast<const float*>(p.q.ptr) + w.b * p.q.sb + static_cast<int64_t>((w.h / blocks) * p.group + r / alpha) * p.q.sh +
+         (r % alpha) * p.q.st;
+}
+
+// The flagged tiles of a CTA, after all others: logits by multiply-adds, each summed in the order of its channels as on the fp32
+// pipe, and their row statistics added to those of the CTA's runs.  By all threads, with the shared memory that the parts have
+// left: a unit's window rows channel-major, a tile's keys row-major, two window rows and eight keys per thread.
+// Scores of 8101 keys x 8 heads x 128 rows with every tile flagged: 115 us, one tile in a head 43 (none: 33, the fp32 pipe 79).  In the epilogue's
+// own loop, a window row and a key at a time, 4430 and 660; eight keys at a time 445, and every call 0.9 us longer by the registers.
+template <int D>
+__device__ __forceinline__ void sp_plain_tiles(const ScoreParams& p, float* qs, float* ks, float2* part, const uint32_t* flagged, int item0,
+                                               int ntiles) {
+  constexpr int kThreads = 512, kGroups = 8, kKeys = kSpKeys / kGroups;        // groups of threads, each with its keys
+  static_assert(kSpRows / 2 * kGroups == kThreads, "two rows per thread");
+  const int tid = threadIdx.x, row = tid % (kSpRows / 2) * 2, kg = tid / (kSpRows / 2);
+  const int blocks = (p.rows + kSpRows - 1) / kSpRows, units = p.num_kv_heads * blocks;
+  const int32_t* off = p.seq.stat_off;
+  int cur_b = -1, cur_h = -1;
+  TcItem w = tc_item(off, p.seq.batch, units, item0);
+  for (int it = 0; it < ntiles; ++it, tc_next<false>(off, p.seq.batch, units, w)) {
+    if (!((flagged[it >> 5] >> (it & 31)) & 1u)) continue;
+    const int r0 = (w.h % blocks) * kSpRows, n = p.seq.n[w.b], key0 = w.c * kSpKeys;
+    __syncthreads();                                           // the tile before has been read
+    if (tid < kThreads) {
+      if (w.b != cur_b || w.h != cur_h) {
+        const int x = tid % kSpRows;
+        for (int c = tid / kSpRows * 4; c < D; c += kThreads / kSpRows * 4) {
+          const float4 f = r0 + x < p.rows ? *reinterpret_cast<const float4*>(sp_q_row(p, w, blocks, r0 + x) + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+          qs[c * kSpRows + x] = f.x;
+          qs[(c + 1) * kSpRows + x] = f.y;
+          qs[(c + 2) * kSpRows + x] = f.z;
+          qs[(c + 3) * kSpRows + x] = f.w;
+        }
+      }
+      for (int i = tid; i < kSpKeys * D / 4; i += kThreads) {
+        const int key = key0 + i / (D / 4);
+        reinterpret_cast<float4*>(ks)[i] = key < n ? *reinterpret_cast<const float4*>(sp_keys(p, w, blocks) + key * p.k.st + i % (D / 4) * 4)
+                                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+    cur_b = w.b;
+    cur_h = w.h;
+    __syncthreads();
+    if (tid < kThreads) {
+      unsigned long long x2[kKeys] = {};
+#pragma unroll 2
+      for (int c = 0; c < D; c += 4) {
+        unsigned long long q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) q[u] = *reinterpret_cast<const unsigned long long*>(qs + (c + u) * kSpRows + row);
+#pragma unroll
+        for (int j = 0; j < kKeys; ++j) {
+          const float4 k = *reinterpret_cast<const float4*>(ks + (kg * kKeys + j) * D + c);
+          x2[j] = fma2(q[0], pack2(k.x, k.x), x2[j]);
+          x2[j] = fma2(q[1], pack2(k.y, k.y), x2[j]);
+          x2[j] = fma2(q[2], pack2(k.z, k.z), x2[j]);
+          x2[j] = fma2(q[3], pack2(k.w, k.w), x2[j]);
+        }
+      }
+      const int first = key0 + kg * kKeys;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int r = r0 + row + i, last = min(p.seq.prefix[w.b] + r % p.seq.alpha, n - 1);
+        float* to = p.logits + ((static_cast<int64_t>(w.b) * p.num_kv_heads + w.h / blocks) * p.ld_logits + first) * p.rows + r;
+        float x[kKeys], m = -INFINITY, z = 0.f;
+#pragma unroll
+        for (int j = 0; j < kKeys; ++j, to += p.rows) {
+          float even, odd;
+          unpack2(x2[j], even, odd);
+          x[j] = (i == 0 ? even : odd) * p.scale_log2;
+          if (r < p.rows) *to = x[j];                          // (within the padded length)
+          if (first + j > last) x[j] = -INFINITY;
+          m = fmaxf(m, x[j]);
+        }
+        const float ref = m == -INFINITY ? 0.f : m;
+#pragma unroll
+        for (int j = 0; j < kKeys; ++j) z += ex2(x[j] - ref);
+        part[kg * kSpRows + row + i] = make_float2(m, z);
+      }
+    }
+    __syncthreads();
+    if (tid < kSpRows && r0 + tid < p.rows) {
+      float2* of_run = p.partial + (static_cast<int64_t>(blockIdx.x) + w.b * units + w.h) * p.rows + r0 + tid;
+      float2 s = *of_run;
+#pragma unroll
+      for (int g = 0; g < kGroups; ++g) {
+        const float2 o = part[g * kSpRows + tid];
+        const float mn = fmaxf(s.x, o.x), ref = mn == -INFINITY ? 0.f : mn;
+        s = make_float2(mn, s.y * ex2(s.x - ref) + o.y * ex2(o.x - ref));
+      }
+      *of_run = s;
+    }
+  }
+}
+
 // grid: at most one CTA per SM, block kSpThreads, dynamic shared memory SpSmem<D>::kTotal.
 template <int D>
-__global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const ScoreParams p) {
+__global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const __grid_constant__ ScoreParams p) {
   using L = SpSmem<D>;
   constexpr int kChunks = D / 8;                               // 16-byte chunks of a part's row
   constexpr int kSteps = kSpKeys * kChunks / kSpConverters;    // chunks of a K tile per converter thread
@@ -131,9 +233,11 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
   uint64_t* bars = reinterpret_cast<uint64_t*>(misc);          // k_full, k_empty, t_full, t_empty (two of each), x_full, x_empty
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 192);                                      // (one a quarter)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 196);
+  volatile int* any_flagged = reinterpret_cast<volatile int*>(misc + 200);
   volatile int* special = reinterpret_cast<volatile int*>(misc + 256);         // [8]: tiles with values that are not split
   volatile int* q_special = reinterpret_cast<volatile int*>(misc + 288);       // [8]: the same of the units' window rows
   float2* halves = reinterpret_cast<float2*>(misc + 1024);                     // [128] statistics of the second team
+  uint32_t* flagged = reinterpret_cast<uint32_t*>(misc + 2048);                // a bit per tile of this CTA
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t bar0 = smem_u32(bars), smem0 = smem_u32(smem);
   auto k_full = [&](int s) { return bar0 + 8u * s; };
@@ -154,10 +258,11 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
     }
     for (int q = 0; q < 4; ++q) { mbar_init(x_full(q), 1); mbar_init(x_empty(q), 1); }
     mbar_init(q_full, 2 * kSpConverters / 32);
-    *abort_flag = 0;
+    *abort_flag = *any_flagged = 0;
     for (int i = 0; i < 8; ++i) special[i] = q_special[i] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  for (int i = threadIdx.x; i < kSpMaxTiles / 32; i += kSpThreads) flagged[i] = 0;
   constexpr uint32_t kCols = kSpStages * kSpAccs * kSpKeys;
   if (warp == 16) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kCols) : "memory");
@@ -181,12 +286,6 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
     ntiles = (part + 1) * nc / p.per_unit - first;
   }
   const int alpha = p.seq.alpha;
-  const float* kptr = static_cast<const float*>(p.k.ptr);
-  const float* qptr = static_cast<const float*>(p.q.ptr);
-  auto head_keys = [&](const TcItem& w) { return kptr + w.b * p.k.sb + (w.h / blocks) * p.k.sh; };
-  auto q_row = [&](const TcItem& w, int r) {
-    return qptr + w.b * p.q.sb + static_cast<int64_t>((w.h / blocks) * p.group + r / alpha) * p.q.sh + (r % alpha) * p.q.st;
-  };
   // Chunk c of row x of a part of `rows` rows: 64 channels to a row of 128 bytes, its 16-byte chunks exchanged by the row.
   auto place = [](int rows, int x, int c) { return (c >> 3) * rows * 128 + x * 128 + (((c & 7) ^ (x & 7)) << 4); };
   // Chunks [begin, end) of the window rows of w's unit, by 256 threads; returns whether this thread saw a value that is not split.
@@ -203,7 +302,7 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
         const int x = (i0 + u * kSpConverters) / kChunks, c = (i0 + u * kSpConverters) % kChunks;
         f[u][0] = f[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (r0 + x < p.rows) {
-          const float4* src = reinterpret_cast<const float4*>(q_row(w, r0 + x) + c * 8);
+          const float4* src = reinterpret_cast<const float4*>(sp_q_row(p, w, blocks, r0 + x) + c * 8);
           f[u][0] = src[0];
           f[u][1] = src[1];
         }
@@ -225,14 +324,14 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
   auto prefetch_tile = [&](const TcItem& w) {
     const int key = w.c * kSpKeys + static_cast<int>(threadIdx.x) / (D / 32);
     if (threadIdx.x < kSpKeys * (D / 32) && key < p.seq.n[w.b])
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(head_keys(w) + key * p.k.st + threadIdx.x % (D / 32) * 32));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(sp_keys(p, w, blocks) + key * p.k.st + threadIdx.x % (D / 32) * 32));
   };
   static_assert(kSpKeys * (D / 32) <= kSpConverters, "a line per thread");
   TcItem ahead = tc_item(off, p.seq.batch, units, item0);
   if (warp >= 8 && warp < 16)
     for (int i = threadIdx.x - kSpConverters; i < kSpRows * (D / 32); i += kSpConverters) {
       const int r = (ahead.h % blocks) * kSpRows + i / (D / 32);
-      if (r < p.rows) asm volatile("prefetch.global.L2 [%0];" ::"l"(q_row(ahead, r) + i % (D / 32) * 32));
+      if (r < p.rows) asm volatile("prefetch.global.L2 [%0];" ::"l"(sp_q_row(p, ahead, blocks, r) + i % (D / 32) * 32));
     }
   if (warp < 8)
     for (int it = 0; it < min(ntiles, kSpPrefetch); ++it, tc_next<false>(off, p.seq.batch, units, ahead)) prefetch_tile(ahead);
@@ -246,7 +345,7 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
     auto load_tile = [&](const TcItem& t) {
       constexpr int kRows = kSpConverters / kChunks;           // per step
       const int n = p.seq.n[t.b], key0 = t.c * kSpKeys + threadIdx.x / kChunks;
-      const float* base = head_keys(t) + key0 * p.k.st + threadIdx.x % kChunks * 8;
+      const float* base = sp_keys(p, t, blocks) + key0 * p.k.st + threadIdx.x % kChunks * 8;
 #pragma unroll
       for (int s = 0; s < kSteps; ++s) {
         if (key0 + s * kRows < n) {
@@ -385,9 +484,18 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc_fence_after();
-        const bool on_pipe = special[it & 7] | q_special[runs & 7];            // the whole tile on the fp32 pipe
+        const bool plain = special[it & 7] | q_special[runs & 7];              // left to sp_plain_tiles
+        if (plain) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) {
+            mbar_arrive(t_empty(team));
+            atomicOr(&flagged[it >> 5], 1u << (it & 31));
+            *any_flagged = 1;
+          }
+        }
 #pragma unroll 1
-        for (int half = 0; half < 2; ++half) {
+        for (int half = plain ? 2 : 0; half < 2; ++half) {
           const int key0 = w.c * kSpKeys + half * 32;
           const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + team * kSpAccs * kSpKeys + half * 32;
           unsigned long long x2[16];
@@ -408,21 +516,6 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
           float x[32];
 #pragma unroll
           for (int j = 0; j < 16; ++j) unpack2(mul2(x2[j], scale), x[2 * j], x[2 * j + 1]);
-          if (on_pipe) {
-            const float* q = q_row(w, min(r, p.rows - 1));
-#pragma unroll 1
-            for (int j = 0; j < 32; ++j) {
-              float dot = 0.f;
-              if (key0 + j < n) {
-                const float* k = head_keys(w) + (key0 + j) * p.k.st;
-#pragma unroll 4
-                for (int c = 0; c < D; ++c) dot = fmaf(q[c], k[c], dot);
-              }
-              dot *= p.scale_log2;
-#pragma unroll
-              for (int i = 0; i < 32; ++i) x[i] = i == j ? dot : x[i];
-            }
-          }
           if (half == 1) {
             tc_fence_before();
             __syncwarp();
@@ -484,6 +577,9 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const Score
   }
   tc_fence_before();
   __syncthreads();
+  if (*any_flagged && !*abort_flag)
+    sp_plain_tiles<D>(p, reinterpret_cast<float*>(smem + L::kQOff), reinterpret_cast<float*>(smem + L::kKOff),
+                      reinterpret_cast<float2*>(smem + L::kKOff + kSpKeys * D * 4), flagged, item0, ntiles);
   if (threadIdx.x == 0 && *abort_flag) atomicOr(p.status, kStatusWaitExpired);
   if (warp == 16) {
     tc_fence_after();
