@@ -428,14 +428,16 @@ int launch_scores_split(ScoreParams& sp, int batch, int max_n, int grid, cudaStr
   return check_launch();
 }
 
-// Row blocks as large as the window rows need (16-bit inputs only come here with more than 256 rows).
+// Row blocks as large as the window rows need (16-bit inputs only come here with more than 256 rows).  sweep_ctas: the caller's cap
+// on persistent sweeps, or 0; the kernels on the fp32 pipe are none.
 template <typename T, int D>
-int launch_scores_generic(ScoreParams& sp, int batch, cudaStream_t st) {
+int launch_scores_generic(ScoreParams& sp, int batch, int sweep_ctas, cudaStream_t st) {
   if constexpr (sizeof(T) == 4) {
     int max_n = 0;
     for (int b = 0; b < batch; ++b) max_n = std::max(max_n, sp.seq.n[b]);
-    const int sms = device_sm_count();
+    int sms = device_sm_count();
     if (sms <= 0) return PKV_ERR_CUDA;
+    if (sweep_ctas > 0) sms = std::min(sms, sweep_ctas);
     if (const int grid = split_grid(sp, batch, max_n, sms)) return launch_scores_split<D>(sp, batch, max_n, grid, st);
     if (sp.rows <= 32) return launch_logit_tiles<T, D, 32, 4, 4>(sp, batch, st);
     if (sp.rows <= 64) return launch_logit_tiles<T, D, 64, 4, 8>(sp, batch, st);
@@ -643,14 +645,15 @@ int run_scores(const pkv_config* c, const pkv_tensor& q, const pkv_tensor& k, co
     return c->head_dim == 64 ? launch_scores_tc<64>(c, q, k, sp, batch, max_n, w.status, st, stats)
                              : launch_scores_tc<128>(c, q, k, sp, batch, max_n, w.status, st, stats);
   }
+  const int sweep_ctas = static_cast<int>(c->sweep_ctas);
   if (c->dtype == PKV_DTYPE_FP32)
-    return c->head_dim == 64 ? launch_scores_generic<float, 64>(sp, batch, st)
-                             : launch_scores_generic<float, 128>(sp, batch, st);
+    return c->head_dim == 64 ? launch_scores_generic<float, 64>(sp, batch, sweep_ctas, st)
+                             : launch_scores_generic<float, 128>(sp, batch, sweep_ctas, st);
   if (c->dtype == PKV_DTYPE_FP16)
-    return c->head_dim == 64 ? launch_scores_generic<__half, 64>(sp, batch, st)
-                             : launch_scores_generic<__half, 128>(sp, batch, st);
-  return c->head_dim == 64 ? launch_scores_generic<__nv_bfloat16, 64>(sp, batch, st)
-                           : launch_scores_generic<__nv_bfloat16, 128>(sp, batch, st);
+    return c->head_dim == 64 ? launch_scores_generic<__half, 64>(sp, batch, sweep_ctas, st)
+                             : launch_scores_generic<__half, 128>(sp, batch, sweep_ctas, st);
+  return c->head_dim == 64 ? launch_scores_generic<__nv_bfloat16, 64>(sp, batch, sweep_ctas, st)
+                           : launch_scores_generic<__nv_bfloat16, 128>(sp, batch, sweep_ctas, st);
 }
 
 // ---------------------------------------------------------------- window attention fused with the scores
