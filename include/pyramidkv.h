@@ -549,8 +549,8 @@ int pyramidkv_compress_model_lanes(const pkv_config* cfg, pkv_lanes* lanes, int3
  *
  * pyramidkv_test_hooks: process-wide knobs read by the calls that follow.  wait_clocks > 0 replaces the bound
  * of every wait inside the tensor-core score kernels (default 2^31 SM clocks).  Bit 0 of withhold_tile makes the
- * copy engine thread of the first CTA of the row-statistics sweep leave out its last K tile, so that the waits
- * for that tile run out, the kernel gives up in an orderly way (every role leaves its loop, the accumulator
+ * copy engine thread of the first CTA of the row-statistics sweep leave out its last K tile (in the kernel that
+ * forms the logits of fp32 inputs: keep it to itself), so that the waits for that tile run out, the kernel gives up in an orderly way (every role leaves its loop, the accumulator
  * memory is released, the status word gets bit 1) and returns.  Bit 1 keeps short contexts on the two-sweep
  * kernels instead of the single-sweep one (same scores within rounding).  Bit 2 is bit 0 for the window-attention
  * kernel of pyramidkv_attend_window.  (0, 0) restores normal operation.

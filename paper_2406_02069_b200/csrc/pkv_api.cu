@@ -420,6 +420,9 @@ int launch_scores_split(ScoreParams& sp, int batch, int max_n, int grid, cudaStr
   }
   sp.stat_grid = grid;
   sp.log2_group = std::log2(static_cast<float>(sp.group));
+  const long long test_wait = g_test_wait_clocks.load();
+  sp.wait_clocks = test_wait > 0 ? test_wait : kTcWaitCycles;
+  sp.withhold = g_test_withhold.load();
   launch_pdl(split_logits_kernel<D>, dim3(grid), kSpThreads, SpSmem<D>::kTotal, st, sp);
   mark(st, "logits_split");
   launch_pdl(split_scores_kernel, dim3((max_n - sp.seq.alpha + kSpSumKeys - 1) / kSpSumKeys, sp.num_kv_heads, batch), kSpSumThreads,

@@ -51,6 +51,8 @@ struct ScoreParams {
   int32_t chunk_tiles;                   // tiles per CTA (1 when there are several row blocks)
   float log2_group;
   int32_t per_unit;                      // pkv_score_split.cuh: CTAs per unit of one length, or 0
+  int32_t withhold;                      // ... test aid: CTA 0 never hands over its last K tile (its waits then run out)
+  long long wait_clocks;                 // ... bound of any one wait, in SM clocks
   uint32_t* status;
 };
 

@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const __gri
     for (int it = 0; it < min(ntiles, kSpPrefetch); ++it, tc_next<false>(off, p.seq.batch, units, ahead)) prefetch_tile(ahead);
   pdl_wait();
 
-  const long long limit = kTcWaitCycles;
+  const long long limit = p.wait_clocks;
   if (warp < 8) {
     // =========================================================== converters
     TcItem w = tc_item(off, p.seq.batch, units, item0);
@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(kSpThreads, 1) split_logits_kernel(const __gri
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
-      if (lane == 0) mbar_arrive(k_full(s));
+      if (lane == 0 && !(p.withhold && blockIdx.x == 0 && it + 1 == ntiles)) mbar_arrive(k_full(s));
     }
   } else if (warp == 16) {
     // =========================================================== MMA issuer
