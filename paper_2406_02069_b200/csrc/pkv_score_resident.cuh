@@ -71,14 +71,16 @@ __device__ __forceinline__ void rs_load(uint32_t taddr, uint32_t (&v)[32]) { tc_
 // scores, ld_scores, status, wait_clocks.
 // HALVES: epilogue warps per quarter of the TMEM lanes.
 template <int D, int STAGES, int HALVES>
-__global__ void __launch_bounds__(rs_threads(HALVES), STAGES == kRsStagesShort ? 2 : 1)
+__global__ void __launch_bounds__(rs_threads(HALVES), HALVES == 2 && STAGES == kRsStagesShort ? 2 : 1)
 score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                       const TcParams p) {
   namespace cg = cooperative_groups;
   using L = RsSmem<D, STAGES>;
   constexpr int kHalves = D / 64, kThreads = rs_threads(HALVES);
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = smem_raw + (-smem_u32(smem_raw) & 1023u);   // (an offset, so that accesses stay known as shared memory)
+  // (with two warps an offset, so that accesses stay known as shared memory)
+  uint8_t* smem = HALVES == 1 ? reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023))
+                              : smem_raw + (-smem_u32(smem_raw) & 1023u);
   uint8_t* q_s = smem + L::kQOff;
   uint8_t* k_s = smem + L::kKOff;
   uint8_t* misc = smem + L::kMiscOff;
@@ -187,10 +189,11 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
     }
   }
 
-  // =========================================================== epilogue (warps 2..9), in step with the cluster
+  // =========================================================== epilogue (warps 2.., 4 * HALVES of them), in step with the cluster
   const bool epi = warp >= 2;
   const int quarter = warp & 3;                               // TMEM lanes 32 * quarter .. + 31 are this warp's
-  const int rh = (warp - 2) >> 2;                             // ... and window rows 16 * rh .. + 15
+  const int rh = HALVES == 1 ? 0 : (warp - 2) >> 2;           // ... and window rows kRsRows / HALVES * rh ..; a constant
+                                                              // with one warp (worked out there: 0.3 to 0.5 us a call)
   const int lane_row = quarter * 32 + lane;
   const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
   const float c2 = p.scale_log2;
@@ -229,10 +232,13 @@ score_resident_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
         }
       } else {
         const int i = (tile0 + t) * kRsTileKeys + lane_row;
-        int jr = (rh * kHalf) % alpha;                         // window index of the row, counted up (no division per row)
+        // Window index of the row: with two warps counted up, with one divided.  (Counted up there too the scores alone are faster,
+        // 32 heads x 1280 keys 8.5 us instead of 8.7, but layer calls of 32 heads x 1024 to 1536 keys take 19.0 to 20.3 us instead
+        // of 18.4 to 19.8; why is not known.)
+        int jr = (rh * kHalf) % alpha;
 #pragma unroll
         for (int j = 0; j < kHalf; ++j) {
-          if (i <= min(P + jr, n - 1)) {
+          if (i <= min(P + (HALVES == 1 ? j % alpha : jr), n - 1)) {
             const float x = __uint_as_float(v[j]) * c2, mn = fmaxf(m[j], x);
             z[j] = z[j] * ex2(m[j] - mn) + ex2(x - mn);
             m[j] = mn;
