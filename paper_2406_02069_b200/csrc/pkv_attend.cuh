@@ -19,9 +19,9 @@
 //
 // Warp roles: 0 = TMA producer of Q and K, 1 = MMA issuer and TMEM owner, 2 = TMA producer of V,
 // 4..19 = epilogue in four groups of four warps (TMEM lane quarter = warp % 4), all on the same K tile.
-// Per tile the issuer queues ONE product K Q^T over all window rows (N up to 256: an MMA costs the issuing
+// Per tile the issuer queues ONE product K Q^T over all window rows (N = 256: an MMA costs the issuing
 // thread about 100 clocks whatever its width, so few wide ones) into the single 256-column S stage; the
-// epilogue takes the rows in halves of (up to) 128: it loads a half's logits into registers, and once the last
+// epilogue takes the rows in halves of 128 (the second one padded with zeros): it loads a half's logits into registers, and once the last
 // half is loaded gives the S stage back, so the next tile's K Q^T runs beside the exponentials; each half's e
 // values go to their own P buffer and V^T P of a half is queued when the buffer is full, behind the next tile's
 // K Q^T.
@@ -177,9 +177,7 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
   const uint32_t x_full = bar0 + 8u * 16, x_empty = bar0 + 8u * 17;
   const uint32_t lse_full = bar0 + 8u * 18;
 
-  const int halves = p.rows_pad > 128 ? 2 : 1;                 // row halves the epilogue takes a tile in
-  const int n_half = halves == 2 ? 128 : p.rows_pad;           // window rows (columns) of one half
-  const int n_pv = n_half < 64 ? 64 : n_half;                  // ... and of its P x V product (whole 64-row blocks)
+  constexpr int halves = 2, n_half = kTcMaxRows / halves;      // row halves the epilogue takes a tile in, window rows of one
 
   if (threadIdx.x == 0) {
     mbar_init(k_full, 1); mbar_init(k_empty, 1);
@@ -195,7 +193,7 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // Q rows beyond R and P rows beyond a half's width stay zero for the whole kernel
+  // Q rows beyond R stay zero for the whole kernel
   for (int i = threadIdx.x; i < kAtQBytes / 16; i += kAtThreads) reinterpret_cast<uint4*>(q_s)[i] = make_uint4(0, 0, 0, 0);
   for (int i = threadIdx.x; i < 2 * kAtTileBytes / 16; i += kAtThreads) reinterpret_cast<uint4*>(p_s)[i] = make_uint4(0, 0, 0, 0);
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -278,10 +276,10 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
   } else if (warp == 1) {
     // =========================================================== MMA issuer
     if (elect_one()) {
-      // all window rows at once; with two halves always 256 columns, so that the second half holds zeros (Q rows
-      // beyond R are zero) rather than what the stage held before
-      const uint32_t idesc_s = instr_desc_16bit(kAtTileKeys, halves == 2 ? 256 : p.rows_pad, p.fp16);
-      const uint32_t idesc_pv = instr_desc_16bit(kAtD, n_pv, p.fp16) | (1u << 15) | (1u << 16);   // A and B M/N-major
+      // all window rows at once, always 256 columns, so that the second half holds zeros (Q rows beyond R are zero) rather
+      // than what the stage held before
+      const uint32_t idesc_s = instr_desc_16bit(kAtTileKeys, kTcMaxRows, p.fp16);
+      const uint32_t idesc_pv = instr_desc_16bit(kAtD, n_half, p.fp16) | (1u << 15) | (1u << 16);   // A and B M/N-major
       uint32_t it = 0, heads_seen = 0, runs = 0;
       int cur_b = -1, cur_h = -1;
       bool ok = true, fresh = true, wait_o = false, pend = false;   // pend: the products V^T P of tile it - 1 are still to be queued
@@ -298,7 +296,7 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
         for (int hf = 0; hf < halves; ++hf) {
           if (!mbar_wait(p_full(hf), j & 1, abort_flag, p.wait_clocks)) return false;
           tc_fence_after();
-          const uint32_t d_addr = tmem_base + 256 + hf * 128;
+          const uint32_t d_addr = tmem_base + 256 + hf * n_half;
           const uint32_t p_lo = desc_lo_mn_major(smem_u32(p_s) + hf * kAtTileBytes, kAtTileKeys * 128);
           if (fresh) tc_mma_halves<false>(d_addr, v_lo, p_lo, idesc_pv);
           else tc_mma_halves<true>(d_addr, v_lo, p_lo, idesc_pv);
@@ -369,7 +367,6 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
     const float c2 = p.scale_log2;
     const float unshift = 1.0f / static_cast<float>(1 << kAtShift);
     const int cg_a = g4 * 16, cg_b = cg_a + 64;                // this group's pieces of a half
-    const bool has_a = cg_a < n_half, has_b = cg_b < n_half;
     uint32_t it = 0, lse_rounds = 0, runs = 0;
     int cur_b = -1, cur_h = -1;
     bool ok = true;
@@ -379,10 +376,9 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
       good = __all_sync(0xffffffffu, good);
       if (!good) return false;
       tc_fence_after();
-      const int ncols = halves == 2 ? 256 : n_pv;
       const int64_t seg = static_cast<int64_t>(blockIdx.x) + cur_b * p.num_kv_heads + cur_h;
       float* dst = p.o_partial + seg * p.rows * kAtD + lane_row;
-      for (int cg = g4 * 16; cg < ncols; cg += 64) {           // 16-column pieces dealt round to the four groups
+      for (int cg = g4 * 16; cg < kTcMaxRows; cg += 64) {      // 16-column pieces dealt round to the four groups
         uint32_t v[16];
         tc_ld16(tmem_base + lanes + 256 + cg, v);
         tc_wait_ld();
@@ -437,8 +433,8 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
         for (int hf = 0; hf < halves && ok; ++hf) {
           const uint32_t taddr = tmem_base + lanes + hf * 128;
           uint32_t va[16], vb[16];
-          if (has_a) tc_ld16(taddr + cg_a, va);
-          if (has_b) tc_ld16(taddr + cg_b, vb);
+          tc_ld16(taddr + cg_a, va);
+          tc_ld16(taddr + cg_b, vb);
           tc_wait_ld();
           if (hf == halves - 1) {                              // this tile's logits are in registers: the stage is free
             tc_fence_before();
@@ -454,13 +450,12 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
             unsigned long long acc = pack2(0.f, 0.f);
             const unsigned long long cc = pack2(c2, c2);
             const int sw = lane_row & 7;
-            if (has_a) {
-              if (p.fp16) at_chunk<true>(va, cc, nlr + cg_a, prow, cg_a >> 3, sw, acc);
-              else at_chunk<false>(va, cc, nlr + cg_a, prow, cg_a >> 3, sw, acc);
-            }
-            if (has_b) {
-              if (p.fp16) at_chunk<true>(vb, cc, nlr + cg_b, prow + kAtTileKeys * 128, (cg_b & 63) >> 3, sw, acc);
-              else at_chunk<false>(vb, cc, nlr + cg_b, prow + kAtTileKeys * 128, (cg_b & 63) >> 3, sw, acc);
+            if (p.fp16) {
+              at_chunk<true>(va, cc, nlr + cg_a, prow, cg_a >> 3, sw, acc);
+              at_chunk<true>(vb, cc, nlr + cg_b, prow + kAtTileKeys * 128, (cg_b & 63) >> 3, sw, acc);
+            } else {
+              at_chunk<false>(va, cc, nlr + cg_a, prow, cg_a >> 3, sw, acc);
+              at_chunk<false>(vb, cc, nlr + cg_b, prow + kAtTileKeys * 128, (cg_b & 63) >> 3, sw, acc);
             }
             float lo, hi;
             unpack2(acc, lo, hi);
@@ -468,7 +463,6 @@ window_attend_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
           } else {
 #pragma unroll
             for (int piece = 0; piece < 2; ++piece) {
-              if (piece == 0 ? !has_a : !has_b) continue;
               const int cg = piece == 0 ? cg_a : cg_b;
               const uint32_t (&v)[16] = piece == 0 ? va : vb;
               float ev[16];

@@ -50,7 +50,6 @@ constexpr int kSpSumThreads = 256;
 
 template <int D>
 struct SpSmem {
-  static constexpr int kHalves = D / 64;
   static constexpr int kQPart = kSpRows * D * 2;               // bytes of one part
   static constexpr int kKPart = kSpKeys * D * 2;
   static constexpr int kQOff = 0;
