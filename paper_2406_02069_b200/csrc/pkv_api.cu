@@ -141,7 +141,7 @@ struct Workspace {
   uint2* sel_cand;           // selection: candidate (key, position) pairs, [heads][sel_cand_stride]
   int64_t sel_cand_stride;
   uint32_t* sel_cnt;         // selection: pairs per cluster rank, [heads][kSelMaxCluster]
-  float* logits;             // fp32-pipe path: [heads][rows][ld_logits] logits between its two passes, or null
+  float* logits;             // scores that do not come from the 16-bit tensor-core kernels: logits between their two passes, or null
   int64_t ld_logits;
   size_t logit_bytes;        // what they take; 0: a path that never stores them
   float* o_partial;          // window attention: per-segment accumulators [kAtMaxGrid + heads][R][d], or null
@@ -377,9 +377,9 @@ int launch_logit_tiles(ScoreParams& sp, int batch, cudaStream_t st) {
 // From 33 window rows on; with up to 32 the fp32 pipe is faster (scores, fp32 pipe / split: 32 rows, 32 heads, 2000 keys,
 // d = 128 28.6 / 30.3 us; 32 rows, 8 heads, 1000 keys 14.0 / 17.9; 16 rows, 2 heads, 512 keys, d = 64 8.8 / 11.2; 64 rows, 2 heads, 8000
 // keys, d = 64 20.5 / 18.1; 64 rows, 8 heads, 4001 keys, d = 128 27.3 / 22.6; 384 rows, 8 heads, 3000 keys 121 / 40).
-constexpr int kSplitMinRows = 32;
+constexpr int kSplitAbove = 32;     // window rows up to which the fp32 pipe takes a call
 int split_grid(const ScoreParams& sp, int batch, int max_n, int sms) {
-  if (!sp.logits || sp.stats_only || sp.lse_in != sp.lse2 || sp.rows <= kSplitMinRows || sp.rows > 8192) return 0;
+  if (!sp.logits || sp.stats_only || sp.lse_in != sp.lse2 || sp.rows <= kSplitAbove || sp.rows > 8192) return 0;
   const long long blocks = (sp.rows + kSpRows - 1) / kSpRows, units = sp.num_kv_heads * blocks * batch;
   long long tiles = 0;
   for (int b = 0; b < batch; ++b) tiles += (sp.seq.n[b] + kSpKeys - 1) / kSpKeys;

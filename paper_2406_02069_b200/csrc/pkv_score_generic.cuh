@@ -44,9 +44,11 @@ struct ScoreParams {
   int64_t ld_scores;
   int32_t stats_only;                    // host side: stop after the row normalisers (no score sweep)
   int32_t stat_grid;                     // 0: partial is [tile][H_kv][rows] (fp32-pipe sweep).  > 0: CTAs of
-                                         // the tensor-core sweep, which writes [segment][rows] with segment =
-                                         // CTA + head for every run of a CTA over one head's chunks
-  float* logits;                         // fp32-pipe path: [batch][H_kv][rows][ld_logits] x values, or null
+                                         // a tensor-core sweep, which writes [segment][rows] with segment =
+                                         // CTA + head for every run of a CTA over one head's chunks (fp32 inputs:
+                                         // over the tiles of one unit, a head's block of 128 rows)
+  float* logits;                         // x values kept between two kernels, or null: [batch][H_kv][rows][ld_logits] (fp32
+                                         // pipe), [batch][H_kv][ld_logits][rows] (fp32 inputs on the tensor cores)
   int64_t ld_logits;
   int32_t chunk_tiles;                   // tiles per CTA (1 when there are several row blocks)
   float log2_group;

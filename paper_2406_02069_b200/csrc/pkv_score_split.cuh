@@ -4,8 +4,8 @@
 //
 //   q . k = sum (q_hi + q_mid + q_lo) (k_hi + k_mid + k_lo)  ~  hh + (hm + mh) + (hl + mm + lh)
 //
-// What is left out is below 2^-25 of a product of two magnitudes, a fraction of the rounding of one fp32 multiply-add.
-// The small products come first and each half of the channels has an accumulator of its own, so that a logit goes through
+// What is left out, (ml + lm) + ll, is at most about 2^-24 of a product of two magnitudes, as much as the rounding of one fp32
+// multiply-add (a middle part is up to 2^-8 of its value, a low part up to 2^-17).  The small products come first and each half of the channels has an accumulator of its own, so that a logit goes through
 // few roundings at full size (the accumulator of the tensor cores cuts off, it does not round).
 //
 //   split_logits_kernel     logits (key-major: the window rows of a key are consecutive) and row statistics, one segment
@@ -25,9 +25,10 @@
 // Tiles of 64 keys and not 128: two stages of parts fit beside Q's, and the tiles spread more evenly over the CTAs.
 //
 // Infinities, NaN and magnitudes of 2^59 or more raise a flag for their tile, whose logits are then formed by plain fp32
-// multiply-adds, once the CTA is through with the others (sp_plain_tiles).  Below that nothing overflows that the multiply-adds would not: the parts of 128 products add up to less
-// than 2^126 in magnitude.  (Parts have either sign: of products near 2^128 some would become infinities of opposite
-// signs, and NaN of a logit that is -inf.)  And parts that are subnormal and lost change no logit by more than 2^-59.
+// multiply-adds, once the CTA is through with the others (sp_plain_tiles).  Below that nothing overflows that the
+// multiply-adds would not: the parts of 128 products add up to less than 2^126 in magnitude.  (Parts have either sign: of
+// products near 2^128 some would become infinities of opposite signs, and NaN of a logit that is -inf.)  And parts that
+// are subnormal and lost change no logit by more than 2^-59.
 #pragma once
 
 #include "pkv_score_generic.cuh"

@@ -41,7 +41,8 @@ def _run(cfg, q, k, lens):
 
 
 # Logits (log2 units): sum |q k| is about 122 at d = 128, times log2(e) / sqrt(d) 16; a relative error of 2^-21 of that (24
-# accumulations that cut off at 2^-23 of a partial sum, far smaller ones before them) is 7.4e-6.  It enters a score through
+# accumulations that cut off at 2^-23 of a partial sum, far smaller ones before them, and 2^-24 of the magnitudes for the
+# products that are left out) is 7.4e-6.  It enters a score through
 # its own logits and the normalisers: 2 x 7.4e-6 ln 2 and a few 2^-22 of the exponentials and sums, below 2e-5.
 REL = 2e-5
 
@@ -58,7 +59,7 @@ def test_scores_are_those_of_64_bit_arithmetic(group, heads, window, d, lens):
         assert torch.all(got[b, h, P:] == -1.0)              # nothing is written behind the prefix
 
 
-# 2^80: split (the parts of the small operand end near 2^-100); 2^95: the large operand is beyond what is split
+# The large operand is beyond what is split (2^59); test_gpu_split_range.py has the powers around that
 @pytest.mark.parametrize("power", [80, -80, 95, -95])
 def test_operands_on_other_scales(power):
     lens = [300, 129]
